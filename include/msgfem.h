@@ -177,7 +177,7 @@ typedef struct {
   int refine;           /* MSGFEM_MIXED: most FP64 correction steps after each FP32 solve: for
                            K, preconditioned CG steps with the FP32 factor as preconditioner;
                            for A11, refinement steps.  A subdomain stops once its relative
-                           residual is below 1e-11 (CG) or 1e-13 (refinement, also when it
+                           residual is below 1e-11 (CG) or 1e-14 (refinement, also when it
                            stops falling); 0 = 10 */
   int instances;        /* batch of S >= 1 copies of the mesh and partition, each with its own
                            element angles (elem_angle_deg holds S consecutive fields);
@@ -255,7 +255,13 @@ enum { MSGFEM_METHOD_MSGFEM = 0, MSGFEM_METHOD_GENEO = 1 };
  * work of the last local stage.  Flop counts use the unpadded layer sizes n of
  * the nL node layers: factorisation of the block-tridiagonal matrix, per
  * matrix, sum_l n^3/3 [diagonal Cholesky] + (nL - 1) 2 n^3 [coupling block,
- * update of the next diagonal block]; one block solve (4 (nL - 1) + 2 nL) n^2 p. */
+ * update of the next diagonal block]; one block solve (4 (nL - 1) + 2 nL) n^2 p.
+ * The default path of the block Krylov solver keeps inverses of the Schur
+ * complements instead of block Cholesky factors: sum_l n^3 + 108 n^2, one block
+ * solve 2 (2 nL - 1) n^2 p.  A request for a Cholesky schedule (factor_schedule =
+ * 1), tile kernel (factor_kernel = 1), tile precision (tile_chol = 1), solve
+ * kernel (solve_kernel > 0) or subspace iteration (solver = 1), and layers too
+ * wide for its solve kernel, use the block Cholesky. */
 typedef struct {
   double assemble_ms;   /* element stiffness, stencils, layer blocks */
   double factor_ms;     /* layer-block Cholesky + inverses of K and A11 */
@@ -268,8 +274,9 @@ typedef struct {
   int solve_calls;      /* block solves in the last local stage */
   double solve_bytes;   /* per local stage, all solve calls: factor blocks read (the
                            inverse diagonal blocks as triangles, the coupling blocks whole,
-                           forward and backward) in the factor's precision, plus the FP64
-                           right-hand side read and solution written */
+                           forward and backward; the inverse form: its blocks whole, 2 nL - 1
+                           of them) in the factor's precision, plus the FP64 right-hand side
+                           read and solution written */
   double stencil_ms;    /* stencil products (K, B, K + sigma B) inside the iteration */
   double ortho_ms;      /* Gram, block updates, CholeskyQR, basis rotations */
   double stencil_flops; /* per local stage: 18 flop per (node, neighbour) pair and column, 24 for the

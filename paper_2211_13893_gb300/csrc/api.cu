@@ -326,12 +326,17 @@ msgfem_status allocate(msgfem* h) {
   TRY(dalloc(h, &h->d_ref, ndof));
   TRY(dalloc(h, &h->d_energy, 2 * 1024));
   TRY(dalloc(h, &h->d_l2, 4 * 1024));
-  // schedules
-  build_factor_schedule(h);
-  build_solve_schedules(h);
-  for (WaveSched& w : h->waves) {
-    TRY(upload_wave_factor(h, w));
-    TRY(upload_wave_solves(h, w));
+  // schedules: of the inverse form, or of the block Cholesky
+  h->inv_on = inv_create(h);
+  if (h->inv_on) {
+    TRY(inv_build(h));
+  } else {
+    build_factor_schedule(h);
+    build_solve_schedules(h);
+    for (WaveSched& w : h->waves) {
+      TRY(upload_wave_factor(h, w));
+      TRY(upload_wave_solves(h, w));
+    }
   }
   TRY(dalloc(h, &h->d_mk, h->N));
   TRY(dalloc(h, &h->d_nwk, h->N));
@@ -442,6 +447,7 @@ MSGFEM_TIMED_ORTHO(rotate, (msgfem* h, int which, int wy, int ncols), (h, which,
 // block); with_inverse adds the n^3 / 3 per layer of the explicit inverses of
 // the diagonal factors that this build forms for its solves
 double factor_flops(const msgfem* h, bool with_inverse = false) {
+  if (h->inv_on) return inv_factor_flops(h, false);
   double f = 0.0;
   for (const auto& s : h->sub)
     for (int n : {s.nK, s.nA}) {
@@ -476,7 +482,7 @@ double solve_flops(const msgfem* h, int mat, int p) {
     if (!active(h, j)) continue;
     const SubDev& s = h->sub[j];
     const double n = mat == 0 ? s.nK : s.nA;
-    f += (4.0 * (s.nzn - 1) + 2.0 * s.nzn) * n * n * p;
+    f += (h->inv_on ? 2.0 * (2.0 * s.nzn - 1) : 4.0 * (s.nzn - 1) + 2.0 * s.nzn) * n * n * p;
   }
   return f;
 }
@@ -491,7 +497,8 @@ double solve_bytes(const msgfem* h, int mat, int p) {
     if (!active(h, j)) continue;
     const SubDev& s = h->sub[j];
     const double n = mat == 0 ? s.nK : s.nA;
-    b += 2.0 * (s.nzn * n * (n + 1) / 2.0 + (s.nzn - 1) * n * n) * es + 2.0 * s.nzn * n * p * 8.0;
+    if (h->inv_on) b += (2.0 * s.nzn - 1) * n * n * es + 2.0 * s.nzn * n * p * 8.0;
+    else b += 2.0 * (s.nzn * n * (n + 1) / 2.0 + (s.nzn - 1) * n * n) * es + 2.0 * s.nzn * n * p * 8.0;
   }
   return b;
 }
@@ -529,6 +536,14 @@ void run_graph(msgfem* h, uint64_t key, Issue issue) {
 // handle's precision; add = 1 accumulates into the destination.
 void timed_solve_w(msgfem* h, int mat, int src, int dst, int neg, int width, int add) {
   const int sp = span_begin(h, TAG_SOLVE);
+  if (h->inv_on) {
+    inv_solve(h, mat, src, dst, neg, width, add);
+    span_end(h, sp);
+    h->prof.solve_flops += solve_flops(h, mat, width == KB ? KB : h->p);
+    h->prof.solve_bytes += solve_bytes(h, mat, width == KB ? KB : h->p);
+    h->prof.solve_calls += 1;
+    return;
+  }
   const uint64_t key = ((uint64_t)1 << 60) | ((uint64_t)h->cur << 48) | ((uint64_t)mat << 40) |
                        ((uint64_t)width << 32) | ((uint64_t)src << 16) | ((uint64_t)dst << 4) | ((uint64_t)neg << 1) |
                        (uint64_t)add;
@@ -670,6 +685,10 @@ static uint64_t factor_graph_key(const msgfem* h, int w) {
 // The layer-block factorisation of wave w: one persistent launch (mixed
 // precision, when chosen) or the captured step schedule.
 static msgfem_status run_factorisation(msgfem* h, const WaveSched& ws, int w) {
+  if (h->inv_on) {
+    run_graph(h, ((uint64_t)2 << 60) | ((uint64_t)w << 48) | ((uint64_t)1 << 45), [&](cudaStream_t cs) { inv_factor(h, w, cs); });
+    return MSGFEM_OK;
+  }
   if (h->mixed && h->factor_persistent) return run_factor_persistent(h, ws, h->stream);
   run_graph(h, factor_graph_key(h, w), [&](cudaStream_t cs) {
     if (h->mixed) run_schedule(ws.factf, cs, &h->gs);
@@ -702,8 +721,7 @@ msgfem_status schwarz_factors(msgfem* h) {
   const WaveSched& ws = h->waves[0];
   std::vector<int> notspd(h->N + 1);
   for (int attempt = 0; attempt < 2; ++attempt) {
-    if (h->mixed) launch_layer_blocks_f32(h);
-    else launch_layer_blocks(h);
+    launch_layer_blocks(h);
     TRY(select_factor_kernel(h));
     TRY(run_factorisation(h, ws, 0));
     CK_LAUNCH();
@@ -1205,6 +1223,7 @@ static msgfem_status local_spaces_run(msgfem_h h, const std::vector<int>& nl, do
   h->prof.factor_flops = factor_flops(h);
   h->prof.factor_flops_inverse = factor_flops(h, true);
   h->prof.factor_flops_executed = 0.0;
+  if (h->inv_on) h->prof.factor_flops_executed = inv_factor_flops(h, true);
   for (const auto& w : h->waves) h->prof.factor_flops_executed += h->mixed ? schedule_flops(w.factf) : schedule_flops(w.fact);
   h->prof.solve_flops = 0.0;
   h->prof.solve_bytes = 0.0;
@@ -1239,8 +1258,7 @@ static msgfem_status local_spaces_run(msgfem_h h, const std::vector<int>& nl, do
     for (int j : ws.members) h->base_act[j] = 1;
     TRY(set_active(h, h->base_act));
     sp = span_begin(h, TAG_ASSEMBLE);
-    if (h->mixed) launch_layer_blocks_f32(h);
-    else launch_layer_blocks(h);
+    launch_layer_blocks(h);
     span_end(h, sp);
     CK_LAUNCH();
     // 2. factorisations of K and A11
@@ -1268,7 +1286,7 @@ static msgfem_status local_spaces_run(msgfem_h h, const std::vector<int>& nl, do
         h->potrf_fp64 = 1;
         CK(cudaMemcpyAsync(h->d_notspd, bad.data(), (h->N + 1) * sizeof(int), cudaMemcpyHostToDevice, st));
         sp = span_begin(h, TAG_ASSEMBLE);
-        launch_layer_blocks_f32(h);
+        launch_layer_blocks(h);
         span_end(h, sp);
         TRY(select_factor_kernel(h));
         sp = span_begin(h, TAG_FACTOR);
@@ -1709,6 +1727,7 @@ static msgfem_status autotune_run(msgfem_h h, int reps, msgfem_tuning* out) {
   if (h->stage < 2) return MSGFEM_ESTATE;
   if (reps <= 0) reps = 3;
   h->factored_wave = -1;   // the timed factorisations leave scratch in the pool
+  h->inv_on = false;       // the block Cholesky's candidates first, then the inverse form against the best
   cudaStream_t st = h->stream;
   CK(cudaStreamSynchronize(st));
   // the task lists are re-uploaded below: drop every captured factorisation and
@@ -1743,8 +1762,7 @@ static msgfem_status autotune_run(msgfem_h h, int reps, msgfem_tuning* out) {
   h->factor_persistent = 0;
   const int fgroups[2] = {16, 32};
   auto factor_once = [&](float* ms) -> msgfem_status {
-    if (h->mixed) launch_layer_blocks_f32(h);
-    else launch_layer_blocks(h);
+    launch_layer_blocks(h);
     CK(cudaEventRecord(f0, st));
     if (h->mixed && h->factor_persistent) TRY(run_factor_persistent(h, wl, st));
     else if (h->mixed) run_schedule(wl.factf, st, &h->gs);
@@ -1856,8 +1874,6 @@ static msgfem_status autotune_run(msgfem_h h, int reps, msgfem_tuning* out) {
     }
     h->factor_persistent = 0;
   }
-  CK(cudaEventDestroy(f0));
-  CK(cudaEventDestroy(f1));
   h->factor_left = best_f;
   h->ngroup_factor = best_fg;
   h->factor_tc = best_k;
@@ -1926,6 +1942,31 @@ static msgfem_status autotune_run(msgfem_h h, int reps, msgfem_tuning* out) {
   }
   drop_graphs();
   h->solve_variant = saved_variant;
+  if (h->inv != nullptr) {
+    // the inverse form: one factorisation and the same operator applications; kept
+    // when a local stage of ten block steps is faster with it
+    h->inv_on = true;
+    float fms = 0.f, oms = 0.f;
+    for (int r = 0; r < 2; ++r) {
+      launch_layer_blocks(h);
+      CK(cudaEventRecord(f0, st));
+      TRY(run_factorisation(h, wl, last));
+      CK(cudaEventRecord(f1, st));
+    }
+    for (int r = 0; r <= reps; ++r) {
+      if (r == 1) CK(cudaEventRecord(e0, st));
+      launch_random_kb(h, MV_WB, h->opt.seed + 7919ull * (r + 1));
+      apply_M_kb(h);
+    }
+    CK(cudaEventRecord(e1, st));
+    CK(cudaEventSynchronize(e1));
+    CK_LAUNCH();
+    CK(cudaEventElapsedTime(&fms, f0, f1));
+    CK(cudaEventElapsedTime(&oms, e0, e1));
+    h->inv_on = fms + 10.0 * oms / reps <= best_fms + 10.0 * best;
+  }
+  CK(cudaEventDestroy(f0));
+  CK(cudaEventDestroy(f1));
   CK(cudaStreamSynchronize(st));
   for (auto& sp : h->spans) {   // the timing's phase spans are dropped
     h->ev_pool.push_back(sp.a);
@@ -2009,6 +2050,7 @@ void msgfem_destroy(msgfem_h h) {
     if (kv.second.first) cudaGraphExecDestroy(kv.second.first);
   if (h->cap) cudaStreamDestroy(h->cap);
   for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
+  inv_destroy(h);
   delete h;
 }
 

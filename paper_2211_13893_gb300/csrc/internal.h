@@ -161,6 +161,8 @@ struct WaveSched {
 // persistent kernel: a list schedule on `workers` resident CTAs (setup.cpp)
 void build_persistent_meta(const ScheduleT<float>& s, std::vector<int4>& meta, int& pcount, int workers);
 
+struct InvForm;   // inverse form of the layer-block solver (k_inv.cu)
+
 struct CoarsePair { int s, t, x0, x1, y0, y1; };   // (i, j) node box of Omega_s cap Omega*_t
 
 // Host copies of the per-subdomain set-up arrays (uploaded once).
@@ -249,6 +251,8 @@ struct msgfem {
   void* d_solve_maps = nullptr;      // the same arrays in 64 x 64 unswizzled boxes (TMA solve stages)
   int* d_kerr = nullptr;             // set by a TMA solve stage that did not arrive in time
   int potrf_fp64 = 0;                // mixed: FP64 tile Cholesky after an FP32 one met a bad pivot
+  InvForm* inv = nullptr;            // inverse form, when the handle is eligible
+  bool inv_on = false;               // factorisations and solves run in the inverse form
   int factor_persistent = 0;         // mixed: FP32 factorisation as one persistent launch
   int refine = 2;                    // FP64 refinement steps per FP32 solve
   std::vector<CoarsePair> pairs;
@@ -366,6 +370,14 @@ template <typename T>
 void run_solve_mv(const SolveScheduleT<T>& s, cudaStream_t st, int src, int dst, int gather_neg, int width = PST,
                   const StreamSet* gs = nullptr, int scatter_add = 0, int variant = SOLVE_DEFAULT);
 void launch_element_stiffness(msgfem* h);
+// inverse form (k_inv.cu): eligibility and geometry, task lists, factorisation of
+// wave w, solves of `width` columns with K (mat 0) or A11 (mat 1), flop counts
+bool inv_create(msgfem* h);
+void inv_destroy(msgfem* h);
+msgfem_status inv_build(msgfem* h);
+void inv_factor(msgfem* h, int w, cudaStream_t st);
+void inv_solve(msgfem* h, int mat, int src, int dst, int neg, int width, int add);
+double inv_factor_flops(const msgfem* h, bool executed);
 // Structured numbering of a hexahedron list (hexmesh.cpp): the (i, j, k) block
 // dimensions and, for every node and element of the list, its structured id.
 struct HexNumbering {
@@ -394,8 +406,8 @@ std::vector<double> global_load(const msgfem* h);
 // node coordinates of node (i, j, k): given, or those of the box (setup.cpp)
 void node_xyz(const msgfem* h, int i, int j, int k, double X[3]);
 void launch_stencil(msgfem* h);
+// layer blocks of the active subdomains in the handle's precision (couplings only for the block Cholesky)
 void launch_layer_blocks(msgfem* h);
-void launch_layer_blocks_f32(msgfem* h);
 void launch_stencil_apply(msgfem* h, int src, int dst, int mode, double alpha);
 void launch_gram(msgfem* h, int wx, int wy, int wg);
 void launch_small_eig(msgfem* h, int p);
@@ -427,9 +439,12 @@ void launch_refine_check(msgfem* h, int wr, int wref, int keep, int step);
 constexpr int KEEP_K = (1 << 1) | (1 << 2);   // rows of K: B1 and B2
 constexpr int KEEP_A11 = 1 << 1;               // rows of A11: B1
 #ifndef MSGFEM_REFINE_TOL
-#define MSGFEM_REFINE_TOL 1e-13
+#define MSGFEM_REFINE_TOL 1e-14
 #endif
-constexpr double REFINE_TOL = MSGFEM_REFINE_TOL;   // relative residual at which refinement stops
+// relative residual at which refinement stops.  The eigen-residual of small clamped
+// subdomains amplifies what is left of the harmonic residual by up to 1e9: with the
+// inverse form a stop at 1e-13 left 6e-5 on one (t2), at 1e-14 4e-6
+constexpr double REFINE_TOL = MSGFEM_REFINE_TOL;
 // relative residual at which the conjugate-gradient K solves of the mixed path stop
 // (the eigensolver's own tolerance is 1e-7 in the energy norm)
 constexpr double PCG_TOL = 1e-11;

@@ -227,17 +227,17 @@ template <> struct Blocks<float> {
 };
 
 // Scatter the stencil into the layer blocks of K (mat 0) and A11 (mat 1).
-// Thread per (node, slot); slots with dk = 0 go to D_k, dk = -1 to E_{k-1}.
+// Thread per (node, slot); slots with dk = 0 go to D_k, dk = -1 to E_{k-1} (with_E).
 template <typename T>
 __global__ void __launch_bounds__(216)
-k_layer_blocks(const SubDev* __restrict__ subs, const int* __restrict__ active) {
+k_layer_blocks(const SubDev* __restrict__ subs, const int* __restrict__ active, int with_E) {
   if (!active[blockIdx.y]) return;
   const SubDev s = subs[blockIdx.y];
   const int tid = threadIdx.x;
   const int node = blockIdx.x * 8 + tid / 27, slot = tid % 27;
   if (node >= s.nnode) return;
   const int dk = slot % 3 - 1;
-  if (dk == 1) return;
+  if (dk == 1 || (dk == -1 && !with_E)) return;
   const int k = node / s.npl, q = node % s.npl;
   if (dk == -1 && k == 0) return;
   const int di = slot / 9 - 1, dj = (slot / 3) % 3 - 1;
@@ -301,21 +301,24 @@ void launch_stencil(msgfem* h) {
 // Layer blocks of the subdomains of the current wave (the active ones).
 template <typename T>
 static void layer_blocks_t(msgfem* h) {
+  const bool with_E = !h->inv_on;   // the inverse form applies the couplings from the stencil
   for (int j = 0; j < h->N; ++j) {
     if (j < (int)h->act_host.size() && !h->act_host[j]) continue;
     const SubDev& s = h->sub[j];
     T* DK = std::is_same<T, float>::value ? (T*)s.DKf : (T*)s.DK;
     T* DA = std::is_same<T, float>::value ? (T*)s.DAf : (T*)s.DA;
-    cudaMemsetAsync(DK, 0, sizeof(T) * (size_t)s.bK * s.bK * (2 * s.nzn - 1), h->stream);
-    cudaMemsetAsync(DA, 0, sizeof(T) * (size_t)s.bA * s.bA * (2 * s.nzn - 1), h->stream);
+    cudaMemsetAsync(DK, 0, sizeof(T) * (size_t)s.bK * s.bK * (with_E ? 2 * s.nzn - 1 : s.nzn), h->stream);
+    cudaMemsetAsync(DA, 0, sizeof(T) * (size_t)s.bA * s.bA * (with_E ? 2 * s.nzn - 1 : s.nzn), h->stream);
   }
   int maxn = 0, maxz = 0;
   for (const auto& s : h->sub) { maxn = std::max(maxn, s.nnode); maxz = std::max(maxz, s.nzn); }
   dim3 grid((maxn + 7) / 8, h->N);
-  k_layer_blocks<T><<<grid, 216, 0, h->stream>>>(h->d_sub, h->d_flags); ++g_launch_count;
+  k_layer_blocks<T><<<grid, 216, 0, h->stream>>>(h->d_sub, h->d_flags, with_E ? 1 : 0); ++g_launch_count;
   dim3 g2(maxz, h->N);
   k_block_identity<T><<<g2, 128, 0, h->stream>>>(h->d_sub, h->d_flags); ++g_launch_count;
 }
 
-void launch_layer_blocks(msgfem* h) { layer_blocks_t<double>(h); }
-void launch_layer_blocks_f32(msgfem* h) { layer_blocks_t<float>(h); }
+void launch_layer_blocks(msgfem* h) {
+  if (h->mixed) layer_blocks_t<float>(h);
+  else layer_blocks_t<double>(h);
+}

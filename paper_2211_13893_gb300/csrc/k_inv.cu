@@ -1,0 +1,1041 @@
+// Inverse form of the layer-block solver (the default of the block Krylov path).
+//
+// K and A11 are block tridiagonal over the node layers, with dense diagonal
+// blocks D_l and couplings C_l = A[layer l, layer l - 1] that hold 27 non-zeros
+// per row (the node stencil).  Instead of the block Cholesky factors L_l and
+// E_l = C_l L_{l-1}^{-T} (dense) this form keeps only the inverses of the Schur
+// complements,
+//   S_l = D_l - C_l S_{l-1}^{-1} C_l^T,
+// and applies the couplings from the stencil:
+//   forward   z_l = b_l - C_l u_{l-1},  u_l = S_l^{-1} z_l
+//   backward  x_l = u_l - S_l^{-1} C_{l+1}^T x_{l+1}.
+// Per layer of n DoFs the factorisation takes n^3 flops (one SPD inverse) plus
+// 54 n^2 fused multiply-adds for the sparse triple product, against 8/3 n^3
+// for the block Cholesky with its block inverses, and a solve reads 2 n^2
+// numbers against 3 n^2.
+//
+// The layers are eliminated from both ends towards the middle layer
+// (two half chains per matrix, the middle Schur complement takes both): the
+// same work in half as many dependent steps.
+//
+// The inverse of a Schur complement is the symmetric sweep operator (block
+// Gauss-Jordan) over its T x T tiles of 64: for k = 0 .. T - 1
+//   P = S_kk^{-1};  W_i = S_ik P;  S_ij -= W_i S_jk^T (i, j != k);
+//   S_ik = W_i, S_ki = W_i^T, S_kk = -P,
+// which leaves -S^{-1} (kept with that sign).  Every sweep touches the whole
+// matrix, so the tasks of a step stay numerous to the end.  Measured on the CPU
+// in the same arithmetic it is as accurate as the block Cholesky with explicit
+// block inverses in FP64, and a better FP32 preconditioner (c2's interior K:
+// 4 CG steps to 1e-11 where the Cholesky form takes 5 to 6).
+//
+// Measured on one GB300 against the block Cholesky (factorisation / all solves of a
+// local stage, ms): 36 x 12 x 39 beam FP64 345 -> 103 / 424 -> 158; 192 x 12 x 39 beam
+// mixed 102 -> 71 / 374 -> 200; C-section of 16 subdomains mixed 85 -> 45 / 409 -> 172;
+// 47 x 7 x 13 beam FP64 whole pass 156 -> 83.
+#include "internal.h"
+
+#include <cooperative_groups.h>
+#include <cstring>
+#include <type_traits>
+
+#include "tc_gemm.cuh"
+
+namespace cg = cooperative_groups;
+
+// One matrix (K or A11) of one subdomain.  The kept DoFs of a layer are all
+// three components of a nic x njc box of in-plane nodes.
+struct InvMat {
+  int sub, mat;
+  int ia, ja, nic, njc;        // kept node box
+  int n, b, nL, mid;           // kept / padded layer size, layers, middle layer
+  int npl, nyn;
+  int pinned;                  // K of a floating subdomain: rows pin[] of layer 0 are out
+  int pin[6];                  // compact rows in layer 0
+  const double* stencil;
+  void* D;                     // [nL][b][b] S_l, then -S_l^{-1}
+  void* E;                     // [nL - 1][b][b] scratch of the triple products
+  void* L;                     // [nL][b][b]: sweep scratch, then the packed couplings
+  void* yc;                    // [nL][b][KB] u of the forward sweep
+};
+
+namespace {
+
+enum { IV_SCHUR_A = 0, IV_SCHUR_B, IV_PIVOT, IV_PANEL, IV_UPDATE };
+struct InvTask {
+  int type, m, layer, k, i, j;
+};
+
+constexpr int NBLK = 8;   // nodes per coupling task
+
+// scratch of the sweep of layer l: the old tile column k and the pivot inverse
+template <typename T>
+__device__ __forceinline__ T* old_col(const InvMat& m, int l) { return static_cast<T*>(m.L) + (size_t)l * m.b * m.b; }
+template <typename T>
+__device__ __forceinline__ T* pivot_inv(const InvMat& m, int l) {
+  return static_cast<T*>(m.L) + (size_t)l * m.b * m.b + (m.b > TILE ? (size_t)m.b * TILE : 0);
+}
+template <typename T>
+__device__ __forceinline__ T* layer_block(const InvMat& m, int l) { return static_cast<T*>(m.D) + (size_t)l * m.b * m.b; }
+// scratch of the triple product that couples layer l to layer l + dk
+template <typename T>
+__device__ __forceinline__ T* triple_scratch(const InvMat& m, int l, int dk) {
+  return static_cast<T*>(m.E) + (size_t)(dk < 0 ? l - 1 : l) * m.b * m.b;
+}
+
+__device__ __forceinline__ bool pinned_row(const InvMat& m, int layer, int row) {
+  if (!m.pinned || layer != 0) return false;
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+    if (m.pin[i] == row) return true;
+  return false;
+}
+
+// Entry (r, c) of the coupling block of kept node p in layer l with neighbour
+// slot s9 (0 .. 8, in-plane) in layer l + dk; zero outside the kept box and at pins.
+__device__ __forceinline__ double coupling(const InvMat& m, int l, int p, int dk, int s9, int r, int c) {
+  const int i = p / m.njc, j = p % m.njc, di = s9 / 3 - 1, dj = s9 % 3 - 1;
+  if (i + di < 0 || i + di >= m.nic || j + dj < 0 || j + dj >= m.njc) return 0.0;
+  if (m.pinned && (pinned_row(m, l, 3 * p + r) || pinned_row(m, l + dk, 3 * (p + di * m.njc + dj) + c))) return 0.0;
+  const size_t node = (size_t)l * m.npl + (size_t)(m.ia + i) * m.nyn + m.ja + j;
+  return m.stencil[node * 243 + (size_t)((di + 1) * 9 + (dj + 1) * 3 + dk + 1) * 9 + r * 3 + c];
+}
+
+// Rows of 8 kept nodes times a row-major matrix X: three outputs per node and
+// column, 27 products each; columns along the lanes (coalesced), the
+// coefficients broadcast from shared memory.  The FP64 form is bound by the
+// FP64 pipe, the FP32 form by the shared-memory broadcasts.
+template <typename T>
+__device__ __forceinline__ void couple_rows(const InvMat& m, int nb, int dk, int layer, int q, const T* X, T* coef,
+                                            T (&acc)[2][3]) {
+  const int tid = threadIdx.x, nn = m.n / 3;
+  for (int e = tid; e < NBLK * 81; e += 256) {
+    const int p = nb * NBLK + e / 81, s9 = (e % 81) / 9, rc = e % 9;
+    coef[e] = p < nn ? (T)coupling(m, layer, p, dk, s9, rc / 3, rc % 3) : (T)0;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int pl = (tid >> 6) * 2 + u, p = nb * NBLK + pl;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) acc[u][r] = (T)0;
+    if (p >= nn || q >= m.n) continue;
+    const int i = p / m.njc, j = p % m.njc;
+#pragma unroll
+    for (int s9 = 0; s9 < 9; ++s9) {
+      const int di = s9 / 3 - 1, dj = s9 % 3 - 1;
+      if (i + di < 0 || i + di >= m.nic || j + dj < 0 || j + dj >= m.njc) continue;
+      const T* x = X + (size_t)(3 * (p + di * m.njc + dj)) * m.b + q;
+      const T x0 = x[0], x1 = x[m.b], x2 = x[2 * (size_t)m.b];
+      const T* c = coef + pl * 81 + s9 * 9;
+#pragma unroll
+      for (int r = 0; r < 3; ++r) acc[u][r] = fma(c[3 * r], x0, fma(c[3 * r + 1], x1, fma(c[3 * r + 2], x2, acc[u][r])));
+    }
+  }
+}
+
+// Inverse of a 64 x 64 SPD tile by the scalar sweep operator in FP64 registers:
+// a 16 x 16 thread grid, each thread the entries (ty + 16 p, tx + 16 q) with
+// p >= q (the tile is symmetric), one barrier per pivot (the pivot column and
+// the pivot's reciprocal are published in a double buffer).  It runs in the same
+// launch as the updates of the other tiles (the next pivot tile is swept by the
+// CTA that updated it), so only narrow steps wait for it.
+template <typename T>
+__device__ void tile_sweep(const T* X, int ldx, T* P, int* notspd, int sub) {
+  __shared__ double v[2][TILE];
+  __shared__ double rinv[2];
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  double a[4][4];
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int q = 0; q <= p; ++q) a[p][q] = (double)X[(ty + 16 * p) * ldx + tx + 16 * q];
+  bool bad = false;
+#pragma unroll
+  for (int kb = 0; kb < 4; ++kb) {
+#pragma unroll 1
+    for (int kr = 0; kr < 16; ++kr) {
+      double* vs = v[kr & 1];
+      if (tx == kr) {
+#pragma unroll
+        for (int p = kb; p < 4; ++p) vs[ty + 16 * p] = a[p][kb];
+        if (ty == kr) {
+          double d = a[kb][kb];
+          if (!(d > 0.0)) { bad = true; d = 1e-300; }
+          rinv[kr & 1] = 1.0 / d;
+        }
+      }
+      if (ty == kr) {
+#pragma unroll
+        for (int q = 0; q < kb; ++q) vs[tx + 16 * q] = a[kb][q];
+      }
+      __syncthreads();
+      const double r = rinv[kr & 1];
+      double vj[4], wi[4];
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        vj[p] = vs[tx + 16 * p];
+        wi[p] = vs[ty + 16 * p] * r;
+      }
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q <= p; ++q) a[p][q] = fma(-wi[p], vj[q], a[p][q]);
+      if (tx == kr) {
+#pragma unroll
+        for (int p = kb; p < 4; ++p) a[p][kb] = wi[p];
+      }
+      if (ty == kr) {
+#pragma unroll
+        for (int q = 0; q <= kb; ++q) a[kb][q] = vj[q] * r;
+        if (tx == kr) a[kb][kb] = -r;
+      }
+    }
+  }
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int q = 0; q <= p; ++q) {
+      const T w = (T)(-a[p][q]);
+      P[(ty + 16 * p) * TILE + tx + 16 * q] = w;
+      if (q < p) P[(tx + 16 * q) * TILE + ty + 16 * p] = w;
+    }
+  if (bad) atomicExch(&notspd[sub], 1);
+}
+
+// shared-memory row stride of a staged operand tile ([k][row])
+template <typename T> struct TileLd;
+template <> struct TileLd<double> { static constexpr int v = 65; };
+template <> struct TileLd<float> { static constexpr int v = 68; };
+template <typename T>
+constexpr int inv_step_smem() { return 2 * TILE * TileLd<T>::v * (int)sizeof(T); }
+
+// rows of a 64 x 64 tile (leading dimension ld) into shared memory as [k][row]
+template <typename T>
+__device__ __forceinline__ void stage_tile(const T* G, int ld, T* S) {
+  using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+  constexpr int N = 16 / sizeof(T), LD = TileLd<T>::v;
+  const int r = threadIdx.x & 63, k0 = (threadIdx.x >> 6) * 16;
+  V x[16 / N];
+#pragma unroll
+  for (int c = 0; c < 16 / N; ++c) x[c] = *reinterpret_cast<const V*>(G + (size_t)r * ld + k0 + c * N);
+#pragma unroll
+  for (int c = 0; c < 16 / N; ++c) {
+    const T* e = reinterpret_cast<const T*>(&x[c]);
+#pragma unroll
+    for (int q = 0; q < N; ++q) S[(k0 + c * N + q) * LD + r] = e[q];
+  }
+}
+
+// output row / column of element (p, q) of thread (ty, tx): FP64 strided by 16
+// (a diagonal tile forms only its 16 x 16 blocks on or below the diagonal),
+// FP32 four contiguous ones (vector loads)
+template <typename T> __device__ __forceinline__ int out_idx(int t, int p) {
+  return sizeof(T) == 8 ? t + 16 * p : 4 * t + p;
+}
+
+// acc = A B^T of two staged 64 x 64 tiles
+template <typename T, bool SYM>
+__device__ __forceinline__ void tile_product(const T* As, const T* Bs, T (&acc)[4][4]) {
+  constexpr int LD = TileLd<T>::v;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[p][q] = (T)0;
+#pragma unroll 16
+  for (int k = 0; k < TILE; ++k) {
+    T a[4], b[4];
+    if constexpr (sizeof(T) == 4) {
+      const float4 av = *reinterpret_cast<const float4*>(As + k * LD + 4 * ty);
+      const float4 bv = *reinterpret_cast<const float4*>(Bs + k * LD + 4 * tx);
+      a[0] = av.x; a[1] = av.y; a[2] = av.z; a[3] = av.w;
+      b[0] = bv.x; b[1] = bv.y; b[2] = bv.z; b[3] = bv.w;
+    } else {
+#pragma unroll
+      for (int p = 0; p < 4; ++p) { a[p] = As[k * LD + ty + 16 * p]; b[p] = Bs[k * LD + tx + 16 * p]; }
+    }
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (!SYM || q <= p) acc[p][q] = fma(a[p], b[q], acc[p][q]);
+  }
+}
+
+// One step of the factorisation: independent tasks, one CTA each.
+template <typename T>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
+k_inv_step(const InvTask* __restrict__ tasks, const InvMat* __restrict__ mats, const int* __restrict__ active,
+           int* __restrict__ notspd) {
+  const InvTask t = tasks[blockIdx.x];
+  const InvMat& m = mats[t.m];
+  if (active != nullptr && !active[m.sub]) return;
+  extern __shared__ __align__(16) unsigned char smem_iv[];
+  T* As = reinterpret_cast<T*>(smem_iv);
+  T* Bs = As + TILE * TileLd<T>::v;
+  constexpr int LD = TileLd<T>::v;
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, b = m.b;
+  T* S = layer_block<T>(m, t.layer);
+  if (t.type == IV_SCHUR_A) {
+    // (C X)^T with X = -S^{-1} of layer layer + k: rows q, columns of layer `layer`
+    T acc[2][3];
+    const int q = t.j * TILE + (tid & 63);
+    couple_rows<T>(m, t.i, t.k, t.layer, q, layer_block<T>(m, t.layer + t.k), As, acc);
+    T* W = triple_scratch<T>(m, t.layer, t.k);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int p = t.i * NBLK + (tid >> 6) * 2 + u;
+      if (p < m.n / 3 && q < m.n)
+#pragma unroll
+        for (int r = 0; r < 3; ++r) W[(size_t)q * b + 3 * p + r] = acc[u][r];
+    }
+    return;
+  }
+  if (t.type == IV_SCHUR_B) {
+    // D += C (C X)^T on and below the diagonal, mirrored
+    T acc[2][3];
+    const int q = t.j * TILE + (tid & 63);
+    couple_rows<T>(m, t.i, t.k, t.layer, q, triple_scratch<T>(m, t.layer, t.k), As, acc);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int p = t.i * NBLK + (tid >> 6) * 2 + u;
+      if (p < m.n / 3 && q < m.n)
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          const int row = 3 * p + r;
+          if (q > row) continue;
+          const T v = S[(size_t)row * b + q] + acc[u][r];
+          S[(size_t)row * b + q] = v;
+          if (q < row) S[(size_t)q * b + row] = v;
+        }
+    }
+    return;
+  }
+  if (t.type == IV_PIVOT) {
+    tile_sweep<T>(S, b, pivot_inv<T>(m, t.layer), notspd, m.sub);
+    return;
+  }
+  const int k = t.k;
+  T* P = pivot_inv<T>(m, t.layer);
+  T* C = old_col<T>(m, t.layer);
+  if (t.type == IV_PANEL) {
+    T* Skk = S + (size_t)k * TILE * b + (size_t)k * TILE;
+    if (t.i == k) {
+      for (int e = tid; e < TILE * TILE; e += 256) Skk[(size_t)(e >> 6) * b + (e & 63)] = -P[e];
+      return;
+    }
+    T* Sik = S + (size_t)t.i * TILE * b + (size_t)k * TILE;
+    T* Ski = S + (size_t)k * TILE * b + (size_t)t.i * TILE;
+    stage_tile<T>(Sik, b, As);
+    stage_tile<T>(P, TILE, Bs);
+    __syncthreads();
+    T acc[4][4];
+    tile_product<T, false>(As, Bs, acc);
+    T* Ci = C + (size_t)t.i * TILE * TILE;
+    for (int e = tid; e < TILE * TILE; e += 256) Ci[e] = As[(e & 63) * LD + (e >> 6)];   // the old tile
+    __syncthreads();
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) As[out_idx<T>(ty, p) * LD + out_idx<T>(tx, q)] = acc[p][q];
+    __syncthreads();
+    for (int e = tid; e < TILE * TILE; e += 256) {
+      const int r = e >> 6, c = e & 63;
+      Sik[(size_t)r * b + c] = As[r * LD + c];
+      Ski[(size_t)r * b + c] = As[c * LD + r];
+    }
+    return;
+  }
+  // IV_UPDATE: S_ij -= W_i old_j^T, mirrored; the next pivot tile is swept at once
+  T* Sij = S + (size_t)t.i * TILE * b + (size_t)t.j * TILE;
+  stage_tile<T>(S + (size_t)t.i * TILE * b + (size_t)k * TILE, b, As);
+  stage_tile<T>(C + (size_t)t.j * TILE * TILE, TILE, Bs);
+  __syncthreads();
+  T acc[4][4];
+  const bool diag = t.i == t.j;
+  if (sizeof(T) == 8 && diag) tile_product<T, sizeof(T) == 8>(As, Bs, acc);
+  else tile_product<T, false>(As, Bs, acc);
+  __syncthreads();
+#pragma unroll
+  for (int p = 0; p < 4; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = out_idx<T>(ty, p), c = out_idx<T>(tx, q);
+      if (diag && c > r) continue;
+      const T v = Sij[(size_t)r * b + c] - acc[p][q];
+      As[r * LD + c] = v;
+      if (diag) As[c * LD + r] = v;
+    }
+  __syncthreads();
+  T* Sji = S + (size_t)t.j * TILE * b + (size_t)t.i * TILE;
+  for (int e = tid; e < TILE * TILE; e += 256) {
+    const int r = e >> 6, c = e & 63;
+    Sij[(size_t)r * b + c] = As[r * LD + c];
+    if (!diag) Sji[(size_t)r * b + c] = As[c * LD + r];
+  }
+  if (diag && t.i == k + 1) tile_sweep<T>(As, LD, P, notspd, m.sub);
+}
+
+// Couplings of every layer in the solver's precision, packed per node for the
+// solves: [layer][2: towards layer - 1, layer + 1][node][9 neighbours][3][3],
+// node counts padded to a multiple of 4 (every rank's share is then a copy on a
+// 16-byte boundary; 2 x 81 padded nodes fit in the b x b slot of a layer).
+__host__ __device__ __forceinline__ int up4(int v) { return (v + 3) & ~3; }
+template <typename T>
+__global__ void k_inv_pack(const InvMat* __restrict__ mats, const int* __restrict__ active) {
+  const InvMat& m = mats[blockIdx.y];
+  if (active != nullptr && !active[m.sub]) return;
+  const int nn = m.n / 3, np = up4(nn);
+  for (int l = blockIdx.x; l < m.nL; l += gridDim.x) {
+    T* out = static_cast<T*>(m.L) + (size_t)l * m.b * m.b;
+    for (int e = threadIdx.x; e < 2 * np * 81; e += blockDim.x) {
+      const int dir = e / (np * 81), p = (e / 81) % np, s = e % 81, dk = dir ? 1 : -1;
+      double v = 0.0;
+      if (p < nn && l + dk >= 0 && l + dk < m.nL) v = coupling(m, l, p, dk, s / 9, (s % 9) / 3, s % 3);
+      out[e] = (T)v;
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Solve of KB right-hand sides.  One thread-block cluster of G CTAs per half
+// chain: rank g holds a contiguous share of the layer's rows (in stages of RS
+// rows) and of its nodes.  Per layer: (1) the sparse step on the own nodes, z to
+// every rank's shared memory; cluster barrier; (2) the own rows of S^{-1} z,
+// results to the ranks whose nodes neighbour them; cluster barrier.  The rows of
+// S^{-1} are contiguous in memory and depend on nothing, so they stream through
+// a ring of bulk copies (cp.async.bulk, one per stage) that runs ahead across
+// the layers: the ring is full again when the barriers are passed.  FP32 is
+// bound by HBM (many subdomains) or by the barriers (few), FP64 by the FP64 pipe.
+struct InvSolveArgs {
+  const InvMat* mats;
+  const int* list;          // matrices (largest first)
+  const SubDev* subs;
+  const int* active;
+  int src, dst, stride, coloff, neg, add;
+  int ring, smem_z, smem_u, smem_c, smem_r;   // stages, byte offsets of the shared arrays
+  int* err;
+};
+
+template <typename T>
+__device__ __forceinline__ int zpos(int row, int col) {
+  // rows in chunks of one 16-byte vector, each chunk padded by 16 bytes (bank
+  // groups of the eight lanes of a 128-bit phase differ)
+  constexpr int VN = 16 / sizeof(T);
+  return (row / VN) * (VN * (KB + 1)) + (row % VN) * KB + col;
+}
+
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src),
+      "r"(bytes), "r"(bar)
+      : "memory");
+}
+
+template <typename T, int RS, bool BACK>
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1)
+k_inv_solve(const InvSolveArgs a) {
+  constexpr int VN = 16 / sizeof(T);
+  constexpr int KS = 8 / (RS / 4);            // warps that share a row group (4 rows), splitting k
+  using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+  cg::cluster_group cl = cg::this_cluster();
+  const int G = (int)cl.num_blocks(), g = (int)cl.block_rank();
+  const int task = blockIdx.x / G, half = task & 1;
+  const InvMat m = a.mats[a.list[task >> 1]];
+  if (a.active != nullptr && !a.active[m.sub]) return;   // uniform over the cluster
+  // layers of this half chain, in order: forward from the end, backward from the middle
+  const int nch = half ? m.nL - 1 - m.mid : m.mid;        // layers without the middle one
+  const int steps = BACK ? nch + 1 : nch;
+  if (!BACK && nch == 0) return;
+  if (BACK && half && nch == 0) return;
+  auto layer_of = [&](int t) {
+    if (BACK) return half ? m.mid + t : m.mid - t;
+    return half ? m.nL - 1 - t : t;
+  };
+  extern __shared__ __align__(128) unsigned char smem_sv[];
+  T* ring = reinterpret_cast<T*>(smem_sv);
+  T* zb = reinterpret_cast<T*>(smem_sv + a.smem_z);
+  T* uw = reinterpret_cast<T*>(smem_sv + a.smem_u);
+  T* cf = reinterpret_cast<T*>(smem_sv + a.smem_c);
+  T* red = reinterpret_cast<T*>(smem_sv + a.smem_r);      // [2][KS][RS][KB]
+  __shared__ __align__(8) unsigned long long bars[9];     // ring slots, couplings
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int b = m.b, nn = m.n / 3;
+  const int NS = (m.n + RS - 1) / RS, s0 = NS * g / G, s1 = NS * (g + 1) / G, ns = s1 - s0;
+  const int npc = up4((nn + G - 1) / G), p0 = min(nn, npc * g), p1 = min(nn, p0 + npc);
+  const int wlo = max(0, p0 - m.njc - 1);                 // first node of the window of neighbour values
+  const uint32_t ring_s = tc::saddr(ring), bar0 = tc::saddr(bars), cf_s = tc::saddr(cf);
+  const uint32_t stage_bytes = (uint32_t)(RS * b * sizeof(T));
+  const int total = ns * steps;
+  bool ok = true;
+  int issued = 0;   // stages requested (thread 0)
+  auto issue = [&](int i) {
+    issued = i + 1;
+    const int l = layer_of(i / ns), s = s0 + i % ns;
+    const uint32_t bar = bar0 + 8 * (i % a.ring);
+    tc::mbar_expect_tx(bar, stage_bytes);
+    bulk_load(ring_s + (uint32_t)(i % a.ring) * stage_bytes, static_cast<const T*>(m.D) + ((size_t)l * b + (size_t)s * RS) * b,
+              stage_bytes, bar);
+  };
+  // couplings of the own nodes in the layer of step t: towards the previous
+  // layer of the chain (forward) or towards the middle (backward)
+  const int cdir = BACK ? (half ? 0 : 1) : (half ? 1 : 0);
+  const uint32_t cbytes = p1 > p0 ? (uint32_t)(up4(p1 - p0) * 81 * sizeof(T)) : 0;
+  auto coupling_ptr = [&](int l, int dir) {
+    return static_cast<const T*>(m.L) + (size_t)l * b * b + ((size_t)dir * up4(nn) + p0) * 81;
+  };
+  if (tid == 0) {
+    for (int i = 0; i < 9; ++i) tc::mbar_init(bar0 + 8 * i, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    for (int i = 0; i < a.ring && i < total; ++i) issue(i);
+  }
+  for (int e = tid; e < ((b + VN - 1) / VN) * VN * (KB + 1); e += 256) zb[e] = (T)0;
+  __syncthreads();
+  const SubDev& sd = a.subs[m.sub];
+  const double* src = mv_ptr(sd, a.src) + a.coloff;
+  double* dst = mv_ptr(sd, a.dst) + a.coloff;
+  T* yc = static_cast<T*>(m.yc);
+  const T sgn = a.neg ? (T)-1 : (T)1;
+  int cphase = 0, ci = 0;   // coupling copies waited for; stages consumed
+  int waited = 0;           // stages whose copies have arrived
+  bool cpend = false;
+  cl.sync();   // no remote store before every CTA of the cluster has cleared its arrays
+  for (int t = 0; t < steps; ++t) {
+    const int l = layer_of(t);
+    // ---- sparse step on the own nodes
+    const bool first = t == 0;
+    if (cpend) {
+      if (ok) ok = tc::mbar_wait(bar0 + 64, cphase & 1);
+      ++cphase;
+    }
+    for (int e = tid; e < (p1 - p0) * KB; e += 256) {
+      const int pl = e / KB, col = e % KB, p = p0 + pl;
+      const int i = p / m.njc, j = p % m.njc;
+      T z[3] = {(T)0, (T)0, (T)0};
+      if (!BACK || first) {
+        const size_t node = (size_t)l * m.npl + (size_t)(m.ia + i) * m.nyn + m.ja + j;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) z[r] = sgn * (T)src[(node * 3 + r) * a.stride + col];
+        if (m.pinned && l == 0)
+#pragma unroll
+          for (int r = 0; r < 3; ++r)
+            if (pinned_row(m, 0, 3 * p + r)) z[r] = (T)0;
+      }
+      auto sub_coupling = [&](const T* c, const T* u) {   // z -= C u, u indexed by row * KB
+        T acc[3] = {(T)0, (T)0, (T)0};
+#pragma unroll
+        for (int s9 = 0; s9 < 9; ++s9) {
+          const int di = s9 / 3 - 1, dj = s9 % 3 - 1;
+          if (i + di < 0 || i + di >= m.nic || j + dj < 0 || j + dj >= m.njc) continue;
+          const T* x = u + (ptrdiff_t)(3 * (p + di * m.njc + dj)) * KB + col;
+          const T x0 = x[0], x1 = x[KB], x2 = x[2 * KB];
+#pragma unroll
+          for (int r = 0; r < 3; ++r)
+            acc[r] = fma(c[s9 * 9 + 3 * r], x0, fma(c[s9 * 9 + 3 * r + 1], x1, fma(c[s9 * 9 + 3 * r + 2], x2, acc[r])));
+        }
+#pragma unroll
+        for (int r = 0; r < 3; ++r) z[r] -= acc[r];
+      };
+      if (BACK && first) {
+        // middle layer: both half chains' u from memory
+        if (m.mid > 0) sub_coupling(coupling_ptr(l, 0) + (size_t)pl * 81, yc + (size_t)(l - 1) * b * KB);
+        if (m.mid + 1 < m.nL) sub_coupling(coupling_ptr(l, 1) + (size_t)pl * 81, yc + (size_t)(l + 1) * b * KB);
+      } else if (!first) {
+        sub_coupling(cf + (size_t)pl * 81, uw - (ptrdiff_t)wlo * 3 * KB);
+      }
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        const int pos = zpos<T>(3 * p + r, col);
+        for (int q = 0; q < G; ++q) cl.map_shared_rank(zb, q)[pos] = z[r];
+      }
+    }
+    cl.sync();
+    // the coupling buffer is free: request the next layer's
+    cpend = t + 1 < steps && cbytes > 0;
+    if (cpend && ok && tid == 0) {
+      tc::fence_async_smem();
+      tc::mbar_expect_tx(bar0 + 64, cbytes);
+      bulk_load(cf_s, coupling_ptr(layer_of(t + 1), cdir), cbytes, bar0 + 64);
+    }
+    // ---- dense step on the own rows
+    const int nchunk = (m.n + VN - 1) / VN;
+    for (int s = s0; s < s1; ++s, ++ci) {
+      const int slot = ci % a.ring;
+      if (ok) {
+        ok = tc::mbar_wait(bar0 + 8 * slot, (ci / a.ring) & 1);
+        if (ok) waited = ci + 1;
+      }
+      const T* st = ring + (size_t)slot * RS * b;
+      const int rg = w / KS, ks = w % KS;
+      T acc[32];
+#pragma unroll
+      for (int e = 0; e < 32; ++e) acc[e] = (T)0;
+      const T* a0 = st + (size_t)rg * 4 * b;
+#pragma unroll 1
+      for (int c = ks * 32 + lane; c < nchunk; c += 32 * KS) {
+        T av[4][VN];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const V x = *reinterpret_cast<const V*>(a0 + (size_t)r * b + c * VN);
+          const T* e = reinterpret_cast<const T*>(&x);
+#pragma unroll
+          for (int q = 0; q < VN; ++q) av[r][q] = e[q];
+        }
+        const T* zp = zb + (size_t)c * VN * (KB + 1);
+#pragma unroll
+        for (int q = 0; q < VN; ++q) {
+          T zv[KB];
+#pragma unroll
+          for (int h = 0; h < KB / VN; ++h) {
+            const V x = *reinterpret_cast<const V*>(zp + q * KB + h * VN);
+            const T* e = reinterpret_cast<const T*>(&x);
+#pragma unroll
+            for (int o = 0; o < VN; ++o) zv[h * VN + o] = e[o];
+          }
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int o = 0; o < KB; ++o) acc[r * KB + o] = fma(av[r][q], zv[o], acc[r * KB + o]);
+        }
+      }
+      // lane L ends with the sum of entry L (row L / KB, column L % KB)
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int e = 0; e < off; ++e) {
+          const T send = up ? acc[e] : acc[e + off];
+          const T keep = up ? acc[e + off] : acc[e];
+          acc[e] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+      }
+      T* rd = red + (size_t)(ci & 1) * KS * RS * KB;
+      rd[((size_t)ks * RS + rg * 4) * KB + lane] = acc[0];
+      __syncthreads();
+      if (tid == 0 && ok && ci + a.ring < total) {
+        tc::fence_async_smem();
+        issue(ci + a.ring);
+      }
+      for (int e = tid; e < RS * KB; e += 256) {
+        const int row = s * RS + e / KB, col = e % KB;
+        if (row >= m.n) continue;
+        T y = rd[e];
+#pragma unroll
+        for (int q = 1; q < KS; ++q) y += rd[q * RS * KB + e];
+        T* yp = yc + ((size_t)l * b + row) * KB + col;
+        T x;   // the block holds -S^{-1}
+        if (BACK && !first) x = *yp + (-y);
+        else x = -y;
+        if (!BACK) *yp = x;
+        else if (!first || half == 0) {
+          const int p = row / 3;
+          const size_t node = (size_t)l * m.npl + (size_t)(m.ia + p / m.njc) * m.nyn + m.ja + p % m.njc;
+          double* o = dst + (node * 3 + row % 3) * a.stride + col;
+          *o = a.add ? *o + (double)x : (double)x;
+        }
+        if (t + 1 < steps) {
+          const int p = row / 3;
+          for (int q = 0; q < G; ++q) {
+            const int q0 = min(nn, npc * q), lo = max(0, q0 - m.njc - 1), hi = min(nn, min(nn, q0 + npc) + m.njc + 1);
+            if (p >= lo && p < hi) cl.map_shared_rank(uw, q)[(size_t)(row - 3 * lo) * KB + col] = x;
+          }
+        }
+      }
+    }
+    cl.sync();
+  }
+  if (!__syncthreads_and(ok) && tid == 0) {
+    // a copy did not arrive within its limit: wait once more for those in flight, then report
+    for (int i = waited; i < issued; ++i) tc::mbar_wait(bar0 + 8 * (i % a.ring), (i / a.ring) & 1);
+    if (cphase > 0) tc::mbar_wait(bar0 + 64, (cphase - 1) & 1);
+    if (a.err != nullptr) atomicExch(a.err, 1);
+  }
+}
+
+}  // namespace
+
+// ---------------------------------------------------------------------------
+// host side
+
+struct InvForm {
+  std::vector<InvMat> mats;        // K and A11 of every subdomain (A11 may have no DoFs: not listed)
+  InvMat* d_mats = nullptr;
+  struct Solve {
+    std::vector<int> list;         // matrices of one kind in a wave, largest first
+    int* d_list = nullptr;
+    int G = 1, ring = 2, smem_z = 0, smem_u = 0, smem_c = 0, smem_r = 0, smem = 0;
+  };
+  struct Wave {
+    std::vector<std::vector<SchedStep>> steps;   // per stream group
+    InvTask* d_tasks = nullptr;
+    std::vector<int> all;          // every matrix of the wave (packing)
+    Solve solve[2];
+  };
+  std::vector<Wave> waves;
+  int rs = 8;                      // rows per stage of the solves (by the widest layer and the type)
+};
+
+namespace {
+
+constexpr int INV_SMEM = 225 * 1024;   // shared memory of one solve CTA
+
+template <typename T>
+const void* solve_kernel_ptr(int rs, bool back) {
+  if (rs == 16) return back ? (const void*)k_inv_solve<T, 16, true> : (const void*)k_inv_solve<T, 16, false>;
+  if (rs == 8) return back ? (const void*)k_inv_solve<T, 8, true> : (const void*)k_inv_solve<T, 8, false>;
+  return back ? (const void*)k_inv_solve<T, 4, true> : (const void*)k_inv_solve<T, 4, false>;
+}
+const void* solve_kernel(const msgfem* h, int rs, bool back) {
+  return h->mixed ? solve_kernel_ptr<float>(rs, back) : solve_kernel_ptr<double>(rs, back);
+}
+
+// shared-memory layout of a solve over the listed matrices with G CTAs per
+// cluster and `ring` stages; the total in bytes
+int solve_layout(const msgfem* h, const InvForm& f, InvForm::Solve& s, int G, int ring) {
+  const int es = h->mixed ? 4 : 8, vn = 16 / es;
+  auto up = [](size_t v) { return (v + 127) / 128 * 128; };
+  size_t st = 0, z = 0, u = 0, c = 0;
+  for (int i : s.list) {
+    const InvMat& m = f.mats[i];
+    const int nn = m.n / 3, npc = up4((nn + G - 1) / G);
+    st = std::max(st, (size_t)f.rs * m.b * es);
+    z = std::max(z, (size_t)((m.b + vn - 1) / vn) * vn * (KB + 1) * es);
+    u = std::max(u, (size_t)std::min(nn, npc + 2 * (m.njc + 1)) * 3 * KB * es);
+    c = std::max(c, (size_t)npc * 81 * es);
+  }
+  s.G = G;
+  s.ring = ring;
+  s.smem_z = (int)up(st * ring);
+  s.smem_u = (int)(s.smem_z + up(z));
+  s.smem_c = (int)(s.smem_u + up(u));
+  s.smem_r = (int)(s.smem_c + up(c));
+  s.smem = (int)(s.smem_r + up((size_t)2 * (8 / (f.rs / 4)) * f.rs * KB * es));
+  return s.smem;
+}
+
+int resident_clusters(const void* kernel, int G, int smem) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(G);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = G;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
+// Cluster size and ring depth of a solve: the largest cluster with which every
+// half chain is resident at once (they run side by side), with the deepest ring
+// that one CTA per SM holds, or half an SM's shared memory when that makes more
+// half chains resident; with more half chains than SMs one CTA each.
+void choose_solve(const msgfem* h, const InvForm& f, InvForm::Solve& s) {
+  const int chains = 2 * (int)s.list.size();
+  int most = 1;
+  for (int i : s.list) most = std::max(most, (f.mats[i].n + f.rs - 1) / f.rs / 2);
+  auto fit = [&](int G, int limit) {
+    int ring = 8;
+    while (ring > 2 && solve_layout(h, f, s, G, ring) > limit) --ring;
+    return solve_layout(h, f, s, G, ring) <= limit;
+  };
+  for (int G : {8, 4, 2, 1}) {
+    if (G > 1 && G > most) continue;
+    for (int limit : {INV_SMEM, 110 * 1024}) {
+      if (!fit(G, limit)) continue;
+      if (resident_clusters(solve_kernel(h, f.rs, true), G, s.smem) >= chains) return;
+    }
+  }
+  if (fit(1, 110 * 1024)) return;
+  for (int G : {1, 2, 4, 8})
+    if (fit(G, INV_SMEM)) return;
+}
+
+}  // namespace
+
+// Eligibility and geometry.  The inverse form serves the block Krylov solver
+// with the default kernels; a request for a particular Cholesky schedule, tile
+// kernel, tile precision or solve kernel keeps the block Cholesky, and so do
+// layers whose solve stages do not fit in shared memory.
+bool inv_create(msgfem* h) {
+  const msgfem_options& o = h->opt;
+  if (o.solver != 0 || o.solve_kernel != 0 || o.factor_schedule != 0 || o.factor_kernel != 0 || o.tile_chol != 0)
+    return false;
+  InvForm* f = new InvForm();
+  const int es = h->mixed ? 4 : 8;
+  int bmax = TILE;
+  bool good = true;
+  for (int j = 0; j < h->N && good; ++j) {
+    const SubDev& s = h->sub[j];
+    const HostSub& hs = h->hsub[j];
+    for (int mat = 0; mat < 2 && good; ++mat) {
+      InvMat m;
+      memset(&m, 0, sizeof(m));
+      m.sub = j;
+      m.mat = mat;
+      m.n = mat == 0 ? s.nK : s.nA;
+      m.b = mat == 0 ? s.bK : s.bA;
+      m.nL = s.nzn;
+      m.mid = s.nzn / 2;
+      m.npl = s.npl;
+      m.nyn = s.nyn;
+      m.stencil = s.stencil;
+      m.D = h->mixed ? (void*)(mat == 0 ? s.DKf : s.DAf) : (void*)(mat == 0 ? s.DK : s.DA);
+      m.E = h->mixed ? (void*)(mat == 0 ? s.EKf : s.EAf) : (void*)(mat == 0 ? s.EK : s.EA);
+      m.L = h->mixed ? (void*)(mat == 0 ? s.LKf : s.LAf) : (void*)(mat == 0 ? s.LK : s.LA);
+      m.yc = h->mixed ? (void*)(mat == 0 ? s.ycK8f : s.ycA8f) : (void*)(mat == 0 ? s.ycK8 : s.ycA8);
+      // the kept nodes must be a box, numbered like the compact rows
+      const std::vector<int>& map = mat == 0 ? hs.mapK : hs.mapA;
+      if (m.n > 0) {
+        const int q0 = map[0] / 3, q1 = map[m.n - 1] / 3;
+        m.ia = q0 / s.nyn;
+        m.ja = q0 % s.nyn;
+        m.nic = q1 / s.nyn - m.ia + 1;
+        m.njc = q1 % s.nyn - m.ja + 1;
+        good = m.nic > 0 && m.njc > 0 && 3 * m.nic * m.njc == m.n;
+        for (int r = 0; r < m.n && good; ++r) {
+          const int p = r / 3;
+          good = map[r] == 3 * ((m.ia + p / m.njc) * s.nyn + m.ja + p % m.njc) + r % 3;
+        }
+      }
+      if (mat == 0 && s.floating) {
+        m.pinned = 1;
+        for (int i = 0; i < 6; ++i) {
+          m.pin[i] = -1;
+          if (s.pin[i] < 0) continue;
+          good = good && s.pin[i] < 3 * s.npl;   // the pins sit in layer 0
+          if (good) m.pin[i] = hs.invK[s.pin[i]];
+        }
+      }
+      bmax = std::max(bmax, m.b);
+      f->mats.push_back(m);
+    }
+  }
+  const int row = bmax * es;
+  f->rs = row <= 3072 ? 16 : row <= 6144 ? 8 : 4;
+  // two stages of the widest layer and its vectors must fit with the widest cluster
+  InvForm::Solve probe;
+  for (int i = 0; i < (int)f->mats.size(); ++i)
+    if (f->mats[i].n > 0) probe.list.push_back(i);
+  good = good && solve_layout(h, *f, probe, 8, 2) <= INV_SMEM;
+  if (!good) {
+    delete f;
+    return false;
+  }
+  h->inv = f;
+  return true;
+}
+
+void inv_destroy(msgfem* h) {
+  delete h->inv;
+  h->inv = nullptr;
+}
+
+// Task lists of every wave (after the waves' storage has been placed).
+msgfem_status inv_build(msgfem* h) {
+  InvForm& f = *h->inv;
+  static bool attr = false;
+  if (!attr) {
+    for (int rs : {4, 8, 16})
+      for (bool back : {false, true}) {
+        CK(cudaFuncSetAttribute(solve_kernel_ptr<float>(rs, back), cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
+        CK(cudaFuncSetAttribute(solve_kernel_ptr<double>(rs, back), cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
+      }
+    CK(cudaFuncSetAttribute(k_inv_step<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, inv_step_smem<double>()));
+    CK(cudaFuncSetAttribute(k_inv_step<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, inv_step_smem<float>()));
+    attr = true;
+  }
+  void* p = nullptr;
+  TRY(dev_alloc_bytes(h, &p, f.mats.size() * sizeof(InvMat)));
+  f.d_mats = static_cast<InvMat*>(p);
+  CK(cudaMemcpy(f.d_mats, f.mats.data(), f.mats.size() * sizeof(InvMat), cudaMemcpyHostToDevice));
+  TRY(kerr_ensure(h));
+  f.waves.resize(h->waves.size());
+  for (size_t w = 0; w < h->waves.size(); ++w) {
+    InvForm::Wave& wv = f.waves[w];
+    for (int j : h->waves[w].members)
+      for (int mat = 0; mat < 2; ++mat)
+        if (f.mats[2 * j + mat].n > 0) {
+          wv.all.push_back(2 * j + mat);
+          wv.solve[mat].list.push_back(2 * j + mat);
+        }
+    int Tmax = 1;
+    for (int i : wv.all) Tmax = std::max(Tmax, f.mats[i].b / TILE);
+    const long long per = 2LL * Tmax + 6;
+    const int ng = std::max(1, std::min(h->ngroup_factor, (int)wv.all.size()));
+    std::vector<std::map<long long, std::vector<InvTask>>> keys(ng);
+    for (size_t c = 0; c < wv.all.size(); ++c) {
+      auto& fk = keys[c % ng];
+      const int mi = wv.all[c];
+      const InvMat& m = f.mats[mi];
+      const int T = m.b / TILE, nbk = (m.n / 3 + NBLK - 1) / NBLK;
+      auto schur = [&](long long key, int l, int dk) {
+        for (int i = 0; i < nbk; ++i)
+          for (int j = 0; j * TILE < m.n; ++j) fk[key].push_back({IV_SCHUR_A, mi, l, dk, i, j});
+      };
+      auto schur_add = [&](long long key, int l, int dk) {
+        for (int i = 0; i < nbk; ++i)
+          for (int j = 0; j * TILE <= 3 * (i * NBLK + NBLK - 1) + 2 && j * TILE < m.n; ++j)
+            fk[key].push_back({IV_SCHUR_B, mi, l, dk, i, j});
+      };
+      auto sweep = [&](long long key, int l) {
+        fk[key].push_back({IV_PIVOT, mi, l, 0, 0, 0});
+        for (int k = 0; k < T; ++k) {
+          for (int i = 0; i < T; ++i) fk[key + 1 + 2 * k].push_back({IV_PANEL, mi, l, k, i, 0});
+          auto& up = fk[key + 2 + 2 * k];
+          if (k + 1 < T) up.push_back({IV_UPDATE, mi, l, k, k + 1, k + 1});   // swept next: first
+          for (int i = 0; i < T; ++i)
+            for (int j = 0; j <= i; ++j)
+              if (i != k && j != k && !(i == k + 1 && j == k + 1)) up.push_back({IV_UPDATE, mi, l, k, i, j});
+        }
+      };
+      int tmid = 0;
+      for (int half = 0; half < 2; ++half) {
+        const int nch = half ? m.nL - 1 - m.mid : m.mid;
+        tmid = std::max(tmid, nch);
+        for (int t = 0; t < nch; ++t) {
+          const int l = half ? m.nL - 1 - t : t, dk = half ? 1 : -1;
+          if (t > 0) {
+            schur(t * per, l, dk);
+            schur_add(t * per + 1, l, dk);
+          }
+          sweep(t * per + 3, l);
+        }
+      }
+      for (int dk : {-1, 1}) {
+        if (m.mid + dk < 0 || m.mid + dk >= m.nL) continue;
+        schur(tmid * per, m.mid, dk);
+        schur_add(tmid * per + (dk < 0 ? 1 : 2), m.mid, dk);
+      }
+      sweep(tmid * per + 3, m.mid);
+    }
+    std::vector<InvTask> tasks;
+    wv.steps.assign(ng, {});
+    for (int g = 0; g < ng; ++g)
+      for (auto& kv : keys[g]) {
+        if (kv.second.empty()) continue;
+        // tasks that sweep a pivot tile first: they are the longest
+        std::stable_partition(kv.second.begin(), kv.second.end(), [](const InvTask& t) {
+          return t.type == IV_PIVOT || (t.type == IV_UPDATE && t.i == t.j && t.i == t.k + 1);
+        });
+        wv.steps[g].push_back({(int)tasks.size(), (int)kv.second.size()});
+        tasks.insert(tasks.end(), kv.second.begin(), kv.second.end());
+      }
+    TRY(dev_alloc_bytes(h, &p, std::max<size_t>(tasks.size(), 1) * sizeof(InvTask)));
+    wv.d_tasks = static_cast<InvTask*>(p);
+    CK(cudaMemcpy(wv.d_tasks, tasks.data(), tasks.size() * sizeof(InvTask), cudaMemcpyHostToDevice));
+    for (InvForm::Solve& s : wv.solve) {
+      if (s.list.empty()) continue;
+      std::stable_sort(s.list.begin(), s.list.end(), [&](int x, int y) {
+        return (double)f.mats[x].n * f.mats[x].n * f.mats[x].nL > (double)f.mats[y].n * f.mats[y].n * f.mats[y].nL;
+      });
+      choose_solve(h, f, s);
+      TRY(dev_alloc_bytes(h, &p, s.list.size() * sizeof(int)));
+      s.d_list = static_cast<int*>(p);
+      CK(cudaMemcpy(s.d_list, s.list.data(), s.list.size() * sizeof(int), cudaMemcpyHostToDevice));
+    }
+    // the packing kernel reads the wave's matrices by list
+  }
+  return MSGFEM_OK;
+}
+
+// Launches of the factorisation of wave w on st (stream groups of h->gs).
+template <typename T>
+static void inv_factor_t(msgfem* h, int w, cudaStream_t st) {
+  const InvForm& f = *h->inv;
+  const InvForm::Wave& wv = f.waves[w];
+  const int ng = (int)wv.steps.size();
+  const bool multi = ng > 1;
+  if (multi) {
+    cudaEventRecord(h->gs.fork, st);
+    for (int g = 0; g < ng; ++g) cudaStreamWaitEvent(h->gs.s[g], h->gs.fork, 0);
+  }
+  size_t maxlen = 0;
+  for (const auto& v : wv.steps) maxlen = std::max(maxlen, v.size());
+  for (size_t k = 0; k < maxlen; ++k)
+    for (int g = 0; g < ng; ++g) {
+      if (k >= wv.steps[g].size()) continue;
+      const SchedStep& s = wv.steps[g][k];
+      k_inv_step<T><<<s.count, 256, inv_step_smem<T>(), multi ? h->gs.s[g] : st>>>(wv.d_tasks + s.first, f.d_mats,
+                                                                                h->d_flags, h->d_notspd);
+      ++g_launch_count;
+    }
+  if (multi)
+    for (int g = 0; g < ng; ++g) {
+      cudaEventRecord(h->gs.join[g], h->gs.s[g]);
+      cudaStreamWaitEvent(st, h->gs.join[g], 0);
+    }
+  // packed couplings, over the sweep's scratch; inactive subdomains (other waves) are skipped
+  int maxl = 1;
+  for (int i : wv.all) maxl = std::max(maxl, f.mats[i].nL);
+  k_inv_pack<T><<<dim3(maxl, (int)f.mats.size()), 256, 0, st>>>(f.d_mats, h->d_flags);
+  ++g_launch_count;
+}
+
+void inv_factor(msgfem* h, int w, cudaStream_t st) {
+  if (h->mixed) inv_factor_t<float>(h, w, st);
+  else inv_factor_t<double>(h, w, st);
+}
+
+// X = M^{-1} B for K (mat 0) or A11 (mat 1) of the current wave, `width` columns.
+void inv_solve(msgfem* h, int mat, int src, int dst, int neg, int width, int add) {
+  const InvForm& f = *h->inv;
+  const InvForm::Solve& s = f.waves[h->cur].solve[mat];
+  if (s.list.empty()) return;
+  for (int c0 = 0; c0 < width; c0 += KB) {
+    InvSolveArgs a = {};
+    a.mats = f.d_mats;
+    a.list = s.d_list;
+    a.subs = h->d_sub;
+    a.active = h->d_flags;
+    a.src = src;
+    a.dst = dst;
+    a.stride = width;
+    a.coloff = c0;
+    a.neg = neg;
+    a.add = add;
+    a.ring = s.ring;
+    a.smem_z = s.smem_z;
+    a.smem_u = s.smem_u;
+    a.smem_c = s.smem_c;
+    a.smem_r = s.smem_r;
+    a.err = h->d_kerr;
+    void* args[] = {&a};
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * (int)s.list.size() * s.G);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = s.smem;
+    cfg.stream = h->stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = s.G;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    for (bool back : {false, true}) {
+      cudaLaunchKernelExC(&cfg, solve_kernel(h, f.rs, back), args);
+      ++g_launch_count;
+    }
+  }
+}
+
+// flops of the inverse form: per layer the SPD inverse n^3 and the triple
+// product 108 n^2 (executed: whole 64 x 64 tiles, both products of the triple product full width)
+double inv_factor_flops(const msgfem* h, bool executed) {
+  double fl = 0.0;
+  for (const InvMat& m : h->inv->mats) {
+    if (m.n == 0) continue;
+    const double n = m.n, T = m.b / TILE, tile = 2.0 * TILE * TILE * TILE;
+    if (!executed) fl += m.nL * (n * n * n + 108.0 * n * n);
+    else fl += m.nL * (T * (T - 1.0 + 0.5 * T * (T - 1.0)) * tile + T * tile * 0.625 + 81.0 * n * n);
+  }
+  return fl;
+}
