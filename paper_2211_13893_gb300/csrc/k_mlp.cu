@@ -1,17 +1,24 @@
 // Warm-start network: a multilayer perceptron with tanh hidden layers, its
 // mean-squared-error gradient and Adam, all in FP32 on the GPU.
 //
-// Every layer is one tiled GEMM (64x64 output tile per CTA, 16-deep K chunks
-// staged in shared memory, 4x4 outputs per thread) with the bias, the tanh
-// and the tanh derivative fused into the epilogue:
+// Every layer is one tiled GEMM (32 x 32 output tile per CTA, 2 x 2 outputs per
+// thread) with the bias, the tanh, the tanh derivative, the loss gradient and the
+// bias gradient fused into it:
 //   forward      Z_l = H_{l-1} W_l^T + b_l, H_l = tanh(Z_l) (linear output layer)
+//   loss grad    G_L = 2 (Y - T) / (B d) in the output layer's epilogue
 //   weight grad  dW_l = G_l^T H_{l-1}, db_l = column sums of G_l
 //   data grad    G_{l-1} = (G_l W_l) * (1 - H_{l-1}^2)
-// with G_L = 2 (Y - T) / (B d).  The network is small (a few hundred
-// thousand weights) and its batches are a few hundred rows, so these GEMMs
-// take microseconds; they are not on the eigensolver's critical path.
+// The products are skinny: a hidden layer of 32 units is a handful of output tiles
+// over an inner dimension of hundreds, so the time is latency, not arithmetic.
+// Long inner dimensions are split over the CTAs of a thread-block cluster (one
+// chunk of 64 each as far as 8 CTAs reach), whose partial tiles are summed in rank
+// order through distributed shared memory.  128 x 672 -> 32 -> 1560 forward pass
+// 55 -> 14 us, a training step at batch 64 245 -> 56 us (64 x 64 tiles, serial
+// chunks of 16 before).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <vector>
 
@@ -40,93 +47,117 @@ struct msgfem_net {
 
 namespace {
 
-constexpr int GT = 64;    // output tile
-constexpr int GK = 16;    // K chunk
-constexpr int LOSS_BLOCKS = 240;
+constexpr int GT = 32;    // output tile
+constexpr int GK = 64;    // K chunk
 
-enum { EPI_PLAIN = 0, EPI_BIAS_TANH = 1, EPI_BIAS = 2, EPI_DTANH = 3 };
+enum { EPI_PLAIN = 0, EPI_BIAS_TANH = 1, EPI_BIAS = 2, EPI_DTANH = 3, EPI_MSE = 4 };
 
 // C[m][n] = sum_k A(m, k) B(k, n) with A(m, k) = A[m lda + k] (or A[k lda + m]
 // when AT) and B(k, n) = B[k ldb + n] (or B[n ldb + k] when BT), followed by
-// the epilogue EPI.  H (EPI_DTANH) is read with the leading dimension of C.
+// the epilogue EPI.  H (EPI_DTANH: the hidden outputs, EPI_MSE: the targets) is read
+// with the leading dimension of C.  EPI_PLAIN also writes the sums of A over k
+// (the bias gradient) to gb; EPI_MSE stores scale (C + bias - H) and adds one
+// partial sum of the squared differences per CTA to part.
+// A cluster of gridDim.z CTAs shares one output tile; rank z sums chunks
+// [z, z + 1) per of the inner dimension.
 template <bool AT, bool BT, int EPI>
 __global__ void __launch_bounds__(256)
 k_gemm(int M, int N, int K, const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
-       float* __restrict__ C, int ldc, const float* __restrict__ bias, const float* __restrict__ H) {
-  __shared__ float As[GK][GT + 4];
-  __shared__ float Bs[GK][GT + 4];
+       float* __restrict__ C, int ldc, const float* __restrict__ bias, const float* __restrict__ H,
+       float* __restrict__ gb, float scale, double* __restrict__ part) {
+  namespace cg = cooperative_groups;
+  __shared__ float As[GK][GT + 1];
+  __shared__ float Bs[GK][GT + 1];
+  __shared__ float Cs[GT][GT + 1];   // partial tile of this rank
+  __shared__ float Ss[GT];           // sums of A over its chunks (EPI_PLAIN)
+  __shared__ double red[8];
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
   const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT;
-  float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += GK) {
+  const int nch = (K + GK - 1) / GK, per = (nch + gridDim.z - 1) / gridDim.z;
+  const int c0 = blockIdx.z * per, c1 = min(c0 + per, nch);
+  float acc[2][2] = {};
+  float asum = 0.f;
+  for (int c = c0; c < c1; ++c) {
+    const int k0 = c * GK;
+    float ra[8], rb[8];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < 8; ++i) {   // every load of the chunk in flight at once
       const int e = tid + 256 * i;
-      int m, k;
-      if (AT) { m = e % GT; k = e / GT; } else { m = e / GK; k = e % GK; }
-      const int gm = m0 + m, gk = k0 + k;
-      float a = 0.f;
-      if (gm < M && gk < K) a = AT ? A[(size_t)gk * lda + gm] : A[(size_t)gm * lda + gk];
-      As[k][m] = a;
-      int n, kb;
-      if (BT) { n = e / GK; kb = e % GK; } else { n = e % GT; kb = e / GT; }
-      const int gn = n0 + n, gkb = k0 + kb;
-      float b = 0.f;
-      if (gn < N && gkb < K) b = BT ? B[(size_t)gn * ldb + gkb] : B[(size_t)gkb * ldb + gn];
-      Bs[kb][n] = b;
+      const int am = AT ? e % GT : e / GK, ak = AT ? e / GT : e % GK;
+      const int bn = BT ? e / GK : e % GT, bk = BT ? e % GK : e / GT;
+      ra[i] = (m0 + am < M && k0 + ak < K)
+                  ? (AT ? A[(size_t)(k0 + ak) * lda + m0 + am] : A[(size_t)(m0 + am) * lda + k0 + ak]) : 0.f;
+      rb[i] = (n0 + bn < N && k0 + bk < K)
+                  ? (BT ? B[(size_t)(n0 + bn) * ldb + k0 + bk] : B[(size_t)(k0 + bk) * ldb + n0 + bn]) : 0.f;
     }
     __syncthreads();
 #pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int e = tid + 256 * i;
+      if (AT) As[e / GT][e % GT] = ra[i]; else As[e % GK][e / GK] = ra[i];
+      if (BT) Bs[e % GK][e / GK] = rb[i]; else Bs[e / GT][e % GT] = rb[i];
+    }
+    __syncthreads();
+#pragma unroll 16
     for (int kk = 0; kk < GK; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+      const float a0 = As[kk][ty], a1 = As[kk][ty + 16], b0 = Bs[kk][tx], b1 = Bs[kk][tx + 16];
+      acc[0][0] = fmaf(a0, b0, acc[0][0]);
+      acc[0][1] = fmaf(a0, b1, acc[0][1]);
+      acc[1][0] = fmaf(a1, b0, acc[1][0]);
+      acc[1][1] = fmaf(a1, b1, acc[1][1]);
     }
-    __syncthreads();
+    if (EPI == EPI_PLAIN && tid < GT)
+      for (int kk = 0; kk < GK; ++kk) asum += As[kk][tid];
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int gm = m0 + ty + 16 * i;
-    if (gm >= M) continue;
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int gn = n0 + tx + 16 * j;
-      if (gn >= N) continue;
-      float v = acc[i][j];
-      if (EPI == EPI_BIAS_TANH) v = tanhf(v + bias[gn]);
-      if (EPI == EPI_BIAS) v += bias[gn];
-      if (EPI == EPI_DTANH) {
-        const float h = H[(size_t)gm * ldc + gn];
-        v *= 1.f - h * h;
-      }
-      C[(size_t)gm * ldc + gn] = v;
+    for (int j = 0; j < 2; ++j) Cs[ty + 16 * i][tx + 16 * j] = acc[i][j];
+  if (EPI == EPI_PLAIN && tid < GT) Ss[tid] = asum;
+  // rank z finishes rows z, z + R, ... of the tile
+  cg::cluster_group cl = cg::this_cluster();
+  const int R = gridDim.z, z = blockIdx.z;
+  if (R > 1) cl.sync();
+  else __syncthreads();
+  double sq = 0.0;
+  for (int e = tid; e < GT * GT; e += 256) {
+    const int r = e / GT, cc = e % GT, gm = m0 + r, gn = n0 + cc;
+    if (r % R != z || gm >= M || gn >= N) continue;
+    float v = 0.f;
+    if (R > 1) {
+      for (int q = 0; q < R; ++q) v += *cl.map_shared_rank(&Cs[r][cc], q);
+    } else {
+      v = Cs[r][cc];
+    }
+    if (EPI == EPI_BIAS_TANH) v = tanhf(v + bias[gn]);
+    if (EPI == EPI_BIAS) v += bias[gn];
+    if (EPI == EPI_DTANH) {
+      const float h = H[(size_t)gm * ldc + gn];
+      v *= 1.f - h * h;
+    }
+    if (EPI == EPI_MSE) {
+      const float d = v + bias[gn] - H[(size_t)gm * ldc + gn];
+      sq += (double)d * (double)d;
+      v = scale * d;
+    }
+    C[(size_t)gm * ldc + gn] = v;
+  }
+  if (EPI == EPI_PLAIN && blockIdx.x == 0 && z == 0 && tid < GT && m0 + tid < M) {
+    float v = 0.f;
+    for (int q = 0; q < R; ++q) v += R > 1 ? *cl.map_shared_rank(&Ss[tid], q) : Ss[tid];
+    gb[m0 + tid] = v;
+  }
+  if (EPI == EPI_MSE) {
+    for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    if ((tid & 31) == 0) red[tid >> 5] = sq;
+    __syncthreads();
+    if (tid == 0) {
+      double t = 0.0;
+      for (int w = 0; w < 8; ++w) t += red[w];
+      part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * R + z] = t;
     }
   }
-}
-
-// G = scale (Y - T) over n entries; per-block partial sums of (Y - T)^2
-__global__ void k_mse_grad(const float* __restrict__ Y, const float* __restrict__ T, long long n, float scale,
-                           float* __restrict__ G, double* __restrict__ part) {
-  __shared__ double red[256];
-  double s = 0.0;
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    const float d = Y[e] - T[e];
-    G[e] = scale * d;
-    s += (double)d * (double)d;
-  }
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[blockIdx.x] = red[0];
+  if (R > 1) cl.sync();   // the partial tiles stay alive until every rank has read them
 }
 
 // loss = sum of the partials / n (fixed order: deterministic)
@@ -143,15 +174,6 @@ __global__ void k_loss_final(const double* __restrict__ part, int np, long long 
   if (threadIdx.x == 0) loss[0] = red[0] / (double)n;
 }
 
-// gb[n] = sum_b G[b][n]
-__global__ void k_colsum(const float* __restrict__ G, int B, int N, float* __restrict__ gb) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  float s = 0.f;
-  for (int b = 0; b < B; ++b) s += G[(size_t)b * N + n];
-  gb[n] = s;
-}
-
 // Adam (Kingma and Ba 2015, Algorithm 1); c1 = 1 / (1 - beta1^t), c2 = 1 / (1 - beta2^t)
 __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
                        float* __restrict__ v, long long n, float lr, float b1, float b2, float eps, float c1,
@@ -166,18 +188,33 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
   }
 }
 
+// CTAs that split the inner dimension: one chunk each, at most 8 (a portable cluster)
+int split_of(int K) { return std::min(8, (K + GK - 1) / GK); }
+
 template <bool AT, bool BT, int EPI>
 void gemm(cudaStream_t st, int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C, int ldc,
-          const float* bias = nullptr, const float* H = nullptr) {
-  dim3 grid((N + GT - 1) / GT, (M + GT - 1) / GT);
-  k_gemm<AT, BT, EPI><<<grid, 256, 0, st>>>(M, N, K, A, lda, B, ldb, C, ldc, bias, H);
+          const float* bias = nullptr, const float* H = nullptr, float* gb = nullptr, float scale = 0.f,
+          double* part = nullptr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((N + GT - 1) / GT, (M + GT - 1) / GT, split_of(K));
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 1;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = cfg.gridDim.z;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k_gemm<AT, BT, EPI>, M, N, K, A, lda, B, ldb, C, ldc, bias, H, gb, scale, part);
   ++g_launch_count;
 }
 
-// forward pass; the output goes to Y (or the handle's output buffer when Y is null)
-void forward(msgfem_net* n, const float* X, int B, float* Y) {
+// forward pass up to layer `layers`; the last layer's output goes to Y (or the
+// handle's output buffer when Y is null)
+void forward(msgfem_net* n, const float* X, int B, float* Y, int layers) {
   const float* h = X;
-  for (int l = 0; l < n->L; ++l) {
+  for (int l = 0; l < layers; ++l) {
     const int in = n->sizes[l], out = n->sizes[l + 1];
     const float* W = n->p + n->woff[l];
     const float* b = n->p + n->boff[l];
@@ -189,22 +226,26 @@ void forward(msgfem_net* n, const float* X, int B, float* Y) {
   }
 }
 
-// forward + backward into n->g; loss into n->loss[0]
-void gradient(msgfem_net* n, const float* X, const float* T, int B) {
-  forward(n, X, B, nullptr);
-  const int dout = n->sizes[n->L];
+// forward + backward into n->g; with want_loss the loss into n->loss[0]
+void gradient(msgfem_net* n, const float* X, const float* T, int B, bool want_loss) {
+  forward(n, X, B, nullptr, n->L - 1);
+  const int dout = n->sizes[n->L], din = n->sizes[n->L - 1];
   const long long cnt = (long long)B * dout;
-  k_mse_grad<<<LOSS_BLOCKS, 256, 0, n->st>>>(n->act[n->L], T, cnt, 2.f / (float)cnt, n->d1, n->part);
-  k_loss_final<<<1, 256, 0, n->st>>>(n->part, LOSS_BLOCKS, cnt, n->loss);
-  g_launch_count += 2;
+  const float* hl = n->L > 1 ? n->act[n->L - 1] : X;
+  gemm<false, true, EPI_MSE>(n->st, B, dout, din, hl, din, n->p + n->woff[n->L - 1], din, n->d1, dout,
+                             n->p + n->boff[n->L - 1], T, nullptr, 2.f / (float)cnt, n->part);
+  if (want_loss) {
+    const int np = ((dout + GT - 1) / GT) * ((B + GT - 1) / GT) * split_of(din);
+    k_loss_final<<<1, 256, 0, n->st>>>(n->part, np, cnt, n->loss);
+    ++g_launch_count;
+  }
   float* G = n->d1;
   float* Gn = n->d2;
   for (int l = n->L - 1; l >= 0; --l) {
     const int in = n->sizes[l], out = n->sizes[l + 1];
     const float* hin = l == 0 ? X : n->act[l];
-    gemm<true, false, EPI_PLAIN>(n->st, out, in, B, G, out, hin, in, n->g + n->woff[l], in);
-    k_colsum<<<(out + 255) / 256, 256, 0, n->st>>>(G, B, out, n->g + n->boff[l]);
-    ++g_launch_count;
+    gemm<true, false, EPI_PLAIN>(n->st, out, in, B, G, out, hin, in, n->g + n->woff[l], in, nullptr, nullptr,
+                                 n->g + n->boff[l]);
     if (l > 0) {
       gemm<false, false, EPI_DTANH>(n->st, B, in, out, G, out, n->p + n->woff[l], in, Gn, in, nullptr, n->act[l]);
       float* tmp = G;
@@ -242,12 +283,14 @@ msgfem_status msgfem_net_create(int n_sizes, const int* sizes, int max_batch, co
   }
   for (int i = 0; i < n_sizes; ++i) wmax = sizes[i] > wmax ? sizes[i] : wmax;
   n->np = off;
+  // partial sums of the loss: one per output-layer CTA of the largest batch
+  const size_t loss_parts = (size_t)((sizes[n->L] + GT - 1) / GT) * ((max_batch + GT - 1) / GT) * split_of(sizes[n->L - 1]);
   n->act.assign(n->L + 1, nullptr);
   bool good = ok(cudaMalloc(&n->p, off * sizeof(float))) && ok(cudaMalloc(&n->g, off * sizeof(float))) &&
               ok(cudaMalloc(&n->m, off * sizeof(float))) && ok(cudaMalloc(&n->v, off * sizeof(float))) &&
               ok(cudaMalloc(&n->d1, (size_t)max_batch * wmax * sizeof(float))) &&
               ok(cudaMalloc(&n->d2, (size_t)max_batch * wmax * sizeof(float))) &&
-              ok(cudaMalloc(&n->part, LOSS_BLOCKS * sizeof(double))) && ok(cudaMalloc(&n->loss, sizeof(double)));
+              ok(cudaMalloc(&n->part, loss_parts * sizeof(double))) && ok(cudaMalloc(&n->loss, sizeof(double)));
   for (int l = 1; good && l <= n->L; ++l) good = ok(cudaMalloc(&n->act[l], (size_t)max_batch * sizes[l] * sizeof(float)));
   if (!good) {
     msgfem_net_destroy(n);
@@ -283,14 +326,14 @@ msgfem_status msgfem_net_set_params(msgfem_net_h n, const float* host_in) {
 
 msgfem_status msgfem_net_forward(msgfem_net_h n, const float* X, int batch, float* Y) {
   if (!n || !X || !Y || batch < 1 || batch > n->bmax) return MSGFEM_EINVAL;
-  forward(n, X, batch, Y);
+  forward(n, X, batch, Y, n->L);
   return ok(cudaGetLastError()) ? MSGFEM_OK : MSGFEM_ECUDA;
 }
 
 msgfem_status msgfem_net_gradient(msgfem_net_h n, const float* X, const float* T, int batch, float* grad_out,
                                   double* loss_out) {
   if (!n || !X || !T || batch < 1 || batch > n->bmax) return MSGFEM_EINVAL;
-  gradient(n, X, T, batch);
+  gradient(n, X, T, batch, loss_out != nullptr);
   if (!ok(cudaGetLastError())) return MSGFEM_ECUDA;
   if (grad_out && !ok(cudaMemcpyAsync(grad_out, n->g, n->np * sizeof(float), cudaMemcpyDeviceToHost, n->st)))
     return MSGFEM_ECUDA;
@@ -304,7 +347,7 @@ msgfem_status msgfem_net_adam_step(msgfem_net_h n, const float* X, const float* 
                                    float beta2, float eps, double* loss_out) {
   if (!n || !X || !T || batch < 1 || batch > n->bmax) return MSGFEM_EINVAL;
   if (!(beta1 >= 0.f && beta1 < 1.f && beta2 >= 0.f && beta2 < 1.f && eps > 0.f)) return MSGFEM_EINVAL;
-  gradient(n, X, T, batch);
+  gradient(n, X, T, batch, loss_out != nullptr);
   n->t += 1;
   double p1 = 1.0, p2 = 1.0;
   for (int i = 0; i < n->t; ++i) { p1 *= beta1; p2 *= beta2; }
