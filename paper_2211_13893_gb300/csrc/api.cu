@@ -310,8 +310,6 @@ msgfem_status allocate(msgfem* h) {
   TRY(dalloc(h, &h->d_flags_saved, h->N + 1));
   TRY(dalloc(h, &h->d_rprev, (size_t)h->N * KB));
   TRY(dalloc(h, &h->d_rref, (size_t)h->N * KB));
-  TRY(dalloc(h, &h->d_pcg, (size_t)h->N * 4 * KB));
-  CK(cudaMemset(h->d_pcg, 0, (size_t)h->N * 4 * KB * sizeof(double)));
   TRY(dalloc(h, &h->d_notspd, h->N + 1));
   TRY(dalloc(h, &h->d_ncols, h->N));
   TRY(dalloc(h, &h->d_coff, h->N));
@@ -587,31 +585,26 @@ void flags_restore(msgfem* h) {
 // kappa(K) u_32 well below 1 and stalls on the long floating subdomains of
 // curved laminates (pinned kappa ~ 2e7); CG converges in a few steps there.
 void solve_K_kb(msgfem* h) {
-  timed_solve8(h, 0, MV_ZB, MV_WB, 0);
-  launch_zero_pins_kb(h, MV_WB);
+  // (the inverse form leaves the pinned rows zero)
+  auto solve_K = [&](int src, int dst) {
+    timed_solve8(h, 0, src, dst, 0);
+    if (!h->inv_on) launch_zero_pins_kb(h, dst);
+  };
+  solve_K(MV_ZB, MV_WB);
   if (!h->mixed) return;
   flags_save(h);
   // x = WB, b = ZB, r = TB, z = P1, p = P2, q = P3; ||b|| recorded once as the reference
-  launch_refine_check_tol(h, MV_ZB, -1, KEEP_K, -1, PCG_TOL);
+  launch_refine_check_tol(h, MV_ZB, KEEP_K, -1, PCG_TOL);
   timed_stencil_kb(h, MV_WB, MV_TB, 0, 1.0);
-  launch_x_minus_y(h, MV_ZB, MV_TB, MV_TB, KB);
-  launch_zero_pins_kb(h, MV_TB);
-  launch_refine_check_tol(h, MV_TB, -1, KEEP_K, 0, PCG_TOL);
-  timed_solve_w(h, 0, MV_TB, MV_P1, 0, KB, 0);
-  launch_zero_pins_kb(h, MV_P1);
-  launch_coldot_kb(h, MV_TB, MV_P1, KEEP_K, 0);
-  launch_pcg_update(h, PCG_DIR0, MV_WB, MV_TB, MV_P1, MV_P2, MV_P3);
+  launch_pcg_residual(h, MV_ZB, MV_TB);
+  launch_refine_decide(h, 0, PCG_TOL);
   for (int it = 0; it < h->refine; ++it) {
+    solve_K(MV_TB, MV_P1);
+    launch_pcg_rz(h, MV_TB, MV_P1, it);
+    launch_pcg_dir(h, MV_P1, MV_P2, it);
     timed_stencil_kb(h, MV_P2, MV_P3, 0, 1.0);
-    launch_zero_pins_kb(h, MV_P3);
-    launch_coldot_kb(h, MV_P2, MV_P3, KEEP_K, 1);
-    launch_pcg_update(h, PCG_STEP, MV_WB, MV_TB, MV_P1, MV_P2, MV_P3);
-    launch_refine_check_tol(h, MV_TB, -1, KEEP_K, 0, PCG_TOL);
-    if (it + 1 == h->refine) break;
-    timed_solve_w(h, 0, MV_TB, MV_P1, 0, KB, 0);
-    launch_zero_pins_kb(h, MV_P1);
-    launch_coldot_kb(h, MV_TB, MV_P1, KEEP_K, 2);
-    launch_pcg_update(h, PCG_DIR, MV_WB, MV_TB, MV_P1, MV_P2, MV_P3);
+    launch_pcg_step(h, MV_WB, MV_TB, MV_P2, MV_P3, it);
+    launch_refine_decide(h, 0, PCG_TOL);
   }
   flags_restore(h);
 }
@@ -624,13 +617,13 @@ void extend_kb(msgfem* h) {
   timed_stencil_kb(h, MV_WB, MV_TB, 0, 1.0);
   if (h->mixed) {
     flags_save(h);
-    launch_refine_check(h, MV_TB, -1, KEEP_A11, -1);
+    launch_refine_check(h, MV_TB, KEEP_A11, -1);
   }
   timed_solve8(h, 1, MV_TB, MV_WB, 1);
   if (!h->mixed) return;
   for (int r = 0; r < h->refine; ++r) {
     timed_stencil_kb(h, MV_WB, MV_TB, 0, 1.0);
-    launch_refine_check(h, MV_TB, -1, KEEP_A11, r);
+    launch_refine_check(h, MV_TB, KEEP_A11, r);
     timed_solve_w(h, 1, MV_TB, MV_WB, 1, KB, 1);
   }
   flags_restore(h);
@@ -851,13 +844,13 @@ msgfem_status run_krylov(msgfem* h, const std::vector<int>& nl, bool& all_done) 
     launch_zero_kb(h, MV_WB);
     if (h->mixed) {
       flags_save(h);
-      launch_refine_check(h, MV_TB, -1, KEEP_A11, -1);   // reference ||b_B1||
+      launch_refine_check(h, MV_TB, KEEP_A11, -1);   // reference ||b_B1||
     }
     timed_solve8(h, 1, MV_TB, MV_WB, 1);
     for (int r = 0; h->mixed && r < h->refine; ++r) {
       timed_stencil_kb(h, MV_WB, MV_TB, 0, 1.0);
       launch_sub_load_kb(h, MV_TB);
-      launch_refine_check(h, MV_TB, -1, KEEP_A11, r);
+      launch_refine_check(h, MV_TB, KEEP_A11, r);
       timed_solve_w(h, 1, MV_TB, MV_WB, 1, KB, 1);
     }
     if (h->mixed) flags_restore(h);

@@ -231,7 +231,6 @@ struct msgfem {
   int* d_flags_saved = nullptr;      // [N + 1] flags saved around an adaptive refinement
   double* d_rprev = nullptr;         // [N][KB] residual norms of the previous refinement step
   double* d_rref = nullptr;          // [N][KB] reference residual norms of the refinement
-  double* d_pcg = nullptr;           // [N][4][KB] CG scalars per column: r.z, p.q, new r.z
   int* d_notspd = nullptr;           // [N + 1]
   int* d_ncols = nullptr;            // [N]
   int* d_mk = nullptr;               // [N] Krylov basis size at the last Rayleigh-Ritz
@@ -427,15 +426,19 @@ void launch_scale_rows_mu(msgfem* h, int which);
 void launch_theta_axpy(msgfem* h, int wx, int wy, int wd, int p);
 void launch_x_minus_y(msgfem* h, int wx, int wy, int wd, int stride);
 void launch_sub_load_kb(msgfem* h, int which);
-// preconditioned CG of the mixed-precision K solves (KB-wide blocks): masked
-// column dots into slot `slot` of d_pcg, and the vector updates
-void launch_coldot_kb(msgfem* h, int wx, int wy, int keep, int slot);
-enum { PCG_STEP = 0, PCG_DIR = 1, PCG_DIR0 = 2 };
-void launch_pcg_update(msgfem* h, int mode, int wx, int wr, int wz, int wp, int wq);
+// preconditioned CG of the mixed-precision K solves (KB-wide blocks; scalars per
+// column as partial sums, r . z of iteration it in one of two alternating slots):
+// r = b - r with its norm; r . z; x and r updates with the new norm; new direction
+void launch_pcg_residual(msgfem* h, int wb, int wr);
+void launch_pcg_rz(msgfem* h, int wr, int wz, int it);
+void launch_pcg_step(msgfem* h, int wx, int wr, int wp, int wq, int it);
+void launch_pcg_dir(msgfem* h, int wz, int wp, int it);
 // adaptive refinement: clear the active flag of subdomains whose residual
 // block wr (rows of the DoF classes in the bit mask keep) is converged or
-// stagnant (step -1 records the reference norm)
-void launch_refine_check(msgfem* h, int wr, int wref, int keep, int step);
+// stagnant (step -1 records the reference norm); launch_refine_decide takes the
+// norms that a CG kernel left
+void launch_refine_check(msgfem* h, int wr, int keep, int step);
+void launch_refine_decide(msgfem* h, int step, double tol);
 constexpr int KEEP_K = (1 << 1) | (1 << 2);   // rows of K: B1 and B2
 constexpr int KEEP_A11 = 1 << 1;               // rows of A11: B1
 #ifndef MSGFEM_REFINE_TOL
@@ -448,7 +451,7 @@ constexpr double REFINE_TOL = MSGFEM_REFINE_TOL;
 // relative residual at which the conjugate-gradient K solves of the mixed path stop
 // (the eigensolver's own tolerance is 1e-7 in the energy norm)
 constexpr double PCG_TOL = 1e-11;
-void launch_refine_check_tol(msgfem* h, int wr, int wref, int keep, int step, double tol);
+void launch_refine_check_tol(msgfem* h, int wr, int keep, int step, double tol);
 void launch_coarse_blocks(msgfem* h);
 void launch_coarse_rhs(msgfem* h);
 void launch_prolong(msgfem* h);

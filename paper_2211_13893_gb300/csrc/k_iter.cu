@@ -651,66 +651,83 @@ __global__ void k_x_minus_y(const SubDev* __restrict__ subs, const int* __restri
     D[e] = X[e] - Yv[e];
 }
 
+// Partial sums of the CG scalars and residual norms: COLDOT_CH blocks per subdomain
+// write one sum per column into a slot of the Gram scratch (slots of N COLDOT_CH KB
+// doubles, four of them within its N PST PST and more); whoever needs a scalar adds
+// the partials in a fixed order.
+constexpr int COLDOT_CH = 32;
+enum { SLOT_RZ0 = 0, SLOT_RZ1 = 1, SLOT_PQ = 2, SLOT_NORM = 3 };
+static_assert(4 * COLDOT_CH * KB <= PST * PST, "the slots must fit in the Gram scratch");
+
+__device__ __forceinline__ double* pcg_slot(double* part, int slot, int n, int sidx) {
+  return part + ((size_t)slot * n + sidx) * COLDOT_CH * KB;
+}
+
+// sum over the block of a per-thread value of column threadIdx.x % KB (256 threads) into out[column]
+__device__ __forceinline__ void block_column_sum(double v, double (*sa)[KB], double* out) {
+  for (int o = 16; o >= KB; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) < KB) sa[threadIdx.x >> 5][threadIdx.x & (KB - 1)] = v;
+  __syncthreads();
+  if (threadIdx.x < KB) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += sa[w][threadIdx.x];
+    out[threadIdx.x] = t;
+  }
+}
+
 // Adaptive iterative refinement of the FP32 solves.  Per active subdomain and
 // column, the residual norm of the KB-wide block R over the rows of the DoF
 // classes in keep (bit c for class c: B1 and B2 for K, B1 for A11; the rows
-// the solve acts on) is compared with a reference norm: the column of the right-hand side
-// block Ref, or, when Ref is absent, the residual recorded at step -1.  A
-// column is done when its relative residual is below tol or fell by less than
-// 10 % since the previous step (the FP64 rounding floor of the residual); a
+// the solve acts on) is compared with a reference norm: the residual recorded at
+// step -1.  A column is done when its relative residual is below tol or fell by
+// less than 10 % since the previous step (the FP64 rounding floor of the residual); a
 // subdomain whose columns are all done leaves the remaining refinement steps:
 // its active flag is cleared and the caller restores the flags afterwards.
 // Columns with a zero reference (unused columns) count as done.
+// Two kernels: the norms by COLDOT_CH blocks per subdomain (one block per subdomain
+// took 208 us on 27,000 rows, bound by one SM's load latency: 57 of 647 ms on the
+// 192 x 12 x 39 beam), the decision by one warp.
 __global__ void __launch_bounds__(256)
-k_refine_check(const SubDev* __restrict__ subs, int* __restrict__ flags, int wr, int wref, int keep, int step,
-               double tol, double* __restrict__ prev, double* __restrict__ refn) {
-  const int sidx = blockIdx.x;
+k_norm_partial(const SubDev* __restrict__ subs, const int* __restrict__ flags, int wr, int keep, double* __restrict__ part,
+               int n) {
+  const int sidx = blockIdx.y;
   if (!flags[sidx]) return;
   const SubDev& s = subs[sidx];
   const double* R = mv_ptr(s, wr);
-  const double* F = wref >= 0 ? mv_ptr(s, wref) : nullptr;
-  // thread t handles column t % KB of rows t / KB, t / KB + 32, ...
-  const int c = threadIdx.x % KB;
-  double r2 = 0.0, f2 = 0.0;
-  for (int row = threadIdx.x / KB; row < s.nfull; row += blockDim.x / KB) {
+  const int per = (s.nfull + COLDOT_CH - 1) / COLDOT_CH;
+  const int r0 = blockIdx.x * per, r1 = min(r0 + per, s.nfull), c = threadIdx.x % KB;
+  double acc = 0.0;
+  for (int row = r0 + threadIdx.x / KB; row < r1; row += 256 / KB) {
     if (!((keep >> s.cls[(row / 3) % s.npl]) & 1)) continue;
-    const double rv = R[(size_t)row * KB + c];
-    r2 += rv * rv;
-    if (F) {
-      const double fv = F[(size_t)row * KB + c];
-      f2 += fv * fv;
-    }
+    const double v = R[(size_t)row * KB + c];
+    acc += v * v;
   }
-  // lanes with equal column are KB apart within a warp
-  for (int o = 16; o >= KB; o >>= 1) {
-    r2 += __shfl_xor_sync(0xffffffffu, r2, o);
-    f2 += __shfl_xor_sync(0xffffffffu, f2, o);
-  }
-  __shared__ double sr[8][KB], sf[8][KB];
-  if ((threadIdx.x & 31) < KB) {
-    sr[threadIdx.x >> 5][c] = r2;
-    sf[threadIdx.x >> 5][c] = f2;
-  }
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  double* pv = prev + (size_t)sidx * KB;
-  double* rf = refn + (size_t)sidx * KB;
-  bool all_done = true;
-  for (int cc = 0; cc < KB; ++cc) {
-    double rt = 0.0, ft = 0.0;
-    for (int w = 0; w < 8; ++w) { rt += sr[w][cc]; ft += sf[w][cc]; }
-    const double rn = sqrt(rt);
+  __shared__ double sa[8][KB];
+  block_column_sum(acc, sa, pcg_slot(part, SLOT_NORM, n, sidx) + blockIdx.x * KB);
+}
+
+__global__ void k_refine_decide(int* __restrict__ flags, const double* __restrict__ part, int n, int step, double tol,
+                                double* __restrict__ prev, double* __restrict__ refn) {
+  const int sidx = blockIdx.x, c = threadIdx.x;
+  if (!flags[sidx]) return;
+  bool done = true;
+  if (c < KB) {
+    const double* p = part + ((size_t)SLOT_NORM * n + sidx) * COLDOT_CH * KB + c;
+    double t = 0.0;
+#pragma unroll 8
+    for (int i = 0; i < COLDOT_CH; ++i) t += p[i * KB];
+    const double rn = sqrt(t);
+    double* pv = prev + (size_t)sidx * KB + c;
+    double* rf = refn + (size_t)sidx * KB + c;
     if (step < 0) {   // record the reference only
-      rf[cc] = rn;
-      pv[cc] = rn;
-      continue;
+      *rf = rn;
+    } else {
+      done = *rf == 0.0 || rn <= tol * *rf || (step > 0 && rn > 0.9 * *pv);
     }
-    const double ref = F ? sqrt(ft) : rf[cc];
-    const bool done = ref == 0.0 || rn <= tol * ref || (step > 0 && rn > 0.9 * pv[cc]);
-    pv[cc] = rn;
-    all_done = all_done && done;
+    *pv = rn;
   }
-  if (step >= 0 && all_done) flags[sidx] = 0;
+  const bool all_done = __all_sync(0xffffffffu, done);
+  if (c == 0 && step >= 0 && all_done) flags[sidx] = 0;
 }
 
 // X[:, 0] -= bload (KB-wide block)
@@ -728,125 +745,166 @@ void launch_x_minus_y(msgfem* h, int wx, int wy, int wd, int stride) {
   k_x_minus_y<<<grid, 256, 0, h->stream>>>(h->d_sub, act(h), wx, wy, wd, stride); ++g_launch_count;
 }
 
-void launch_refine_check(msgfem* h, int wr, int wref, int keep, int step) {
-  launch_refine_check_tol(h, wr, wref, keep, step, REFINE_TOL);
+void launch_refine_check(msgfem* h, int wr, int keep, int step) {
+  launch_refine_check_tol(h, wr, keep, step, REFINE_TOL);
 }
 
-void launch_refine_check_tol(msgfem* h, int wr, int wref, int keep, int step, double tol) {
-  k_refine_check<<<h->N, 256, 0, h->stream>>>(h->d_sub, h->d_flags, wr, wref, keep, step, tol, h->d_rprev,
-                                               h->d_rref);
+void launch_refine_check_tol(msgfem* h, int wr, int keep, int step, double tol) {
+  k_norm_partial<<<dim3(COLDOT_CH, h->N), 256, 0, h->stream>>>(h->d_sub, h->d_flags, wr, keep, h->d_gram_part, h->N);
+  ++g_launch_count;
+  launch_refine_decide(h, step, tol);
+}
+
+void launch_refine_decide(msgfem* h, int step, double tol) {
+  k_refine_decide<<<h->N, 32, 0, h->stream>>>(h->d_flags, h->d_gram_part, h->N, step, tol, h->d_rprev, h->d_rref);
   ++g_launch_count;
 }
 
 namespace {
-// d[slot][c] = sum over rows of the DoF classes in `keep` of X[r][c] Y[r][c]
-// (KB-wide blocks): COLDOT_CH blocks per active subdomain write partial sums,
-// then one thread per (subdomain, column) adds them in a fixed order.
-constexpr int COLDOT_CH = 16;
+__device__ __forceinline__ bool pinned_full_row(const SubDev& s, int row) {
+  if (!s.floating || row >= 3 * s.npl) return false;
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+    if (s.pin[i] == row) return true;
+  return false;
+}
 
+// partial sums of X[r][c] Y[r][c] over the rows of the DoF classes in `keep`
 __global__ void __launch_bounds__(256)
 k_coldot_kb_partial(const SubDev* __restrict__ subs, const int* __restrict__ flags, int wx, int wy, int keep,
-                    double* __restrict__ part) {
+                    double* __restrict__ part, int slot, int n) {
   const int sidx = blockIdx.y;
   if (!flags[sidx]) return;
   const SubDev& s = subs[sidx];
   const double* X = mv_ptr(s, wx);
   const double* Y = mv_ptr(s, wy);
   const int per = (s.nfull + COLDOT_CH - 1) / COLDOT_CH;
-  const int r0 = blockIdx.x * per, r1 = min(r0 + per, s.nfull);
-  const int c = threadIdx.x % KB;
+  const int r0 = blockIdx.x * per, r1 = min(r0 + per, s.nfull), c = threadIdx.x % KB;
   double acc = 0.0;
-  for (int row = r0 + threadIdx.x / KB; row < r1; row += blockDim.x / KB) {
+  for (int row = r0 + threadIdx.x / KB; row < r1; row += 256 / KB) {
     if (!((keep >> s.cls[(row / 3) % s.npl]) & 1)) continue;
     acc += X[(size_t)row * KB + c] * Y[(size_t)row * KB + c];
   }
-  for (int o = 16; o >= KB; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
   __shared__ double sa[8][KB];
-  if ((threadIdx.x & 31) < KB) sa[threadIdx.x >> 5][c] = acc;
-  __syncthreads();
-  if (threadIdx.x < KB) {
-    double t = 0.0;
-    for (int w = 0; w < 8; ++w) t += sa[w][threadIdx.x];
-    part[((size_t)sidx * COLDOT_CH + blockIdx.x) * KB + threadIdx.x] = t;
-  }
+  block_column_sum(acc, sa, pcg_slot(part, slot, n, sidx) + blockIdx.x * KB);
 }
 
-__global__ void k_coldot_kb_reduce(const int* __restrict__ flags, const double* __restrict__ part,
-                                   double* __restrict__ pcg, int slot, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n * KB) return;
-  const int sidx = i / KB, c = i % KB;
-  if (!flags[sidx]) return;
-  double t = 0.0;
-  for (int b = 0; b < COLDOT_CH; ++b) t += part[((size_t)sidx * COLDOT_CH + b) * KB + c];
-  pcg[((size_t)sidx * 4 + slot) * KB + c] = t;
-}
-
-// CG updates per column (scalars from d_pcg slots 0: r.z, 1: p.q, 2: new r.z):
-//   PCG_STEP: alpha = rz / pq; x += alpha p; r -= alpha q
-//   PCG_DIR:  beta = rz_new / rz; p = z + beta p
-//   PCG_DIR0: p = z
-// A non-positive or non-finite ratio gives a zero step (the column then stalls
-// and its refinement check stops it).
+// Residual of the K system: R = B - R (R holds K x on entry), zero at the pins, with
+// the partial sums of its squared norm over the rows in `keep`.
 __global__ void __launch_bounds__(256)
-k_pcg_update(const SubDev* __restrict__ subs, const int* __restrict__ flags, const double* __restrict__ pcg,
-             int mode, int wx, int wr, int wz, int wp, int wq) {
+k_pcg_residual(const SubDev* __restrict__ subs, const int* __restrict__ flags, int wb, int wr, int keep,
+               double* __restrict__ part, int n) {
   const int sidx = blockIdx.y;
   if (!flags[sidx]) return;
   const SubDev& s = subs[sidx];
-  const double* d = pcg + (size_t)sidx * 4 * KB;
-  double* X = mv_ptr(s, wx);
+  const double* B = mv_ptr(s, wb);
   double* R = mv_ptr(s, wr);
-  const double* Z = mv_ptr(s, wz);
-  double* P = mv_ptr(s, wp);
-  const double* Q = mv_ptr(s, wq);
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < (size_t)s.nfull * KB;
-       e += (size_t)gridDim.x * blockDim.x) {
-    const int c = (int)(e % KB);
-    if (mode == PCG_STEP) {
-      const double rz = d[c], pq = d[KB + c];
-      double a = rz / pq;
-      if (!(pq > 0.0) || !(rz > 0.0) || !isfinite(a)) a = 0.0;
-      X[e] += a * P[e];
-      R[e] -= a * Q[e];
-    } else if (mode == PCG_DIR) {
-      const double rz = d[c], rzn = d[2 * KB + c];
-      double b = rzn / rz;
-      if (!(rz > 0.0) || !isfinite(b)) b = 0.0;
-      P[e] = Z[e] + b * P[e];
-    } else {
-      P[e] = Z[e];
-    }
+  const int per = (s.nfull + COLDOT_CH - 1) / COLDOT_CH;
+  const int r0 = blockIdx.x * per, r1 = min(r0 + per, s.nfull), c = threadIdx.x % KB;
+  double acc = 0.0;
+  for (int row = r0 + threadIdx.x / KB; row < r1; row += 256 / KB) {
+    const size_t e = (size_t)row * KB + c;
+    const double v = pinned_full_row(s, row) ? 0.0 : B[e] - R[e];
+    R[e] = v;
+    if ((keep >> s.cls[(row / 3) % s.npl]) & 1) acc += v * v;
   }
+  __shared__ double sa[8][KB];
+  block_column_sum(acc, sa, pcg_slot(part, SLOT_NORM, n, sidx) + blockIdx.x * KB);
 }
 
-// slot 0 <- slot 2 (r.z of the new residual becomes the current one)
-__global__ void k_pcg_shift(const int* __restrict__ flags, double* __restrict__ pcg, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n * KB) return;
-  const int sidx = i / KB, c = i % KB;
+// CG step per column: alpha = rz / pq; x += alpha p; r -= alpha q (zero at the
+// pins), with the partial sums of |r|^2 over the rows in `keep`.  A non-positive or
+// non-finite ratio gives a zero step (the column then stalls and its refinement check
+// stops it).
+__global__ void __launch_bounds__(256)
+k_pcg_step(const SubDev* __restrict__ subs, const int* __restrict__ flags, int wx, int wr, int wp, int wq, int keep,
+           double* __restrict__ part, int slot_rz, int n) {
+  const int sidx = blockIdx.y;
   if (!flags[sidx]) return;
-  pcg[(size_t)sidx * 4 * KB + c] = pcg[((size_t)sidx * 4 + 2) * KB + c];
+  const SubDev& s = subs[sidx];
+  __shared__ double al[KB], sa[8][KB];
+  if (threadIdx.x < KB) {
+    const double* prz = pcg_slot(part, slot_rz, n, sidx) + threadIdx.x;
+    const double* ppq = pcg_slot(part, SLOT_PQ, n, sidx) + threadIdx.x;
+    double rz = 0.0, pq = 0.0;
+#pragma unroll 8
+    for (int i = 0; i < COLDOT_CH; ++i) { rz += prz[i * KB]; pq += ppq[i * KB]; }
+    double a = rz / pq;
+    if (!(pq > 0.0) || !(rz > 0.0) || !isfinite(a)) a = 0.0;
+    al[threadIdx.x] = a;
+  }
+  __syncthreads();
+  double* X = mv_ptr(s, wx);
+  double* R = mv_ptr(s, wr);
+  const double* P = mv_ptr(s, wp);
+  const double* Q = mv_ptr(s, wq);
+  const int per = (s.nfull + COLDOT_CH - 1) / COLDOT_CH;
+  const int r0 = blockIdx.x * per, r1 = min(r0 + per, s.nfull), c = threadIdx.x % KB;
+  const double a = al[c];
+  double acc = 0.0;
+  for (int row = r0 + threadIdx.x / KB; row < r1; row += 256 / KB) {
+    const size_t e = (size_t)row * KB + c;
+    X[e] += a * P[e];
+    const double v = pinned_full_row(s, row) ? 0.0 : R[e] - a * Q[e];
+    R[e] = v;
+    if ((keep >> s.cls[(row / 3) % s.npl]) & 1) acc += v * v;
+  }
+  block_column_sum(acc, sa, pcg_slot(part, SLOT_NORM, n, sidx) + blockIdx.x * KB);
+}
+
+// New direction: p = z + (rz_new / rz) p, or p = z (first)
+__global__ void __launch_bounds__(256)
+k_pcg_dir(const SubDev* __restrict__ subs, const int* __restrict__ flags, int wz, int wp, double* __restrict__ part,
+          int slot_old, int slot_new, int n, int first) {
+  const int sidx = blockIdx.y;
+  if (!flags[sidx]) return;
+  const SubDev& s = subs[sidx];
+  __shared__ double be[KB];
+  if (threadIdx.x < KB) {
+    double b = 0.0;
+    if (!first) {
+      const double* po = pcg_slot(part, slot_old, n, sidx) + threadIdx.x;
+      const double* pn = pcg_slot(part, slot_new, n, sidx) + threadIdx.x;
+      double rz = 0.0, rzn = 0.0;
+#pragma unroll 8
+      for (int i = 0; i < COLDOT_CH; ++i) { rz += po[i * KB]; rzn += pn[i * KB]; }
+      b = rzn / rz;
+      if (!(rz > 0.0) || !isfinite(b)) b = 0.0;
+    }
+    be[threadIdx.x] = b;
+  }
+  __syncthreads();
+  const double* Z = mv_ptr(s, wz);
+  double* P = mv_ptr(s, wp);
+  const double b = be[threadIdx.x % KB];
+  for (size_t e = (size_t)blockIdx.x * 256 + threadIdx.x; e < (size_t)s.nfull * KB; e += (size_t)gridDim.x * 256)
+    P[e] = first ? Z[e] : Z[e] + b * P[e];
 }
 }  // namespace
 
-// (partial sums in the Gram scratch: N * COLDOT_CH * KB doubles, far below its size)
-void launch_coldot_kb(msgfem* h, int wx, int wy, int keep, int slot) {
-  dim3 grid(COLDOT_CH, h->N);
-  k_coldot_kb_partial<<<grid, 256, 0, h->stream>>>(h->d_sub, h->d_flags, wx, wy, keep, h->d_gram_part);
-  ++g_launch_count;
-  k_coldot_kb_reduce<<<(h->N * KB + 255) / 256, 256, 0, h->stream>>>(h->d_flags, h->d_gram_part, h->d_pcg, slot, h->N);
+void launch_pcg_residual(msgfem* h, int wb, int wr) {
+  k_pcg_residual<<<dim3(COLDOT_CH, h->N), 256, 0, h->stream>>>(h->d_sub, h->d_flags, wb, wr, KEEP_K, h->d_gram_part, h->N);
   ++g_launch_count;
 }
 
-void launch_pcg_update(msgfem* h, int mode, int wx, int wr, int wz, int wp, int wq) {
-  dim3 grid(64, h->N);
-  k_pcg_update<<<grid, 256, 0, h->stream>>>(h->d_sub, h->d_flags, h->d_pcg, mode, wx, wr, wz, wp, wq);
+void launch_pcg_rz(msgfem* h, int wr, int wz, int it) {
+  k_coldot_kb_partial<<<dim3(COLDOT_CH, h->N), 256, 0, h->stream>>>(h->d_sub, h->d_flags, wr, wz, KEEP_K, h->d_gram_part,
+                                                                  it & 1 ? SLOT_RZ1 : SLOT_RZ0, h->N);
   ++g_launch_count;
-  if (mode == PCG_DIR) {
-    k_pcg_shift<<<(h->N * KB + 255) / 256, 256, 0, h->stream>>>(h->d_flags, h->d_pcg, h->N);
-    ++g_launch_count;
-  }
+}
+
+void launch_pcg_step(msgfem* h, int wx, int wr, int wp, int wq, int it) {
+  k_coldot_kb_partial<<<dim3(COLDOT_CH, h->N), 256, 0, h->stream>>>(h->d_sub, h->d_flags, wp, wq, KEEP_K, h->d_gram_part,
+                                                                  SLOT_PQ, h->N);
+  k_pcg_step<<<dim3(COLDOT_CH, h->N), 256, 0, h->stream>>>(h->d_sub, h->d_flags, wx, wr, wp, wq, KEEP_K, h->d_gram_part,
+                                                         it & 1 ? SLOT_RZ1 : SLOT_RZ0, h->N);
+  g_launch_count += 2;
+}
+
+void launch_pcg_dir(msgfem* h, int wz, int wp, int it) {
+  k_pcg_dir<<<dim3(64, h->N), 256, 0, h->stream>>>(h->d_sub, h->d_flags, wz, wp, h->d_gram_part,
+                                                  it & 1 ? SLOT_RZ0 : SLOT_RZ1, it & 1 ? SLOT_RZ1 : SLOT_RZ0, h->N, it == 0);
+  ++g_launch_count;
 }
 
 void launch_sub_load_kb(msgfem* h, int which) {

@@ -38,16 +38,19 @@ def _run(cfg, **kw):
 @pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("name", list(CASES))
 def test_inverse_form_equals_block_cholesky(name, precision):
+    from paper_2211_13893_gb300 import plan
     cfg = replace(get_config("t3"), name=name, **CASES[name])
     tol = 1e-8 if precision == 0 else 1e-5
     la, ua, pa = _run(cfg, precision=precision)
     lb, ub, pb = _run(cfg, precision=precision, factor_schedule=1)
     assert pa["factor_flops"] != pb["factor_flops"]     # the two paths did run
-    assert (np.abs(la - lb) / np.abs(lb).max(axis=1, keepdims=True)).max() <= tol
+    scale = np.maximum(np.abs(lb).max(axis=1, keepdims=True), 1.0)   # a floating row may hold rigid zeros only
+    assert (np.abs(la - lb) / scale).max() <= tol
     assert np.abs(ua - ub).max() <= tol * np.abs(ub).max()
-    lc, uc, pc = _run(cfg, precision=precision, wave_mb=0.6 * pa["pool_mb"])
+    largest = plan(cfg, precision)["largest_mb"]
+    lc, uc, pc = _run(cfg, precision=precision, wave_mb=1.01 * largest)
     assert pc["waves"] >= 2
-    assert (np.abs(la - lc) / np.abs(lb).max(axis=1, keepdims=True)).max() <= tol
+    assert (np.abs(la - lc) / scale).max() <= tol
     assert np.abs(ua - uc).max() <= tol * np.abs(ub).max()
 
 
