@@ -40,6 +40,7 @@ void launch_zero_pins_kb(msgfem* h, int which);
 void launch_load_col_kb(msgfem* h, int which, double sign);
 void launch_take_col_kb(msgfem* h, int which);
 void launch_zero_kb(msgfem* h, int which);
+size_t rr_bytes(int N);
 void launch_rr_krylov(msgfem* h, const int* d_m, const int* d_nw);
 void launch_ritz(msgfem* h, const int* d_m, const int* d_nw, int scale, bool masked, int src, int dst);
 void launch_restart(msgfem* h, int m, int k);
@@ -336,6 +337,7 @@ msgfem_status allocate(msgfem* h) {
       TRY(upload_wave_solves(h, w));
     }
   }
+  if (h->opt.solver == 0) TRY(dev_alloc_bytes(h, &h->d_rr, rr_bytes(h->N)));
   TRY(dalloc(h, &h->d_mk, h->N));
   TRY(dalloc(h, &h->d_nwk, h->N));
   return MSGFEM_OK;

@@ -233,6 +233,7 @@ struct msgfem {
   double* d_rref = nullptr;          // [N][KB] reference residual norms of the refinement
   int* d_notspd = nullptr;           // [N + 1]
   int* d_ncols = nullptr;            // [N]
+  void* d_rr = nullptr;              // Rayleigh-Ritz work arrays (rr_bytes)
   int* d_mk = nullptr;               // [N] Krylov basis size at the last Rayleigh-Ritz
   int* d_nwk = nullptr;              // [N] wanted Ritz pairs
   // Waves: subdomains whose layer blocks, factors and solve buffers share one

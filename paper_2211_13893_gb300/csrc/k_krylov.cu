@@ -19,6 +19,15 @@ namespace {
 
 constexpr double KSIGMA = 1e-2;   // N = S + KSIGMA T
 
+// Rayleigh-Ritz work arrays: wanted mu (descending) and their indices [N][PST], the
+// rotations' tangents [N][rounds][MQ / 2], rounds run [N]
+struct RrWork {
+  double* mu;
+  float* log;
+  int* perm;
+  int* rounds;
+};
+
 // y = alpha [D_mu] K [D_mu] x on KB-wide blocks: 4 nodes per warp, lane % 8 = column.
 __global__ void __launch_bounds__(256)
 k_stencil_kb(const SubDev* __restrict__ subs, const int* __restrict__ active, int src, int dst, int mode,
@@ -345,131 +354,209 @@ __global__ void k_take_col_kb(const SubDev* __restrict__ subs, const int* __rest
 }
 
 // Rayleigh-Ritz on the leading m x m block of H (symmetrised): parallel cyclic
-// Jacobi in dynamic shared memory; the nw largest mu give theta = 1/mu
-// ascending, Yk[:, i] their coefficient vectors, resid[i] = theta_i
-// ||R_{m+1} y_last||.
-__global__ void __launch_bounds__(256)
-k_rr_krylov(const SubDev* __restrict__ subs, const int* __restrict__ active, const int* __restrict__ mvec,
-            const int* __restrict__ nwvec) {
+// Jacobi; the nw largest mu give theta = 1/mu ascending, Yk[:, i] their coefficient
+// vectors, resid[i] = theta_i ||R_{m+1} y_last||.
+//
+// One SM's FP64 pipe (1.6 FMA per clock) bounds it, so the arithmetic is kept small
+// and the vectors leave the iteration:
+//  * a round's m / 2 disjoint rotations update the symmetric matrix as 2 x 2 blocks
+//    of pairs (k <= l), read and written once;
+//  * rotations are scaled, A = D S D with J = c [1 t; -t 1]: the c go into D and an
+//    entry costs one FMA per side (8 per 2 x 2 block instead of 16);
+//  * the angle needs no FP64 accuracy (a rotation by a slightly wrong angle is still
+//    a similarity): t is formed in FP32, c = (1 + t^2)^{-1/2} to FP64 by Newton steps;
+//  * only t is logged (4 bytes per rotation); the wanted vectors are formed after
+//    the iteration by applying the rotations backwards to unit vectors, four columns
+//    per CTA (k_rr_vectors).
+// 65 calls (m = 24 to 96) of the GenEO comparison on eight subdomains 452 -> 142 ms,
+// 9 calls on the C-section's 16 subdomains 50.6 -> 16.8 ms (every rotation applied to
+// rows, columns and vectors before).
+constexpr int RR_SWEEPS = 30;
+constexpr int RR_ROUNDS = RR_SWEEPS * (MQ - 1);
+
+// pair k of round r of the round-robin order of mm (even) indices
+__device__ __forceinline__ void rr_pair(int k, int r, int mm, int& a, int& b) {
+  a = (k == 0) ? 0 : ((r + k - 1) % (mm - 1)) + 1;
+  b = ((r + mm - 2 - k) % (mm - 1)) + 1;
+  if (a > b) { const int t = a; a = b; b = t; }
+}
+
+// w^{-1/2} for w in [1, 2]: FP32 seed, two Newton steps
+__device__ __forceinline__ double rr_rsqrt(double w) {
+  double y = (double)rsqrtf((float)w);
+  y = y * fma(-0.5 * w * y, y, 1.5);
+  return y * fma(-0.5 * w * y, y, 1.5);
+}
+
+__global__ void __launch_bounds__(512)
+k_rr_jacobi(const SubDev* __restrict__ subs, const int* __restrict__ active, const int* __restrict__ mvec,
+            const int* __restrict__ nwvec, RrWork wk) {
   const int sidx = blockIdx.x;
   if (active != nullptr && !active[sidx]) return;
   const SubDev& s = subs[sidx];
   const int m = mvec[sidx], nw = nwvec[sidx];
   if (m <= 0 || nw <= 0) return;
   extern __shared__ double sh[];
-  double (*A)[MQ + 1] = reinterpret_cast<double (*)[MQ + 1]>(sh);
-  double (*V)[MQ + 1] = reinterpret_cast<double (*)[MQ + 1]>(sh + MQ * (MQ + 1));
-  __shared__ double cs[MQ / 2], sn[MQ / 2];
-  __shared__ int pa[MQ / 2], pb[MQ / 2], perm[MQ];
+  double (*A)[MQ + 1] = reinterpret_cast<double (*)[MQ + 1]>(sh);   // entries (i, j), j <= i
+  __shared__ double d[MQ], id[MQ], al[MQ / 2], be[MQ / 2];
+  __shared__ int pa[MQ / 2], pb[MQ / 2];
+  __shared__ double red_off[16], red_tot[16];
   __shared__ int again;
-  const int tid = threadIdx.x;
-  for (int e = tid; e < m * m; e += 256) {
+  const int tid = threadIdx.x, np = m / 2;      // m is a multiple of KB
+  float* log = wk.log + (size_t)sidx * RR_ROUNDS * (MQ / 2);
+  for (int e = tid; e < m * m; e += 512) {
     const int r = e / m, c = e % m;
-    A[r][c] = 0.5 * (s.H[(size_t)r * MQ + c] + s.H[(size_t)c * MQ + r]);
-    V[r][c] = (r == c) ? 1.0 : 0.0;
+    if (c <= r) A[r][c] = 0.5 * (s.H[(size_t)r * MQ + c] + s.H[(size_t)c * MQ + r]);
   }
+  if (tid < m) { d[tid] = 1.0; id[tid] = 1.0; }
   __syncthreads();
-  const int mm = (m + 1) & ~1;
-  __shared__ double red_off[8], red_tot[8];
-  for (int sweep = 0; sweep < 30; ++sweep) {
-    {
-      // off-diagonal and total Frobenius mass, reduced over the block
-      double off = 0.0, tot = 0.0;
-      for (int e = tid; e < m * m; e += 256) {
-        const int i = e / m, j = e % m;
-        const double v = A[i][j] * A[i][j];
-        tot += v;
-        if (i != j) off += v;
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        off += __shfl_xor_sync(0xffffffffu, off, o);
-        tot += __shfl_xor_sync(0xffffffffu, tot, o);
-      }
-      if ((tid & 31) == 0) {
-        red_off[tid >> 5] = off;
-        red_tot[tid >> 5] = tot;
-      }
-      __syncthreads();
-      if (tid == 0) {
-        double so = 0.0, st = 0.0;
-        for (int w = 0; w < 8; ++w) { so += red_off[w]; st += red_tot[w]; }
-        again = so > 1e-30 * st;
-      }
-      __syncthreads();
+  int rounds = 0;
+  for (int sweep = 0; sweep < RR_SWEEPS; ++sweep) {
+    // apply the scaling, off-diagonal and total Frobenius mass
+    double off = 0.0, tot = 0.0;
+    for (int e = tid; e < m * m; e += 512) {
+      const int i = e / m, j = e % m;
+      if (j > i) continue;
+      const double v = A[i][j] * d[i] * d[j];
+      A[i][j] = v;
+      if (i != j) off += 2.0 * v * v;
+      else tot += v * v;
     }
+    tot += off;
+    for (int o = 16; o > 0; o >>= 1) {
+      off += __shfl_xor_sync(0xffffffffu, off, o);
+      tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    }
+    if ((tid & 31) == 0) { red_off[tid >> 5] = off; red_tot[tid >> 5] = tot; }
+    __syncthreads();
+    if (tid < m) { d[tid] = 1.0; id[tid] = 1.0; }
+    if (tid == 0) {
+      double so = 0.0, st = 0.0;
+      for (int w = 0; w < 16; ++w) { so += red_off[w]; st += red_tot[w]; }
+      again = so > 1e-30 * st;
+    }
+    __syncthreads();
     if (!again) break;
-    for (int round = 0; round < mm - 1; ++round) {
-      if (tid < mm / 2) {
-        int a = (tid == 0) ? 0 : ((round + tid - 1) % (mm - 1)) + 1;
-        int b = ((round + mm - 2 - tid) % (mm - 1)) + 1;
-        if (a > b) { const int t = a; a = b; b = t; }
-        pa[tid] = a;
-        pb[tid] = b;
-        double c = 1.0, sv = 0.0;
-        if (b < m) {
-          const double apq = A[a][b];
-          if (fabs(apq) > 1e-300) {
-            const double tau = (A[b][b] - A[a][a]) / (2.0 * apq);
-            const double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-            c = 1.0 / sqrt(1.0 + t * t);
-            sv = t * c;
-          }
+    for (int round = 0; round < m - 1; ++round, ++rounds) {
+      if (tid < np) {
+        int p, q;
+        rr_pair(tid, round, m, p, q);
+        pa[tid] = p;
+        pb[tid] = q;
+        // t = sign / (|tau| + sqrt(1 + tau^2)), tau = (a_qq - a_pp) / (2 a_pq)
+        const double dp = d[p], dq = d[q];
+        const double diff = A[q][q] * dq * dq - A[p][p] * dp * dp, twice = 2.0 * A[q][p] * dp * dq;
+        float t = 0.f;
+        if (fabs(twice) > 1e-36) {
+          const float tau = (float)(diff) / (float)twice;
+          t = copysignf(1.f, tau) / (fabsf(tau) + sqrtf(fmaf(tau, tau, 1.f)));
+          if (!(fabsf(t) <= 1.f)) t = 0.f;
         }
-        cs[tid] = c;
-        sn[tid] = sv;
+        const double td = (double)t, w = fma(td, td, 1.0), c = rr_rsqrt(w);
+        al[tid] = td * dq * id[p];
+        be[tid] = td * dp * id[q];
+        d[p] = c * dp;
+        d[q] = c * dq;
+        id[p] *= w * c;
+        id[q] *= w * c;
+        log[(size_t)rounds * (MQ / 2) + tid] = t;
       }
       __syncthreads();
-      for (int e = tid; e < (mm / 2) * m; e += 256) {
-        const int k = e / m, col = e % m;
-        const int a = pa[k], b = pb[k];
-        if (b >= m) continue;
-        const double x = A[a][col], y = A[b][col];
-        A[a][col] = cs[k] * x - sn[k] * y;
-        A[b][col] = sn[k] * x + cs[k] * y;
-      }
-      __syncthreads();
-      for (int e = tid; e < (mm / 2) * m; e += 256) {
-        const int k = e / m, row = e % m;
-        const int a = pa[k], b = pb[k];
-        if (b >= m) continue;
-        const double x = A[row][a], y = A[row][b];
-        A[row][a] = cs[k] * x - sn[k] * y;
-        A[row][b] = sn[k] * x + cs[k] * y;
-        const double vx = V[row][a], vy = V[row][b];
-        V[row][a] = cs[k] * vx - sn[k] * vy;
-        V[row][b] = sn[k] * vx + cs[k] * vy;
+      // blocks (k, l), k <= l: rows k and np - 1 - k hold np + 1 of them together
+      for (int e = tid; e < np / 2 * (np + 1); e += 512) {
+        const int r = e / (np + 1), c = e % (np + 1);
+        const int k = c < np - r ? r : np - 1 - r, l = c < np - r ? r + c : k + c - (np - r);
+        const int p0 = pa[k], q0 = pb[k], p1 = pa[l], q1 = pb[l];
+        double* xa = p0 > p1 ? &A[p0][p1] : &A[p1][p0];
+        double* xb = p0 > q1 ? &A[p0][q1] : &A[q1][p0];
+        double* xc = q0 > p1 ? &A[q0][p1] : &A[p1][q0];
+        double* xd = q0 > q1 ? &A[q0][q1] : &A[q1][q0];
+        const double a = *xa, b = *xb, cc = *xc, dd = *xd;
+        const double ak = al[k], bk = be[k], aL = al[l], bL = be[l];
+        const double a1 = fma(-ak, cc, a), c1 = fma(bk, a, cc), b1 = fma(-ak, dd, b), d1 = fma(bk, b, dd);
+        *xa = fma(-aL, b1, a1);
+        *xd = fma(bL, c1, d1);
+        if (k != l) *xc = fma(-aL, d1, c1);   // (k, k): the same entry as b
+        *xb = fma(bL, a1, b1);
       }
       __syncthreads();
     }
   }
-  if (tid == 0) {
-    for (int i = 0; i < m; ++i) perm[i] = i;
-    for (int i = 0; i < m; ++i)   // descending mu
-      for (int j = i + 1; j < m; ++j)
-        if (A[perm[j]][perm[j]] > A[perm[i]][perm[i]]) { const int t = perm[i]; perm[i] = perm[j]; perm[j] = t; }
+  // descending mu by counting; ties by index
+  __shared__ double mu[MQ];
+  if (tid < m) mu[tid] = A[tid][tid] * d[tid] * d[tid];
+  __syncthreads();
+  if (tid < m) {
+    int rank = 0;
+    for (int j = 0; j < m; ++j) rank += (mu[j] > mu[tid] || (mu[j] == mu[tid] && j < tid)) ? 1 : 0;
+    if (rank < nw && rank < PST) {
+      wk.perm[sidx * PST + rank] = tid;
+      wk.mu[sidx * PST + rank] = mu[tid];
+    }
+  }
+  if (tid == 0) wk.rounds[sidx] = rounds;
+}
+
+constexpr int RR_CHUNK = 32;   // rounds whose rotations are staged at once
+
+__global__ void __launch_bounds__(4 * (MQ / 2))
+k_rr_vectors(const SubDev* __restrict__ subs, const int* __restrict__ active, const int* __restrict__ mvec,
+             const int* __restrict__ nwvec, RrWork wk) {
+  const int sidx = blockIdx.y;
+  if (active != nullptr && !active[sidx]) return;
+  const SubDev& s = subs[sidx];
+  const int m = mvec[sidx], nw = nwvec[sidx];
+  if (m <= 0 || nw <= 0) return;
+  __shared__ double x[MQ][4];
+  __shared__ double2 cs[RR_CHUNK][MQ / 2];
+  const int tid = threadIdx.x, k = tid >> 2, c = tid & 3, col = blockIdx.x * 4 + c, np = m / 2;
+  const bool live = col < nw;
+  const int src = live ? wk.perm[sidx * PST + col] : -1;
+  for (int a = k; a < MQ; a += MQ / 2) x[a][c] = (a == src) ? 1.0 : 0.0;
+  if (blockIdx.x * 4 < nw) {
+    const float* log = wk.log + (size_t)sidx * RR_ROUNDS * (MQ / 2);
+    // V e = J_1 (J_2 ( ... J_n e)), each round's disjoint rotations at once
+    for (int r1 = wk.rounds[sidx]; r1 > 0; r1 -= RR_CHUNK) {
+      const int r0 = max(0, r1 - RR_CHUNK);
+      __syncthreads();
+      for (int e = tid; e < (r1 - r0) * np; e += blockDim.x) {
+        const int r = e / np, i = e % np;
+        const double t = (double)log[(size_t)(r0 + r) * (MQ / 2) + i], cv = rr_rsqrt(fma(t, t, 1.0));
+        cs[r][i] = make_double2(cv, cv * t);
+      }
+      __syncthreads();
+      for (int r = r1 - 1; r >= r0; --r) {
+        if (k < np) {
+          int p, q;
+          rr_pair(k, r % (m - 1), m, p, q);
+          const double2 g = cs[r - r0][k];
+          const double xp = x[p][c], xq = x[q][c];
+          x[p][c] = fma(g.x, xp, g.y * xq);
+          x[q][c] = fma(g.x, xq, -g.y * xp);
+        }
+        __syncthreads();
+      }
+    }
   }
   __syncthreads();
-  for (int e = tid; e < MQ * PST; e += 256) {
-    const int a = e / PST, i = e % PST;
-    s.Yk[e] = (a < m && i < nw) ? V[a][perm[i]] : 0.0;
-  }
-  if (tid < nw) {
+  for (int a = k; a < MQ; a += MQ / 2)
+    if (col < PST) s.Yk[(size_t)a * PST + col] = (live && a < m) ? x[a][c] : 0.0;
+  if (k == 0 && live) {
     // Ritz values of M in the N = S + sigma T inner product lie in [0, 1 / sigma];
     // a wanted one below 1e-14 (lambda above 1e14) comes from a basis that broke down
-    const double mu = A[perm[tid]][perm[tid]];
+    const double mu = wk.mu[sidx * PST + col];
     const bool valid = mu > 1e-14;
     const double th = valid ? 1.0 / mu : 1e300;
     double r2 = 0.0;
-    if (m + KB <= MQ + KB)
-      for (int r = 0; r < KB; ++r) {
-        double v = 0.0;
-        for (int c = 0; c < KB; ++c) v += s.H[(size_t)(m + r) * MQ + (m - KB + c)] * V[m - KB + c][perm[tid]];
-        r2 += v * v;
-      }
-    s.theta[tid] = th;
+    for (int r = 0; r < KB; ++r) {
+      double v = 0.0;
+      for (int j = 0; j < KB; ++j) v += s.H[(size_t)(m + r) * MQ + (m - KB + j)] * x[m - KB + j][c];
+      r2 += v * v;
+    }
+    s.theta[col] = th;
     // no positive Ritz value (a basis that broke down, e.g. from a non-finite
     // start block whose columns were all dropped): never converged
-    s.resid[tid] = valid ? th * sqrt(r2) : INFINITY;
+    s.resid[col] = valid ? th * sqrt(r2) : INFINITY;
   }
 }
 
@@ -625,14 +712,27 @@ void launch_zero_kb(msgfem* h, int which) {
   k_zero_kb<<<grid, 256, 0, h->stream>>>(h->d_sub, h->d_flags, which, 0); ++g_launch_count;
 }
 
+// bytes of the Rayleigh-Ritz work arrays of N subdomains
+size_t rr_bytes(int N) {
+  return (size_t)N * (PST * (sizeof(double) + sizeof(int)) + RR_ROUNDS * (MQ / 2) * sizeof(float) + 8);
+}
+
 void launch_rr_krylov(msgfem* h, const int* d_m, const int* d_nw) {
   static bool attr = false;
-  const int smem = 2 * MQ * (MQ + 1) * (int)sizeof(double);
+  const int smem = MQ * (MQ + 1) * (int)sizeof(double);
   if (!attr) {
-    cudaFuncSetAttribute(k_rr_krylov, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaFuncSetAttribute(k_rr_jacobi, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     attr = true;
   }
-  k_rr_krylov<<<h->N, 256, smem, h->stream>>>(h->d_sub, h->d_flags, d_m, d_nw); ++g_launch_count;
+  RrWork wk;
+  char* base = static_cast<char*>(h->d_rr);
+  wk.mu = reinterpret_cast<double*>(base);
+  wk.log = reinterpret_cast<float*>(wk.mu + (size_t)h->N * PST);
+  wk.perm = reinterpret_cast<int*>(wk.log + (size_t)h->N * RR_ROUNDS * (MQ / 2));
+  wk.rounds = wk.perm + (size_t)h->N * PST;
+  k_rr_jacobi<<<h->N, 512, smem, h->stream>>>(h->d_sub, h->d_flags, d_m, d_nw, wk);
+  k_rr_vectors<<<dim3(PST / 4, h->N), 4 * (MQ / 2), 0, h->stream>>>(h->d_sub, h->d_flags, d_m, d_nw, wk);
+  g_launch_count += 2;
 }
 
 void launch_ritz(msgfem* h, const int* d_m, const int* d_nw, int scale, bool masked, int src, int dst) {
