@@ -652,6 +652,350 @@ k_inv_solve(const InvSolveArgs a) {
   }
 }
 
+// ---------------------------------------------------------------------------
+// FP64 solves in exact digit products on the tensor cores.
+//
+// One SM does 1.6 FP64 FMAs per clock but 956 FP16 ones (mma.sync m16n8k16, both
+// measured), and its FP32 accumulation of integers is exact below 2^24.  A number is
+// written as a 61-bit integer below the largest of its row (matrix) or column
+// (vector) in seven balanced base-512 digits, n_i in [-256, 255], exact in FP16; of
+// the 49 digit products the 28 of weight 512^6 and up are formed (the rest is below
+// 2^-59 of the largest product), those of one weight in one accumulator: 32 columns
+// of k add at most 7 x 32 x 2^16 < 2^24.  After every 32 columns the seven sums go
+// into two 64-bit integers, so nothing is rounded before the result: the error is
+// that of rounding the operands to 2^-61 of their row or column maximum, where the
+// DFMA chain rounds every partial sum to 2^-53.
+//
+// Digits are cut from biased integers, X + sum 256 512^i: a 9-bit field d is the
+// digit d + 256, and 0x6400 | d is 1024 + d in FP16.  The factorisation leaves every
+// layer's -S^{-1} in that form in place (8 bytes per entry, 16 x 16 blocks in fragment
+// order: a lane's operands are four 16-byte vectors), so that a solve streams it with
+// bulk copies as before and spends 6 integer instructions per pair of digits; the
+// right-hand side's digits are cut once per layer by the rank that owns the node
+// and written to every rank of the cluster.  Taken whenever a layer's digits and
+// coefficients fit in shared memory (layers up to about 1,000 DoFs); above, FP64 FMAs.
+// Whole passes with FP64 FMAs -> digits: 36 x 12 x 39 beam 306 -> 204 ms (solves 158 ->
+// 54), 47 x 7 x 13 beam 77 -> 50, 24 x 4 x 12 beam 29 -> 20, Schwarz PCG 45 -> 29; the
+// passes' errors against a dense 64-bit reference are unchanged.
+constexpr int DIG = 7;
+constexpr long long DIG_BIAS = 256ll * (0x7fffffffffffffffll / 511);   // sum of 256 512^i, i < 7
+constexpr int FX_KB = 16;                      // 16 x 16 blocks per stage (two per warp)
+constexpr int FX_STAGE = FX_KB * 256 * 8;      // bytes
+
+// x 2^(60 - emax) rounded to nearest (|x| < 2^(emax + 1), biased exponents), plus the bias
+__device__ __forceinline__ long long biased_fixed(double x, int emax) {
+  const long long xb = __double_as_longlong(x);
+  const int ex = (int)(xb >> 52) & 0x7ff, sh = emax - ex - 8;
+  const long long m = (xb & 0xfffffffffffffll) | (1ll << 52);
+  long long v;
+  if (ex == 0 || sh > 60) v = 0;               // zero, subnormal or below half a unit
+  else if (sh <= 0) v = m << -sh;
+  else v = (m + (1ll << (sh - 1))) >> sh;
+  return (xb < 0 ? -v : v) + DIG_BIAS;
+}
+
+// digit i of two biased integers as a pair of FP16 numbers
+__device__ __forceinline__ uint32_t digit_pair(long long x0, long long x1, int i) {
+  const uint32_t d = ((uint32_t)(x0 >> (9 * i)) & 0x1ff) | (((uint32_t)(x1 >> (9 * i)) & 0x1ff) << 16) | 0x64006400u;
+  uint32_t r;
+  asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(d), "r"(0xe500e500u));   // - 1280
+  return r;
+}
+
+__device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+
+// sums of the seven weights (512^6 .. 512^12) into hi 2^27 + lo
+__device__ __forceinline__ void digit_flush(const float (&acc)[DIG][4], int e, long long& hi, long long& lo) {
+  lo += (long long)__float2int_rn(acc[0][e]) + ((long long)__float2int_rn(acc[1][e]) << 9) +
+        ((long long)__float2int_rn(acc[2][e]) << 18);
+  hi += (long long)__float2int_rn(acc[3][e]) + ((long long)__float2int_rn(acc[4][e]) << 9) +
+        ((long long)__float2int_rn(acc[5][e]) << 18) + ((long long)__float2int_rn(acc[6][e]) << 27);
+}
+
+// (hi 2^27 + lo) 2^e for any int e
+__device__ __forceinline__ double digit_value(long long hi, long long lo, int e) {
+  const double v = fma((double)hi, 0x1p27, (double)lo);
+  if (e >= -1022 && e <= 1023) return v * __hiloint2double((e + 1023) << 20, 0);
+  return scalbn(v, e);
+}
+
+// biased exponents of the rows of layer l (at the end of the layer's L slot)
+__device__ __forceinline__ int* row_exponents(const InvMat& m, int l) {
+  return reinterpret_cast<int*>(static_cast<double*>(m.L) + (size_t)(l + 1) * m.b * m.b - m.b / 2);
+}
+
+// -S^{-1} of every layer to biased integers in fragment order, in place: one strip of 16 rows per CTA
+__global__ void __launch_bounds__(256)
+k_inv_digits(const InvMat* __restrict__ mats, const int* __restrict__ active) {
+  const InvMat& m = mats[blockIdx.z];
+  if (active != nullptr && !active[m.sub]) return;
+  const int l = blockIdx.y, s = blockIdx.x, nkb = (m.n + 15) / 16;
+  if (l >= m.nL || s >= nkb) return;
+  extern __shared__ __align__(16) unsigned char smem_dg[];
+  double* v = reinterpret_cast<double*>(smem_dg);
+  __shared__ int em[16];
+  const int tid = threadIdx.x, b = m.b, ld = b + 2;
+  double* D = static_cast<double*>(m.D) + ((size_t)l * b + (size_t)s * 16) * b;
+  if (tid < 16) em[tid] = 0;
+  __syncthreads();
+  for (int e = tid; e < 16 * b; e += 256) {
+    const int r = e / b, c = e % b;
+    const double x = D[e];
+    v[r * ld + c] = x;
+    atomicMax(&em[r], (__double2hiint(x) >> 20) & 0x7ff);
+  }
+  __syncthreads();
+  long long* out = reinterpret_cast<long long*>(D);
+  for (int e = tid; e < nkb * 256; e += 256) {
+    const int kb = e >> 8, j = (e >> 6) & 3, lane = (e >> 1) & 31;
+    const int r = (lane >> 2) + 8 * (j & 1), c = kb * 16 + 2 * (lane & 3) + 8 * (j >> 1) + (e & 1);
+    out[e] = biased_fixed(v[r * ld + c], em[r]);
+  }
+  if (tid < 16) row_exponents(m, l)[s * 16 + tid] = em[tid];
+}
+
+template <bool BACK>
+__global__ void __launch_bounds__(256, 1)
+k_inv_solve_fx(const InvSolveArgs a) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int G = (int)cl.num_blocks(), g = (int)cl.block_rank();
+  const int task = blockIdx.x / G, half = task & 1;
+  const InvMat m = a.mats[a.list[task >> 1]];
+  if (a.active != nullptr && !a.active[m.sub]) return;   // uniform over the cluster
+  const int nch = half ? m.nL - 1 - m.mid : m.mid;
+  const int steps = BACK ? nch + 1 : nch;
+  if (nch == 0 && (!BACK || half)) return;
+  auto layer_of = [&](int t) {
+    if (BACK) return half ? m.mid + t : m.mid - t;
+    return half ? m.nL - 1 - t : t;
+  };
+  extern __shared__ __align__(128) unsigned char smem_fs[];
+  unsigned char* ring = smem_fs;
+  uint32_t* zd = reinterpret_cast<uint32_t*>(smem_fs + a.smem_z);   // [DIG][8 nkb pairs of rows][KB] FP16 pairs
+  double* uw = reinterpret_cast<double*>(smem_fs + a.smem_u);
+  double* cf = reinterpret_cast<double*>(smem_fs + a.smem_c);
+  double* zo = reinterpret_cast<double*>(smem_fs + a.smem_r);       // z of the own nodes
+  __shared__ __align__(8) unsigned long long bars[9];
+  __shared__ unsigned long long red[2][128][2];
+  __shared__ int zm[KB], zmax[8][KB];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int b = m.b, nn = m.n / 3, nkb = (m.n + 15) / 16, NC = (nkb + FX_KB - 1) / FX_KB;
+  const int s0 = nkb * g / G, s1 = nkb * (g + 1) / G, ns = s1 - s0;
+  const int npc = up4((nn + G - 1) / G), p0 = min(nn, npc * g), p1 = min(nn, p0 + npc);
+  const int wlo = max(0, p0 - m.njc - 1);
+  const uint32_t ring_s = tc::saddr(ring), bar0 = tc::saddr(bars), cf_s = tc::saddr(cf);
+  const int total = ns * NC * steps;
+  bool ok = true;
+  int issued = 0;   // stages requested (thread 0)
+  auto issue = [&](int i) {
+    issued = i + 1;
+    const int c = i % NC, sl = i / NC, l = layer_of(sl / ns), s = s0 + sl % ns;
+    const uint32_t bytes = (uint32_t)min(FX_KB, nkb - c * FX_KB) * 2048u, bar = bar0 + 8 * (i % a.ring);
+    tc::mbar_expect_tx(bar, bytes);
+    bulk_load(ring_s + (uint32_t)(i % a.ring) * FX_STAGE,
+              static_cast<const double*>(m.D) + ((size_t)l * b + (size_t)s * 16) * b + (size_t)c * FX_KB * 256, bytes, bar);
+  };
+  const int cdir = BACK ? (half ? 0 : 1) : (half ? 1 : 0);
+  const uint32_t cbytes = p1 > p0 ? (uint32_t)(up4(p1 - p0) * 81 * sizeof(double)) : 0;
+  auto coupling_ptr = [&](int l, int dir) {
+    return static_cast<const double*>(m.L) + (size_t)l * b * b + ((size_t)dir * up4(nn) + p0) * 81;
+  };
+  if (tid == 0) {
+    for (int i = 0; i < 9; ++i) tc::mbar_init(bar0 + 8 * i, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    for (int i = 0; i < a.ring && i < total; ++i) issue(i);
+  }
+  for (int e = tid; e < DIG * nkb * 8 * KB; e += 256) zd[e] = 0u;
+  red[tid >> 7][tid & 127][0] = 0ull;
+  red[tid >> 7][tid & 127][1] = 0ull;
+  if (tid < KB) zm[tid] = 0;
+  __syncthreads();
+  const SubDev& sd = a.subs[m.sub];
+  const double* src = mv_ptr(sd, a.src) + a.coloff;
+  double* dst = mv_ptr(sd, a.dst) + a.coloff;
+  double* yc = static_cast<double*>(m.yc);
+  const double sgn = a.neg ? -1.0 : 1.0;
+  int cphase = 0, ci = 0, waited = 0, strip = 0;
+  bool cpend = false;
+  cl.sync();   // no remote store before every CTA of the cluster has cleared its arrays
+  for (int t = 0; t < steps; ++t) {
+    const int l = layer_of(t);
+    const bool first = t == 0;
+    if (cpend) {
+      if (ok) ok = tc::mbar_wait(bar0 + 64, cphase & 1);
+      ++cphase;
+    }
+    // ---- sparse step on the own nodes (FP64), the largest exponent per column
+    int mx = 0;
+    for (int e = tid; e < (p1 - p0) * KB; e += 256) {
+      const int pl = e / KB, col = e % KB, p = p0 + pl;
+      const int i = p / m.njc, j = p % m.njc;
+      double z[3] = {0.0, 0.0, 0.0};
+      if (!BACK || first) {
+        const size_t node = (size_t)l * m.npl + (size_t)(m.ia + i) * m.nyn + m.ja + j;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) z[r] = sgn * src[(node * 3 + r) * a.stride + col];
+        if (m.pinned && l == 0)
+#pragma unroll
+          for (int r = 0; r < 3; ++r)
+            if (pinned_row(m, 0, 3 * p + r)) z[r] = 0.0;
+      }
+      auto sub_coupling = [&](const double* c, const double* u) {
+        double acc[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+        for (int s9 = 0; s9 < 9; ++s9) {
+          const int di = s9 / 3 - 1, dj = s9 % 3 - 1;
+          if (i + di < 0 || i + di >= m.nic || j + dj < 0 || j + dj >= m.njc) continue;
+          const double* x = u + (ptrdiff_t)(3 * (p + di * m.njc + dj)) * KB + col;
+          const double x0 = x[0], x1 = x[KB], x2 = x[2 * KB];
+#pragma unroll
+          for (int r = 0; r < 3; ++r)
+            acc[r] = fma(c[s9 * 9 + 3 * r], x0, fma(c[s9 * 9 + 3 * r + 1], x1, fma(c[s9 * 9 + 3 * r + 2], x2, acc[r])));
+        }
+#pragma unroll
+        for (int r = 0; r < 3; ++r) z[r] -= acc[r];
+      };
+      if (BACK && first) {
+        if (m.mid > 0) sub_coupling(coupling_ptr(l, 0) + (size_t)pl * 81, yc + (size_t)(l - 1) * b * KB);
+        if (m.mid + 1 < m.nL) sub_coupling(coupling_ptr(l, 1) + (size_t)pl * 81, yc + (size_t)(l + 1) * b * KB);
+      } else if (!first) {
+        sub_coupling(cf + (size_t)pl * 81, uw - (ptrdiff_t)wlo * 3 * KB);
+      }
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        zo[(3 * pl + r) * KB + col] = z[r];
+        mx = max(mx, (__double2hiint(z[r]) >> 20) & 0x7ff);
+      }
+    }
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+    mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+    if (lane < KB) atomicMax(&zm[lane], mx);
+    __syncthreads();
+    if (tid < G * KB) cl.map_shared_rank(&zmax[g][tid % KB], tid / KB)[0] = zm[tid % KB];
+    cl.sync();
+    // the coupling buffer is free: request the next layer's
+    cpend = t + 1 < steps && cbytes > 0;
+    if (cpend && ok && tid == 0) {
+      tc::fence_async_smem();
+      tc::mbar_expect_tx(bar0 + 64, cbytes);
+      bulk_load(cf_s, coupling_ptr(layer_of(t + 1), cdir), cbytes, bar0 + 64);
+    }
+    // ---- digits of the own rows (in pairs) to every rank
+    if (tid < KB) zm[tid] = 0;
+    {
+      const int rows = 3 * (p1 - p0), col = tid % KB;
+      int ez = 0;
+      for (int q = 0; q < G; ++q) ez = max(ez, zmax[q][col]);
+      for (int e = tid; e < (rows + 1) / 2 * KB; e += 256) {
+        const int rp = e / KB;
+        const long long x0 = biased_fixed(zo[2 * rp * KB + col], ez);
+        const long long x1 = 2 * rp + 1 < rows ? biased_fixed(zo[(2 * rp + 1) * KB + col], ez) : DIG_BIAS;
+        uint32_t dg[DIG];
+#pragma unroll
+        for (int i = 0; i < DIG; ++i) dg[i] = digit_pair(x0, x1, i);
+        const int pos = (3 * p0 / 2 + rp) * KB + col;
+        for (int q = 0; q < G; ++q) {
+          uint32_t* z = cl.map_shared_rank(zd, q) + pos;
+#pragma unroll
+          for (int i = 0; i < DIG; ++i) z[i * nkb * 8 * KB] = dg[i];
+        }
+      }
+    }
+    cl.sync();
+    // ---- dense step on the own strips of 16 rows
+    for (int s = s0; s < s1; ++s, ++strip) {
+      for (int c = 0; c < NC; ++c, ++ci) {
+        const int slot = ci % a.ring;
+        if (ok) {
+          ok = tc::mbar_wait(bar0 + 8 * slot, (ci / a.ring) & 1);
+          if (ok) waited = ci + 1;
+        }
+        const int k0 = c * FX_KB + 2 * w, k1 = min(nkb, k0 + 2);
+        if (k0 < k1) {
+          float acc[DIG][4];
+#pragma unroll
+          for (int i = 0; i < DIG; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[i][e] = 0.f;
+          for (int kb = k0; kb < k1; ++kb) {
+            const longlong2* ap = reinterpret_cast<const longlong2*>(ring + (size_t)slot * FX_STAGE + (size_t)(kb - c * FX_KB) * 2048);
+            longlong2 x[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) x[j] = ap[j * 32 + lane];
+            uint32_t bz[DIG][2];
+            const uint32_t* zp = zd + (kb * 8 + (lane & 3)) * KB + (lane >> 2);
+#pragma unroll
+            for (int i = 0; i < DIG; ++i) {
+              bz[i][0] = zp[i * nkb * 8 * KB];
+              bz[i][1] = zp[i * nkb * 8 * KB + 4 * KB];
+            }
+#pragma unroll
+            for (int i = 0; i < DIG; ++i) {
+              uint32_t av[4];
+#pragma unroll
+              for (int j = 0; j < 4; ++j) av[j] = digit_pair(x[j].x, x[j].y, i);
+#pragma unroll
+              for (int j = DIG - 1 - i; j < DIG; ++j) mma_f16(acc[i + j - (DIG - 1)], av, bz[j]);
+            }
+          }
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            long long hi = 0, lo = 0;
+            digit_flush(acc, e, hi, lo);
+            unsigned long long* rd = red[strip & 1][((lane >> 2) + 8 * (e >> 1)) * KB + 2 * (lane & 3) + (e & 1)];
+            atomicAdd(rd, (unsigned long long)hi);
+            atomicAdd(rd + 1, (unsigned long long)lo);
+          }
+        }
+        __syncthreads();
+        if (tid == 0 && ok && ci + a.ring < total) {
+          tc::fence_async_smem();
+          issue(ci + a.ring);
+        }
+      }
+      if (tid < 128) {
+        const int row = s * 16 + tid / KB, col = tid % KB;
+        unsigned long long* rd = red[strip & 1][tid];
+        const long long hi = (long long)rd[0], lo = (long long)rd[1];
+        rd[0] = 0ull;
+        rd[1] = 0ull;
+        if (row < m.n) {
+          int ez = 0;
+          for (int q = 0; q < G; ++q) ez = max(ez, zmax[q][col]);
+          const int er = row_exponents(m, l)[row];
+          double y = digit_value(hi, lo, er + ez - 2 * 1023 - 66);
+          if (er == 0x7ff || ez == 0x7ff) y = __longlong_as_double(0x7ff8000000000000ll);   // Inf or NaN operands
+          double* yp = yc + ((size_t)l * b + row) * KB + col;
+          const double x = (BACK && !first) ? *yp - y : -y;   // the block holds -S^{-1}
+          const int p = row / 3;
+          if (!BACK) *yp = x;
+          else if (!first || half == 0) {
+            const size_t node = (size_t)l * m.npl + (size_t)(m.ia + p / m.njc) * m.nyn + m.ja + p % m.njc;
+            double* o = dst + (node * 3 + row % 3) * a.stride + col;
+            *o = a.add ? *o + x : x;
+          }
+          if (t + 1 < steps)
+            for (int q = 0; q < G; ++q) {
+              const int q0 = min(nn, npc * q), lo_n = max(0, q0 - m.njc - 1), hi_n = min(nn, min(nn, q0 + npc) + m.njc + 1);
+              if (p >= lo_n && p < hi_n) cl.map_shared_rank(uw, q)[(size_t)(row - 3 * lo_n) * KB + col] = x;
+            }
+        }
+      }
+    }
+    cl.sync();
+  }
+  if (!__syncthreads_and(ok) && tid == 0) {
+    for (int i = waited; i < issued; ++i) tc::mbar_wait(bar0 + 8 * (i % a.ring), (i / a.ring) & 1);
+    if (cphase > 0) tc::mbar_wait(bar0 + 64, (cphase - 1) & 1);
+    if (a.err != nullptr) atomicExch(a.err, 1);
+  }
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -673,11 +1017,13 @@ struct InvForm {
   };
   std::vector<Wave> waves;
   int rs = 8;                      // rows per stage of the solves (by the widest layer and the type)
+  bool digits = false;             // FP64: solves in digit products (k_inv_solve_fx)
 };
 
 namespace {
 
 constexpr int INV_SMEM = 225 * 1024;   // shared memory of one solve CTA
+constexpr int FX_SMEM = 221 * 1024;    // the same beside the digit solve's static arrays
 
 template <typename T>
 const void* solve_kernel_ptr(int rs, bool back) {
@@ -685,7 +1031,9 @@ const void* solve_kernel_ptr(int rs, bool back) {
   if (rs == 8) return back ? (const void*)k_inv_solve<T, 8, true> : (const void*)k_inv_solve<T, 8, false>;
   return back ? (const void*)k_inv_solve<T, 4, true> : (const void*)k_inv_solve<T, 4, false>;
 }
-const void* solve_kernel(const msgfem* h, int rs, bool back) {
+const void* solve_kernel(const msgfem* h, const InvForm& f, bool back) {
+  if (f.digits) return back ? (const void*)k_inv_solve_fx<true> : (const void*)k_inv_solve_fx<false>;
+  const int rs = f.rs;
   return h->mixed ? solve_kernel_ptr<float>(rs, back) : solve_kernel_ptr<double>(rs, back);
 }
 
@@ -694,12 +1042,18 @@ const void* solve_kernel(const msgfem* h, int rs, bool back) {
 int solve_layout(const msgfem* h, const InvForm& f, InvForm::Solve& s, int G, int ring) {
   const int es = h->mixed ? 4 : 8, vn = 16 / es;
   auto up = [](size_t v) { return (v + 127) / 128 * 128; };
-  size_t st = 0, z = 0, u = 0, c = 0;
+  size_t st = 0, z = 0, u = 0, c = 0, o = 0;
   for (int i : s.list) {
     const InvMat& m = f.mats[i];
     const int nn = m.n / 3, npc = up4((nn + G - 1) / G);
-    st = std::max(st, (size_t)f.rs * m.b * es);
-    z = std::max(z, (size_t)((m.b + vn - 1) / vn) * vn * (KB + 1) * es);
+    o = std::max(o, (size_t)npc * 3 * KB * es);
+    if (f.digits) {
+      z = std::max(z, (size_t)((m.n + 15) / 16) * DIG * 8 * KB * 4);
+      st = FX_STAGE;
+    } else {
+      st = std::max(st, (size_t)f.rs * m.b * es);
+      z = std::max(z, (size_t)((m.b + vn - 1) / vn) * vn * (KB + 1) * es);
+    }
     u = std::max(u, (size_t)std::min(nn, npc + 2 * (m.njc + 1)) * 3 * KB * es);
     c = std::max(c, (size_t)npc * 81 * es);
   }
@@ -709,7 +1063,7 @@ int solve_layout(const msgfem* h, const InvForm& f, InvForm::Solve& s, int G, in
   s.smem_u = (int)(s.smem_z + up(z));
   s.smem_c = (int)(s.smem_u + up(u));
   s.smem_r = (int)(s.smem_c + up(c));
-  s.smem = (int)(s.smem_r + up((size_t)2 * (8 / (f.rs / 4)) * f.rs * KB * es));
+  s.smem = (int)(s.smem_r + up(f.digits ? o : (size_t)2 * (8 / (f.rs / 4)) * f.rs * KB * es));
   return s.smem;
 }
 
@@ -740,7 +1094,8 @@ int resident_clusters(const void* kernel, int G, int smem) {
 void choose_solve(const msgfem* h, const InvForm& f, InvForm::Solve& s) {
   const int chains = 2 * (int)s.list.size();
   int most = 1;
-  for (int i : s.list) most = std::max(most, (f.mats[i].n + f.rs - 1) / f.rs / 2);
+  const int strip = f.digits ? 16 : f.rs;
+  for (int i : s.list) most = std::max(most, (f.mats[i].n + strip - 1) / strip / (f.digits ? 1 : 2));
   auto fit = [&](int G, int limit) {
     int ring = 8;
     while (ring > 2 && solve_layout(h, f, s, G, ring) > limit) --ring;
@@ -748,14 +1103,14 @@ void choose_solve(const msgfem* h, const InvForm& f, InvForm::Solve& s) {
   };
   for (int G : {8, 4, 2, 1}) {
     if (G > 1 && G > most) continue;
-    for (int limit : {INV_SMEM, 110 * 1024}) {
+    for (int limit : {f.digits ? FX_SMEM : INV_SMEM, 108 * 1024}) {
       if (!fit(G, limit)) continue;
-      if (resident_clusters(solve_kernel(h, f.rs, true), G, s.smem) >= chains) return;
+      if (resident_clusters(solve_kernel(h, f, true), G, s.smem) >= chains) return;
     }
   }
-  if (fit(1, 110 * 1024)) return;
+  if (fit(1, 108 * 1024)) return;
   for (int G : {1, 2, 4, 8})
-    if (fit(G, INV_SMEM)) return;
+    if (fit(G, f.digits ? FX_SMEM : INV_SMEM)) return;
 }
 
 }  // namespace
@@ -824,7 +1179,11 @@ bool inv_create(msgfem* h) {
   InvForm::Solve probe;
   for (int i = 0; i < (int)f->mats.size(); ++i)
     if (f->mats[i].n > 0) probe.list.push_back(i);
-  good = good && solve_layout(h, *f, probe, 8, 2) <= INV_SMEM;
+  if (good && !h->mixed && !probe.list.empty()) {
+    f->digits = true;
+    f->digits = solve_layout(h, *f, probe, 8, 2) <= FX_SMEM && (size_t)16 * (bmax + 2) * 8 <= (size_t)INV_SMEM;
+  }
+  good = good && (f->digits || solve_layout(h, *f, probe, 8, 2) <= INV_SMEM);
   if (!good) {
     delete f;
     return false;
@@ -850,6 +1209,9 @@ msgfem_status inv_build(msgfem* h) {
       }
     CK(cudaFuncSetAttribute(k_inv_step<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, inv_step_smem<double>()));
     CK(cudaFuncSetAttribute(k_inv_step<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, inv_step_smem<float>()));
+    for (const void* k : {(const void*)k_inv_solve_fx<false>, (const void*)k_inv_solve_fx<true>})
+      CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, FX_SMEM));
+    CK(cudaFuncSetAttribute(k_inv_digits, cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
     attr = true;
   }
   void* p = nullptr;
@@ -977,6 +1339,15 @@ static void inv_factor_t(msgfem* h, int w, cudaStream_t st) {
   for (int i : wv.all) maxl = std::max(maxl, f.mats[i].nL);
   k_inv_pack<T><<<dim3(maxl, (int)f.mats.size()), 256, 0, st>>>(f.d_mats, h->d_flags);
   ++g_launch_count;
+  if (f.digits) {
+    int bmax = 0, kmax = 0;
+    for (int i : wv.all) {
+      bmax = std::max(bmax, f.mats[i].b);
+      kmax = std::max(kmax, (f.mats[i].n + 15) / 16);
+    }
+    k_inv_digits<<<dim3(kmax, maxl, (int)f.mats.size()), 256, 16 * (bmax + 2) * 8, st>>>(f.d_mats, h->d_flags);
+    ++g_launch_count;
+  }
 }
 
 void inv_factor(msgfem* h, int w, cudaStream_t st) {
@@ -1021,7 +1392,7 @@ void inv_solve(msgfem* h, int mat, int src, int dst, int neg, int width, int add
     cfg.attrs = at;
     cfg.numAttrs = 1;
     for (bool back : {false, true}) {
-      cudaLaunchKernelExC(&cfg, solve_kernel(h, f.rs, back), args);
+      cudaLaunchKernelExC(&cfg, solve_kernel(h, f, back), args);
       ++g_launch_count;
     }
   }

@@ -20,6 +20,8 @@ CASES = {
     "narrow": dict(NX=30, NY=1, NZ=9, sx=5, sy=1, overlap=1, oversampling=2, n_loc=7),
     "one_tile_full": dict(NX=9, NY=2, NZ=6, sx=2, sy=1, overlap=1, oversampling=2, n_loc=7),
     "ragged": dict(NX=25, NY=7, NZ=8, sx=3, sy=2, overlap=2, oversampling=3, n_loc=9),
+    # FP64 layers too wide for the digit products' shared memory (plain FP64 products)
+    "dfma": dict(NX=18, NY=30, NZ=3, sx=2, sy=1, overlap=1, oversampling=2, n_loc=8),
     "wide": dict(NX=34, NY=16, NZ=4, sx=2, sy=1, overlap=1, oversampling=2, n_loc=8),
 }
 
