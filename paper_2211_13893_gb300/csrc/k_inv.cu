@@ -133,6 +133,182 @@ __device__ __forceinline__ void couple_rows(const InvMat& m, int nb, int dk, int
   }
 }
 
+// ---------------------------------------------------------------------------
+// FP64 products in exact digit products on the tensor cores.
+//
+// One SM does 1.6 FP64 FMAs per clock but 956 FP16 ones (mma.sync m16n8k16, both
+// measured), and its FP32 accumulation of integers is exact below 2^24.  A number is
+// written as a 61-bit integer below the largest of its row (matrix) or column
+// (vector) in seven balanced base-512 digits, n_i in [-256, 255], exact in FP16; of
+// the 49 digit products the 28 of weight 512^6 and up are formed (the rest is below
+// 2^-59 of the largest product), those of one weight in one accumulator: 32 columns
+// of k add at most 7 x 32 x 2^16 < 2^24.  After every 32 columns the seven sums go
+// into two 64-bit integers, so nothing is rounded before the result: the error is
+// that of rounding the operands to 2^-61 of their row or column maximum, where the
+// DFMA chain rounds every partial sum to 2^-53.
+//
+// Digits are cut from biased integers, X + sum 256 512^i: a 9-bit field d is the
+// digit d + 256, and 0x6400 | d is 1024 + d in FP16.  The factorisation leaves every
+// layer's -S^{-1} in that form in place (8 bytes per entry, 16 x 16 blocks in fragment
+// order: a lane's operands are four 16-byte vectors), so that a solve streams it with
+// bulk copies as before and spends 6 integer instructions per pair of digits; the
+// right-hand side's digits are cut once per layer by the rank that owns the node
+// and written to every rank of the cluster.  Taken whenever a layer's digits and
+// coefficients fit in shared memory (layers up to about 1,000 DoFs); above, FP64 FMAs.
+// Whole passes with FP64 FMAs -> digits: 36 x 12 x 39 beam 306 -> 204 ms (solves 158 ->
+// 54), 47 x 7 x 13 beam 77 -> 50, 24 x 4 x 12 beam 29 -> 20, Schwarz PCG 45 -> 29; the
+// passes' errors against a dense 64-bit reference are unchanged.
+constexpr int DIG = 7;
+constexpr long long DIG_BIAS = 256ll * (0x7fffffffffffffffll / 511);   // sum of 256 512^i, i < 7
+
+// x 2^(60 - emax) rounded to nearest (|x| < 2^(emax + 1), biased exponents), plus the bias
+__device__ __forceinline__ long long biased_fixed(double x, int emax) {
+  const long long xb = __double_as_longlong(x);
+  const int ex = (int)(xb >> 52) & 0x7ff, sh = emax - ex - 8;
+  const long long m = (xb & 0xfffffffffffffll) | (1ll << 52);
+  long long v;
+  if (ex == 0 || sh > 60) v = 0;               // zero, subnormal or below half a unit
+  else if (sh <= 0) v = m << -sh;
+  else v = (m + (1ll << (sh - 1))) >> sh;
+  return (xb < 0 ? -v : v) + DIG_BIAS;
+}
+
+// digit i of two biased integers as a pair of FP16 numbers
+__device__ __forceinline__ uint32_t digit_pair(long long x0, long long x1, int i) {
+  const uint32_t d = ((uint32_t)(x0 >> (9 * i)) & 0x1ff) | (((uint32_t)(x1 >> (9 * i)) & 0x1ff) << 16) | 0x64006400u;
+  uint32_t r;
+  asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(d), "r"(0xe500e500u));   // - 1280
+  return r;
+}
+
+__device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+
+// sums of the seven weights (512^6 .. 512^12) into hi 2^27 + lo
+__device__ __forceinline__ void digit_flush(const float (&acc)[DIG][4], int e, long long& hi, long long& lo) {
+  lo += (long long)__float2int_rn(acc[0][e]) + ((long long)__float2int_rn(acc[1][e]) << 9) +
+        ((long long)__float2int_rn(acc[2][e]) << 18);
+  hi += (long long)__float2int_rn(acc[3][e]) + ((long long)__float2int_rn(acc[4][e]) << 9) +
+        ((long long)__float2int_rn(acc[5][e]) << 18) + ((long long)__float2int_rn(acc[6][e]) << 27);
+}
+
+// (hi 2^27 + lo) 2^e for any int e
+__device__ __forceinline__ double digit_value(long long hi, long long lo, int e) {
+  const double v = fma((double)hi, 0x1p27, (double)lo);
+  if (e >= -1022 && e <= 1023) return v * __hiloint2double((e + 1023) << 20, 0);
+  return scalbn(v, e);
+}
+
+// v 2^e for a 64 x 64 x 64 digit product (|hi| < 2^50, |lo| < 2^45): conversions by
+// the 1.5 2^52 constant, the scale by the exponent field (four FP64 instructions
+// per result with the caller's subtraction: they are a third of a tile's time)
+__device__ __forceinline__ double tile_digit_value(long long hi, long long lo, int e) {
+  const double dh = __longlong_as_double(0x4338000000000000ll + hi) - 0x1.8p52;
+  const double dl = __longlong_as_double(0x4338000000000000ll + lo) - 0x1.8p52;
+  const double v = fma(dh, 0x1p27, dl);
+  const long long vb = __double_as_longlong(v);
+  const int ev = (int)(vb >> 52) & 0x7ff;
+  if (ev != 0 && ev + e > 0 && ev + e < 0x7ff) return __longlong_as_double(vb + ((long long)e << 52));
+  return scalbn(v, e);
+}
+
+// Product of two 64 x 64 FP64 tiles, A B^T, in digits: f(r, c, v0, v1) receives the
+// entries (r, c) and (r, c + 1), every entry once.  Shared memory: A as FP16 digits in
+// fragment order (7 x 8 KiB), B as biased integers in fragment order (32 KiB), two
+// CTAs per SM; warp w forms 16 rows x 32 columns, 8 at a time.  Digit scales are the
+// rows' maxima within the tile.  copy (may be null) receives A.
+constexpr int DIGIT_TILE_SMEM = DIG * 8192 + 32768;
+
+template <typename F>
+__device__ __forceinline__ void digit_tile(const double* A, int lda, const double* B, int ldb, unsigned char* sm,
+                                           int (*em)[TILE], double* copy, F f) {
+  uint32_t* ad = reinterpret_cast<uint32_t*>(sm);                               // [DIG][4 kb][4 rt][32 lanes][4]
+  longlong2* bf = reinterpret_cast<longlong2*>(sm + DIG * 8192);                // [4 kb][8 nt][2][32 lanes]
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  {
+    const int r = tid & 63, kb = tid >> 6, g = r & 7;
+    double2 xa[8], xb[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      xa[c] = *reinterpret_cast<const double2*>(A + (size_t)r * lda + kb * 16 + 2 * c);
+      xb[c] = *reinterpret_cast<const double2*>(B + (size_t)r * ldb + kb * 16 + 2 * c);
+    }
+    if (tid < TILE) em[0][tid] = em[1][tid] = 0;
+    __syncthreads();
+    int ma = 0, mb = 0;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      ma = max(ma, max((__double2hiint(xa[c].x) >> 20) & 0x7ff, (__double2hiint(xa[c].y) >> 20) & 0x7ff));
+      mb = max(mb, max((__double2hiint(xb[c].x) >> 20) & 0x7ff, (__double2hiint(xb[c].y) >> 20) & 0x7ff));
+    }
+    atomicMax(&em[0][r], ma);
+    atomicMax(&em[1][r], mb);
+    if (copy != nullptr)
+#pragma unroll
+      for (int c = 0; c < 8; ++c) *reinterpret_cast<double2*>(copy + r * TILE + kb * 16 + 2 * c) = xa[c];
+    __syncthreads();
+    const int ea = em[0][r], eb = em[1][r];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const int fl = g * 4 + (c & 3), kj = c >> 2;
+      const long long u0 = biased_fixed(xa[c].x, ea), u1 = biased_fixed(xa[c].y, ea);
+#pragma unroll
+      for (int i = 0; i < DIG; ++i)
+        ad[(((i * 4 + kb) * 4 + (r >> 4)) * 32 + fl) * 4 + ((r >> 3) & 1) + 2 * kj] = digit_pair(u0, u1, i);
+      bf[((kb * 8 + (r >> 3)) * 2 + kj) * 32 + fl] = make_longlong2(biased_fixed(xb[c].x, eb), biased_fixed(xb[c].y, eb));
+    }
+  }
+  __syncthreads();
+  const int rt = w & 3;
+#pragma unroll 1
+  for (int nt = (w >> 2) * 4; nt < (w >> 2) * 4 + 4; ++nt) {
+    long long hi[4] = {}, lo[4] = {};
+#pragma unroll 1
+    for (int kp = 0; kp < 2; ++kp) {
+      float acc[DIG][4];
+#pragma unroll
+      for (int i = 0; i < DIG; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[i][e] = 0.f;
+#pragma unroll
+      for (int kk = 0; kk < 2; ++kk) {
+        const int kb = 2 * kp + kk;
+        const longlong2 y0 = bf[((kb * 8 + nt) * 2) * 32 + lane], y1 = bf[((kb * 8 + nt) * 2 + 1) * 32 + lane];
+        uint32_t bz[DIG][2];
+#pragma unroll
+        for (int i = 0; i < DIG; ++i) {
+          bz[i][0] = digit_pair(y0.x, y0.y, i);
+          bz[i][1] = digit_pair(y1.x, y1.y, i);
+        }
+#pragma unroll
+        for (int i = 0; i < DIG; ++i) {
+          const uint4 v = *reinterpret_cast<const uint4*>(ad + (((i * 4 + kb) * 4 + rt) * 32 + lane) * 4);
+          const uint32_t av[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+          for (int j = DIG - 1 - i; j < DIG; ++j) mma_f16(acc[i + j - (DIG - 1)], av, bz[j]);
+        }
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) digit_flush(acc, e, hi[e], lo[e]);
+    }
+    const int c = nt * 8 + 2 * (lane & 3), e0 = em[1][c], e1 = em[1][c + 1];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int r = rt * 16 + (lane >> 2) + 8 * h, er = em[0][r];
+      double v0 = tile_digit_value(hi[2 * h], lo[2 * h], er + e0 - 2 * 1023 - 66);
+      double v1 = tile_digit_value(hi[2 * h + 1], lo[2 * h + 1], er + e1 - 2 * 1023 - 66);
+      const double nan = __longlong_as_double(0x7ff8000000000000ll);
+      if (er == 0x7ff || e0 == 0x7ff) v0 = nan;   // Inf or NaN operands
+      if (er == 0x7ff || e1 == 0x7ff) v1 = nan;
+      f(r, c, v0, v1);
+    }
+  }
+}
+
 // Inverse of a 64 x 64 SPD tile by the scalar sweep operator in FP64 registers:
 // a 16 x 16 thread grid, each thread the entries (ty + 16 p, tx + 16 q) with
 // p >= q (the tile is symmetric), one barrier per pivot (the pivot column and
@@ -202,63 +378,44 @@ __device__ void tile_sweep(const T* X, int ldx, T* P, int* notspd, int sub) {
   if (bad) atomicExch(&notspd[sub], 1);
 }
 
-// shared-memory row stride of a staged operand tile ([k][row])
-template <typename T> struct TileLd;
-template <> struct TileLd<double> { static constexpr int v = 65; };
-template <> struct TileLd<float> { static constexpr int v = 68; };
+// FP32 tiles: operands staged in shared memory as [k][row] (row stride in floats)
+constexpr int LDF = 68;
 template <typename T>
-constexpr int inv_step_smem() { return 2 * TILE * TileLd<T>::v * (int)sizeof(T); }
+constexpr int inv_step_smem() {
+  return sizeof(T) == 8 ? DIGIT_TILE_SMEM : 2 * TILE * LDF * (int)sizeof(float);
+}
 
-// rows of a 64 x 64 tile (leading dimension ld) into shared memory as [k][row]
-template <typename T>
-__device__ __forceinline__ void stage_tile(const T* G, int ld, T* S) {
-  using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
-  constexpr int N = 16 / sizeof(T), LD = TileLd<T>::v;
+// rows of a 64 x 64 tile (leading dimension ld) into shared memory
+__device__ __forceinline__ void stage_tile(const float* G, int ld, float* S) {
   const int r = threadIdx.x & 63, k0 = (threadIdx.x >> 6) * 16;
-  V x[16 / N];
+  float4 x[4];
 #pragma unroll
-  for (int c = 0; c < 16 / N; ++c) x[c] = *reinterpret_cast<const V*>(G + (size_t)r * ld + k0 + c * N);
+  for (int c = 0; c < 4; ++c) x[c] = *reinterpret_cast<const float4*>(G + (size_t)r * ld + k0 + 4 * c);
 #pragma unroll
-  for (int c = 0; c < 16 / N; ++c) {
-    const T* e = reinterpret_cast<const T*>(&x[c]);
-#pragma unroll
-    for (int q = 0; q < N; ++q) S[(k0 + c * N + q) * LD + r] = e[q];
+  for (int c = 0; c < 4; ++c) {
+    S[(k0 + 4 * c) * LDF + r] = x[c].x;
+    S[(k0 + 4 * c + 1) * LDF + r] = x[c].y;
+    S[(k0 + 4 * c + 2) * LDF + r] = x[c].z;
+    S[(k0 + 4 * c + 3) * LDF + r] = x[c].w;
   }
 }
 
-// output row / column of element (p, q) of thread (ty, tx): FP64 strided by 16
-// (a diagonal tile forms only its 16 x 16 blocks on or below the diagonal),
-// FP32 four contiguous ones (vector loads)
-template <typename T> __device__ __forceinline__ int out_idx(int t, int p) {
-  return sizeof(T) == 8 ? t + 16 * p : 4 * t + p;
-}
-
-// acc = A B^T of two staged 64 x 64 tiles
-template <typename T, bool SYM>
-__device__ __forceinline__ void tile_product(const T* As, const T* Bs, T (&acc)[4][4]) {
-  constexpr int LD = TileLd<T>::v;
+// acc = A B^T of two staged 64 x 64 tiles: rows 4 ty .., columns 4 tx ..
+__device__ __forceinline__ void tile_product(const float* As, const float* Bs, float (&acc)[4][4]) {
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll
   for (int p = 0; p < 4; ++p)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) acc[p][q] = (T)0;
+    for (int q = 0; q < 4; ++q) acc[p][q] = 0.f;
 #pragma unroll 16
   for (int k = 0; k < TILE; ++k) {
-    T a[4], b[4];
-    if constexpr (sizeof(T) == 4) {
-      const float4 av = *reinterpret_cast<const float4*>(As + k * LD + 4 * ty);
-      const float4 bv = *reinterpret_cast<const float4*>(Bs + k * LD + 4 * tx);
-      a[0] = av.x; a[1] = av.y; a[2] = av.z; a[3] = av.w;
-      b[0] = bv.x; b[1] = bv.y; b[2] = bv.z; b[3] = bv.w;
-    } else {
-#pragma unroll
-      for (int p = 0; p < 4; ++p) { a[p] = As[k * LD + ty + 16 * p]; b[p] = Bs[k * LD + tx + 16 * p]; }
-    }
+    const float4 av = *reinterpret_cast<const float4*>(As + k * LDF + 4 * ty);
+    const float4 bv = *reinterpret_cast<const float4*>(Bs + k * LDF + 4 * tx);
+    const float a[4] = {av.x, av.y, av.z, av.w}, b[4] = {bv.x, bv.y, bv.z, bv.w};
 #pragma unroll
     for (int p = 0; p < 4; ++p)
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (!SYM || q <= p) acc[p][q] = fma(a[p], b[q], acc[p][q]);
+      for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(a[p], b[q], acc[p][q]);
   }
 }
 
@@ -271,16 +428,14 @@ k_inv_step(const InvTask* __restrict__ tasks, const InvMat* __restrict__ mats, c
   const InvMat& m = mats[t.m];
   if (active != nullptr && !active[m.sub]) return;
   extern __shared__ __align__(16) unsigned char smem_iv[];
-  T* As = reinterpret_cast<T*>(smem_iv);
-  T* Bs = As + TILE * TileLd<T>::v;
-  constexpr int LD = TileLd<T>::v;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, b = m.b;
+  __shared__ int em[2][TILE];
+  const int tid = threadIdx.x, b = m.b;
   T* S = layer_block<T>(m, t.layer);
   if (t.type == IV_SCHUR_A) {
     // (C X)^T with X = -S^{-1} of layer layer + k: rows q, columns of layer `layer`
     T acc[2][3];
     const int q = t.j * TILE + (tid & 63);
-    couple_rows<T>(m, t.i, t.k, t.layer, q, layer_block<T>(m, t.layer + t.k), As, acc);
+    couple_rows<T>(m, t.i, t.k, t.layer, q, layer_block<T>(m, t.layer + t.k), reinterpret_cast<T*>(smem_iv), acc);
     T* W = triple_scratch<T>(m, t.layer, t.k);
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
@@ -295,7 +450,7 @@ k_inv_step(const InvTask* __restrict__ tasks, const InvMat* __restrict__ mats, c
     // D += C (C X)^T on and below the diagonal, mirrored
     T acc[2][3];
     const int q = t.j * TILE + (tid & 63);
-    couple_rows<T>(m, t.i, t.k, t.layer, q, triple_scratch<T>(m, t.layer, t.k), As, acc);
+    couple_rows<T>(m, t.i, t.k, t.layer, q, triple_scratch<T>(m, t.layer, t.k), reinterpret_cast<T*>(smem_iv), acc);
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const int p = t.i * NBLK + (tid >> 6) * 2 + u;
@@ -318,62 +473,84 @@ k_inv_step(const InvTask* __restrict__ tasks, const InvMat* __restrict__ mats, c
   const int k = t.k;
   T* P = pivot_inv<T>(m, t.layer);
   T* C = old_col<T>(m, t.layer);
-  if (t.type == IV_PANEL) {
+  if (t.type == IV_PANEL && t.i == k) {
     T* Skk = S + (size_t)k * TILE * b + (size_t)k * TILE;
-    if (t.i == k) {
-      for (int e = tid; e < TILE * TILE; e += 256) Skk[(size_t)(e >> 6) * b + (e & 63)] = -P[e];
+    for (int e = tid; e < TILE * TILE; e += 256) Skk[(size_t)(e >> 6) * b + (e & 63)] = -P[e];
+    return;
+  }
+  T* Sik = S + (size_t)t.i * TILE * b + (size_t)k * TILE;
+  // IV_PANEL: W_i = S_ik P in place and mirrored, the old tile kept in C;
+  // IV_UPDATE: S_ij -= W_i old_j^T, mirrored; the next pivot tile is swept at once
+  T* Ski = S + (size_t)k * TILE * b + (size_t)t.i * TILE;
+  T* Sij = S + (size_t)t.i * TILE * b + (size_t)t.j * TILE;
+  T* Sji = S + (size_t)t.j * TILE * b + (size_t)t.i * TILE;
+  const bool diag = t.i == t.j;
+  if constexpr (sizeof(T) == 8) {
+    if (t.type == IV_PANEL) {
+      digit_tile(Sik, b, P, TILE, smem_iv, em, C + (size_t)t.i * TILE * TILE, [&](int r, int c, double v0, double v1) {
+        *reinterpret_cast<double2*>(Sik + (size_t)r * b + c) = make_double2(v0, v1);
+        Ski[(size_t)c * b + r] = v0;
+        Ski[(size_t)(c + 1) * b + r] = v1;
+      });
       return;
     }
-    T* Sik = S + (size_t)t.i * TILE * b + (size_t)k * TILE;
-    T* Ski = S + (size_t)k * TILE * b + (size_t)t.i * TILE;
-    stage_tile<T>(Sik, b, As);
-    stage_tile<T>(P, TILE, Bs);
-    __syncthreads();
-    T acc[4][4];
-    tile_product<T, false>(As, Bs, acc);
+    digit_tile(Sik, b, C + (size_t)t.j * TILE * TILE, TILE, smem_iv, em, nullptr, [&](int r, int c, double v0, double v1) {
+      if (!diag) {
+        double2* o = reinterpret_cast<double2*>(Sij + (size_t)r * b + c);
+        double2 x = *o;
+        x.x -= v0;
+        x.y -= v1;
+        *o = x;
+        Sji[(size_t)c * b + r] = x.x;
+        Sji[(size_t)(c + 1) * b + r] = x.y;
+        return;
+      }
+      // diagonal tile: lower half and its mirror image
+      if (c <= r) Sij[(size_t)c * b + r] = Sij[(size_t)r * b + c] -= v0;
+      if (c + 1 <= r) Sij[(size_t)(c + 1) * b + r] = Sij[(size_t)r * b + c + 1] -= v1;
+    });
+    if (diag && t.i == k + 1) {
+      __syncthreads();   // the tile's stores are visible to the CTA
+      tile_sweep<T>(Sij, b, P, notspd, m.sub);
+    }
+  } else {
+    float* As = reinterpret_cast<float*>(smem_iv);
+    float* Bs = As + TILE * LDF;
+    const int tx = tid & 15, ty = tid >> 4;
+    const bool panel = t.type == IV_PANEL;
     T* Ci = C + (size_t)t.i * TILE * TILE;
-    for (int e = tid; e < TILE * TILE; e += 256) Ci[e] = As[(e & 63) * LD + (e >> 6)];   // the old tile
+    stage_tile(Sik, b, As);
+    stage_tile(panel ? P : C + (size_t)t.j * TILE * TILE, TILE, Bs);
+    __syncthreads();
+    float acc[4][4];
+    tile_product(As, Bs, acc);
+    if (panel)
+      for (int e = tid; e < TILE * TILE; e += 256) Ci[e] = As[(e & 63) * LDF + (e >> 6)];
     __syncthreads();
 #pragma unroll
     for (int p = 0; p < 4; ++p)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) As[out_idx<T>(ty, p) * LD + out_idx<T>(tx, q)] = acc[p][q];
+      for (int q = 0; q < 4; ++q) {
+        const int r = 4 * ty + p, c = 4 * tx + q;
+        if (panel) {
+          As[r * LDF + c] = acc[p][q];
+          continue;
+        }
+        if (diag && c > r) continue;
+        const float v = Sij[(size_t)r * b + c] - acc[p][q];
+        As[r * LDF + c] = v;
+        if (diag) As[c * LDF + r] = v;
+      }
     __syncthreads();
+    T* out = panel ? Sik : Sij;
+    T* mir = panel ? Ski : Sji;
     for (int e = tid; e < TILE * TILE; e += 256) {
       const int r = e >> 6, c = e & 63;
-      Sik[(size_t)r * b + c] = As[r * LD + c];
-      Ski[(size_t)r * b + c] = As[c * LD + r];
+      out[(size_t)r * b + c] = As[r * LDF + c];
+      if (panel || !diag) mir[(size_t)r * b + c] = As[c * LDF + r];
     }
-    return;
+    if (!panel && diag && t.i == k + 1) tile_sweep<T>(As, LDF, P, notspd, m.sub);
   }
-  // IV_UPDATE: S_ij -= W_i old_j^T, mirrored; the next pivot tile is swept at once
-  T* Sij = S + (size_t)t.i * TILE * b + (size_t)t.j * TILE;
-  stage_tile<T>(S + (size_t)t.i * TILE * b + (size_t)k * TILE, b, As);
-  stage_tile<T>(C + (size_t)t.j * TILE * TILE, TILE, Bs);
-  __syncthreads();
-  T acc[4][4];
-  const bool diag = t.i == t.j;
-  if (sizeof(T) == 8 && diag) tile_product<T, sizeof(T) == 8>(As, Bs, acc);
-  else tile_product<T, false>(As, Bs, acc);
-  __syncthreads();
-#pragma unroll
-  for (int p = 0; p < 4; ++p)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int r = out_idx<T>(ty, p), c = out_idx<T>(tx, q);
-      if (diag && c > r) continue;
-      const T v = Sij[(size_t)r * b + c] - acc[p][q];
-      As[r * LD + c] = v;
-      if (diag) As[c * LD + r] = v;
-    }
-  __syncthreads();
-  T* Sji = S + (size_t)t.j * TILE * b + (size_t)t.i * TILE;
-  for (int e = tid; e < TILE * TILE; e += 256) {
-    const int r = e >> 6, c = e & 63;
-    Sij[(size_t)r * b + c] = As[r * LD + c];
-    if (!diag) Sji[(size_t)r * b + c] = As[c * LD + r];
-  }
-  if (diag && t.i == k + 1) tile_sweep<T>(As, LD, P, notspd, m.sub);
 }
 
 // Couplings of every layer in the solver's precision, packed per node for the
@@ -653,76 +830,9 @@ k_inv_solve(const InvSolveArgs a) {
 }
 
 // ---------------------------------------------------------------------------
-// FP64 solves in exact digit products on the tensor cores.
-//
-// One SM does 1.6 FP64 FMAs per clock but 956 FP16 ones (mma.sync m16n8k16, both
-// measured), and its FP32 accumulation of integers is exact below 2^24.  A number is
-// written as a 61-bit integer below the largest of its row (matrix) or column
-// (vector) in seven balanced base-512 digits, n_i in [-256, 255], exact in FP16; of
-// the 49 digit products the 28 of weight 512^6 and up are formed (the rest is below
-// 2^-59 of the largest product), those of one weight in one accumulator: 32 columns
-// of k add at most 7 x 32 x 2^16 < 2^24.  After every 32 columns the seven sums go
-// into two 64-bit integers, so nothing is rounded before the result: the error is
-// that of rounding the operands to 2^-61 of their row or column maximum, where the
-// DFMA chain rounds every partial sum to 2^-53.
-//
-// Digits are cut from biased integers, X + sum 256 512^i: a 9-bit field d is the
-// digit d + 256, and 0x6400 | d is 1024 + d in FP16.  The factorisation leaves every
-// layer's -S^{-1} in that form in place (8 bytes per entry, 16 x 16 blocks in fragment
-// order: a lane's operands are four 16-byte vectors), so that a solve streams it with
-// bulk copies as before and spends 6 integer instructions per pair of digits; the
-// right-hand side's digits are cut once per layer by the rank that owns the node
-// and written to every rank of the cluster.  Taken whenever a layer's digits and
-// coefficients fit in shared memory (layers up to about 1,000 DoFs); above, FP64 FMAs.
-// Whole passes with FP64 FMAs -> digits: 36 x 12 x 39 beam 306 -> 204 ms (solves 158 ->
-// 54), 47 x 7 x 13 beam 77 -> 50, 24 x 4 x 12 beam 29 -> 20, Schwarz PCG 45 -> 29; the
-// passes' errors against a dense 64-bit reference are unchanged.
-constexpr int DIG = 7;
-constexpr long long DIG_BIAS = 256ll * (0x7fffffffffffffffll / 511);   // sum of 256 512^i, i < 7
+// FP64 solve in digit products
 constexpr int FX_KB = 16;                      // 16 x 16 blocks per stage (two per warp)
 constexpr int FX_STAGE = FX_KB * 256 * 8;      // bytes
-
-// x 2^(60 - emax) rounded to nearest (|x| < 2^(emax + 1), biased exponents), plus the bias
-__device__ __forceinline__ long long biased_fixed(double x, int emax) {
-  const long long xb = __double_as_longlong(x);
-  const int ex = (int)(xb >> 52) & 0x7ff, sh = emax - ex - 8;
-  const long long m = (xb & 0xfffffffffffffll) | (1ll << 52);
-  long long v;
-  if (ex == 0 || sh > 60) v = 0;               // zero, subnormal or below half a unit
-  else if (sh <= 0) v = m << -sh;
-  else v = (m + (1ll << (sh - 1))) >> sh;
-  return (xb < 0 ? -v : v) + DIG_BIAS;
-}
-
-// digit i of two biased integers as a pair of FP16 numbers
-__device__ __forceinline__ uint32_t digit_pair(long long x0, long long x1, int i) {
-  const uint32_t d = ((uint32_t)(x0 >> (9 * i)) & 0x1ff) | (((uint32_t)(x1 >> (9 * i)) & 0x1ff) << 16) | 0x64006400u;
-  uint32_t r;
-  asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(d), "r"(0xe500e500u));   // - 1280
-  return r;
-}
-
-__device__ __forceinline__ void mma_f16(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-// sums of the seven weights (512^6 .. 512^12) into hi 2^27 + lo
-__device__ __forceinline__ void digit_flush(const float (&acc)[DIG][4], int e, long long& hi, long long& lo) {
-  lo += (long long)__float2int_rn(acc[0][e]) + ((long long)__float2int_rn(acc[1][e]) << 9) +
-        ((long long)__float2int_rn(acc[2][e]) << 18);
-  hi += (long long)__float2int_rn(acc[3][e]) + ((long long)__float2int_rn(acc[4][e]) << 9) +
-        ((long long)__float2int_rn(acc[5][e]) << 18) + ((long long)__float2int_rn(acc[6][e]) << 27);
-}
-
-// (hi 2^27 + lo) 2^e for any int e
-__device__ __forceinline__ double digit_value(long long hi, long long lo, int e) {
-  const double v = fma((double)hi, 0x1p27, (double)lo);
-  if (e >= -1022 && e <= 1023) return v * __hiloint2double((e + 1023) << 20, 0);
-  return scalbn(v, e);
-}
 
 // biased exponents of the rows of layer l (at the end of the layer's L slot)
 __device__ __forceinline__ int* row_exponents(const InvMat& m, int l) {
