@@ -1490,32 +1490,53 @@ msgfem_status msgfem_coarse_assemble_threshold(msgfem_h h, double t, int* coarse
   for (int j = 0; j < h->N; ++j) { h->coff[j] = Nc; Nc += h->basis_m[j]; }
   const int NcPad = (Nc + TILE - 1) / TILE * TILE;
   if (NcPad != h->NcPad) {
-    h->NcPad = NcPad;
-    TRY(dalloc(h, &h->d_AH, (size_t)NcPad * NcPad));
-    TRY(dalloc(h, &h->d_AHinv, (size_t)NcPad * NcPad));
-    {
-      // the coarse inverse's split rows: scratch tiles and the identity strip
-      size_t tiles = 0;
-      int maxc = 1;
-      coarse_inverse_split_sizes(NcPad / TILE, COARSE_INV_SPLIT, &tiles, &maxc);
-      TRY(dalloc(h, &h->d_cscr, std::max<size_t>(tiles, 1) * TILE * TILE));
-      std::vector<double> id((size_t)TILE * maxc * TILE, 0.0);
-      for (int r = 0; r < TILE; ++r)
-        for (int c = 0; c < maxc; ++c) id[(size_t)r * maxc * TILE + (size_t)c * TILE + r] = 1.0;
-      TRY(dalloc(h, &h->d_cid, id.size()));
-      CK(cudaMemcpy(h->d_cid, id.data(), id.size() * sizeof(double), cudaMemcpyHostToDevice));
+    h->NcPad = 0;
+    if (NcPad > h->NcCap) {   // a smaller coarse space keeps the arrays
+      h->NcCap = 0;
+      for (double** p : {&h->d_AH, &h->d_AHinv, &h->d_AHkeep, &h->d_bH, &h->d_cH, &h->d_yH, &h->d_rH, &h->d_cscr, &h->d_cid}) {
+        dfree(h, *p);
+        *p = nullptr;
+      }
+      TRY(dalloc(h, &h->d_AH, (size_t)NcPad * NcPad));
+      TRY(dalloc(h, &h->d_AHinv, (size_t)NcPad * NcPad));
+      TRY(dalloc(h, &h->d_bH, (size_t)NcPad * PST));
+      TRY(dalloc(h, &h->d_cH, (size_t)NcPad * PST));
+      TRY(dalloc(h, &h->d_yH, (size_t)NcPad * PST));
+      TRY(dalloc(h, &h->d_rH, (size_t)NcPad * PST));
+      if (h->inv) TRY(dalloc(h, &h->d_AHkeep, (size_t)NcPad * NcPad));
+      h->NcCap = NcPad;
     }
-    TRY(dalloc(h, &h->d_bH, (size_t)NcPad * PST));
-    TRY(dalloc(h, &h->d_cH, (size_t)NcPad * PST));
-    TRY(dalloc(h, &h->d_yH, (size_t)NcPad * PST));
-    TRY(dalloc(h, &h->d_rH, (size_t)NcPad * PST));
-    build_coarse_schedules(h);
-    TRY(dalloc(h, &h->cfact.d_gemm, h->cfact.gemm.size()));
-    CK(cudaMemcpy(h->cfact.d_gemm, h->cfact.gemm.data(), h->cfact.gemm.size() * sizeof(GemmTask),
-                  cudaMemcpyHostToDevice));
-    TRY(dalloc(h, &h->csolve.d_tasks, h->csolve.tasks.size()));
-    CK(cudaMemcpy(h->csolve.d_tasks, h->csolve.tasks.data(), h->csolve.tasks.size() * sizeof(SolveTask),
-                  cudaMemcpyHostToDevice));
+    h->NcPad = NcPad;
+    if (h->inv) {
+      TRY(coarse_inv_build(h));
+    } else {
+      {
+        // the coarse inverse's split rows: scratch tiles and the identity strip
+        size_t tiles = 0;
+        int maxc = 1;
+        coarse_inverse_split_sizes(NcPad / TILE, COARSE_INV_SPLIT, &tiles, &maxc);
+        dfree(h, h->d_cscr);
+        dfree(h, h->d_cid);
+        h->d_cscr = h->d_cid = nullptr;
+        TRY(dalloc(h, &h->d_cscr, std::max<size_t>(tiles, 1) * TILE * TILE));
+        std::vector<double> id((size_t)TILE * maxc * TILE, 0.0);
+        for (int r = 0; r < TILE; ++r)
+          for (int c = 0; c < maxc; ++c) id[(size_t)r * maxc * TILE + (size_t)c * TILE + r] = 1.0;
+        TRY(dalloc(h, &h->d_cid, id.size()));
+        CK(cudaMemcpy(h->d_cid, id.data(), id.size() * sizeof(double), cudaMemcpyHostToDevice));
+      }
+      build_coarse_schedules(h);
+      dfree(h, h->cfact.d_gemm);
+      dfree(h, h->csolve.d_tasks);
+      h->cfact.d_gemm = nullptr;
+      h->csolve.d_tasks = nullptr;
+      TRY(dalloc(h, &h->cfact.d_gemm, h->cfact.gemm.size()));
+      CK(cudaMemcpy(h->cfact.d_gemm, h->cfact.gemm.data(), h->cfact.gemm.size() * sizeof(GemmTask),
+                    cudaMemcpyHostToDevice));
+      TRY(dalloc(h, &h->csolve.d_tasks, h->csolve.tasks.size()));
+      CK(cudaMemcpy(h->csolve.d_tasks, h->csolve.tasks.data(), h->csolve.tasks.size() * sizeof(SolveTask),
+                    cudaMemcpyHostToDevice));
+    }
   }
   h->Nc = Nc;
   CK(cudaMemcpyAsync(h->d_coff, h->coff.data(), h->N * sizeof(int), cudaMemcpyHostToDevice, st));
@@ -1524,7 +1545,12 @@ msgfem_status msgfem_coarse_assemble_threshold(msgfem_h h, double t, int* coarse
   launch_coarse_blocks(h);
   launch_coarse_rhs(h);
   CK(cudaMemsetAsync(h->d_notspd + h->N, 0, sizeof(int), st));
-  run_schedule(h->cfact, st);
+  if (h->inv) {
+    CK(cudaMemcpyAsync(h->d_AHkeep, h->d_AH, (size_t)NcPad * NcPad * sizeof(double), cudaMemcpyDeviceToDevice, st));
+    coarse_inv_factor(h);
+  } else {
+    run_schedule(h->cfact, st);
+  }
   span_end(h, sp_c);
   CK_LAUNCH();
   spans_collect(h);
@@ -1546,7 +1572,7 @@ msgfem_status msgfem_solve(msgfem_h h, double* u_out, const double* u_ref, doubl
   cudaStream_t st = h->stream;
   set_dense_context(h->d_flags, h->d_notspd, h->d_sub);
   const int sp_c = span_begin(h, TAG_COARSE);
-  run_solve_mv(h->csolve, st, 0, 0, 0);
+  launch_coarse_solve(h, st, 1);
   launch_prolong(h);
   span_end(h, sp_c);
   CK_LAUNCH();

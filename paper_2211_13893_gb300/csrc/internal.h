@@ -258,12 +258,13 @@ struct msgfem {
   std::vector<CoarsePair> pairs;
   CoarsePair* d_pairs = nullptr;
   double* d_pair_part = nullptr;
-  int Nc = 0, NcPad = 0;
+  int Nc = 0, NcPad = 0, NcCap = 0;  // coarse size, padded to tiles, padded size the arrays hold
   std::vector<int> coff;
   int* d_coff = nullptr;
   int* d_m = nullptr;
   double* d_AH = nullptr;
   double* d_AHinv = nullptr;
+  double* d_AHkeep = nullptr; // inverse form: A_H itself, for the correction of the coarse solve
   double* d_cscr = nullptr;   // scratch tiles of the coarse inverse's split rows
   double* d_cid = nullptr;    // identity strip [I I ... I] of the coarse inverse
   double* d_bH = nullptr;
@@ -378,6 +379,12 @@ msgfem_status inv_build(msgfem* h);
 void inv_factor(msgfem* h, int w, cudaStream_t st);
 void inv_solve(msgfem* h, int mat, int src, int dst, int neg, int width, int add);
 double inv_factor_flops(const msgfem* h, bool executed);
+// the coarse matrix in the same form: tasks for the current NcPad, sweep of d_AH in place
+msgfem_status coarse_inv_build(msgfem* h);
+void coarse_inv_factor(msgfem* h);
+// c = A_H^{-1} b on stream st (column 0 of cH and bH) by the block Cholesky or, when the
+// handle has the inverse form, by the inverse, with `refine` corrections by the kept A_H
+void launch_coarse_solve(msgfem* h, cudaStream_t st, int refine);
 // Structured numbering of a hexahedron list (hexmesh.cpp): the (i, j, k) block
 // dimensions and, for every node and element of the list, its structured id.
 struct HexNumbering {
@@ -455,6 +462,7 @@ constexpr double PCG_TOL = 1e-11;
 void launch_refine_check_tol(msgfem* h, int wr, int keep, int step, double tol);
 void launch_coarse_blocks(msgfem* h);
 void launch_coarse_rhs(msgfem* h);
+void launch_coarse_restrict(msgfem* h, const double* r, cudaStream_t st);
 void launch_prolong(msgfem* h);
 int energy_blocks(msgfem* h);
 void launch_energy(msgfem* h, const double* d_ref, const double* d_u, double* d_out);

@@ -87,21 +87,58 @@ __global__ void k_symmetrize(double* AH, int Nc, int ld) {
   }
 }
 
-// b^H rows of subdomain s: sum_r CB[r][a] b[r]; one block per subdomain.
-__global__ void k_coarse_rhs(const SubDev* __restrict__ subs, const int* __restrict__ coff,
-                             const int* __restrict__ msz, double* __restrict__ bH) {
-  const SubDev& s = subs[blockIdx.x];
+// V_s^T v over chunks of rows, v = the subdomain's load (r = NULL) or the global
+// vector r: RCH blocks per subdomain write partial sums (one block per subdomain took
+// 155 to 770 us, bound by one SM's load latency), added in a fixed order.
+constexpr int RCH = 32;
+
+__global__ void __launch_bounds__(256)
+k_restrict_partial(const SubDev* __restrict__ subs, const double* __restrict__ r, int NY, int NZ, double* __restrict__ part) {
+  const SubDev& s = subs[blockIdx.y];
   __shared__ double red[8][PST];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int per = (s.nfull + RCH - 1) / RCH, r0 = blockIdx.x * per, r1 = min(r0 + per, s.nfull);
   double acc = 0.0;
-  for (int r = w; r < s.nfull; r += 8) acc = fma(s.CB[(size_t)r * PST + lane], s.bload[r], acc);
+#pragma unroll 4
+  for (int row = r0 + w; row < r1; row += 8) {
+    double v;
+    if (r == nullptr) {
+      v = s.bload[row];
+    } else {
+      const int n = row / 3, k = n / s.npl, q = n % s.npl;
+      v = r[3 * ((size_t)((s.I0 + q / s.nyn) * (NY + 1) + s.J0 + q % s.nyn) * (NZ + 1) + k) + row % 3];
+    }
+    acc = fma(s.CB[(size_t)row * PST + lane], v, acc);
+  }
   red[w][lane] = acc;
   __syncthreads();
   if (w == 0) {
     double t = 0.0;
     for (int i = 0; i < 8; ++i) t += red[i][lane];
-    if (lane < msz[blockIdx.x]) bH[(size_t)(coff[blockIdx.x] + lane) * PST] = t;
+    part[((size_t)blockIdx.y * RCH + blockIdx.x) * PST + lane] = t;
   }
+}
+
+__global__ void k_restrict_sum(const int* __restrict__ coff, const int* __restrict__ msz, const double* __restrict__ part,
+                               double* __restrict__ bH) {
+  const int s = blockIdx.x, lane = threadIdx.x;
+  double t = 0.0;
+#pragma unroll 8
+  for (int c = 0; c < RCH; ++c) t += part[((size_t)s * RCH + c) * PST + lane];
+  if (lane < msz[s]) bH[(size_t)(coff[s] + lane) * PST] = t;
+}
+
+// column 0 of [n][PST] blocks: y = alpha A x + beta y0, a warp per row
+__global__ void __launch_bounds__(256)
+k_coarse_matvec(const double* __restrict__ A, int n, double alpha, const double* __restrict__ x, double beta,
+                const double* __restrict__ y0, double* __restrict__ y) {
+  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (row >= n) return;
+  double t = 0.0;
+#pragma unroll 4
+  for (int j = lane; j < n; j += 32) t = fma(A[(size_t)row * n + j], x[(size_t)j * PST], t);
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (lane == 0) y[(size_t)row * PST] = fma(alpha, t, beta != 0.0 ? beta * y0[(size_t)row * PST] : 0.0);
 }
 
 // u^G on global DoFs: sum over subdomains whose Omega box holds the node.
@@ -217,9 +254,32 @@ void launch_coarse_blocks(msgfem* h) {
   k_symmetrize<<<256, 256, 0, h->stream>>>(h->d_AH, h->Nc, h->NcPad); ++g_launch_count;
 }
 
+// b^H = V^T v (column 0 of bH): the handle's load, or the global vector r
+void launch_coarse_restrict(msgfem* h, const double* r, cudaStream_t st) {
+  k_restrict_partial<<<dim3(RCH, h->N), 256, 0, st>>>(h->d_sub, r, h->NY, h->NZ, h->d_gram_part);
+  k_restrict_sum<<<h->N, PST, 0, st>>>(h->d_coff, h->d_m, h->d_gram_part, h->d_bH);
+  g_launch_count += 2;
+}
+
 void launch_coarse_rhs(msgfem* h) {
   cudaMemsetAsync(h->d_bH, 0, sizeof(double) * (size_t)h->NcPad * PST, h->stream);
-  k_coarse_rhs<<<h->N, 256, 0, h->stream>>>(h->d_sub, h->d_coff, h->d_m, h->d_bH); ++g_launch_count;
+  launch_coarse_restrict(h, nullptr, h->stream);
+}
+
+void launch_coarse_solve(msgfem* h, cudaStream_t st, int refine) {
+  if (h->inv == nullptr) {
+    run_solve_mv(h->csolve, st, 0, 0, 0);
+    return;
+  }
+  // d_AH holds -A_H^{-1}
+  const int n = h->NcPad, grid = (n + 7) / 8;
+  k_coarse_matvec<<<grid, 256, 0, st>>>(h->d_AH, n, -1.0, h->d_bH, 0.0, nullptr, h->d_cH);
+  ++g_launch_count;
+  for (int i = 0; i < refine; ++i) {
+    k_coarse_matvec<<<grid, 256, 0, st>>>(h->d_AHkeep, n, -1.0, h->d_cH, 1.0, h->d_bH, h->d_rH);
+    k_coarse_matvec<<<grid, 256, 0, st>>>(h->d_AH, n, -1.0, h->d_rH, 1.0, h->d_cH, h->d_cH);
+    g_launch_count += 2;
+  }
 }
 
 void launch_prolong(msgfem* h) {

@@ -1126,6 +1126,10 @@ struct InvForm {
     Solve solve[2];
   };
   std::vector<Wave> waves;
+  // coarse matrix: sweep tasks of its T x T tiles (coarse_inv_build)
+  InvMat* d_cmat = nullptr;
+  InvTask* d_ctasks = nullptr;
+  std::vector<SchedStep> csteps;
   int rs = 8;                      // rows per stage of the solves (by the widest layer and the type)
   bool digits = false;             // FP64: solves in digit products (k_inv_solve_fx)
 };
@@ -1505,6 +1509,59 @@ void inv_solve(msgfem* h, int mat, int src, int dst, int neg, int width, int add
       cudaLaunchKernelExC(&cfg, solve_kernel(h, f, back), args);
       ++g_launch_count;
     }
+  }
+}
+
+// The coarse matrix as one block: its sweep's tasks for the current NcPad, in place in
+// d_AH, scratch in d_AHinv.  (The block Cholesky with its block inverse took T tile
+// Cholesky steps and T inverse rows of up to T products on one CTA each: 6.6 ms at 10
+// tiles, sweeps 1.1 ms.)
+msgfem_status coarse_inv_build(msgfem* h) {
+  InvForm& f = *h->inv;
+  const int T = h->NcPad / TILE;
+  dev_free_bytes(h, f.d_cmat);
+  dev_free_bytes(h, f.d_ctasks);
+  f.d_cmat = nullptr;
+  f.d_ctasks = nullptr;
+  InvMat m;
+  memset(&m, 0, sizeof(m));
+  m.sub = h->N;      // entry N of the flags: the coarse problem
+  m.n = m.b = h->NcPad;
+  m.nL = 1;
+  m.D = h->d_AH;
+  m.L = h->d_AHinv;
+  std::vector<InvTask> tasks;
+  f.csteps.clear();
+  auto step = [&](size_t first) { f.csteps.push_back({(int)first, (int)(tasks.size() - first)}); };
+  tasks.push_back({IV_PIVOT, 0, 0, 0, 0, 0});
+  step(0);
+  for (int k = 0; k < T; ++k) {
+    size_t first = tasks.size();
+    for (int i = 0; i < T; ++i) tasks.push_back({IV_PANEL, 0, 0, k, i, 0});
+    step(first);
+    first = tasks.size();
+    if (k + 1 < T) tasks.push_back({IV_UPDATE, 0, 0, k, k + 1, k + 1});   // swept next: first
+    for (int i = 0; i < T; ++i)
+      for (int j = 0; j <= i; ++j)
+        if (i != k && j != k && !(i == k + 1 && j == k + 1)) tasks.push_back({IV_UPDATE, 0, 0, k, i, j});
+    if (tasks.size() > first) step(first);
+  }
+  void* p = nullptr;
+  TRY(dev_alloc_bytes(h, &p, sizeof(InvMat)));
+  f.d_cmat = static_cast<InvMat*>(p);
+  TRY(dev_alloc_bytes(h, &p, tasks.size() * sizeof(InvTask)));
+  f.d_ctasks = static_cast<InvTask*>(p);
+  CK(cudaMemcpy(f.d_cmat, &m, sizeof(InvMat), cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(f.d_ctasks, tasks.data(), tasks.size() * sizeof(InvTask), cudaMemcpyHostToDevice));
+  return MSGFEM_OK;
+}
+
+void coarse_inv_factor(msgfem* h) {
+  const InvForm& f = *h->inv;
+  for (const SchedStep& s : f.csteps) {
+    k_inv_step<double><<<s.count, 256, inv_step_smem<double>(), h->stream>>>(f.d_ctasks + s.first, f.d_cmat, h->d_flags,
+                                                                           h->d_notspd);
+    ++g_launch_count;
   }
 }
 

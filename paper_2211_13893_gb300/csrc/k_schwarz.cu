@@ -93,28 +93,6 @@ __global__ void k_local_scatter(const SubDev* __restrict__ subs, int N, int whic
   }
 }
 
-// r_H = V^T r into column 0 of bH (the coarse handle's weighted basis CB)
-__global__ void k_coarse_restrict(const SubDev* __restrict__ subs, const int* __restrict__ coff,
-                                  const int* __restrict__ msz, const double* __restrict__ r, double* __restrict__ bH,
-                                  int NY, int NZ) {
-  const SubDev& s = subs[blockIdx.x];
-  __shared__ double red[8][PST];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  double acc = 0.0;
-  for (int row = w; row < s.nfull; row += 8) {
-    const int n = row / 3, c = row % 3;
-    const double rv = r[3 * (size_t)global_node(s, n / s.npl, n % s.npl, NY, NZ) + c];
-    acc = fma(s.CB[(size_t)row * PST + lane], rv, acc);
-  }
-  red[w][lane] = acc;
-  __syncthreads();
-  if (w == 0) {
-    double t = 0.0;
-    for (int i = 0; i < 8; ++i) t += red[i][lane];
-    if (lane < msz[blockIdx.x]) bH[(size_t)(coff[blockIdx.x] + lane) * PST] = t;
-  }
-}
-
 // z += V c (column 0 of cH), subdomains summed in index order
 __global__ void k_prolong_add(const SubDev* __restrict__ subs, int N, const int* __restrict__ coff,
                               const int* __restrict__ msz, const double* __restrict__ cH, double* __restrict__ z,
@@ -326,9 +304,8 @@ msgfem_status schwarz_run(msgfem_h hl, msgfem_h hc, const double* b_in, const do
     ++g_launch_count;
     if (hc) {
       set_dense_context(hc->d_flags, hc->d_notspd, hc->d_sub);
-      k_coarse_restrict<<<hc->N, 256, 0, st>>>(hc->d_sub, hc->d_coff, hc->d_m, r, hc->d_bH, NY, NZ);
-      ++g_launch_count;
-      run_solve_mv(hc->csolve, st, 0, 0, 0);
+      launch_coarse_restrict(hc, r, st);
+      launch_coarse_solve(hc, st, 0);
       k_prolong_add<<<(ndof + 255) / 256, 256, 0, st>>>(hc->d_sub, hc->N, hc->d_coff, hc->d_m, hc->d_cH, z, NY, NZ,
                                                          ndof);
       ++g_launch_count;
