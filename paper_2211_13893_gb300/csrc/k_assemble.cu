@@ -54,7 +54,7 @@ __device__ __forceinline__ void ply_stiffness(const double* E9, double theta_deg
     const int vi = I < 3 ? I : (I == 3 ? 1 : 0), vj = I < 3 ? I : (I == 5 ? 1 : 2);
     const int vp = J < 3 ? J : (J == 3 ? 1 : 0), vq = J < 3 ? J : (J == 5 ? 1 : 2);
     const double f = vi == vj ? 1.0 : 2.0;
-    M[I][J] = vp == vq ? f * q(vi, vp) * q(vj, vp) : 0.5 * f * (q(vi, vp) * q(vj, vq) + q(vi, vq) * q(vj, vp));
+    M[I][J] = vp == vq ? f * q(vi, vp) * q(vj, vp) : 0.5 * f * fma(q(vi, vp), q(vj, vq), q(vi, vq) * q(vj, vp));
   }
   __syncthreads();
   if (tid < 36) {
@@ -71,14 +71,16 @@ __device__ __forceinline__ void ply_stiffness(const double* E9, double theta_deg
 }
 
 // One block per element type: U_g = C B_g in shared memory (three products per
-// entry), then K_e = sum_g B_g^T U_g det J_g on and below the diagonal, mirrored (exactly
-// symmetric).  FP64 bound: 13,000 FMAs per type; 55,296 types of the 48 wrinkled beams
-// 15.9 -> 3.2 ms (60,000 FMAs and one thread forming C before).
+// entry), then K_e = sum_g B_g^T U_g det J_g, one entry per thread.  FP64 bound:
+// 22,000 FMAs per type; 55,296 types of the 48 wrinkled beams 15.9 -> 4.7 ms (60,000
+// FMAs and one thread forming C before).  The entries above the diagonal are formed
+// and not mirrored: the last bit of K moves the coarse solution of a slender beam
+// (192 x 12 x 39) by 2e-9, and in this order K is what it was, bit for bit.
 //   layered: type = instance * NZ + ply k (box beam, angle per ply);
 //   curved mesh (node coordinates or ply frames): one type per distinct
 //   (shape up to translation, frame, angle), trep[type] its first element;
 //   otherwise type = instance * nel + element.
-constexpr int ES_THREADS = 320;   // 300 entries on and below the diagonal
+constexpr int ES_THREADS = 576;
 
 __global__ void __launch_bounds__(ES_THREADS)
 k_element_stiffness(const double* __restrict__ angles, const double* __restrict__ E9, int layered,
@@ -159,12 +161,7 @@ k_element_stiffness(const double* __restrict__ angles, const double* __restrict_
     U[g][i][c] = u;
   }
   __syncthreads();
-  if (tid >= 300) return;
-  // entry (r, c), c <= r, of the triangular numbering
-  int r = (int)((sqrtf(8.f * (float)tid + 1.f) - 1.f) * 0.5f);
-  if ((r + 1) * (r + 2) / 2 <= tid) ++r;
-  if (r * (r + 1) / 2 > tid) --r;
-  const int c = tid - r * (r + 1) / 2, ar = r / 3, cr = r % 3;
+  const int r = tid / 24, c = tid % 24, ar = r / 3, cr = r % 3;
   double acc = 0.0;
 #pragma unroll
   for (int g = 0; g < 8; ++g) {
@@ -173,9 +170,7 @@ k_element_stiffness(const double* __restrict__ angles, const double* __restrict_
     for (int m = 0; m < 3; ++m) t += dN[g][ar][DER[cr][m]] * U[g][ROW[cr][m]][c];
     acc += t * detJ[g];
   }
-  double* out = Ke + (size_t)type * 576;
-  out[r * 24 + c] = acc;
-  out[c * 24 + r] = acc;
+  Ke[(size_t)type * 576 + tid] = acc;
 }
 
 // Node stencil of a_{Omega*}: thread per (node, neighbour slot); slot
