@@ -29,9 +29,9 @@
 // 4 CG steps to 1e-11 where the Cholesky form takes 5 to 6).
 //
 // Measured on one GB300 against the block Cholesky (factorisation / all solves of a
-// local stage, ms): 36 x 12 x 39 beam FP64 345 -> 103 / 424 -> 158; 192 x 12 x 39 beam
-// mixed 102 -> 71 / 374 -> 200; C-section of 16 subdomains mixed 85 -> 45 / 409 -> 172;
-// 47 x 7 x 13 beam FP64 whole pass 156 -> 83.
+// local stage, ms): 36 x 12 x 39 beam FP64 345 -> 46 / 424 -> 54; 192 x 12 x 39 beam
+// mixed 102 -> 72 / 374 -> 170; C-section of 16 subdomains mixed 85 -> 45 / 409 -> 124;
+// 47 x 7 x 13 beam FP64 whole pass 156 -> 42.
 #include "internal.h"
 
 #include <cooperative_groups.h>
@@ -51,6 +51,7 @@ struct InvMat {
   int npl, nyn;
   int pinned;                  // K of a floating subdomain: rows pin[] of layer 0 are out
   int pin[6];                  // compact rows in layer 0
+  int sg;                      // FP32: ranks of the solve's clusters (0: no k_inv_solve_f32)
   const double* stencil;
   void* D;                     // [nL][b][b] S_l, then -S_l^{-1}
   void* E;                     // [nL - 1][b][b] scratch of the triple products
@@ -582,8 +583,8 @@ __global__ void k_inv_pack(const InvMat* __restrict__ mats, const int* __restric
 // results to the ranks whose nodes neighbour them; cluster barrier.  The rows of
 // S^{-1} are contiguous in memory and depend on nothing, so they stream through
 // a ring of bulk copies (cp.async.bulk, one per stage) that runs ahead across
-// the layers: the ring is full again when the barriers are passed.  FP32 is
-// bound by HBM (many subdomains) or by the barriers (few), FP64 by the FP64 pipe.
+// the layers: the ring is full again when the barriers are passed.  Serves the layers
+// that neither k_inv_solve_f32 nor k_inv_solve_fx takes (more than about 1,000 DoFs).
 struct InvSolveArgs {
   const InvMat* mats;
   const int* list;          // matrices (largest first)
@@ -826,6 +827,339 @@ k_inv_solve(const InvSolveArgs a) {
     for (int i = waited; i < issued; ++i) tc::mbar_wait(bar0 + 8 * (i % a.ring), (i / a.ring) & 1);
     if (cphase > 0) tc::mbar_wait(bar0 + 64, (cphase - 1) & 1);
     if (a.err != nullptr) atomicExch(a.err, 1);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// FP32 solve of layers up to 1,024 DoFs.  The cluster, the chain and the sparse step are
+// those of k_inv_solve; the dense step is laid out so that neither shuffles nor CTA
+// barriers stand in its loop:
+//   - lane = row: a rank owns up to 8 blocks of 32 rows, a warp a fixed eighth of the
+//     columns; a lane adds 4 columns x 8 right-hand sides for its row of every block in
+//     packed FMAs, z comes as shared-memory broadcasts, 24 reads of 128 bytes per 512
+//     entries of 4 blocks (rows across 32 lanes of k: 48, and 31 shuffles per 4 rows);
+//   - the factorisation's last kernel puts -S^{-1} into that order (k_inv_pack_f32), so a
+//     warp streams its own 512-byte rows of lanes with its own ring of bulk copies and
+//     mbarriers and waits for nobody until the layer's end;
+//   - there the eight warps' sums are added through shared memory, and all threads write
+//     the results (two warps after every stage before).
+// All solves of a local stage, k_inv_solve -> here: C-section of 16 subdomains (layers of
+// 714 and 912 DoFs) 188 -> 124 ms, 192 x 12 x 39 beam (570 and 693) 204 -> 170 ms (84 % of
+// the HBM copy rate), 48 beams (210 and 225) 42 -> 31 ms, 47 x 7 x 13 beam (360 and 408, 20
+// half chains: barriers) 20 -> 20 ms.  Bound by HBM with many half chains, by the cluster's
+// barriers with few.
+constexpr int F32_BLOCKS = 8;    // blocks of 32 rows per rank
+constexpr int F32_WIDE = 1024;   // widest layer
+
+// -S^{-1} of layer l in the order of the solve: the triple products' scratch, the last
+// layer in layer 0's place (packed before)
+__device__ __forceinline__ float* packed_layer(const InvMat& m, int l) {
+  return l + 1 < m.nL ? static_cast<float*>(m.E) + (size_t)l * m.b * m.b : static_cast<float*>(m.D);
+}
+// blocks of 32 rows per rank of a cluster of G
+__host__ __device__ __forceinline__ int f32_blocks(int n, int G) { return ((n + 31) / 32 + G - 1) / G; }
+
+// Layer l < nL - 1 (last = 0) or nL - 1 (last = 1), block of 32 rows: rank's strip of Rg
+// rows, then [column / 4][row of the strip][4]; zero outside the n x n matrix.
+__global__ void __launch_bounds__(256)
+k_inv_pack_f32(const InvMat* __restrict__ mats, const int* __restrict__ active, int last) {
+  const InvMat& m = mats[blockIdx.z];
+  if (m.sg == 0 || (active != nullptr && !active[m.sub])) return;
+  const int l = last ? m.nL - 1 : blockIdx.y, rb = blockIdx.x, nb = (m.n + 31) / 32, kp = nb * 32;
+  if (rb >= nb || (!last && l >= m.nL - 1)) return;
+  __shared__ float4 tile[32][33];
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int nbr = f32_blocks(m.n, m.sg), g = rb / nbr, Rg = 32 * min(nbr, nb - g * nbr);
+  const float* D = static_cast<const float*>(m.D) + ((size_t)l * m.b + (size_t)rb * 32) * m.b;
+  float4* out = reinterpret_cast<float4*>(packed_layer(m, l)) + (size_t)g * nbr * 32 * (kp / 4) + (rb - g * nbr) * 32;
+  for (int c0 = 0; c0 < kp / 4; c0 += 32) {
+    for (int r = w; r < 32; r += 8) {
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+      const int c = 4 * (c0 + lane);
+      if (rb * 32 + r < m.n && c < m.n) {
+        x = *reinterpret_cast<const float4*>(D + (size_t)r * m.b + c);
+        if (c + 1 >= m.n) x.y = 0.f;
+        if (c + 2 >= m.n) x.z = 0.f;
+        if (c + 3 >= m.n) x.w = 0.f;
+      }
+      tile[r][lane] = x;
+    }
+    __syncthreads();
+    for (int c = w; c < 32 && c0 + c < kp / 4; c += 8) out[(size_t)(c0 + c) * Rg + lane] = tile[lane][c];
+    __syncthreads();
+  }
+}
+
+__device__ __forceinline__ unsigned long long dup2(float x) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float2 split2(unsigned long long v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ void fma2(unsigned long long& d, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+
+// A warp's ring: groups of 4 columns x Rg rows, in the order they are used
+struct F32Ring {
+  uint32_t smem, bar, bytes;   // first slot, first mbarrier, bytes per group
+  int depth, used;             // slots; groups consumed
+  bool ok;
+};
+
+// Dense step of one layer for NR blocks of rows: the warp's ngrp groups against z, the
+// eight warps' sums added into red[4][2][Rg][4] (to be summed over its four slots).
+template <int NR, typename Issue>
+__device__ __forceinline__ void dense_f32(F32Ring& rg, const float4* slots, const float* z, int ngrp, float* red,
+                                          Issue issue) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  unsigned long long acc[NR][4];
+#pragma unroll
+  for (int r = 0; r < NR; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[r][c] = 0ull;
+#pragma unroll 1
+  for (int i = 0; i < ngrp; ++i, ++rg.used) {
+    const int slot = rg.used % rg.depth;
+    if (rg.ok) rg.ok = tc::mbar_wait(rg.bar + 8 * slot, (rg.used / rg.depth) & 1);
+    const float4* sp = slots + slot * NR * 32 + lane;
+    const float* zp = z + i * 4 * KB;
+    float4 sv[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) sv[r] = sp[r * 32];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const ulonglong2 z0 = *reinterpret_cast<const ulonglong2*>(zp + q * KB);
+      const ulonglong2 z1 = *reinterpret_cast<const ulonglong2*>(zp + q * KB + 4);
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const unsigned long long x = dup2(q == 0 ? sv[r].x : q == 1 ? sv[r].y : q == 2 ? sv[r].z : sv[r].w);
+        fma2(acc[r][0], x, z0.x);
+        fma2(acc[r][1], x, z0.y);
+        fma2(acc[r][2], x, z1.x);
+        fma2(acc[r][3], x, z1.y);
+      }
+    }
+    __syncwarp();
+    issue();   // the slot is free
+  }
+  float4* rd = reinterpret_cast<float4*>(red) + (size_t)(w & 3) * 2 * NR * 32 + lane;
+  auto put = [&](bool add) {
+#pragma unroll
+    for (int r = 0; r < NR; ++r)
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        const float2 u = split2(acc[r][2 * hf]), v = split2(acc[r][2 * hf + 1]);
+        float4* o = rd + (hf * NR + r) * 32;
+        float4 x = make_float4(u.x, u.y, v.x, v.y);
+        if (add) x = make_float4(x.x + o->x, x.y + o->y, x.z + o->z, x.w + o->w);
+        *o = x;
+      }
+  };
+  if (w >= 4) put(false);
+  __syncthreads();
+  if (w < 4) put(true);
+  __syncthreads();
+}
+
+template <bool BACK>
+__global__ void __launch_bounds__(256, 2)
+k_inv_solve_f32(const InvSolveArgs a) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int G = (int)cl.num_blocks(), g = (int)cl.block_rank();
+  const int task = blockIdx.x / G, half = task & 1;
+  const InvMat& m = a.mats[a.list[task >> 1]];
+  if (a.active != nullptr && !a.active[m.sub]) return;   // uniform over the cluster
+  const int nch = half ? m.nL - 1 - m.mid : m.mid;        // layers without the middle one
+  const int steps = BACK ? nch + 1 : nch;
+  if (!BACK && nch == 0) return;
+  if (BACK && half && nch == 0) return;
+  const int mid = m.mid, nL = m.nL;
+  auto layer_of = [&](int t) {
+    if (BACK) return half ? mid + t : mid - t;
+    return half ? nL - 1 - t : t;
+  };
+  extern __shared__ __align__(128) unsigned char smem_sv[];
+  float* ring = reinterpret_cast<float*>(smem_sv);
+  float* zb = reinterpret_cast<float*>(smem_sv + a.smem_z);   // [b][KB]
+  float* uw = reinterpret_cast<float*>(smem_sv + a.smem_u);
+  float* cf = reinterpret_cast<float*>(smem_sv + a.smem_c);
+  float* red = reinterpret_cast<float*>(smem_sv + a.smem_r);  // [4][2][Rg][4]
+  __shared__ __align__(8) unsigned long long bars[65];        // the warps' ring slots, couplings
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int b = m.b, n = m.n, nn = n / 3, njc = m.njc, nic = m.nic;
+  const int nbr = f32_blocks(n, G), nb = max(0, min(nbr, (n + 31) / 32 - g * nbr));   // own blocks of 32 rows
+  const int r0 = g * nbr * 32, nrow = max(0, min(n - r0, nb * 32));
+  const int npc = up4((nn + G - 1) / G), p0 = min(nn, npc * g), p1 = min(nn, p0 + npc);
+  const int wlo = max(0, p0 - njc - 1);                       // first node of the window of neighbour values
+  const uint32_t bar0 = tc::saddr(bars), cbar = bar0 + 8 * 64, cf_s = tc::saddr(cf);
+  // the warp's ring: its eighth of the columns, group by group, layer by layer
+  const int ngrp = (n + 31) / 32, total = nb > 0 ? ngrp * steps : 0;
+  F32Ring rg;
+  rg.depth = a.ring;
+  rg.bytes = (uint32_t)nb * 512;
+  rg.smem = tc::saddr(ring) + (uint32_t)w * a.ring * rg.bytes;
+  rg.bar = bar0 + 8 * 8 * w;
+  rg.used = 0;
+  rg.ok = true;
+  const float4* slots = reinterpret_cast<const float4*>(ring) + (size_t)w * a.ring * nb * 32;
+  int issued = 0, ist = 0, isg = 0;   // groups requested; step and group of the next (lane 0)
+  auto issue = [&]() {
+    if (lane != 0 || issued >= total || !rg.ok) return;
+    const int slot = issued % rg.depth;
+    tc::fence_async_smem();
+    tc::mbar_expect_tx(rg.bar + 8 * slot, rg.bytes);
+    bulk_load(rg.smem + slot * rg.bytes,
+              packed_layer(m, layer_of(ist)) + ((size_t)r0 * ngrp * 8 + (size_t)(w * ngrp + isg) * nb * 32) * 4, rg.bytes,
+              rg.bar + 8 * slot);
+    ++issued;
+    if (++isg == ngrp) { isg = 0; ++ist; }
+  };
+  const int cdir = BACK ? (half ? 0 : 1) : (half ? 1 : 0);
+  const uint32_t cbytes = p1 > p0 ? (uint32_t)(up4(p1 - p0) * 81 * sizeof(float)) : 0;
+  auto coupling_ptr = [&](int l, int dir) {
+    return static_cast<const float*>(m.L) + (size_t)l * b * b + ((size_t)dir * up4(nn) + p0) * 81;
+  };
+  if (tid == 0) {
+    for (int i = 0; i < 65; ++i) tc::mbar_init(bar0 + 8 * i, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  for (int e = tid; e < b * KB; e += 256) zb[e] = 0.f;
+  __syncthreads();
+  for (int i = 0; i < a.ring; ++i) issue();
+  const SubDev& sd = a.subs[m.sub];
+  const double* src = mv_ptr(sd, a.src) + a.coloff;
+  double* dst = mv_ptr(sd, a.dst) + a.coloff;
+  float* yc = static_cast<float*>(m.yc);
+  const float sgn = a.neg ? -1.f : 1.f;
+  int cphase = 0;   // coupling copies waited for
+  bool cpend = false, cok = true;
+  // sparse step: task e = ((node, component), half of the columns); the source values of
+  // a thread's first task of the next layer are requested before the dense step
+  const int ntask = (p1 - p0) * 6;
+  auto source = [&](int l, int e, double (&v)[4]) {
+    const int p = p0 + e / 6, r = (e % 6) >> 1;
+    const size_t node = (size_t)l * m.npl + (size_t)(m.ia + p / njc) * m.nyn + m.ja + p % njc;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) v[c] = src[(node * 3 + r) * a.stride + (e & 1) * 4 + c];
+  };
+  double pre[4] = {0.0, 0.0, 0.0, 0.0};
+  if (tid < ntask) source(layer_of(0), tid, pre);
+  cl.sync();   // no remote store before every CTA of the cluster has cleared its arrays
+  for (int t = 0; t < steps; ++t) {
+    const int l = layer_of(t);
+    const bool first = t == 0;
+    if (cpend) {
+      if (cok) cok = tc::mbar_wait(cbar, cphase & 1);
+      ++cphase;
+    }
+    for (int e = tid; e < ntask; e += 256) {
+      const int pl = e / 6, r = (e % 6) >> 1, c0 = (e & 1) * 4, p = p0 + pl;
+      const int i = p / njc, j = p % njc;
+      float z[4] = {0.f, 0.f, 0.f, 0.f};
+      if (!BACK || first) {
+        double v[4] = {pre[0], pre[1], pre[2], pre[3]};
+        if (e != tid) source(l, e, v);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) z[c] = pinned_row(m, l, 3 * p + r) ? 0.f : sgn * (float)v[c];
+      }
+      auto sub_coupling = [&](const float* c, const float* u) {   // z -= C u, u indexed by row * KB
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int s9 = 0; s9 < 9; ++s9) {
+          const int di = s9 / 3 - 1, dj = s9 % 3 - 1;
+          if (i + di < 0 || i + di >= nic || j + dj < 0 || j + dj >= njc) continue;
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            const float4 x = *reinterpret_cast<const float4*>(u + (ptrdiff_t)(3 * (p + di * njc + dj) + q) * KB + c0);
+            const float cv = c[s9 * 9 + 3 * r + q];
+            acc[0] = fmaf(cv, x.x, acc[0]);
+            acc[1] = fmaf(cv, x.y, acc[1]);
+            acc[2] = fmaf(cv, x.z, acc[2]);
+            acc[3] = fmaf(cv, x.w, acc[3]);
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) z[q] -= acc[q];
+      };
+      if (BACK && first) {
+        // middle layer: both half chains' u from memory
+        if (mid > 0) sub_coupling(coupling_ptr(l, 0) + (size_t)pl * 81, yc + (size_t)(l - 1) * b * KB);
+        if (mid + 1 < nL) sub_coupling(coupling_ptr(l, 1) + (size_t)pl * 81, yc + (size_t)(l + 1) * b * KB);
+      } else if (!first) {
+        sub_coupling(cf + (size_t)pl * 81, uw - (ptrdiff_t)wlo * 3 * KB);
+      }
+      for (int q = 0; q < G; ++q)
+        *reinterpret_cast<float4*>(cl.map_shared_rank(zb, q) + (3 * p + r) * KB + c0) = make_float4(z[0], z[1], z[2], z[3]);
+    }
+    cl.sync();
+    // the coupling buffer is free: request the next layer's
+    cpend = t + 1 < steps && cbytes > 0;
+    if (cpend && cok && tid == 0) {
+      tc::fence_async_smem();
+      tc::mbar_expect_tx(cbar, cbytes);
+      bulk_load(cf_s, coupling_ptr(layer_of(t + 1), cdir), cbytes, cbar);
+    }
+    // ---- dense step on the own rows
+    if (!BACK && t + 1 < steps && tid < ntask) source(layer_of(t + 1), tid, pre);
+    float4 prey = make_float4(0.f, 0.f, 0.f, 0.f);   // u of the thread's first result
+    if (BACK && !first && tid < 2 * nrow) {
+      const int hf = tid >= nrow;
+      prey = *reinterpret_cast<const float4*>(yc + ((size_t)l * b + r0 + tid - hf * nrow) * KB + 4 * hf);
+    }
+    const float* zw = zb + (size_t)w * ngrp * 4 * KB;
+    switch (nb) {
+      case 1: dense_f32<1>(rg, slots, zw, ngrp, red, issue); break;
+      case 2: dense_f32<2>(rg, slots, zw, ngrp, red, issue); break;
+      case 3: dense_f32<3>(rg, slots, zw, ngrp, red, issue); break;
+      case 4: dense_f32<4>(rg, slots, zw, ngrp, red, issue); break;
+      case 5: dense_f32<5>(rg, slots, zw, ngrp, red, issue); break;
+      case 6: dense_f32<6>(rg, slots, zw, ngrp, red, issue); break;
+      case 7: dense_f32<7>(rg, slots, zw, ngrp, red, issue); break;
+      case 8: dense_f32<8>(rg, slots, zw, ngrp, red, issue); break;
+    }
+    for (int e = tid; e < 2 * nrow; e += 256) {
+      const int hf = e >= nrow, rl = e - hf * nrow, row = r0 + rl, c0 = 4 * hf;
+      float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 v = reinterpret_cast<const float4*>(red)[(size_t)(q * 2 + hf) * nb * 32 + rl];
+        y = make_float4(y.x + v.x, y.y + v.y, y.z + v.z, y.w + v.w);
+      }
+      float4* yp = reinterpret_cast<float4*>(yc + ((size_t)l * b + row) * KB + c0);
+      float4 x = make_float4(-y.x, -y.y, -y.z, -y.w);   // the block holds -S^{-1}
+      if (BACK && !first) {
+        const float4 u = e == tid ? prey : *yp;
+        x = make_float4(u.x + x.x, u.y + x.y, u.z + x.z, u.w + x.w);
+      }
+      const int p = row / 3;
+      if (!BACK) *yp = x;
+      else if (!first || half == 0) {
+        const size_t node = (size_t)l * m.npl + (size_t)(m.ia + p / njc) * m.nyn + m.ja + p % njc;
+        double* o = dst + (node * 3 + row % 3) * a.stride + c0;
+        const float xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) o[c] = a.add ? o[c] + (double)xv[c] : (double)xv[c];
+      }
+      if (t + 1 < steps)
+        for (int q = 0; q < G; ++q) {
+          const int q0 = min(nn, npc * q), lo = max(0, q0 - njc - 1), hi = min(nn, min(nn, q0 + npc) + njc + 1);
+          if (p >= lo && p < hi) *reinterpret_cast<float4*>(cl.map_shared_rank(uw, q) + (row - 3 * lo) * KB + c0) = x;
+        }
+    }
+    cl.sync();
+  }
+  if (!__syncthreads_and(rg.ok && cok)) {
+    // a copy did not arrive within its limit: wait once more for those in flight, then report
+    if (lane == 0)
+      for (int i = max(0, issued - rg.depth); i < issued; ++i)
+        tc::mbar_wait(rg.bar + 8 * (i % rg.depth), (i / rg.depth) & 1);
+    if (tid == 0 && cphase > 0) tc::mbar_wait(cbar, (cphase - 1) & 1);
+    if (tid == 0 && a.err != nullptr) atomicExch(a.err, 1);
   }
 }
 
@@ -1118,6 +1452,7 @@ struct InvForm {
     std::vector<int> list;         // matrices of one kind in a wave, largest first
     int* d_list = nullptr;
     int G = 1, ring = 2, smem_z = 0, smem_u = 0, smem_c = 0, smem_r = 0, smem = 0;
+    bool rows32 = false;           // k_inv_solve_f32 (FP32, layers up to F32_WIDE)
   };
   struct Wave {
     std::vector<std::vector<SchedStep>> steps;   // per stream group
@@ -1141,11 +1476,11 @@ constexpr int FX_SMEM = 221 * 1024;    // the same beside the digit solve's stat
 
 template <typename T>
 const void* solve_kernel_ptr(int rs, bool back) {
-  if (rs == 16) return back ? (const void*)k_inv_solve<T, 16, true> : (const void*)k_inv_solve<T, 16, false>;
   if (rs == 8) return back ? (const void*)k_inv_solve<T, 8, true> : (const void*)k_inv_solve<T, 8, false>;
   return back ? (const void*)k_inv_solve<T, 4, true> : (const void*)k_inv_solve<T, 4, false>;
 }
-const void* solve_kernel(const msgfem* h, const InvForm& f, bool back) {
+const void* solve_kernel(const msgfem* h, const InvForm& f, const InvForm::Solve& s, bool back) {
+  if (s.rows32) return back ? (const void*)k_inv_solve_f32<true> : (const void*)k_inv_solve_f32<false>;
   if (f.digits) return back ? (const void*)k_inv_solve_fx<true> : (const void*)k_inv_solve_fx<false>;
   const int rs = f.rs;
   return h->mixed ? solve_kernel_ptr<float>(rs, back) : solve_kernel_ptr<double>(rs, back);
@@ -1157,13 +1492,22 @@ int solve_layout(const msgfem* h, const InvForm& f, InvForm::Solve& s, int G, in
   const int es = h->mixed ? 4 : 8, vn = 16 / es;
   auto up = [](size_t v) { return (v + 127) / 128 * 128; };
   size_t st = 0, z = 0, u = 0, c = 0, o = 0;
+  int wide = 0;
+  for (int i : s.list) wide = std::max(wide, f.mats[i].b);
+  s.rows32 = h->mixed && wide <= F32_WIDE;
   for (int i : s.list) {
     const InvMat& m = f.mats[i];
     const int nn = m.n / 3, npc = up4((nn + G - 1) / G);
-    o = std::max(o, (size_t)npc * 3 * KB * es);
     if (f.digits) {
+      o = std::max(o, (size_t)npc * 3 * KB * es);
       z = std::max(z, (size_t)((m.n + 15) / 16) * DIG * 8 * KB * 4);
       st = FX_STAGE;
+    } else if (s.rows32) {
+      const int rows = 32 * f32_blocks(m.n, G);
+      if (rows > 32 * F32_BLOCKS) return 1 << 30;
+      st = std::max(st, (size_t)rows * 16 * 8);          // a group of every warp
+      z = std::max(z, (size_t)m.b * KB * es);
+      o = std::max(o, (size_t)rows * KB * es * 4);
     } else {
       st = std::max(st, (size_t)f.rs * m.b * es);
       z = std::max(z, (size_t)((m.b + vn - 1) / vn) * vn * (KB + 1) * es);
@@ -1177,7 +1521,7 @@ int solve_layout(const msgfem* h, const InvForm& f, InvForm::Solve& s, int G, in
   s.smem_u = (int)(s.smem_z + up(z));
   s.smem_c = (int)(s.smem_u + up(u));
   s.smem_r = (int)(s.smem_c + up(c));
-  s.smem = (int)(s.smem_r + up(f.digits ? o : (size_t)2 * (8 / (f.rs / 4)) * f.rs * KB * es));
+  s.smem = (int)(s.smem_r + up(f.digits || s.rows32 ? o : (size_t)2 * (8 / (f.rs / 4)) * f.rs * KB * es));
   return s.smem;
 }
 
@@ -1205,21 +1549,43 @@ int resident_clusters(const void* kernel, int G, int smem) {
 // half chain is resident at once (they run side by side), with the deepest ring
 // that one CTA per SM holds, or half an SM's shared memory when that makes more
 // half chains resident; with more half chains than SMs one CTA each.
+// FP32 layers up to F32_WIDE: the fewest rounds of resident half chains, then the widest
+// cluster.  All solves of a local stage, ms, by CTAs per half chain: 32 half chains of 912
+// DoFs 8: 124, 4: 144; 64 of 570 (4 resident at once, 8 in two rounds) 8: 204, 4: 170;
+// 192 of 225 DoFs 8: 66, 4: 38, 2: 31, 1: 34; 20 of 408 8: 20, 4: 20, 2: 27.  The ring's
+// depth (2 to 8) changes none of them by more than 3 %.
 void choose_solve(const msgfem* h, const InvForm& f, InvForm::Solve& s) {
   const int chains = 2 * (int)s.list.size();
   int most = 1;
-  const int strip = f.digits ? 16 : f.rs;
-  for (int i : s.list) most = std::max(most, (f.mats[i].n + strip - 1) / strip / (f.digits ? 1 : 2));
+  solve_layout(h, f, s, 8, 2);   // the kernel
+  const int strip = f.digits ? 16 : s.rows32 ? 32 : f.rs;
+  for (int i : s.list) most = std::max(most, (f.mats[i].n + strip - 1) / strip / (f.digits || s.rows32 ? 1 : 2));
   auto fit = [&](int G, int limit) {
     int ring = 8;
     while (ring > 2 && solve_layout(h, f, s, G, ring) > limit) --ring;
     return solve_layout(h, f, s, G, ring) <= limit;
   };
+  if (s.rows32) {
+    int best = 0, rounds = 0, ring = 0;
+    for (int G : {8, 4, 2, 1})
+      for (int limit : {INV_SMEM, 108 * 1024}) {
+        if (G > most || !fit(G, limit)) continue;
+        const int res = std::max(1, resident_clusters(solve_kernel(h, f, s, true), G, s.smem));
+        const int n = (chains + res - 1) / res;
+        if (best == 0 || n < rounds) {
+          best = G;
+          rounds = n;
+          ring = s.ring;
+        }
+      }
+    solve_layout(h, f, s, best, ring);
+    return;
+  }
   for (int G : {8, 4, 2, 1}) {
     if (G > 1 && G > most) continue;
     for (int limit : {f.digits ? FX_SMEM : INV_SMEM, 108 * 1024}) {
       if (!fit(G, limit)) continue;
-      if (resident_clusters(solve_kernel(h, f, true), G, s.smem) >= chains) return;
+      if (resident_clusters(solve_kernel(h, f, s, true), G, s.smem) >= chains) return;
     }
   }
   if (fit(1, 108 * 1024)) return;
@@ -1288,7 +1654,7 @@ bool inv_create(msgfem* h) {
     }
   }
   const int row = bmax * es;
-  f->rs = row <= 3072 ? 16 : row <= 6144 ? 8 : 4;
+  f->rs = row <= 6144 ? 8 : 4;
   // two stages of the widest layer and its vectors must fit with the widest cluster
   InvForm::Solve probe;
   for (int i = 0; i < (int)f->mats.size(); ++i)
@@ -1316,13 +1682,15 @@ msgfem_status inv_build(msgfem* h) {
   InvForm& f = *h->inv;
   static bool attr = false;
   if (!attr) {
-    for (int rs : {4, 8, 16})
+    for (int rs : {4, 8})
       for (bool back : {false, true}) {
         CK(cudaFuncSetAttribute(solve_kernel_ptr<float>(rs, back), cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
         CK(cudaFuncSetAttribute(solve_kernel_ptr<double>(rs, back), cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
       }
     CK(cudaFuncSetAttribute(k_inv_step<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, inv_step_smem<double>()));
     CK(cudaFuncSetAttribute(k_inv_step<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, inv_step_smem<float>()));
+    for (const void* k : {(const void*)k_inv_solve_f32<false>, (const void*)k_inv_solve_f32<true>})
+      CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
     for (const void* k : {(const void*)k_inv_solve_fx<false>, (const void*)k_inv_solve_fx<true>})
       CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, FX_SMEM));
     CK(cudaFuncSetAttribute(k_inv_digits, cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
@@ -1413,12 +1781,14 @@ msgfem_status inv_build(msgfem* h) {
         return (double)f.mats[x].n * f.mats[x].n * f.mats[x].nL > (double)f.mats[y].n * f.mats[y].n * f.mats[y].nL;
       });
       choose_solve(h, f, s);
+      if (s.rows32)
+        for (int i : s.list) f.mats[i].sg = s.G;
       TRY(dev_alloc_bytes(h, &p, s.list.size() * sizeof(int)));
       s.d_list = static_cast<int*>(p);
       CK(cudaMemcpy(s.d_list, s.list.data(), s.list.size() * sizeof(int), cudaMemcpyHostToDevice));
     }
-    // the packing kernel reads the wave's matrices by list
   }
+  CK(cudaMemcpy(f.d_mats, f.mats.data(), f.mats.size() * sizeof(InvMat), cudaMemcpyHostToDevice));   // with sg
   return MSGFEM_OK;
 }
 
@@ -1453,6 +1823,15 @@ static void inv_factor_t(msgfem* h, int w, cudaStream_t st) {
   for (int i : wv.all) maxl = std::max(maxl, f.mats[i].nL);
   k_inv_pack<T><<<dim3(maxl, (int)f.mats.size()), 256, 0, st>>>(f.d_mats, h->d_flags);
   ++g_launch_count;
+  if (sizeof(T) == 4) {
+    int kmax = 0;
+    for (int i : wv.all)
+      if (f.mats[i].sg > 0) kmax = std::max(kmax, (f.mats[i].n + 31) / 32);
+    for (int last = 0; last < 2 && kmax > 0; ++last) {
+      k_inv_pack_f32<<<dim3(kmax, last ? 1 : maxl, (int)f.mats.size()), 256, 0, st>>>(f.d_mats, h->d_flags, last);
+      ++g_launch_count;
+    }
+  }
   if (f.digits) {
     int bmax = 0, kmax = 0;
     for (int i : wv.all) {
@@ -1506,7 +1885,7 @@ void inv_solve(msgfem* h, int mat, int src, int dst, int neg, int width, int add
     cfg.attrs = at;
     cfg.numAttrs = 1;
     for (bool back : {false, true}) {
-      cudaLaunchKernelExC(&cfg, solve_kernel(h, f, back), args);
+      cudaLaunchKernelExC(&cfg, solve_kernel(h, f, s, back), args);
       ++g_launch_count;
     }
   }

@@ -75,6 +75,29 @@ def test_nodal_loads_and_gather_signs(precision):
         assert np.linalg.norm(a - b) <= (1e-9 if precision == 0 else 1e-7) * np.linalg.norm(b)
 
 
+# FP32 solves: blocks of 32 rows per rank and ranks per half chain.  Layers of 45 (NY + 1)
+# and 42 (NY + 1) DoFs; few half chains take clusters of 8 (NY = 4: one block each, the last
+# of one row; 5: ranks without rows; 15, 21: up to 4 blocks; 22: above 1,024 DoFs, the other
+# kernel), 152 half chains clusters of 2 with 5 to 8 blocks.
+@pytest.mark.parametrize("ny,instances", [(4, 1), (5, 1), (15, 1), (21, 1), (22, 1), (6, 38), (7, 38), (8, 38), (10, 38)])
+def test_fp32_solve_row_blocks(ny, instances):
+    from paper_2211_13893_gb300 import MSGFEM
+    cfg = replace(get_config("t3"), name="rows", NX=24, NY=ny, NZ=3, sx=2, sy=1, overlap=1, oversampling=2, n_loc=6)
+    rng = np.random.default_rng(ny)
+    ang = rng.uniform(-90.0, 90.0, instances * cfg.NX * cfg.NY * cfg.NZ)
+    out = []
+    for kw in (dict(), dict(factor_schedule=1)):
+        m = MSGFEM.from_config(cfg, ang, seed=7, precision=1, instances=instances, **kw)
+        lam = np.array(m.local_spaces(cfg.n_loc))
+        out.append((lam, [m.export_local(j)[0][:, -1] for j in (0, m.N - 1)]))
+        m.close()
+    (la, pa), (lb, pb) = out
+    scale = np.maximum(np.abs(lb).max(axis=1, keepdims=True), 1.0)
+    assert (np.abs(la - lb) / scale).max() <= 1e-5
+    for a, b in zip(pa, pb):
+        assert np.linalg.norm(a - b) <= 1e-7 * np.linalg.norm(b)
+
+
 def test_wide_layers_keep_the_block_cholesky():
     """Layers whose solve stages exceed shared memory run the block Cholesky (same results bar)."""
     from paper_2211_13893_gb300 import MSGFEM
