@@ -423,11 +423,11 @@ void timed_stencil_kb(msgfem* h, int src, int dst, int mode, double alpha) {
   span_end(h, sp);
   h->prof.stencil_flops += stencil_flops(h, KB, mode);
 }
-void timed_stencil_apply(msgfem* h, int src, int dst, int mode, double alpha) {
+void timed_stencil_apply(msgfem* h, int src, int dst, int mode, double alpha, int ncols = PST) {
   const int sp = span_begin(h, TAG_STENCIL);
-  launch_stencil_apply(h, src, dst, mode, alpha);
+  launch_stencil_apply(h, src, dst, mode, alpha, ncols);
   span_end(h, sp);
-  h->prof.stencil_flops += stencil_flops(h, PST, mode);
+  h->prof.stencil_flops += stencil_flops(h, std::min(PST, (ncols + KB - 1) / KB * KB), mode);
 }
 #define MSGFEM_TIMED_ORTHO(name, params, args) \
   void timed_##name params { const int sp = span_begin(h, TAG_ORTHO); launch_##name args; span_end(h, sp); }
@@ -534,10 +534,11 @@ void run_graph(msgfem* h, uint64_t key, Issue issue) {
 
 // One block solve (K: mat 0, A11: mat 1) of PST or KB right-hand sides in the
 // handle's precision; add = 1 accumulates into the destination.
-void timed_solve_w(msgfem* h, int mat, int src, int dst, int neg, int width, int add) {
+// ncols: the columns that are read afterwards (the inverse form leaves the others alone).
+void timed_solve_w(msgfem* h, int mat, int src, int dst, int neg, int width, int add, int ncols = PST) {
   const int sp = span_begin(h, TAG_SOLVE);
   if (h->inv_on) {
-    inv_solve(h, mat, src, dst, neg, width, add);
+    inv_solve(h, mat, src, dst, neg, width, add, ncols);
     span_end(h, sp);
     h->prof.solve_flops += solve_flops(h, mat, width == KB ? KB : h->p);
     h->prof.solve_bytes += solve_bytes(h, mat, width == KB ? KB : h->p);
@@ -974,8 +975,8 @@ msgfem_status run_krylov(msgfem* h, const std::vector<int>& nl, bool& all_done) 
   TRY(set_active(h, h->base_act));
   CK(cudaMemcpyAsync(h->d_mk, h->m_final.data(), h->N * sizeof(int), cudaMemcpyHostToDevice, st));
   launch_ritz(h, h->d_mk, h->d_nwk, 1, false, MV_QB, MV_PHI);
-  timed_stencil_apply(h, MV_PHI, MV_Z, 3, 1.0);
-  timed_stencil_apply(h, MV_PHI, MV_KPHI, 0, 1.0);
+  timed_stencil_apply(h, MV_PHI, MV_Z, 3, 1.0, nwmax);
+  timed_stencil_apply(h, MV_PHI, MV_KPHI, 0, 1.0, nwmax);
   CK_LAUNCH();
   return MSGFEM_OK;
 }
@@ -1233,7 +1234,7 @@ static msgfem_status local_spaces_run(msgfem_h h, const std::vector<int>& nl, do
   // rigid modes, B-orthonormal (floating)
   int sp_iter = span_begin(h, TAG_ITERATE);
   launch_rigid_modes(h);
-  timed_stencil_apply(h, MV_R, MV_BR, 3, 1.0);
+  timed_stencil_apply(h, MV_R, MV_BR, 3, 1.0, 6);
   timed_gram(h, MV_R, MV_BR, GM_G1);
   launch_chol_inv_small(h, GM_G1, nullptr, 6, 0);
   timed_rotate(h, MV_R, GM_Y, 6);
@@ -1341,13 +1342,15 @@ static msgfem_status local_spaces_run(msgfem_h h, const std::vector<int>& nl, do
       // GenEO: ||K phi - lambda B phi|| / (||K phi|| + lambda ||B phi||) over B1 and B2
       launch_colnorms(h, MV_KPHI, MV_Z, p, KEEP_K, -1.0);
     } else {
-      timed_solve(h, 1, MV_Z, MV_T1, 0);
+      // of the wanted eigenvectors only (the subspace iteration's block has further columns)
+      const int nc = h->opt.solver == 0 ? n_loc : PST;
+      timed_solve_w(h, 1, MV_Z, MV_T1, 0, PST, 0, nc);
       for (int r = 0; h->mixed && r < std::min(h->refine, 5); ++r) {   // refine y~: residual Z - K y~ on B1
-        timed_stencil_apply(h, MV_T1, MV_W, 0, 1.0);
+        timed_stencil_apply(h, MV_T1, MV_W, 0, 1.0, nc);
         launch_x_minus_y(h, MV_Z, MV_W, MV_W, PST);
-        timed_solve_w(h, 1, MV_W, MV_T1, 0, PST, 1);
+        timed_solve_w(h, 1, MV_W, MV_T1, 0, PST, 1, nc);
       }
-      timed_stencil_apply(h, MV_T1, MV_W, 0, 1.0);
+      timed_stencil_apply(h, MV_T1, MV_W, 0, 1.0, nc);
       launch_colnorms(h, MV_KPHI, MV_W, p);
     }
     span_end(h, sp_iter);
@@ -1464,9 +1467,10 @@ msgfem_status msgfem_coarse_assemble_threshold(msgfem_h h, double t, int* coarse
     if (h->sub[j].loaded && !h->geneo)
       CK(cudaMemcpy2DAsync(h->sub[j].CB + h->m_sel[j], PST * sizeof(double), h->sub[j].psi, sizeof(double),
                            sizeof(double), h->sub[j].nfull, cudaMemcpyDeviceToDevice, st));
+  const int mmax = *std::max_element(ncols.begin(), ncols.end());
   // Gram-Schmidt in the B inner product (CholeskyQR, twice); psi dropped if dependent
   for (int pass = 0; pass < 2; ++pass) {
-    timed_stencil_apply(h, MV_CB, MV_CW, 3, 1.0);
+    timed_stencil_apply(h, MV_CB, MV_CW, 3, 1.0, mmax);
     timed_gram(h, MV_CB, MV_CW, GM_G1);
     launch_chol_inv_small(h, GM_G1, h->d_ncols, 0, pass == 0 ? 1 : 0);
     timed_rotate(h, MV_CB, GM_Y, PST);
@@ -1482,7 +1486,7 @@ msgfem_status msgfem_coarse_assemble_threshold(msgfem_h h, double t, int* coarse
     }
   }
   launch_scale_rows_mu(h, MV_CB);
-  timed_stencil_apply(h, MV_CB, MV_CW, 0, 1.0);
+  timed_stencil_apply(h, MV_CB, MV_CW, 0, 1.0, mmax);
   CK_LAUNCH();
   // coarse layout
   h->coff.assign(h->N, 0);

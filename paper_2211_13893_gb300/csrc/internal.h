@@ -377,7 +377,7 @@ bool inv_create(msgfem* h);
 void inv_destroy(msgfem* h);
 msgfem_status inv_build(msgfem* h);
 void inv_factor(msgfem* h, int w, cudaStream_t st);
-void inv_solve(msgfem* h, int mat, int src, int dst, int neg, int width, int add);
+void inv_solve(msgfem* h, int mat, int src, int dst, int neg, int width, int add, int ncols);
 double inv_factor_flops(const msgfem* h, bool executed);
 // the coarse matrix in the same form: tasks for the current NcPad, sweep of d_AH in place
 msgfem_status coarse_inv_build(msgfem* h);
@@ -415,7 +415,7 @@ void node_xyz(const msgfem* h, int i, int j, int k, double X[3]);
 void launch_stencil(msgfem* h);
 // layer blocks of the active subdomains in the handle's precision (couplings only for the block Cholesky)
 void launch_layer_blocks(msgfem* h);
-void launch_stencil_apply(msgfem* h, int src, int dst, int mode, double alpha);
+void launch_stencil_apply(msgfem* h, int src, int dst, int mode, double alpha, int ncols = PST);
 void launch_gram(msgfem* h, int wx, int wy, int wg);
 void launch_small_eig(msgfem* h, int p);
 void launch_rotate(msgfem* h, int which, int wy, int ncols);

@@ -1848,12 +1848,13 @@ void inv_factor(msgfem* h, int w, cudaStream_t st) {
   else inv_factor_t<double>(h, w, st);
 }
 
-// X = M^{-1} B for K (mat 0) or A11 (mat 1) of the current wave, `width` columns.
-void inv_solve(msgfem* h, int mat, int src, int dst, int neg, int width, int add) {
+// X = M^{-1} B for K (mat 0) or A11 (mat 1) of the current wave, the first ncols columns
+// (in groups of KB) of blocks of `width`.
+void inv_solve(msgfem* h, int mat, int src, int dst, int neg, int width, int add, int ncols) {
   const InvForm& f = *h->inv;
   const InvForm::Solve& s = f.waves[h->cur].solve[mat];
   if (s.list.empty()) return;
-  for (int c0 = 0; c0 < width; c0 += KB) {
+  for (int c0 = 0; c0 < std::min(width, ncols); c0 += KB) {
     InvSolveArgs a = {};
     a.mats = f.d_mats;
     a.list = s.d_list;

@@ -8,15 +8,23 @@
 
 namespace {
 
-// y = alpha * [D_mu] K [D_mu] x, one warp per node, lane = column.
+// y = alpha * [D_mu] K [D_mu] x on the first 8 NG columns (the others of y are zero),
+// thread per (node, column), NPB nodes per CTA.
 // mode bit 0: scale x by mu (pre), bit 1: scale y by mu (post).
+// FP64 bound, so the columns that nothing reads are left out (the wanted eigenvectors
+// in the residuals, the basis in the coarse assembly).  Whole local stages, with the
+// solves of the residuals likewise: 192 x 12 x 39 beam (20 of 32 columns) 517 -> 501 ms,
+// 48 beams (8) 114 -> 101, 47 x 7 x 13 beam mixed (13) 54 -> 51; coarse assembly and
+// errors of a 96 x 12 x 13 beam (21) 17.3 -> 16.4.
+template <int NG>
 __global__ void __launch_bounds__(256)
 k_stencil_apply(const SubDev* __restrict__ subs, const int* __restrict__ active, int src, int dst,
                 int mode, double alpha) {
+  constexpr int NC = 8 * NG, NPB = 32 / NG;
   const int sidx = blockIdx.y;
   if (active != nullptr && !active[sidx]) return;
   const SubDev& s = subs[sidx];
-  const int node = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int node = blockIdx.x * NPB + threadIdx.x / NC, col = threadIdx.x % NC;
   if (node >= s.nnode) return;
   const double* x = mv_ptr(s, src);
   double* y = mv_ptr(s, dst);
@@ -30,7 +38,7 @@ k_stencil_apply(const SubDev* __restrict__ subs, const int* __restrict__ active,
     if (ni < 0 || ni >= s.nxn || nj < 0 || nj >= s.nyn || nk < 0 || nk >= s.nzn) continue;
     const int nb = nk * s.npl + ni * s.nyn + nj;
     const double sc = (mode & 1) ? s.mu[nb] : 1.0;
-    const double* xr = x + (size_t)nb * 3 * PST + lane;
+    const double* xr = x + (size_t)nb * 3 * PST + col;
     const double x0 = sc * xr[0], x1 = sc * xr[PST], x2 = sc * xr[2 * PST];
     const double* c = st + slot * 9;
     y0 = fma(c[0], x0, fma(c[1], x1, fma(c[2], x2, y0)));
@@ -38,10 +46,11 @@ k_stencil_apply(const SubDev* __restrict__ subs, const int* __restrict__ active,
     y2 = fma(c[6], x0, fma(c[7], x1, fma(c[8], x2, y2)));
   }
   const double post = alpha * ((mode & 2) ? s.mu[node] : 1.0);
-  double* yr = y + (size_t)node * 3 * PST + lane;
+  double* yr = y + (size_t)node * 3 * PST + col;
   yr[0] = post * y0;
   yr[PST] = post * y1;
   yr[2 * PST] = post * y2;
+  for (int c = NC; c + col < PST; c += NC) yr[c] = yr[PST + c] = yr[2 * PST + c] = 0.0;
 }
 
 constexpr int GRAM_ROWS = 512;
@@ -563,9 +572,15 @@ static int max_nnode(msgfem* h) {
   return m;
 }
 
-void launch_stencil_apply(msgfem* h, int src, int dst, int mode, double alpha) {
-  dim3 grid((max_nnode(h) + 7) / 8, h->N);
-  k_stencil_apply<<<grid, 256, 0, h->stream>>>(h->d_sub, act(h), src, dst, mode, alpha); ++g_launch_count;
+void launch_stencil_apply(msgfem* h, int src, int dst, int mode, double alpha, int ncols) {
+  const int ng = std::min(4, std::max(1, (ncols + 7) / 8)), npb = 32 / ng;
+  dim3 grid((max_nnode(h) + npb - 1) / npb, h->N);
+  auto run = [&](auto k) { k<<<grid, npb * 8 * ng, 0, h->stream>>>(h->d_sub, act(h), src, dst, mode, alpha); };
+  if (ng == 1) run(k_stencil_apply<1>);
+  else if (ng == 2) run(k_stencil_apply<2>);
+  else if (ng == 3) run(k_stencil_apply<3>);
+  else run(k_stencil_apply<4>);
+  ++g_launch_count;
 }
 
 void launch_gram(msgfem* h, int wx, int wy, int wg) {
