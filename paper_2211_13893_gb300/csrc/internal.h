@@ -254,6 +254,7 @@ struct msgfem {
   InvForm* inv = nullptr;            // inverse form, when the handle is eligible
   bool inv_on = false;               // factorisations and solves run in the inverse form
   int factor_persistent = 0;         // mixed: FP32 factorisation as one persistent launch
+  int refine_last[2] = {0, 0};       // steps the last adaptive refinement took (K, A11): when to look at its flags
   int refine = 2;                    // FP64 refinement steps per FP32 solve
   std::vector<CoarsePair> pairs;
   CoarsePair* d_pairs = nullptr;
