@@ -306,7 +306,7 @@ msgfem_status allocate(msgfem* h) {
   int maxnode = 0;
   for (const auto& s : h->sub) maxnode = std::max(maxnode, s.nnode);
   const size_t nchunk = (3 * (size_t)maxnode + 511) / 512;
-  TRY(dalloc(h, &h->d_gram_part, nchunk * h->N * PST * PST));
+  TRY(dalloc(h, &h->d_gram_part, std::max(nchunk * h->N * PST * PST, (size_t)GRAM_KB_PARTS * MQ * KB)));
   TRY(dalloc(h, &h->d_flags, h->N + 1));
   TRY(dalloc(h, &h->d_flags_saved, h->N + 1));
   TRY(dalloc(h, &h->d_rprev, (size_t)h->N * KB));
@@ -540,8 +540,9 @@ void timed_solve_w(msgfem* h, int mat, int src, int dst, int neg, int width, int
   if (h->inv_on) {
     inv_solve(h, mat, src, dst, neg, width, add, ncols);
     span_end(h, sp);
-    h->prof.solve_flops += solve_flops(h, mat, width == KB ? KB : h->p);
-    h->prof.solve_bytes += solve_bytes(h, mat, width == KB ? KB : h->p);
+    const int cols = width == KB ? KB : std::min(h->p, ncols);
+    h->prof.solve_flops += solve_flops(h, mat, cols);
+    h->prof.solve_bytes += solve_bytes(h, mat, cols);
     h->prof.solve_calls += 1;
     return;
   }

@@ -26,6 +26,7 @@
 #define PST 32
 #define KB 8      // block width of the block Krylov eigensolver
 #define MQ 96     // largest Krylov basis (12 blocks)
+#define GRAM_KB_PARTS 1024   // partial sums of a block Gram product that d_gram_part holds for any size
 
 // Tile task: C(64x64) = [C +] sign * [P *] A(64 x K) * op(B), or with
 // G_POTRF the Cholesky factor and inverse of the SPD tile C (in place) with the

@@ -81,13 +81,22 @@ k_stencil_kb(const SubDev* __restrict__ subs, const int* __restrict__ active, in
   yr[2 * KB] = post * y2;
 }
 
-constexpr int KROWS = 512;
+// Rows per partial sum of a Gram product: the fewest of 64 .. 512 with at most
+// GRAM_KB_PARTS partial sums over all subdomains (whose slots d_gram_part holds in any
+// case).  FP64 bound once every SM has work; 512 rows leave few subdomains on few SMs:
+// 40 x 6 x 12 beam, 8 subdomains, 8 to 96 columns: 407 products 24 -> 5 ms.
+int gram_kb_rows(const msgfem* h, int nfull) {
+  int rows = 64;
+  while (rows < 512 && (size_t)h->N * ((nfull + rows - 1) / rows) > GRAM_KB_PARTS) rows *= 2;
+  return rows;
+}
 
 // Partial sums of G[a][b] = sum_r X[r][a] Y[r][b], a < nx (X of stride xs),
-// b < KB (Y of stride KB).
+// b < KB (Y of stride KB), over krows rows (a multiple of 32).  Up to 16 columns of X the
+// threads form 2 or 4 groups that share the rows.
 __global__ void __launch_bounds__(256)
 k_gram_kb_partial(const SubDev* __restrict__ subs, const int* __restrict__ active, int wx, int xs, int nx, int wy,
-                  int only_floating, double* __restrict__ part, int nchunk) {
+                  int only_floating, double* __restrict__ part, int nchunk, int krows) {
   const int sidx = blockIdx.y;
   if (active != nullptr && !active[sidx]) return;
   const SubDev& s = subs[sidx];
@@ -97,10 +106,11 @@ k_gram_kb_partial(const SubDev* __restrict__ subs, const int* __restrict__ activ
   const double* X = mv_ptr(s, wx);
   const double* Yv = mv_ptr(s, wy);
   const int tid = threadIdx.x;
-  const int nout = nx * KB;
+  const int nout = nx * KB, groups = nx <= 8 ? 4 : (nx <= 16 ? 2 : 1), per = 256 / groups;
+  const int g = tid / per, nr = 32 / groups, f0 = g * nr;
   double acc[3] = {0.0, 0.0, 0.0};
-  const int r0 = blockIdx.x * KROWS;
-  const int r1 = min(r0 + KROWS, s.nfull);
+  const int r0 = blockIdx.x * krows;
+  const int r1 = min(r0 + krows, s.nfull);
   for (int rb = r0; rb < r1; rb += 32) {
     for (int e = tid; e < 32 * nx; e += 256) {
       const int rr = rb + e / nx;
@@ -112,30 +122,41 @@ k_gram_kb_partial(const SubDev* __restrict__ subs, const int* __restrict__ activ
     }
     __syncthreads();
     for (int i = 0; i < 3; ++i) {
-      const int o = tid + 256 * i;
+      const int o = tid % per + 256 * i;
       if (o >= nout) break;
       const int a = o / KB, b = o % KB;
       double v = acc[i];
 #pragma unroll 8
-      for (int r = 0; r < 32; ++r) v = fma(Xs[r][a], Ys[r][b], v);
+      for (int r = 0; r < nr; ++r) v = fma(Xs[f0 + r][a], Ys[f0 + r][b], v);
       acc[i] = v;
     }
     __syncthreads();
   }
   double* out = part + ((size_t)sidx * nchunk + blockIdx.x) * MQ * KB;
+  if (groups > 1) {   // nout <= per: one output per thread
+    double* sum = &Xs[0][0];
+    sum[tid] = acc[0];
+    __syncthreads();
+    if (tid < nout) {
+      double v = sum[tid];
+      for (int q = 1; q < groups; ++q) v += sum[tid + q * per];
+      out[tid] = v;
+    }
+    return;
+  }
   for (int i = 0; i < 3; ++i) {
     const int o = tid + 256 * i;
-    if (o < nout) out[o] = r0 < s.nfull ? acc[i] : 0.0;
+    if (o < nout) out[o] = acc[i];
   }
 }
 
 __global__ void k_gram_kb_reduce(const SubDev* __restrict__ subs, const int* __restrict__ active, int nx,
-                                 int only_floating, const double* __restrict__ part, int nchunk) {
+                                 int only_floating, const double* __restrict__ part, int nchunk, int krows) {
   const int sidx = blockIdx.x;
   if (active != nullptr && !active[sidx]) return;
   const SubDev& s = subs[sidx];
   if (only_floating && !s.floating) return;
-  const int nc = (s.nfull + KROWS - 1) / KROWS;
+  const int nc = (s.nfull + krows - 1) / krows;
   for (int o = threadIdx.x; o < nx * KB; o += blockDim.x) {
     double acc = 0.0;
     for (int c = 0; c < nc; ++c) acc += part[((size_t)sidx * nchunk + c) * MQ * KB + o];
@@ -184,59 +205,72 @@ __global__ void k_h_accum(const SubDev* __restrict__ subs, const int* __restrict
 // Gram-Schmidt (the Krylov space is exhausted) -- and keeps R1 = L^T in
 // Y[KB:2KB][0:KB].  Pass 2 re-orthonormalises the surviving columns and, for
 // j >= 0, stores R_{j+1} = L2^T R1 in H[(j+1) KB + r][j KB + c].
+// One warp per subdomain, a lane per row of the column's elimination and per column of
+// the inverse (50 us in one thread,
+// 16 here).
 __global__ void k_cholqr_kb(const SubDev* __restrict__ subs, const int* __restrict__ active, int j, int pass) {
   const int sidx = blockIdx.x;
   if (active != nullptr && !active[sidx]) return;
   const SubDev& s = subs[sidx];
-  if (threadIdx.x != 0) return;
-  double G[KB][KB], L[KB][KB], U[KB][KB], n0[KB];
-  for (int a = 0; a < KB; ++a)
-    for (int b = 0; b < KB; ++b) { G[a][b] = 0.5 * (s.Hc[a * KB + b] + s.Hc[b * KB + a]); L[a][b] = 0.0; U[a][b] = 0.0; }
-  for (int c = 0; c < KB; ++c) {
-    n0[c] = G[c][c];
-    if (pass == 1 && j >= 0)
-      for (int a = 0; a < (j + 1) * KB; ++a) {
-        const double hc = s.H[(size_t)a * MQ + j * KB + c];
-        n0[c] += hc * hc;
-      }
+  __shared__ double G[KB][KB], L[KB][KB], U[KB][KB], R1[KB][KB];
+  const int lane = threadIdx.x;
+  for (int e = lane; e < KB * KB; e += 32) {
+    const int a = e / KB, b = e % KB;
+    G[a][b] = 0.5 * (s.Hc[a * KB + b] + s.Hc[b * KB + a]);
+    L[a][b] = U[a][b] = 0.0;
+    R1[a][b] = pass == 2 ? s.Y[(KB + a) * PST + b] : 0.0;
   }
-  bool dead[KB];
+  __syncwarp();
+  // lanes c, c + 8, c + 16, c + 24: squared norm of column c before Gram-Schmidt
+  double n0 = 0.0;
+  if (pass == 1 && j >= 0)
+    for (int a = lane / KB; a < (j + 1) * KB; a += 32 / KB) {
+      const double hc = s.H[(size_t)a * MQ + j * KB + lane % KB];
+      n0 += hc * hc;
+    }
+  n0 += __shfl_xor_sync(0xffffffffu, n0, 8);
+  n0 += __shfl_xor_sync(0xffffffffu, n0, 16);
+  n0 += G[lane % KB][lane % KB];
+  unsigned dead = 0;   // the same in every lane
   for (int c = 0; c < KB; ++c) {
     double v = G[c][c];
     for (int k = 0; k < c; ++k) v -= L[c][k] * L[c][k];
-    dead[c] = !(G[c][c] > 0.0) || !(v > 1e-12 * G[c][c]) || !(v > 1e-20 * n0[c]);
-    if (dead[c]) {
-      s.status[3] = 1;
+    const double nc = __shfl_sync(0xffffffffu, n0, c);
+    if (!(G[c][c] > 0.0) || !(v > 1e-12 * G[c][c]) || !(v > 1e-20 * nc)) {
+      dead |= 1u << c;
+      if (lane == 0) s.status[3] = 1;
       continue;
     }
-    L[c][c] = sqrt(v);
-    for (int r = c + 1; r < KB; ++r) {
-      double w = G[r][c];
-      for (int k = 0; k < c; ++k) w -= L[r][k] * L[c][k];
-      L[r][c] = w / L[c][c];
+    const double d = sqrt(v);
+    double w = d;
+    if (lane > c && lane < KB) {
+      w = G[lane][c];
+      for (int k = 0; k < c; ++k) w -= L[lane][k] * L[c][k];
+      w /= d;
     }
+    if (lane >= c && lane < KB) L[lane][c] = w;
+    __syncwarp();
   }
-  for (int c = 0; c < KB; ++c) {
-    if (dead[c]) continue;
+  if (lane < KB && !((dead >> lane) & 1)) {
+    const int c = lane;
     for (int i = c; i >= 0; --i) {
-      if (dead[i]) continue;
+      if ((dead >> i) & 1) continue;
       double v = (i == c) ? 1.0 : 0.0;
       for (int k = i + 1; k <= c; ++k) v -= L[k][i] * U[k][c];
       U[i][c] = v / L[i][i];
     }
   }
-  for (int a = 0; a < KB; ++a)
-    for (int b = 0; b < KB; ++b) s.Y[a * PST + b] = U[a][b];
-  if (pass == 1) {
-    for (int r = 0; r < KB; ++r)
-      for (int c = 0; c < KB; ++c) s.Y[(KB + r) * PST + c] = L[c][r];
-  } else if (j >= 0) {
-    for (int r = 0; r < KB; ++r)
-      for (int c = 0; c < KB; ++c) {
-        double v = 0.0;
-        for (int k = 0; k < KB; ++k) v += L[k][r] * s.Y[(KB + k) * PST + c];   // (L2^T R1)[r][c]
-        s.H[(size_t)((j + 1) * KB + r) * MQ + j * KB + c] = v;
-      }
+  __syncwarp();
+  for (int e = lane; e < KB * KB; e += 32) {
+    const int r = e / KB, c = e % KB;
+    s.Y[r * PST + c] = U[r][c];
+    if (pass == 1) {
+      s.Y[(KB + r) * PST + c] = L[c][r];
+    } else if (j >= 0) {
+      double v = 0.0;
+      for (int k = 0; k < KB; ++k) v += L[k][r] * R1[k][c];   // (L2^T R1)[r][c]
+      s.H[(size_t)((j + 1) * KB + r) * MQ + j * KB + c] = v;
+    }
   }
 }
 
@@ -657,15 +691,23 @@ void launch_stencil_kb(msgfem* h, int src, int dst, int mode, double alpha) {
 
 // Hc[0:nx][0:KB] = X[:, 0:nx]^T Y
 void launch_gram_kb(msgfem* h, int wx, int xs, int nx, int wy, int only_floating) {
-  const int nchunk = (3 * max_nnode_k(h) + KROWS - 1) / KROWS;
+  const int nfull = 3 * max_nnode_k(h), krows = gram_kb_rows(h, nfull), nchunk = (nfull + krows - 1) / krows;
   dim3 grid(nchunk, h->N);
   k_gram_kb_partial<<<grid, 256, 0, h->stream>>>(h->d_sub, h->d_flags, wx, xs, nx, wy, only_floating,
-                                                 h->d_gram_part, nchunk); ++g_launch_count;
-  k_gram_kb_reduce<<<h->N, 256, 0, h->stream>>>(h->d_sub, h->d_flags, nx, only_floating, h->d_gram_part, nchunk); ++g_launch_count;
+                                                 h->d_gram_part, nchunk, krows); ++g_launch_count;
+  k_gram_kb_reduce<<<h->N, 256, 0, h->stream>>>(h->d_sub, h->d_flags, nx, only_floating, h->d_gram_part, nchunk, krows);
+  ++g_launch_count;
+}
+
+// CTAs per subdomain of the row-wise block kernels (32 rows per pass): 256 rows each, or
+// down to 32 while that leaves less than about eight CTAs per SM.
+static int row_ctas(msgfem* h) {
+  const int rows = 3 * max_nnode_k(h);
+  return std::max(1, std::min((rows + 31) / 32, std::max((rows + 255) / 256, 1216 / h->N)));
 }
 
 void launch_update_kb(msgfem* h, int wx, int xs, int nx, int wy, int only_floating) {
-  dim3 grid(std::max(1, (3 * max_nnode_k(h) + 255) / 256), h->N);
+  dim3 grid(row_ctas(h), h->N);
   k_update_kb<<<grid, 256, 0, h->stream>>>(h->d_sub, h->d_flags, wx, xs, nx, wy, only_floating); ++g_launch_count;
 }
 
@@ -676,7 +718,7 @@ void launch_h_accum(msgfem* h, int m, int j, int add) {
 void launch_cholqr_kb(msgfem* h, int j, int pass) { k_cholqr_kb<<<h->N, 32, 0, h->stream>>>(h->d_sub, h->d_flags, j, pass); ++g_launch_count; }
 
 void launch_rotate_kb(msgfem* h, int which) {
-  dim3 grid(std::max(1, (3 * max_nnode_k(h) + 255) / 256), h->N);
+  dim3 grid(row_ctas(h), h->N);
   k_rotate_kb<<<grid, 256, 0, h->stream>>>(h->d_sub, h->d_flags, which); ++g_launch_count;
 }
 
