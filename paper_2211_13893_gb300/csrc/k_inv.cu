@@ -29,9 +29,9 @@
 // 4 CG steps to 1e-11 where the Cholesky form takes 5 to 6).
 //
 // Measured on one GB300 against the block Cholesky (factorisation / all solves of a
-// local stage, ms): 36 x 12 x 39 beam FP64 345 -> 46 / 424 -> 54; 192 x 12 x 39 beam
+// local stage, ms): 36 x 12 x 39 beam FP64 345 -> 46 / 424 -> 41; 192 x 12 x 39 beam
 // mixed 102 -> 72 / 374 -> 170; C-section of 16 subdomains mixed 85 -> 45 / 409 -> 124;
-// 47 x 7 x 13 beam FP64 whole pass 156 -> 42.
+// 47 x 7 x 13 beam FP64 whole pass 156 -> 34.
 #include "internal.h"
 
 #include <cooperative_groups.h>
@@ -152,12 +152,12 @@ __device__ __forceinline__ void couple_rows(const InvMat& m, int nb, int dk, int
 // digit d + 256, and 0x6400 | d is 1024 + d in FP16.  The factorisation leaves every
 // layer's -S^{-1} in that form in place (8 bytes per entry, 16 x 16 blocks in fragment
 // order: a lane's operands are four 16-byte vectors), so that a solve streams it with
-// bulk copies as before and spends 6 integer instructions per pair of digits; the
+// bulk copies as before and spends five instructions per pair of digits; the
 // right-hand side's digits are cut once per layer by the rank that owns the node
 // and written to every rank of the cluster.  Taken whenever a layer's digits and
 // coefficients fit in shared memory (layers up to about 1,000 DoFs); above, FP64 FMAs.
 // Whole passes with FP64 FMAs -> digits: 36 x 12 x 39 beam 306 -> 204 ms (solves 158 ->
-// 54), 47 x 7 x 13 beam 77 -> 50, 24 x 4 x 12 beam 29 -> 20, Schwarz PCG 45 -> 29; the
+// 54, 41 since), 47 x 7 x 13 beam 77 -> 50, 24 x 4 x 12 beam 29 -> 20, Schwarz PCG 45 -> 29; the
 // passes' errors against a dense 64-bit reference are unchanged.
 constexpr int DIG = 7;
 constexpr long long DIG_BIAS = 256ll * (0x7fffffffffffffffll / 511);   // sum of 256 512^i, i < 7
@@ -176,7 +176,7 @@ __device__ __forceinline__ long long biased_fixed(double x, int emax) {
 
 // digit i of two biased integers as a pair of FP16 numbers
 __device__ __forceinline__ uint32_t digit_pair(long long x0, long long x1, int i) {
-  const uint32_t d = ((uint32_t)(x0 >> (9 * i)) & 0x1ff) | (((uint32_t)(x1 >> (9 * i)) & 0x1ff) << 16) | 0x64006400u;
+  const uint32_t d = (__byte_perm((uint32_t)(x0 >> (9 * i)), (uint32_t)(x1 >> (9 * i)), 0x5410) & 0x01ff01ffu) | 0x64006400u;
   uint32_t r;
   asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(d), "r"(0xe500e500u));   // - 1280
   return r;
@@ -1165,8 +1165,9 @@ k_inv_solve_f32(const InvSolveArgs a) {
 
 // ---------------------------------------------------------------------------
 // FP64 solve in digit products
-constexpr int FX_KB = 16;                      // 16 x 16 blocks per stage (two per warp)
-constexpr int FX_STAGE = FX_KB * 256 * 8;      // bytes
+constexpr int FX_WARPS = 16;                    // two groups of eight
+constexpr int FX_STAGE = FX_WARPS * 2048;       // bytes of a ring level: a 16 x 16 block for each warp
+constexpr int FX_RED = 2 * 4 * 128 * 16;        // bytes of the partial sums of the groups' strips
 
 // biased exponents of the rows of layer l (at the end of the layer's L slot)
 __device__ __forceinline__ int* row_exponents(const InvMat& m, int l) {
@@ -1203,8 +1204,18 @@ k_inv_digits(const InvMat* __restrict__ mats, const int* __restrict__ active) {
   if (tid < 16) row_exponents(m, l)[s * 16 + tid] = em[tid];
 }
 
+// Two groups of eight warps take the rank's strips in turn; a warp owns an eighth of the
+// columns and streams its blocks through its own ring (nobody else waits for them); the
+// eight sums of a strip, 64-bit integers, meet in shared memory once per strip and the
+// results are written once per layer.
+// Bound by the integer and FP16 pipes (five instructions per pair of digits) and, per
+// layer, the FP64 sparse step (6 us of 37 on 693 DoFs and 8 ranks) and three barriers.  A
+// stage of 16 blocks per CTA with shared 64-bit atomics and a CTA barrier per stage took
+// 1.00 ms per half solve of the 36 x 12 x 39 beam, 0.75 here (0.86 with one group of eight
+// warps); whole passes 139.4 -> 127.6 ms, 47 x 7 x 13 beam 37.0 -> 34.2, GenEO comparison
+// 211 -> 207, Schwarz PCG 15.9 -> 15.4.
 template <bool BACK>
-__global__ void __launch_bounds__(256, 1)
+__global__ void __launch_bounds__(32 * FX_WARPS, 1)
 k_inv_solve_fx(const InvSolveArgs a) {
   cg::cluster_group cl = cg::this_cluster();
   const int G = (int)cl.num_blocks(), g = (int)cl.block_rank();
@@ -1223,26 +1234,37 @@ k_inv_solve_fx(const InvSolveArgs a) {
   uint32_t* zd = reinterpret_cast<uint32_t*>(smem_fs + a.smem_z);   // [DIG][8 nkb pairs of rows][KB] FP16 pairs
   double* uw = reinterpret_cast<double*>(smem_fs + a.smem_u);
   double* cf = reinterpret_cast<double*>(smem_fs + a.smem_c);
-  double* zo = reinterpret_cast<double*>(smem_fs + a.smem_r);       // z of the own nodes
-  __shared__ __align__(8) unsigned long long bars[9];
-  __shared__ unsigned long long red[2][128][2];
+  longlong2* red = reinterpret_cast<longlong2*>(smem_fs + a.smem_r);          // [2 groups][4][128]
+  double* zo = reinterpret_cast<double*>(smem_fs + a.smem_r + FX_RED);        // z of the own nodes, then the results
+  __shared__ __align__(8) unsigned long long bars[8 * FX_WARPS + 1];
   __shared__ int zm[KB], zmax[8][KB];
-  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int b = m.b, nn = m.n / 3, nkb = (m.n + 15) / 16, NC = (nkb + FX_KB - 1) / FX_KB;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, grp = w >> 3, wg = w & 7, gt = tid & 255;
+  const int b = m.b, nn = m.n / 3, nkb = (m.n + 15) / 16;
   const int s0 = nkb * g / G, s1 = nkb * (g + 1) / G, ns = s1 - s0;
   const int npc = up4((nn + G - 1) / G), p0 = min(nn, npc * g), p1 = min(nn, p0 + npc);
   const int wlo = max(0, p0 - m.njc - 1);
-  const uint32_t ring_s = tc::saddr(ring), bar0 = tc::saddr(bars), cf_s = tc::saddr(cf);
-  const int total = ns * NC * steps;
-  bool ok = true;
-  int issued = 0;   // stages requested (thread 0)
-  auto issue = [&](int i) {
-    issued = i + 1;
-    const int c = i % NC, sl = i / NC, l = layer_of(sl / ns), s = s0 + sl % ns;
-    const uint32_t bytes = (uint32_t)min(FX_KB, nkb - c * FX_KB) * 2048u, bar = bar0 + 8 * (i % a.ring);
-    tc::mbar_expect_tx(bar, bytes);
-    bulk_load(ring_s + (uint32_t)(i % a.ring) * FX_STAGE,
-              static_cast<const double*>(m.D) + ((size_t)l * b + (size_t)s * 16) * b + (size_t)c * FX_KB * 256, bytes, bar);
+  const uint32_t bar0 = tc::saddr(bars), cbar = bar0 + 8 * 8 * FX_WARPS, cf_s = tc::saddr(cf);
+  // the warp's ring: its blocks of the group's strips, layer by layer
+  const int kw0 = nkb * wg / 8, nw = nkb * (wg + 1) / 8 - kw0, nsg = (ns + 1 - grp) / 2;
+  const int total = nsg * nw * steps, depth = a.ring;
+  const uint32_t ring_s = tc::saddr(ring) + (uint32_t)w * depth * 2048, wbar = bar0 + 8 * 8 * w;
+  const longlong2* slots = reinterpret_cast<const longlong2*>(ring) + (size_t)w * depth * 128;
+  bool ok = true, cok = true;
+  int used = 0, issued = 0, ist = 0, iss = 0, isb = 0;   // blocks consumed, requested; step, strip, block of the next
+  auto issue = [&]() {
+    if (lane != 0 || issued >= total || !ok) return;
+    const int slot = issued % depth;
+    tc::fence_async_smem();
+    tc::mbar_expect_tx(wbar + 8 * slot, 2048u);
+    bulk_load(ring_s + slot * 2048u,
+              static_cast<const double*>(m.D) + ((size_t)layer_of(ist) * b + (size_t)(s0 + grp + 2 * iss) * 16) * b +
+                  (size_t)(kw0 + isb) * 256,
+              2048u, wbar + 8 * slot);
+    ++issued;
+    if (++isb == nw) {
+      isb = 0;
+      if (++iss == nsg) { iss = 0; ++ist; }
+    }
   };
   const int cdir = BACK ? (half ? 0 : 1) : (half ? 1 : 0);
   const uint32_t cbytes = p1 > p0 ? (uint32_t)(up4(p1 - p0) * 81 * sizeof(double)) : 0;
@@ -1250,33 +1272,31 @@ k_inv_solve_fx(const InvSolveArgs a) {
     return static_cast<const double*>(m.L) + (size_t)l * b * b + ((size_t)dir * up4(nn) + p0) * 81;
   };
   if (tid == 0) {
-    for (int i = 0; i < 9; ++i) tc::mbar_init(bar0 + 8 * i, 1);
+    for (int i = 0; i < 8 * FX_WARPS + 1; ++i) tc::mbar_init(bar0 + 8 * i, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    for (int i = 0; i < a.ring && i < total; ++i) issue(i);
   }
-  for (int e = tid; e < DIG * nkb * 8 * KB; e += 256) zd[e] = 0u;
-  red[tid >> 7][tid & 127][0] = 0ull;
-  red[tid >> 7][tid & 127][1] = 0ull;
+  for (int e = tid; e < DIG * nkb * 8 * KB; e += 32 * FX_WARPS) zd[e] = 0u;
   if (tid < KB) zm[tid] = 0;
   __syncthreads();
+  for (int i = 0; i < depth; ++i) issue();
   const SubDev& sd = a.subs[m.sub];
   const double* src = mv_ptr(sd, a.src) + a.coloff;
   double* dst = mv_ptr(sd, a.dst) + a.coloff;
   double* yc = static_cast<double*>(m.yc);
   const double sgn = a.neg ? -1.0 : 1.0;
-  int cphase = 0, ci = 0, waited = 0, strip = 0;
+  int cphase = 0;
   bool cpend = false;
   cl.sync();   // no remote store before every CTA of the cluster has cleared its arrays
   for (int t = 0; t < steps; ++t) {
     const int l = layer_of(t);
     const bool first = t == 0;
     if (cpend) {
-      if (ok) ok = tc::mbar_wait(bar0 + 64, cphase & 1);
+      if (cok) cok = tc::mbar_wait(cbar, cphase & 1);
       ++cphase;
     }
     // ---- sparse step on the own nodes (FP64), the largest exponent per column
     int mx = 0;
-    for (int e = tid; e < (p1 - p0) * KB; e += 256) {
+    for (int e = tid; e < (p1 - p0) * KB; e += 32 * FX_WARPS) {
       const int pl = e / KB, col = e % KB, p = p0 + pl;
       const int i = p / m.njc, j = p % m.njc;
       double z[3] = {0.0, 0.0, 0.0};
@@ -1324,10 +1344,10 @@ k_inv_solve_fx(const InvSolveArgs a) {
     cl.sync();
     // the coupling buffer is free: request the next layer's
     cpend = t + 1 < steps && cbytes > 0;
-    if (cpend && ok && tid == 0) {
+    if (cpend && cok && tid == 0) {
       tc::fence_async_smem();
-      tc::mbar_expect_tx(bar0 + 64, cbytes);
-      bulk_load(cf_s, coupling_ptr(layer_of(t + 1), cdir), cbytes, bar0 + 64);
+      tc::mbar_expect_tx(cbar, cbytes);
+      bulk_load(cf_s, coupling_ptr(layer_of(t + 1), cdir), cbytes, cbar);
     }
     // ---- digits of the own rows (in pairs) to every rank
     if (tid < KB) zm[tid] = 0;
@@ -1335,7 +1355,7 @@ k_inv_solve_fx(const InvSolveArgs a) {
       const int rows = 3 * (p1 - p0), col = tid % KB;
       int ez = 0;
       for (int q = 0; q < G; ++q) ez = max(ez, zmax[q][col]);
-      for (int e = tid; e < (rows + 1) / 2 * KB; e += 256) {
+      for (int e = tid; e < (rows + 1) / 2 * KB; e += 32 * FX_WARPS) {
         const int rp = e / KB;
         const long long x0 = biased_fixed(zo[2 * rp * KB + col], ez);
         const long long x1 = 2 * rp + 1 < rows ? biased_fixed(zo[(2 * rp + 1) * KB + col], ez) : DIG_BIAS;
@@ -1352,91 +1372,101 @@ k_inv_solve_fx(const InvSolveArgs a) {
     }
     cl.sync();
     // ---- dense step on the own strips of 16 rows
-    for (int s = s0; s < s1; ++s, ++strip) {
-      for (int c = 0; c < NC; ++c, ++ci) {
-        const int slot = ci % a.ring;
-        if (ok) {
-          ok = tc::mbar_wait(bar0 + 8 * slot, (ci / a.ring) & 1);
-          if (ok) waited = ci + 1;
-        }
-        const int k0 = c * FX_KB + 2 * w, k1 = min(nkb, k0 + 2);
-        if (k0 < k1) {
-          float acc[DIG][4];
+    int ezc = 0;   // of the column of the strip's sums that this thread adds up
+    for (int q = 0; q < G; ++q) ezc = max(ezc, zmax[q][(gt >> 1) % KB]);
+    auto group_sync = [&]() { asm volatile("bar.sync %0, 256;" ::"r"(1 + grp) : "memory"); };
+    longlong2* rd = red + grp * 4 * 128;
+    for (int s = s0 + grp; s < s1; s += 2) {
+      const int er = row_exponents(m, l)[s * 16 + (gt >> 1) / KB];
+      long long hi[4] = {}, lo[4] = {};
+      for (int k0 = 0; k0 < nw; k0 += 2) {
+        float acc[DIG][4];
 #pragma unroll
-          for (int i = 0; i < DIG; ++i)
+        for (int i = 0; i < DIG; ++i)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) acc[i][e] = 0.f;
-          for (int kb = k0; kb < k1; ++kb) {
-            const longlong2* ap = reinterpret_cast<const longlong2*>(ring + (size_t)slot * FX_STAGE + (size_t)(kb - c * FX_KB) * 2048);
-            longlong2 x[4];
+          for (int e = 0; e < 4; ++e) acc[i][e] = 0.f;
+        for (int kb = k0; kb < min(nw, k0 + 2); ++kb, ++used) {
+          const int slot = used % depth;
+          if (ok) ok = tc::mbar_wait(wbar + 8 * slot, (used / depth) & 1);
+          const longlong2* ap = slots + slot * 128;
+          longlong2 x[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) x[j] = ap[j * 32 + lane];
-            uint32_t bz[DIG][2];
-            const uint32_t* zp = zd + (kb * 8 + (lane & 3)) * KB + (lane >> 2);
+          for (int j = 0; j < 4; ++j) x[j] = ap[j * 32 + lane];
+          uint32_t bz[DIG][2];
+          const uint32_t* zp = zd + ((kw0 + kb) * 8 + (lane & 3)) * KB + (lane >> 2);
 #pragma unroll
-            for (int i = 0; i < DIG; ++i) {
-              bz[i][0] = zp[i * nkb * 8 * KB];
-              bz[i][1] = zp[i * nkb * 8 * KB + 4 * KB];
-            }
-#pragma unroll
-            for (int i = 0; i < DIG; ++i) {
-              uint32_t av[4];
-#pragma unroll
-              for (int j = 0; j < 4; ++j) av[j] = digit_pair(x[j].x, x[j].y, i);
-#pragma unroll
-              for (int j = DIG - 1 - i; j < DIG; ++j) mma_f16(acc[i + j - (DIG - 1)], av, bz[j]);
-            }
+          for (int i = 0; i < DIG; ++i) {
+            bz[i][0] = zp[i * nkb * 8 * KB];
+            bz[i][1] = zp[i * nkb * 8 * KB + 4 * KB];
           }
+          __syncwarp();
+          issue();   // the slot is free
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            long long hi = 0, lo = 0;
-            digit_flush(acc, e, hi, lo);
-            unsigned long long* rd = red[strip & 1][((lane >> 2) + 8 * (e >> 1)) * KB + 2 * (lane & 3) + (e & 1)];
-            atomicAdd(rd, (unsigned long long)hi);
-            atomicAdd(rd + 1, (unsigned long long)lo);
+          for (int i = 0; i < DIG; ++i) {
+            uint32_t av[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) av[j] = digit_pair(x[j].x, x[j].y, i);
+#pragma unroll
+            for (int j = DIG - 1 - i; j < DIG; ++j) mma_f16(acc[i + j - (DIG - 1)], av, bz[j]);
           }
         }
-        __syncthreads();
-        if (tid == 0 && ok && ci + a.ring < total) {
-          tc::fence_async_smem();
-          issue(ci + a.ring);
-        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) digit_flush(acc, e, hi[e], lo[e]);
       }
-      if (tid < 128) {
-        const int row = s * 16 + tid / KB, col = tid % KB;
-        unsigned long long* rd = red[strip & 1][tid];
-        const long long hi = (long long)rd[0], lo = (long long)rd[1];
-        rd[0] = 0ull;
-        rd[1] = 0ull;
-        if (row < m.n) {
-          int ez = 0;
-          for (int q = 0; q < G; ++q) ez = max(ez, zmax[q][col]);
-          const int er = row_exponents(m, l)[row];
-          double y = digit_value(hi, lo, er + ez - 2 * 1023 - 66);
-          if (er == 0x7ff || ez == 0x7ff) y = __longlong_as_double(0x7ff8000000000000ll);   // Inf or NaN operands
-          double* yp = yc + ((size_t)l * b + row) * KB + col;
-          const double x = (BACK && !first) ? *yp - y : -y;   // the block holds -S^{-1}
-          const int p = row / 3;
-          if (!BACK) *yp = x;
-          else if (!first || half == 0) {
-            const size_t node = (size_t)l * m.npl + (size_t)(m.ia + p / m.njc) * m.nyn + m.ja + p % m.njc;
-            double* o = dst + (node * 3 + row % 3) * a.stride + col;
-            *o = a.add ? *o + x : x;
-          }
-          if (t + 1 < steps)
-            for (int q = 0; q < G; ++q) {
-              const int q0 = min(nn, npc * q), lo_n = max(0, q0 - m.njc - 1), hi_n = min(nn, min(nn, q0 + npc) + m.njc + 1);
-              if (p >= lo_n && p < hi_n) cl.map_shared_rank(uw, q)[(size_t)(row - 3 * lo_n) * KB + col] = x;
-            }
+      auto entry = [&](int e) {
+        return (wg & 3) * 128 + ((lane >> 2) + 8 * (e >> 1)) * KB + 2 * (lane & 3) + (e & 1);
+      };
+      group_sync();   // the previous strip's sums have been read
+      if (wg >= 4)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) rd[entry(e)] = make_longlong2(hi[e], lo[e]);
+      group_sync();
+      if (wg < 4)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const longlong2 v = rd[entry(e)];
+          rd[entry(e)] = make_longlong2(hi[e] + v.x, lo[e] + v.y);
         }
+      group_sync();
+      // threads 2 i, 2 i + 1 of the group: the high and the low sum of entry i
+      const long long* part = reinterpret_cast<const long long*>(rd) + gt;
+      long long sum = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) sum += part[q * 256];
+      const long long other = __shfl_xor_sync(0xffffffffu, sum, 1);
+      if (!(tid & 1)) {
+        double y = digit_value(sum, other, er + ezc - 2 * 1023 - 66);
+        if (er == 0x7ff || ezc == 0x7ff) y = __longlong_as_double(0x7ff8000000000000ll);   // Inf or NaN operands
+        zo[(s - s0) * 128 + (gt >> 1)] = y;
       }
+    }
+    __syncthreads();
+    for (int e = tid; e < ns * 128; e += 32 * FX_WARPS) {
+      const int row = s0 * 16 + e / KB, col = e % KB;
+      if (row >= m.n) continue;
+      const double y = zo[e];
+      double* yp = yc + ((size_t)l * b + row) * KB + col;
+      const double x = (BACK && !first) ? *yp - y : -y;   // the block holds -S^{-1}
+      const int p = row / 3;
+      if (!BACK) *yp = x;
+      else if (!first || half == 0) {
+        const size_t node = (size_t)l * m.npl + (size_t)(m.ia + p / m.njc) * m.nyn + m.ja + p % m.njc;
+        double* o = dst + (node * 3 + row % 3) * a.stride + col;
+        *o = a.add ? *o + x : x;
+      }
+      if (t + 1 < steps)
+        for (int q = 0; q < G; ++q) {
+          const int q0 = min(nn, npc * q), lo_n = max(0, q0 - m.njc - 1), hi_n = min(nn, min(nn, q0 + npc) + m.njc + 1);
+          if (p >= lo_n && p < hi_n) cl.map_shared_rank(uw, q)[(size_t)(row - 3 * lo_n) * KB + col] = x;
+        }
     }
     cl.sync();
   }
-  if (!__syncthreads_and(ok) && tid == 0) {
-    for (int i = waited; i < issued; ++i) tc::mbar_wait(bar0 + 8 * (i % a.ring), (i / a.ring) & 1);
-    if (cphase > 0) tc::mbar_wait(bar0 + 64, (cphase - 1) & 1);
-    if (a.err != nullptr) atomicExch(a.err, 1);
+  if (!__syncthreads_and(ok && cok)) {
+    if (lane == 0)
+      for (int i = max(0, issued - depth); i < issued; ++i) tc::mbar_wait(wbar + 8 * (i % depth), (i / depth) & 1);
+    if (tid == 0 && cphase > 0) tc::mbar_wait(cbar, (cphase - 1) & 1);
+    if (tid == 0 && a.err != nullptr) atomicExch(a.err, 1);
   }
 }
 
@@ -1472,7 +1502,6 @@ struct InvForm {
 namespace {
 
 constexpr int INV_SMEM = 225 * 1024;   // shared memory of one solve CTA
-constexpr int FX_SMEM = 221 * 1024;    // the same beside the digit solve's static arrays
 
 template <typename T>
 const void* solve_kernel_ptr(int rs, bool back) {
@@ -1485,6 +1514,10 @@ const void* solve_kernel(const msgfem* h, const InvForm& f, const InvForm::Solve
   const int rs = f.rs;
   return h->mixed ? solve_kernel_ptr<float>(rs, back) : solve_kernel_ptr<double>(rs, back);
 }
+
+int solve_threads(const InvForm& f) { return f.digits ? 32 * FX_WARPS : 256; }
+// fewest ring levels of a solve
+int ring_min(const InvForm& f) { return f.digits ? 1 : 2; }
 
 // shared-memory layout of a solve over the listed matrices with G CTAs per
 // cluster and `ring` stages; the total in bytes
@@ -1499,7 +1532,7 @@ int solve_layout(const msgfem* h, const InvForm& f, InvForm::Solve& s, int G, in
     const InvMat& m = f.mats[i];
     const int nn = m.n / 3, npc = up4((nn + G - 1) / G);
     if (f.digits) {
-      o = std::max(o, (size_t)npc * 3 * KB * es);
+      o = std::max(o, FX_RED + (size_t)std::max(npc * 3, ((m.n + 15) / 16 + G - 1) / G * 16) * KB * es);
       z = std::max(z, (size_t)((m.n + 15) / 16) * DIG * 8 * KB * 4);
       st = FX_STAGE;
     } else if (s.rows32) {
@@ -1525,10 +1558,10 @@ int solve_layout(const msgfem* h, const InvForm& f, InvForm::Solve& s, int G, in
   return s.smem;
 }
 
-int resident_clusters(const void* kernel, int G, int smem) {
+int resident_clusters(const void* kernel, int G, int smem, int threads) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(G);
-  cfg.blockDim = dim3(256);
+  cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1549,7 +1582,7 @@ int resident_clusters(const void* kernel, int G, int smem) {
 // half chain is resident at once (they run side by side), with the deepest ring
 // that one CTA per SM holds, or half an SM's shared memory when that makes more
 // half chains resident; with more half chains than SMs one CTA each.
-// FP32 layers up to F32_WIDE: the fewest rounds of resident half chains, then the widest
+// FP32 layers up to F32_WIDE and digit solves: the fewest rounds of resident half chains, then the widest
 // cluster.  All solves of a local stage, ms, by CTAs per half chain: 32 half chains of 912
 // DoFs 8: 124, 4: 144; 64 of 570 (4 resident at once, 8 in two rounds) 8: 204, 4: 170;
 // 192 of 225 DoFs 8: 66, 4: 38, 2: 31, 1: 34; 20 of 408 8: 20, 4: 20, 2: 27.  The ring's
@@ -1562,15 +1595,15 @@ void choose_solve(const msgfem* h, const InvForm& f, InvForm::Solve& s) {
   for (int i : s.list) most = std::max(most, (f.mats[i].n + strip - 1) / strip / (f.digits || s.rows32 ? 1 : 2));
   auto fit = [&](int G, int limit) {
     int ring = 8;
-    while (ring > 2 && solve_layout(h, f, s, G, ring) > limit) --ring;
+    while (ring > ring_min(f) && solve_layout(h, f, s, G, ring) > limit) --ring;
     return solve_layout(h, f, s, G, ring) <= limit;
   };
-  if (s.rows32) {
+  if (s.rows32 || f.digits) {
     int best = 0, rounds = 0, ring = 0;
     for (int G : {8, 4, 2, 1})
       for (int limit : {INV_SMEM, 108 * 1024}) {
         if (G > most || !fit(G, limit)) continue;
-        const int res = std::max(1, resident_clusters(solve_kernel(h, f, s, true), G, s.smem));
+        const int res = std::max(1, resident_clusters(solve_kernel(h, f, s, true), G, s.smem, solve_threads(f)));
         const int n = (chains + res - 1) / res;
         if (best == 0 || n < rounds) {
           best = G;
@@ -1583,14 +1616,14 @@ void choose_solve(const msgfem* h, const InvForm& f, InvForm::Solve& s) {
   }
   for (int G : {8, 4, 2, 1}) {
     if (G > 1 && G > most) continue;
-    for (int limit : {f.digits ? FX_SMEM : INV_SMEM, 108 * 1024}) {
+    for (int limit : {INV_SMEM, 108 * 1024}) {
       if (!fit(G, limit)) continue;
-      if (resident_clusters(solve_kernel(h, f, s, true), G, s.smem) >= chains) return;
+      if (resident_clusters(solve_kernel(h, f, s, true), G, s.smem, solve_threads(f)) >= chains) return;
     }
   }
   if (fit(1, 108 * 1024)) return;
   for (int G : {1, 2, 4, 8})
-    if (fit(G, f.digits ? FX_SMEM : INV_SMEM)) return;
+    if (fit(G, INV_SMEM)) return;
 }
 
 }  // namespace
@@ -1661,7 +1694,7 @@ bool inv_create(msgfem* h) {
     if (f->mats[i].n > 0) probe.list.push_back(i);
   if (good && !h->mixed && !probe.list.empty()) {
     f->digits = true;
-    f->digits = solve_layout(h, *f, probe, 8, 2) <= FX_SMEM && (size_t)16 * (bmax + 2) * 8 <= (size_t)INV_SMEM;
+    f->digits = solve_layout(h, *f, probe, 8, 1) <= INV_SMEM && (size_t)16 * (bmax + 2) * 8 <= (size_t)INV_SMEM;
   }
   good = good && (f->digits || solve_layout(h, *f, probe, 8, 2) <= INV_SMEM);
   if (!good) {
@@ -1692,7 +1725,7 @@ msgfem_status inv_build(msgfem* h) {
     for (const void* k : {(const void*)k_inv_solve_f32<false>, (const void*)k_inv_solve_f32<true>})
       CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
     for (const void* k : {(const void*)k_inv_solve_fx<false>, (const void*)k_inv_solve_fx<true>})
-      CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, FX_SMEM));
+      CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
     CK(cudaFuncSetAttribute(k_inv_digits, cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
     attr = true;
   }
@@ -1875,7 +1908,7 @@ void inv_solve(msgfem* h, int mat, int src, int dst, int neg, int width, int add
     void* args[] = {&a};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (int)s.list.size() * s.G);
-    cfg.blockDim = dim3(256);
+    cfg.blockDim = dim3(solve_threads(f));
     cfg.dynamicSmemBytes = s.smem;
     cfg.stream = h->stream;
     cudaLaunchAttribute at[1];
