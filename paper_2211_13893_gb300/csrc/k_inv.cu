@@ -29,9 +29,9 @@
 // 4 CG steps to 1e-11 where the Cholesky form takes 5 to 6).
 //
 // Measured on one GB300 against the block Cholesky (factorisation / all solves of a
-// local stage, ms): 36 x 12 x 39 beam FP64 345 -> 46 / 424 -> 41; 192 x 12 x 39 beam
+// local stage, ms): 36 x 12 x 39 beam FP64 345 -> 41 / 424 -> 41; 192 x 12 x 39 beam
 // mixed 102 -> 72 / 374 -> 170; C-section of 16 subdomains mixed 85 -> 45 / 409 -> 124;
-// 47 x 7 x 13 beam FP64 whole pass 156 -> 34.
+// 47 x 7 x 13 beam FP64 whole pass 156 -> 33.
 #include "internal.h"
 
 #include <cooperative_groups.h>
@@ -310,31 +310,94 @@ __device__ __forceinline__ void digit_tile(const double* A, int lda, const doubl
   }
 }
 
-// Inverse of a 64 x 64 SPD tile by the scalar sweep operator in FP64 registers:
-// a 16 x 16 thread grid, each thread the entries (ty + 16 p, tx + 16 q) with
-// p >= q (the tile is symmetric), one barrier per pivot (the pivot column and
-// the pivot's reciprocal are published in a double buffer).  It runs in the same
-// launch as the updates of the other tiles (the next pivot tile is swept by the
-// CTA that updated it), so only narrow steps wait for it.
-template <typename T>
-__device__ void tile_sweep(const T* X, int ldx, T* P, int* notspd, int sub) {
-  __shared__ double v[2][TILE];
-  __shared__ double rinv[2];
+// Product of two 32 x 32 matrices in shared memory, A B^T, in digits: A(r, k) = A[r ar +
+// k ac], B likewise; f(r, c, v) receives every entry once.  A warp forms 16 rows x 8
+// columns and cuts its operands' digits itself (row maxima over its quads of lanes).
+template <typename F>
+__device__ __forceinline__ void digit_32(const double* A, int ar, int ac, const double* B, int br, int bc, F f) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  const double* a0 = A + ((w & 1) * 16 + g) * ar;
+  const double* a1 = a0 + 8 * ar;
+  const double* b0 = B + ((w >> 1) * 8 + g) * br;
+  auto col = [&](int q) { return (q >> 2) * 16 + 2 * t + (q & 1) + 8 * ((q >> 1) & 1); };
+  int e0 = 0, e1 = 0, eb = 0;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    e0 = max(e0, (__double2hiint(a0[col(q) * ac]) >> 20) & 0x7ff);
+    e1 = max(e1, (__double2hiint(a1[col(q) * ac]) >> 20) & 0x7ff);
+    eb = max(eb, (__double2hiint(b0[col(q) * bc]) >> 20) & 0x7ff);
+  }
+#pragma unroll
+  for (int o = 1; o < 4; o <<= 1) {
+    e0 = max(e0, __shfl_xor_sync(0xffffffffu, e0, o));
+    e1 = max(e1, __shfl_xor_sync(0xffffffffu, e1, o));
+    eb = max(eb, __shfl_xor_sync(0xffffffffu, eb, o));
+  }
+  float acc[DIG][4];
+#pragma unroll
+  for (int i = 0; i < DIG; ++i)
+#pragma unroll
+    for (int e = 0; e < 4; ++e) acc[i][e] = 0.f;
+#pragma unroll 1
+  for (int kk = 0; kk < 2; ++kk) {
+    long long xa[2][4], xb[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int c = col(4 * kk + q);
+      xa[0][q] = biased_fixed(a0[c * ac], e0);
+      xa[1][q] = biased_fixed(a1[c * ac], e1);
+      xb[q] = biased_fixed(b0[c * bc], eb);
+    }
+    uint32_t bz[DIG][2];
+#pragma unroll
+    for (int i = 0; i < DIG; ++i) {
+      bz[i][0] = digit_pair(xb[0], xb[1], i);
+      bz[i][1] = digit_pair(xb[2], xb[3], i);
+    }
+#pragma unroll
+    for (int i = 0; i < DIG; ++i) {
+      const uint32_t av[4] = {digit_pair(xa[0][0], xa[0][1], i), digit_pair(xa[1][0], xa[1][1], i),
+                              digit_pair(xa[0][2], xa[0][3], i), digit_pair(xa[1][2], xa[1][3], i)};
+#pragma unroll
+      for (int j = DIG - 1 - i; j < DIG; ++j) mma_f16(acc[i + j - (DIG - 1)], av, bz[j]);
+    }
+  }
+  const int ec[2] = {__shfl_sync(0xffffffffu, eb, 8 * t), __shfl_sync(0xffffffffu, eb, 8 * t + 4)};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    long long hi = 0, lo = 0;
+    digit_flush(acc, e, hi, lo);
+    const int er = e < 2 ? e0 : e1;
+    double v = tile_digit_value(hi, lo, er + ec[e & 1] - 2 * 1023 - 66);
+    if (er == 0x7ff || ec[e & 1] == 0x7ff) v = __longlong_as_double(0x7ff8000000000000ll);   // Inf or NaN operands
+    f((w & 1) * 16 + g + 8 * (e >> 1), (w >> 1) * 8 + 2 * t + (e & 1), v);
+  }
+}
+
+constexpr int LDH = 33;   // row stride of the 32 x 32 matrices of tile_sweep
+
+// Inverse of a 32 x 32 SPD matrix in shared memory, in place, by the scalar sweep operator
+// in FP64 registers: a 16 x 16 thread grid, each thread the entries (ty + 16 p, tx + 16 q)
+// with p >= q.  Per pivot the column and the pivot's reciprocal are published, one warp
+// scales the column (every thread scaling its own two values took as long as the update:
+// a warp's FP64 instruction occupies the SM's pipe for 20 clocks), and all update.  True
+// in the threads that met a non-positive pivot.
+__device__ __forceinline__ bool sweep_32(double* M, double (*v)[32], double* rinv, double* ws) {
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  double a[4][4];
+  double a[2][2];
 #pragma unroll
-  for (int p = 0; p < 4; ++p)
+  for (int p = 0; p < 2; ++p)
 #pragma unroll
-    for (int q = 0; q <= p; ++q) a[p][q] = (double)X[(ty + 16 * p) * ldx + tx + 16 * q];
+    for (int q = 0; q <= p; ++q) a[p][q] = M[(ty + 16 * p) * LDH + tx + 16 * q];
   bool bad = false;
 #pragma unroll
-  for (int kb = 0; kb < 4; ++kb) {
+  for (int kb = 0; kb < 2; ++kb) {
 #pragma unroll 1
     for (int kr = 0; kr < 16; ++kr) {
       double* vs = v[kr & 1];
       if (tx == kr) {
 #pragma unroll
-        for (int p = kb; p < 4; ++p) vs[ty + 16 * p] = a[p][kb];
+        for (int p = kb; p < 2; ++p) vs[ty + 16 * p] = a[p][kb];
         if (ty == kr) {
           double d = a[kb][kb];
           if (!(d > 0.0)) { bad = true; d = 1e-300; }
@@ -347,35 +410,102 @@ __device__ void tile_sweep(const T* X, int ldx, T* P, int* notspd, int sub) {
       }
       __syncthreads();
       const double r = rinv[kr & 1];
-      double vj[4], wi[4];
+      if (tid < 32) ws[tid] = vs[tid] * r;
+      __syncthreads();
+      double vj[2], wi[2];
 #pragma unroll
-      for (int p = 0; p < 4; ++p) {
+      for (int p = 0; p < 2; ++p) {
         vj[p] = vs[tx + 16 * p];
-        wi[p] = vs[ty + 16 * p] * r;
+        wi[p] = ws[ty + 16 * p];
       }
 #pragma unroll
-      for (int p = 0; p < 4; ++p)
+      for (int p = 0; p < 2; ++p)
 #pragma unroll
         for (int q = 0; q <= p; ++q) a[p][q] = fma(-wi[p], vj[q], a[p][q]);
       if (tx == kr) {
 #pragma unroll
-        for (int p = kb; p < 4; ++p) a[p][kb] = wi[p];
+        for (int p = kb; p < 2; ++p) a[p][kb] = wi[p];
       }
       if (ty == kr) {
 #pragma unroll
-        for (int q = 0; q <= kb; ++q) a[kb][q] = vj[q] * r;
+        for (int q = 0; q <= kb; ++q) a[kb][q] = ws[tx + 16 * q];
         if (tx == kr) a[kb][kb] = -r;
       }
     }
   }
 #pragma unroll
-  for (int p = 0; p < 4; ++p)
+  for (int p = 0; p < 2; ++p)
 #pragma unroll
     for (int q = 0; q <= p; ++q) {
-      const T w = (T)(-a[p][q]);
-      P[(ty + 16 * p) * TILE + tx + 16 * q] = w;
-      if (q < p) P[(tx + 16 * q) * TILE + ty + 16 * p] = w;
+      M[(ty + 16 * p) * LDH + tx + 16 * q] = -a[p][q];
+      if (q < p) M[(tx + 16 * q) * LDH + ty + 16 * p] = -a[p][q];
     }
+  __syncthreads();
+  return bad;
+}
+
+// Inverse of a 64 x 64 SPD tile X (its lower half), FP64 for either type, by blocks of 32:
+//   W = A21 A11^{-1}, S = A22 - W A21^T, V = S^{-1} W,
+//   X^{-1} = [A11^{-1} + W^T V, -V^T; -V, S^{-1}],
+// the two inverses by scalar sweeps, the products in digits.  A chain of these inverses is
+// the critical path of a factorisation (the CTA that updates the next pivot tile inverts
+// it).  One SM's FP64 pipe (1.6 FMAs per clock) bounded 64 scalar pivots at 53 us; here
+// about 31.  Whole passes: 24 x 4 x 12 beam 14.5 -> 13.7 ms, 47 x 7 x 13 beam 34.2 -> 32.7
+// (mixed 46.3 -> 44.9), 36 x 12 x 39 beam 127.6 -> 121.7, C-section 328 -> 322.
+// sm: 4 x 32 x 33 doubles; X may lie in it.
+template <typename T>
+__device__ void tile_sweep(const T* X, int ldx, T* P, unsigned char* sm, int* notspd, int sub) {
+  __shared__ double v[2][32], ws[32];
+  __shared__ double rinv[2];
+  double* M11 = reinterpret_cast<double*>(sm);
+  double* M21 = M11 + 32 * LDH;
+  double* M22 = M21 + 32 * LDH;
+  double* W = M22 + 32 * LDH;
+  const int tid = threadIdx.x;
+  {
+    T x[12];   // rows of the lower half, 32 x 32 blocks 11, 21, 22
+#pragma unroll
+    for (int i = 0; i < 12; ++i) {
+      const int e = (i & 3) * 256 + tid, r = e >> 5, c = e & 31, blk = i >> 2;
+      const int rr = max(r, c), cc = min(r, c);   // diagonal blocks: from the lower half
+      x[i] = blk == 1 ? X[(size_t)(32 + r) * ldx + c] : X[(size_t)(blk * 16 + rr) * ldx + blk * 16 + cc];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 12; ++i) {
+      const int e = (i & 3) * 256 + tid;
+      M11[(i >> 2) * 32 * LDH + (e >> 5) * LDH + (e & 31)] = (double)x[i];
+    }
+    __syncthreads();
+  }
+  bool bad = sweep_32(M11, v, rinv, ws);
+  digit_32(M21, LDH, 1, M11, LDH, 1, [&](int r, int c, double y) { W[r * LDH + c] = y; });
+  __syncthreads();
+  digit_32(W, LDH, 1, M21, LDH, 1, [&](int r, int c, double y) {
+    if (c > r) return;
+    M22[r * LDH + c] -= y;
+    if (c < r) M22[c * LDH + r] = M22[r * LDH + c];
+  });
+  __syncthreads();
+  bad |= sweep_32(M22, v, rinv, ws);
+  double* V = M21;
+  digit_32(M22, LDH, 1, W, 1, LDH, [&](int r, int c, double y) {
+    V[r * LDH + c] = y;
+    P[(32 + r) * TILE + c] = (T)-y;
+  });
+  __syncthreads();
+  digit_32(W, 1, LDH, V, 1, LDH, [&](int r, int c, double y) {
+    if (c > r) return;
+    const T p = (T)(M11[r * LDH + c] + y);
+    P[r * TILE + c] = p;
+    if (c < r) P[c * TILE + r] = p;
+  });
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int e = i * 256 + tid, r = e >> 5, c = e & 31;
+    P[(32 + r) * TILE + 32 + c] = (T)M22[r * LDH + c];
+    P[r * TILE + 32 + c] = (T)-V[c * LDH + r];
+  }
   if (bad) atomicExch(&notspd[sub], 1);
 }
 
@@ -468,7 +598,7 @@ k_inv_step(const InvTask* __restrict__ tasks, const InvMat* __restrict__ mats, c
     return;
   }
   if (t.type == IV_PIVOT) {
-    tile_sweep<T>(S, b, pivot_inv<T>(m, t.layer), notspd, m.sub);
+    tile_sweep<T>(S, b, pivot_inv<T>(m, t.layer), smem_iv, notspd, m.sub);
     return;
   }
   const int k = t.k;
@@ -512,7 +642,7 @@ k_inv_step(const InvTask* __restrict__ tasks, const InvMat* __restrict__ mats, c
     });
     if (diag && t.i == k + 1) {
       __syncthreads();   // the tile's stores are visible to the CTA
-      tile_sweep<T>(Sij, b, P, notspd, m.sub);
+      tile_sweep<T>(Sij, b, P, smem_iv, notspd, m.sub);
     }
   } else {
     float* As = reinterpret_cast<float*>(smem_iv);
@@ -550,7 +680,7 @@ k_inv_step(const InvTask* __restrict__ tasks, const InvMat* __restrict__ mats, c
       out[(size_t)r * b + c] = As[r * LDF + c];
       if (panel || !diag) mir[(size_t)r * b + c] = As[c * LDF + r];
     }
-    if (!panel && diag && t.i == k + 1) tile_sweep<T>(As, LDF, P, notspd, m.sub);
+    if (!panel && diag && t.i == k + 1) tile_sweep<T>(As, LDF, P, smem_iv, notspd, m.sub);
   }
 }
 
@@ -1713,22 +1843,19 @@ void inv_destroy(msgfem* h) {
 // Task lists of every wave (after the waves' storage has been placed).
 msgfem_status inv_build(msgfem* h) {
   InvForm& f = *h->inv;
-  static bool attr = false;
-  if (!attr) {
-    for (int rs : {4, 8})
-      for (bool back : {false, true}) {
-        CK(cudaFuncSetAttribute(solve_kernel_ptr<float>(rs, back), cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
-        CK(cudaFuncSetAttribute(solve_kernel_ptr<double>(rs, back), cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
-      }
-    CK(cudaFuncSetAttribute(k_inv_step<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, inv_step_smem<double>()));
-    CK(cudaFuncSetAttribute(k_inv_step<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, inv_step_smem<float>()));
-    for (const void* k : {(const void*)k_inv_solve_f32<false>, (const void*)k_inv_solve_f32<true>})
-      CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
-    for (const void* k : {(const void*)k_inv_solve_fx<false>, (const void*)k_inv_solve_fx<true>})
-      CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
-    CK(cudaFuncSetAttribute(k_inv_digits, cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
-    attr = true;
-  }
+  // shared-memory limits (of the current device)
+  for (int rs : {4, 8})
+    for (bool back : {false, true}) {
+      CK(cudaFuncSetAttribute(solve_kernel_ptr<float>(rs, back), cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
+      CK(cudaFuncSetAttribute(solve_kernel_ptr<double>(rs, back), cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
+    }
+  CK(cudaFuncSetAttribute(k_inv_step<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, inv_step_smem<double>()));
+  CK(cudaFuncSetAttribute(k_inv_step<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, inv_step_smem<float>()));
+  for (const void* k : {(const void*)k_inv_solve_f32<false>, (const void*)k_inv_solve_f32<true>})
+    CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
+  for (const void* k : {(const void*)k_inv_solve_fx<false>, (const void*)k_inv_solve_fx<true>})
+    CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
+  CK(cudaFuncSetAttribute(k_inv_digits, cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
   void* p = nullptr;
   TRY(dev_alloc_bytes(h, &p, f.mats.size() * sizeof(InvMat)));
   f.d_mats = static_cast<InvMat*>(p);
