@@ -51,6 +51,8 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12   # SMs x DFMA/clk x 2 flop x max SM clock (derived, 1.26)
+# FP64 products in exact FP16 digit products: 28 mma.sync FMAs each, 956 per clock and SM (measured)
+DIGIT_PEAK_TFLOPS = 152 * 956 / 28 * 2 * 2.070e9 / 1e12   # 21.5
 
 
 def _hbm_peak():
@@ -106,8 +108,16 @@ def job_rate(world, units_per_rank, steps, total_ms):
     return world * units_per_rank * steps / (total_ms / 1000.0)
 
 
-def _solve_kernel_name(tuning):
-    """Kernel of the FP32 8-column block solves for the autotuner's choice (default: the cp.async ring)."""
+def _inverse_form(prof):
+    """Whether the handle keeps inverses of the Schur complements (then the two counts are the same)."""
+    return prof["factor_flops_inverse"] == prof["factor_flops"]
+
+
+def _solve_kernel_name(tuning, prof):
+    """Kernel of the FP32 8-column block solves: the inverse form's, or the autotuner's choice
+    among the block Cholesky's (default: the cp.async ring)."""
+    if _inverse_form(prof):
+        return "k_inv_solve_f32 (FP32 block solves, 8 right-hand sides, inverse Schur complements)"
     k = (tuning or {}).get("solve_kernel", 1)
     return {1: "k_solve_async (FP32 block solves, 8 right-hand sides, cp.async ring)",
             2: "k_solve_stream<float, 1> (FP32 block solves, 8 right-hand sides, register streaming)",
@@ -333,17 +343,28 @@ def run_ours(args):
     fact_inv_tf = fact_tf * prof["factor_flops_inverse"] / prof["factor_flops"] if prof["factor_flops"] else 0.0
     fact_x_tf = fact_tf * prof["factor_flops_executed"] / prof["factor_flops"] if prof["factor_flops"] else 0.0
     solve_tf = prof["solve_flops"] * args.steps / (prof["solve_ms"] / 1000.0) / 1e12 if prof["solve_ms"] else 0.0
-    if prof["solve_ms"] >= prof["factor_ms"]:
+    inverse = _inverse_form(prof)
+    peak = DIGIT_PEAK_TFLOPS if inverse else FP64_PEAK_TFLOPS
+    if inverse and prof["solve_ms"] >= prof["factor_ms"]:
+        dom, achieved, share = "k_inv_solve_fx (block solves in digit products)", solve_tf, prof["solve_ms"] / total_ms
+    elif inverse:
+        dom, achieved, share = "k_inv_step<double> (sweeps of the Schur complements)", fact_tf, prof["factor_ms"] / total_ms
+    elif prof["solve_ms"] >= prof["factor_ms"]:
         dom, achieved, share = "k_solve_stream<double> (block triangular solves)", solve_tf, prof["solve_ms"] / total_ms
     else:
         dom, achieved, share = "k_tile_task<double> (layer-block Cholesky tile tasks)", fact_tf, prof["factor_ms"] / total_ms
-    roof = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-            "frac": achieved / FP64_PEAK_TFLOPS, "traffic": NCU_TRAFFIC.get(args.config), "kernel": dom,
+    roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
+            "frac": achieved / peak, "traffic": None if inverse else NCU_TRAFFIC.get(args.config), "kernel": dom,
             "traffic_note": "bytes per factorisation graph replay (one per step), from an ncu capture on p2 scaled "
                             "to the workload's subdomains",
-            "peak_note": "FP64 DFMA: 152 SMs x 2 DFMA/clk x 2 flop x 2070 MHz (derived); measured by the FMA probe "
+            "peak_note": "FP64 as 28 exact FP16 digit products: 152 SMs x 956 / 28 FMA/clk (measured mma.sync rate) x 2 "
+                         "flop x 2070 MHz" if inverse else
+                         "FP64 DFMA: 152 SMs x 2 DFMA/clk x 2 flop x 2070 MHz (derived); measured by the FMA probe "
                          "in this run: see probe",
-            "achieved_note": "algorithmic flops of the block-tridiagonal Cholesky of K and A11 (per matrix sum_l "
+            "achieved_note": "algorithmic flops of the inverse form (per matrix sum_l n^3 + 108 n^2; a solve "
+                             "2 (2 nL - 1) n^2 per column) over the phase's CUDA-event time on the launching stream"
+                             if inverse else
+                             "algorithmic flops of the block-tridiagonal Cholesky of K and A11 (per matrix sum_l "
                              "n^3/3 + (nL-1) 2 n^3, unpadded layer sizes) over the factorisation phase's CUDA-event "
                              "time on the launching stream",
             "probe": probe,
@@ -511,7 +532,7 @@ def run_c4(args, dev, stream, flush, rank, world):
            "unconverged_subdomains": [j for j, i in enumerate(infos) if i["residual"] > 1e-5],
            "roofline": {"bound": "hbm", "achieved": solve_gbs, "peak": hbm, "unit": "GB/s",
                         "frac": solve_gbs / hbm, "peak_note": hbm_note,
-                        "kernel": _solve_kernel_name(tuning),
+                        "kernel": _solve_kernel_name(tuning, prof),
                         "time_share": prof["solve_ms"] / total if total else None},
            "sampled_parity": sample, "autotune": tuning}
     m.close()
@@ -578,7 +599,7 @@ def run_mixed(args, cfg, ang_dev, stream, dev, rank, lam_fp64, u_fp64, flush, wo
            "ortho_ms_per_step": prof["ortho_ms"] / args.steps, "autotune": tuning,
            "roofline": {"bound": "hbm", "achieved": solve_gbs, "peak": hbm, "unit": "GB/s",
                         "frac": solve_gbs / hbm, "peak_note": hbm_note,
-                        "kernel": _solve_kernel_name(tuning),
+                        "kernel": _solve_kernel_name(tuning, prof),
                         "time_share": prof["solve_ms"] / total if total else None,
                         "calls_per_step": prof["solve_calls"]},
            "warm": warm}

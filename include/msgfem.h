@@ -245,7 +245,9 @@ typedef struct {
                            topological order and waits, bounded by two seconds, on the
                            completion counter of the previous step of the task's chain)
                            instead of the graph-captured step schedule; the factors are the
-                           same bit for bit.  0 = the step schedule.  msgfem_autotune sets it */
+                           same bit for bit.  0 = the step schedule.  msgfem_autotune sets it.
+                           Of the block Cholesky: no effect on a handle that keeps inverses of
+                           the Schur complements (see msgfem_profile) */
 } msgfem_options;
 
 enum { MSGFEM_METHOD_MSGFEM = 0, MSGFEM_METHOD_GENEO = 1 };
@@ -264,8 +266,8 @@ enum { MSGFEM_METHOD_MSGFEM = 0, MSGFEM_METHOD_GENEO = 1 };
  * wide for its solve kernel, use the block Cholesky. */
 typedef struct {
   double assemble_ms;   /* element stiffness, stencils, layer blocks */
-  double factor_ms;     /* layer-block Cholesky + inverses of K and A11 */
-  double solve_ms;      /* all block triangular solves of the iteration */
+  double factor_ms;     /* factorisations of K and A11 */
+  double solve_ms;      /* all block solves of the iteration */
   double iterate_ms;    /* the whole eigen-iteration including solves */
   double coarse_ms;     /* coarse_assemble + solve */
   double factor_flops;  /* per local stage */
@@ -284,7 +286,8 @@ typedef struct {
   int waves;            /* waves of subdomains per local stage (msgfem_options.wave_mb) */
   double pool_mb;       /* size of the shared layer-block / factor / solve-buffer pool (MiB) */
   double factor_flops_inverse;   /* factor_flops plus the n^3/3 per layer of the explicit
-                                    inverses of the diagonal factors that the solves use */
+                                    inverses of the diagonal factors that the solves use
+                                    (the inverse form: factor_flops) */
   double factor_flops_executed;  /* flops the factorisation's 64 x 64 tile tasks execute
                                     (padding, whole diagonal tiles and inverses included) */
 } msgfem_profile;
@@ -510,7 +513,10 @@ msgfem_status msgfem_solution_errors(msgfem_h h, const double* u_ref, double* er
  * N-product stencil, the 8-column K solve with, in mixed precision, its PCG
  * refinement, and the A-harmonic extension by A11 solves), after one untimed
  * application, then regroups the solve schedules of every wave and sets the
- * kernel to the fastest combination; later calls use it.  The working blocks
+ * kernel to the fastest combination; later calls use it.  A handle that keeps
+ * inverses of the Schur complements times the block Cholesky's candidates like
+ * that, then its own factorisation and operator, and goes back to them when they
+ * are faster.  The working blocks
  * the timing reads and writes are scratch of the eigensolver; results of the
  * previous local stage, the phase timers and the launch count are kept.
  * tuning (may be NULL) receives the choice and the measured times.  Errors:

@@ -30,7 +30,7 @@
 //
 // Measured on one GB300 against the block Cholesky (factorisation / all solves of a
 // local stage, ms): 36 x 12 x 39 beam FP64 345 -> 41 / 424 -> 41; 192 x 12 x 39 beam
-// mixed 102 -> 72 / 374 -> 170; C-section of 16 subdomains mixed 85 -> 45 / 409 -> 124;
+// mixed 102 -> 72 / 374 -> 163; C-section of 16 subdomains mixed 85 -> 42 / 409 -> 124;
 // 47 x 7 x 13 beam FP64 whole pass 156 -> 33.
 #include "internal.h"
 
@@ -973,11 +973,13 @@ k_inv_solve(const InvSolveArgs a) {
 //     mbarriers and waits for nobody until the layer's end;
 //   - there the eight warps' sums are added through shared memory, and all threads write
 //     the results (two warps after every stage before).
-// All solves of a local stage, k_inv_solve -> here: C-section of 16 subdomains (layers of
-// 714 and 912 DoFs) 188 -> 124 ms, 192 x 12 x 39 beam (570 and 693) 204 -> 170 ms (84 % of
-// the HBM copy rate), 48 beams (210 and 225) 42 -> 31 ms, 47 x 7 x 13 beam (360 and 408, 20
-// half chains: barriers) 20 -> 20 ms.  Bound by HBM with many half chains, by the cluster's
-// barriers with few.
+// All solves of a local stage, k_inv_solve -> here: C-section of 16 subdomains (layers up
+// to 714 and 912 DoFs) 188 -> 124 ms, 192 x 12 x 39 beam (570 and 693) 204 -> 163 ms
+// (3.0 TB/s, 44 % of the HBM copy rate), 48 beams (210 and 225) 42 -> 25 ms, 47 x 7 x 13
+// beam (360 and 408, 20 half chains) 20 -> 17 ms.  Bound by the steps' latency: of a step of
+// 21 us on 912 DoFs the products take about 8 in issue slots (two CTAs per SM), the sparse
+// step, two cluster barriers and the wait for the slowest rank the rest (issue slots 36 %
+// busy, DRAM 32 %, barriers the largest stall).
 constexpr int F32_BLOCKS = 8;    // blocks of 32 rows per rank
 constexpr int F32_WIDE = 1024;   // widest layer
 
