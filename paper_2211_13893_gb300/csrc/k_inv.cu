@@ -30,7 +30,7 @@
 //
 // Measured on one GB300 against the block Cholesky (factorisation / all solves of a
 // local stage, ms): 36 x 12 x 39 beam FP64 345 -> 41 / 424 -> 41; 192 x 12 x 39 beam
-// mixed 102 -> 72 / 374 -> 163; C-section of 16 subdomains mixed 85 -> 42 / 409 -> 124;
+// mixed 102 -> 72 / 374 -> 154; C-section of 16 subdomains mixed 85 -> 42 / 409 -> 124;
 // 47 x 7 x 13 beam FP64 whole pass 156 -> 33.
 #include "internal.h"
 
@@ -974,8 +974,8 @@ k_inv_solve(const InvSolveArgs a) {
 //   - there the eight warps' sums are added through shared memory, and all threads write
 //     the results (two warps after every stage before).
 // All solves of a local stage, k_inv_solve -> here: C-section of 16 subdomains (layers up
-// to 714 and 912 DoFs) 188 -> 124 ms, 192 x 12 x 39 beam (570 and 693) 204 -> 163 ms
-// (3.0 TB/s, 44 % of the HBM copy rate), 48 beams (210 and 225) 42 -> 25 ms, 47 x 7 x 13
+// to 714 and 912 DoFs) 188 -> 124 ms, 192 x 12 x 39 beam (570 and 693) 204 -> 154 ms
+// (3.1 TB/s, 46 % of the HBM copy rate), 48 beams (210 and 225) 42 -> 23 ms, 47 x 7 x 13
 // beam (360 and 408, 20 half chains) 20 -> 17 ms.  Bound by the steps' latency: of a step of
 // 21 us on 912 DoFs the products take about 8 in issue slots (two CTAs per SM), the sparse
 // step, two cluster barriers and the wait for the slowest rank the rest (issue slots 36 %
@@ -1649,7 +1649,7 @@ const void* solve_kernel(const msgfem* h, const InvForm& f, const InvForm::Solve
 
 int solve_threads(const InvForm& f) { return f.digits ? 32 * FX_WARPS : 256; }
 // fewest ring levels of a solve
-int ring_min(const InvForm& f) { return f.digits ? 1 : 2; }
+int ring_min(const InvForm& f, const InvForm::Solve& s) { return f.digits || s.rows32 ? 1 : 2; }
 
 // shared-memory layout of a solve over the listed matrices with G CTAs per
 // cluster and `ring` stages; the total in bytes
@@ -1718,7 +1718,8 @@ int resident_clusters(const void* kernel, int G, int smem, int threads) {
 // cluster.  All solves of a local stage, ms, by CTAs per half chain: 32 half chains of 912
 // DoFs 8: 124, 4: 144; 64 of 570 (4 resident at once, 8 in two rounds) 8: 204, 4: 170;
 // 192 of 225 DoFs 8: 66, 4: 38, 2: 31, 1: 34; 20 of 408 8: 20, 4: 20, 2: 27.  The ring's
-// depth (2 to 8) changes none of them by more than 3 %.
+// depth (2 to 8) changes none of them by more than 3 %, so one level is enough where it
+// saves a round: 64 half chains of 693 and 570 DoFs 163 -> 154, 192 of 225 24.6 -> 23.5.
 void choose_solve(const msgfem* h, const InvForm& f, InvForm::Solve& s) {
   const int chains = 2 * (int)s.list.size();
   int most = 1;
@@ -1727,7 +1728,7 @@ void choose_solve(const msgfem* h, const InvForm& f, InvForm::Solve& s) {
   for (int i : s.list) most = std::max(most, (f.mats[i].n + strip - 1) / strip / (f.digits || s.rows32 ? 1 : 2));
   auto fit = [&](int G, int limit) {
     int ring = 8;
-    while (ring > ring_min(f) && solve_layout(h, f, s, G, ring) > limit) --ring;
+    while (ring > ring_min(f, s) && solve_layout(h, f, s, G, ring) > limit) --ring;
     return solve_layout(h, f, s, G, ring) <= limit;
   };
   if (s.rows32 || f.digits) {
