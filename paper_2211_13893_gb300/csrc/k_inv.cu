@@ -31,7 +31,7 @@
 // Measured on one GB300 against the block Cholesky (factorisation / all solves of a
 // local stage, ms): 36 x 12 x 39 beam FP64 345 -> 41 / 424 -> 41; 192 x 12 x 39 beam
 // mixed 102 -> 72 / 374 -> 154; C-section of 16 subdomains mixed 85 -> 42 / 409 -> 124;
-// 47 x 7 x 13 beam FP64 whole pass 156 -> 33.
+// 47 x 7 x 13 beam FP64 whole pass 156 -> 31.
 #include "internal.h"
 
 #include <cooperative_groups.h>
@@ -1720,6 +1720,9 @@ int resident_clusters(const void* kernel, int G, int smem, int threads) {
 // 192 of 225 DoFs 8: 66, 4: 38, 2: 31, 1: 34; 20 of 408 8: 20, 4: 20, 2: 27.  The ring's
 // depth (2 to 8) changes none of them by more than 3 %, so one level is enough where it
 // saves a round: 64 half chains of 693 and 570 DoFs 163 -> 154, 192 of 225 24.6 -> 23.5.
+// Sizes that are no powers of two serve what just misses one (FP64, 20 half chains: 6
+// instead of 4, 47 x 7 x 13 beam 32.7 -> 30.6 ms; layers of fewer blocks than 8: Schwarz
+// PCG 15.5 -> 14.4, GenEO comparison 206 -> 202).
 void choose_solve(const msgfem* h, const InvForm& f, InvForm::Solve& s) {
   const int chains = 2 * (int)s.list.size();
   int most = 1;
@@ -1733,7 +1736,7 @@ void choose_solve(const msgfem* h, const InvForm& f, InvForm::Solve& s) {
   };
   if (s.rows32 || f.digits) {
     int best = 0, rounds = 0, ring = 0;
-    for (int G : {8, 4, 2, 1})
+    for (int G = 8; G >= 1; --G)
       for (int limit : {INV_SMEM, 108 * 1024}) {
         if (G > most || !fit(G, limit)) continue;
         const int res = std::max(1, resident_clusters(solve_kernel(h, f, s, true), G, s.smem, solve_threads(f)));

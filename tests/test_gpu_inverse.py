@@ -98,6 +98,28 @@ def test_fp32_solve_row_blocks(ny, instances):
         assert np.linalg.norm(a - b) <= 1e-7 * np.linalg.norm(b)
 
 
+# Clusters that are no powers of two: layers of 3 to 7 blocks (32 rows in FP32, 16 in FP64),
+# and 20 half chains, for which clusters of 8 are not resident at once.
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("ny,instances", [(1, 1), (2, 1), (3, 1), (4, 5)])
+def test_cluster_sizes(ny, instances, precision):
+    from paper_2211_13893_gb300 import MSGFEM
+    cfg = replace(get_config("t3"), name="ranks", NX=24, NY=ny, NZ=4, sx=2, sy=1, overlap=1, oversampling=2, n_loc=6)
+    rng = np.random.default_rng(ny)
+    ang = rng.uniform(-90.0, 90.0, instances * cfg.NX * cfg.NY * cfg.NZ)
+    out = []
+    for kw in (dict(), dict(factor_schedule=1)):
+        m = MSGFEM.from_config(cfg, ang, seed=7, precision=precision, instances=instances, **kw)
+        lam = np.array(m.local_spaces(cfg.n_loc))
+        out.append((lam, [m.export_local(j)[0][:, -1] for j in (0, m.N - 1)]))
+        m.close()
+    (la, pa), (lb, pb) = out
+    scale = np.maximum(np.abs(lb).max(axis=1, keepdims=True), 1.0)
+    assert (np.abs(la - lb) / scale).max() <= (1e-8 if precision == 0 else 1e-5)
+    for a, b in zip(pa, pb):
+        assert np.linalg.norm(a - b) <= (1e-9 if precision == 0 else 1e-7) * np.linalg.norm(b)
+
+
 def test_wide_layers_keep_the_block_cholesky():
     """Layers whose solve stages exceed shared memory run the block Cholesky (same results bar)."""
     from paper_2211_13893_gb300 import MSGFEM
