@@ -263,7 +263,9 @@ enum { MSGFEM_METHOD_MSGFEM = 0, MSGFEM_METHOD_GENEO = 1 };
  * solve 2 (2 nL - 1) n^2 p.  A request for a Cholesky schedule (factor_schedule =
  * 1), tile kernel (factor_kernel = 1), tile precision (tile_chol = 1), solve
  * kernel (solve_kernel > 0) or subspace iteration (solver = 1), and layers too
- * wide for its solve kernel, use the block Cholesky. */
+ * wide for its solve kernel, use the block Cholesky; so does a call that finds the
+ * Schur complements not positive definite or too ill-conditioned for explicit
+ * inverses (the flop counts are then those of the block Cholesky). */
 typedef struct {
   double assemble_ms;   /* element stiffness, stencils, layer blocks */
   double factor_ms;     /* factorisations of K and A11 */

@@ -246,6 +246,34 @@ msgfem_status upload_wave_solves(msgfem* h, WaveSched& w) {
   return MSGFEM_OK;
 }
 
+// Captured factorisation and solve graphs: their task lists are being replaced.
+void drop_graphs(msgfem* h) {
+  for (auto it = h->graphs.begin(); it != h->graphs.end();) {
+    if ((it->first >> 60) == 1 || (it->first >> 60) == 2) {
+      if (it->second.first) cudaGraphExecDestroy(it->second.first);
+      it = h->graphs.erase(it);
+    } else {
+      ++it;
+    }
+  }
+}
+
+// Task lists of the block Cholesky for every wave, unless they are in place: at set-up
+// on a handle without the inverse form, else when a call first needs them.
+msgfem_status chol_lists(msgfem* h) {
+  if (h->chol_ready) return MSGFEM_OK;
+  CK(cudaStreamSynchronize(h->stream));
+  drop_graphs(h);
+  build_factor_schedule(h);
+  build_solve_schedules(h);
+  for (WaveSched& w : h->waves) {
+    TRY(upload_wave_factor(h, w));
+    TRY(upload_wave_solves(h, w));
+  }
+  h->chol_ready = true;
+  return MSGFEM_OK;
+}
+
 msgfem_status allocate(msgfem* h) {
   for (int j = 0; j < h->N; ++j) {
     SubDev& s = h->sub[j];
@@ -326,17 +354,9 @@ msgfem_status allocate(msgfem* h) {
   TRY(dalloc(h, &h->d_energy, 2 * 1024));
   TRY(dalloc(h, &h->d_l2, 4 * 1024));
   // schedules: of the inverse form, or of the block Cholesky
-  h->inv_on = inv_create(h);
-  if (h->inv_on) {
-    TRY(inv_build(h));
-  } else {
-    build_factor_schedule(h);
-    build_solve_schedules(h);
-    for (WaveSched& w : h->waves) {
-      TRY(upload_wave_factor(h, w));
-      TRY(upload_wave_solves(h, w));
-    }
-  }
+  h->inv_use = h->inv_on = inv_create(h);
+  if (h->inv_on) TRY(inv_build(h));
+  else TRY(chol_lists(h));
   if (h->opt.solver == 0) TRY(dev_alloc_bytes(h, &h->d_rr, rr_bytes(h->N)));
   TRY(dalloc(h, &h->d_mk, h->N));
   TRY(dalloc(h, &h->d_nwk, h->N));
@@ -703,11 +723,25 @@ static msgfem_status run_factorisation(msgfem* h, const WaveSched& ws, int w) {
     run_graph(h, ((uint64_t)2 << 60) | ((uint64_t)w << 48) | ((uint64_t)1 << 45), [&](cudaStream_t cs) { inv_factor(h, w, cs); });
     return MSGFEM_OK;
   }
+  TRY(chol_lists(h));
   if (h->mixed && h->factor_persistent) return run_factor_persistent(h, ws, h->stream);
   run_graph(h, factor_graph_key(h, w), [&](cudaStream_t cs) {
     if (h->mixed) run_schedule(ws.factf, cs, &h->gs);
     else run_schedule(ws.fact, cs, &h->gs);
   });
+  return MSGFEM_OK;
+}
+
+// Whether the factors of wave w stay: always, but for factors of the inverse form that are
+// not sound (inv_sound).  Those are dropped, and the rest of the call factorises by the
+// block Cholesky.
+static msgfem_status keep_factors(msgfem* h, int w, bool* keep) {
+  *keep = true;
+  if (!h->inv_on) return MSGFEM_OK;
+  TRY(inv_sound(h, w, keep));
+  if (*keep) return MSGFEM_OK;
+  h->inv_on = false;
+  CK(cudaMemsetAsync(h->d_notspd, 0, (h->N + 1) * sizeof(int), h->stream));
   return MSGFEM_OK;
 }
 
@@ -734,11 +768,15 @@ msgfem_status schwarz_factors(msgfem* h) {
   }
   const WaveSched& ws = h->waves[0];
   std::vector<int> notspd(h->N + 1);
-  for (int attempt = 0; attempt < 2; ++attempt) {
+  h->inv_on = h->inv_use;
+  for (;;) {
     launch_layer_blocks(h);
     TRY(select_factor_kernel(h));
     TRY(run_factorisation(h, ws, 0));
     CK_LAUNCH();
+    bool keep = true;
+    TRY(keep_factors(h, 0, &keep));
+    if (!keep) continue;
     CK(cudaMemcpyAsync(notspd.data(), h->d_notspd, (h->N + 1) * sizeof(int), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     bool any = false;
@@ -1181,6 +1219,15 @@ msgfem_status msgfem_local_spaces_var(msgfem_h h, const int* n_loc, double* lamb
   return ke != MSGFEM_OK ? ke : st;
 }
 
+// Factorisation work of the form in use (the form the call ends with)
+static void count_factor_flops(msgfem* h) {
+  h->prof.factor_flops = factor_flops(h);
+  h->prof.factor_flops_inverse = factor_flops(h, true);
+  h->prof.factor_flops_executed = 0.0;
+  if (h->inv_on) h->prof.factor_flops_executed = inv_factor_flops(h, true);
+  for (const auto& w : h->waves) h->prof.factor_flops_executed += h->mixed ? schedule_flops(w.factf) : schedule_flops(w.fact);
+}
+
 // nl: eigenpairs per subdomain; n_loc below is the largest of them
 static msgfem_status local_spaces_run(msgfem_h h, const std::vector<int>& nl, double* lambda_out) {
   if (!h) return MSGFEM_EINVAL;
@@ -1224,6 +1271,7 @@ static msgfem_status local_spaces_run(msgfem_h h, const std::vector<int>& nl, do
   // being replaced: a failure leaves the handle needing a new local stage
   h->stage = 1;
   h->factored_wave = -1;
+  h->inv_on = h->inv_use;
   h->potrf_fp64 = 0;   // with tile_chol 1 each local stage first tries FP32 tile Cholesky
   h->n_loc = n_loc;
   h->nloc_j = nl;
@@ -1234,11 +1282,7 @@ static msgfem_status local_spaces_run(msgfem_h h, const std::vector<int>& nl, do
   TRY(set_active(h, act));
   CK(cudaMemsetAsync(h->d_notspd, 0, (h->N + 1) * sizeof(int), st));
   for (auto& s : h->sub) CK(cudaMemsetAsync(s.status, 0, 4 * sizeof(int), st));
-  h->prof.factor_flops = factor_flops(h);
-  h->prof.factor_flops_inverse = factor_flops(h, true);
-  h->prof.factor_flops_executed = 0.0;
-  if (h->inv_on) h->prof.factor_flops_executed = inv_factor_flops(h, true);
-  for (const auto& w : h->waves) h->prof.factor_flops_executed += h->mixed ? schedule_flops(w.factf) : schedule_flops(w.fact);
+  count_factor_flops(h);
   h->prof.solve_flops = 0.0;
   h->prof.solve_bytes = 0.0;
   h->prof.stencil_flops = 0.0;
@@ -1271,19 +1315,26 @@ static msgfem_status local_spaces_run(msgfem_h h, const std::vector<int>& nl, do
     h->base_act.assign(h->N, 0);
     for (int j : ws.members) h->base_act[j] = 1;
     TRY(set_active(h, h->base_act));
-    sp = span_begin(h, TAG_ASSEMBLE);
-    launch_layer_blocks(h);
-    span_end(h, sp);
-    CK_LAUNCH();
-    // 2. factorisations of K and A11
-    TRY(select_factor_kernel(h));
-    sp = span_begin(h, TAG_FACTOR);
-    nvtxRangePushA("msgfem_factor");   // lets a kernel profiler select the factorisation (graph or launches)
-    const msgfem_status fst = run_factorisation(h, ws, (int)w);
-    nvtxRangePop();
-    TRY(fst);
-    span_end(h, sp);
-    CK_LAUNCH();
+    for (bool keep = false; !keep;) {
+      sp = span_begin(h, TAG_ASSEMBLE);
+      launch_layer_blocks(h);
+      span_end(h, sp);
+      CK_LAUNCH();
+      // 2. factorisations of K and A11
+      TRY(select_factor_kernel(h));
+      sp = span_begin(h, TAG_FACTOR);
+      nvtxRangePushA("msgfem_factor");   // lets a kernel profiler select the factorisation (graph or launches)
+      const msgfem_status fst = run_factorisation(h, ws, (int)w);
+      nvtxRangePop();
+      TRY(fst);
+      span_end(h, sp);
+      CK_LAUNCH();
+      TRY(keep_factors(h, (int)w, &keep));
+      if (!keep) {
+        TRY(chol_lists(h));
+        count_factor_flops(h);
+      }
+    }
     if (tile_chol_fp32(h)) {
       // a non-positive pivot in an FP32 tile Cholesky: the wave (and the later
       // ones) are factorised again with FP64 tiles before any solve reads them
@@ -2006,8 +2057,9 @@ static msgfem_status autotune_run(msgfem_h h, int reps, msgfem_tuning* out) {
     CK_LAUNCH();
     CK(cudaEventElapsedTime(&fms, f0, f1));
     CK(cudaEventElapsedTime(&oms, e0, e1));
-    h->inv_on = fms + 10.0 * oms / reps <= best_fms + 10.0 * best;
+    h->inv_use = fms + 10.0 * oms / reps <= best_fms + 10.0 * best;
   }
+  h->inv_on = h->inv_use;
   CK(cudaEventDestroy(f0));
   CK(cudaEventDestroy(f1));
   CK(cudaStreamSynchronize(st));
@@ -2032,6 +2084,7 @@ static msgfem_status autotune_run(msgfem_h h, int reps, msgfem_tuning* out) {
     build_wave_solve_schedules(h, w);
     TRY(upload_wave_solves(h, w));
   }
+  h->chol_ready = true;
   h->cur = 0;
   h->base_act.assign(h->N, 1);
   TRY(set_active(h, h->base_act));

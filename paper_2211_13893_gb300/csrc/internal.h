@@ -253,7 +253,9 @@ struct msgfem {
   int* d_kerr = nullptr;             // set by a TMA solve stage that did not arrive in time
   int potrf_fp64 = 0;                // mixed: FP64 tile Cholesky after an FP32 one met a bad pivot
   InvForm* inv = nullptr;            // inverse form, when the handle is eligible
-  bool inv_on = false;               // factorisations and solves run in the inverse form
+  bool inv_use = false;              // factorisations start in the inverse form (eligible, and kept by the autotuner)
+  bool inv_on = false;               // the current factors are in the inverse form
+  bool chol_ready = false;           // the block Cholesky's task lists of every wave are in place
   int factor_persistent = 0;         // mixed: FP32 factorisation as one persistent launch
   int refine_last[2] = {0, 0};       // steps the last adaptive refinement took (K, A11): when to look at its flags
   int refine = 2;                    // FP64 refinement steps per FP32 solve
@@ -379,6 +381,9 @@ bool inv_create(msgfem* h);
 void inv_destroy(msgfem* h);
 msgfem_status inv_build(msgfem* h);
 void inv_factor(msgfem* h, int w, cudaStream_t st);
+// whether the factorisation of wave w met positive pivots only and its Schur complements
+// are conditioned well enough for their inverses (reads back: synchronises)
+msgfem_status inv_sound(msgfem* h, int w, bool* sound);
 void inv_solve(msgfem* h, int mat, int src, int dst, int neg, int width, int add, int ncols);
 double inv_factor_flops(const msgfem* h, bool executed);
 // the coarse matrix in the same form: tasks for the current NcPad, sweep of d_AH in place

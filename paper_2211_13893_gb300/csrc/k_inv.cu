@@ -604,6 +604,13 @@ k_inv_step(const InvTask* __restrict__ tasks, const InvMat* __restrict__ mats, c
   const int k = t.k;
   T* P = pivot_inv<T>(m, t.layer);
   T* C = old_col<T>(m, t.layer);
+  if (t.type == IV_PANEL && k == 0 && m.yc != nullptr) {   // the diagonal before any update (k_inv_condition)
+    if (tid < TILE) {
+      const size_t r = (size_t)t.i * TILE + tid;
+      static_cast<T*>(m.yc)[(size_t)t.layer * b + r] = S[r * b + r];
+    }
+    __syncthreads();
+  }
   if (t.type == IV_PANEL && t.i == k) {
     T* Skk = S + (size_t)k * TILE * b + (size_t)k * TILE;
     for (int e = tid; e < TILE * TILE; e += 256) Skk[(size_t)(e >> 6) * b + (e & 63)] = -P[e];
@@ -682,6 +689,28 @@ k_inv_step(const InvTask* __restrict__ tasks, const InvMat* __restrict__ mats, c
     }
     if (!panel && diag && t.i == k + 1) tile_sweep<T>(As, LDF, P, smem_iv, notspd, m.sub);
   }
+}
+
+// Conditioning of the Schur complements: the largest S_ii (S^{-1})_ii of the matrix's
+// layers into cond[2 sub + mat] (zeroed before; as the bits of a positive float), infinity
+// when a pivot was not positive or the value is no number.  D holds -S^{-1}, yc the
+// diagonals of S.
+template <typename T>
+__global__ void __launch_bounds__(128)
+k_inv_condition(const InvMat* __restrict__ mats, const int* __restrict__ active, const int* __restrict__ notspd,
+                int* __restrict__ cond) {
+  const InvMat& m = mats[blockIdx.x];
+  const int l = blockIdx.y;
+  if (l >= m.nL || (active != nullptr && !active[m.sub])) return;
+  const T* D = layer_block<T>(m, l);
+  const T* d = static_cast<const T*>(m.yc) + (size_t)l * m.b;
+  float g = notspd[m.sub] ? INFINITY : 0.f;
+  for (int r = threadIdx.x; r < m.n; r += 128) {
+    const float v = (float)(-D[(size_t)r * m.b + r] * d[r]);
+    g = v >= 0.f ? fmaxf(g, v) : INFINITY;
+  }
+  for (int o = 16; o > 0; o >>= 1) g = fmaxf(g, __shfl_xor_sync(0xffffffffu, g, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(&cond[2 * m.sub + m.mat], __float_as_int(g));
 }
 
 // Couplings of every layer in the solver's precision, packed per node for the
@@ -1629,11 +1658,27 @@ struct InvForm {
   std::vector<SchedStep> csteps;
   int rs = 8;                      // rows per stage of the solves (by the widest layer and the type)
   bool digits = false;             // FP64: solves in digit products (k_inv_solve_fx)
+  int* d_cond = nullptr;           // [2 N + 2] conditioning of the matrices' Schur complements (float bits)
 };
 
 namespace {
 
 constexpr int INV_SMEM = 225 * 1024;   // shared memory of one solve CTA
+
+// Conditioning of the layers' Schur complements, gam = max_i S_ii (S^{-1})_ii, up to which
+// their explicit inverses serve; beyond it a call goes over to the block Cholesky.  A
+// product with S^{-1} is off by about eps gam, the block Cholesky's by less where the
+// material or the mesh makes gam large.
+// FP64, energy error of the particular functions against a refined 64-bit solution,
+// inverse form / block Cholesky by gam of A11: up to 700 0.6 to 1.9 (E1 / E2 from 2 to
+// 2,500; bricks of aspect ratio 1 to 60), nu = 0.499 at 150 3.2; E1 / E2 = 25,000 on cubes
+// 4,000 13; nu = 0.49999 3,700 120; E1 / E2 = 250,000 42,000 190.  K (whose solves only
+// steer the iteration; its eigen-residuals were level up to 170,000, fifty times larger at
+// 3e7) has 20 to 4,400 on plies with aspect ratios up to 15 and curved sections.
+// Mixed (CG and refinement take the factors as a preconditioner): steps and residuals as
+// with the block Cholesky up to 26,000; at 170,000 a run ended at 3e-2 instead of 1e-6,
+// and from 65,000 on pivots turn non-positive where the block Cholesky's do not.
+constexpr float INV_COND_A11 = 1e3f, INV_COND_K = 1e5f, INV_COND_F32 = 5e4f;
 
 template <typename T>
 const void* solve_kernel_ptr(int rs, bool back) {
@@ -1866,6 +1911,8 @@ msgfem_status inv_build(msgfem* h) {
   TRY(dev_alloc_bytes(h, &p, f.mats.size() * sizeof(InvMat)));
   f.d_mats = static_cast<InvMat*>(p);
   CK(cudaMemcpy(f.d_mats, f.mats.data(), f.mats.size() * sizeof(InvMat), cudaMemcpyHostToDevice));
+  TRY(dev_alloc_bytes(h, &p, (2 * (size_t)h->N + 2) * sizeof(int)));
+  f.d_cond = static_cast<int*>(p);
   TRY(kerr_ensure(h));
   f.waves.resize(h->waves.size());
   for (size_t w = 0; w < h->waves.size(); ++w) {
@@ -1984,9 +2031,13 @@ static void inv_factor_t(msgfem* h, int w, cudaStream_t st) {
       cudaEventRecord(h->gs.join[g], h->gs.s[g]);
       cudaStreamWaitEvent(st, h->gs.join[g], 0);
     }
-  // packed couplings, over the sweep's scratch; inactive subdomains (other waves) are skipped
+  // inactive subdomains (other waves) are skipped by the kernels below
   int maxl = 1;
   for (int i : wv.all) maxl = std::max(maxl, f.mats[i].nL);
+  cudaMemsetAsync(f.d_cond, 0, 2 * (size_t)h->N * sizeof(int), st);
+  k_inv_condition<T><<<dim3((int)f.mats.size(), maxl), 128, 0, st>>>(f.d_mats, h->d_flags, h->d_notspd, f.d_cond);
+  ++g_launch_count;
+  // packed couplings, over the sweep's scratch
   k_inv_pack<T><<<dim3(maxl, (int)f.mats.size()), 256, 0, st>>>(f.d_mats, h->d_flags);
   ++g_launch_count;
   if (sizeof(T) == 4) {
@@ -2012,6 +2063,19 @@ static void inv_factor_t(msgfem* h, int w, cudaStream_t st) {
 void inv_factor(msgfem* h, int w, cudaStream_t st) {
   if (h->mixed) inv_factor_t<float>(h, w, st);
   else inv_factor_t<double>(h, w, st);
+}
+
+msgfem_status inv_sound(msgfem* h, int w, bool* sound) {
+  const InvForm& f = *h->inv;
+  std::vector<float> g(2 * (size_t)h->N);
+  CK(cudaMemcpyAsync(g.data(), f.d_cond, g.size() * sizeof(float), cudaMemcpyDeviceToHost, h->stream));
+  CK(cudaStreamSynchronize(h->stream));
+  *sound = true;
+  for (int i : f.waves[w].all) {
+    const InvMat& m = f.mats[i];
+    *sound = *sound && g[2 * m.sub + m.mat] <= (h->mixed ? INV_COND_F32 : m.mat == 0 ? INV_COND_K : INV_COND_A11);
+  }
+  return MSGFEM_OK;
 }
 
 // X = M^{-1} B for K (mat 0) or A11 (mat 1) of the current wave, the first ncols columns
