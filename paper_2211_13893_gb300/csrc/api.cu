@@ -1494,6 +1494,38 @@ static msgfem_status local_spaces_run(msgfem_h h, const std::vector<int>& nl, do
   return MSGFEM_OK;
 }
 
+// Task lists (and the block Cholesky's scratch) of the coarse matrix for the current NcPad.
+static msgfem_status coarse_build(msgfem* h) {
+  if (h->inv) return coarse_inv_build(h);
+  const int NcPad = h->NcPad;
+  {
+    // the coarse inverse's split rows: scratch tiles and the identity strip
+    size_t tiles = 0;
+    int maxc = 1;
+    coarse_inverse_split_sizes(NcPad / TILE, COARSE_INV_SPLIT, &tiles, &maxc);
+    dfree(h, h->d_cscr);
+    dfree(h, h->d_cid);
+    h->d_cscr = h->d_cid = nullptr;
+    TRY(dalloc(h, &h->d_cscr, std::max<size_t>(tiles, 1) * TILE * TILE));
+    std::vector<double> id((size_t)TILE * maxc * TILE, 0.0);
+    for (int r = 0; r < TILE; ++r)
+      for (int c = 0; c < maxc; ++c) id[(size_t)r * maxc * TILE + (size_t)c * TILE + r] = 1.0;
+    TRY(dalloc(h, &h->d_cid, id.size()));
+    CK(cudaMemcpy(h->d_cid, id.data(), id.size() * sizeof(double), cudaMemcpyHostToDevice));
+  }
+  build_coarse_schedules(h);
+  dfree(h, h->cfact.d_gemm);
+  dfree(h, h->csolve.d_tasks);
+  h->cfact.d_gemm = nullptr;
+  h->csolve.d_tasks = nullptr;
+  TRY(dalloc(h, &h->cfact.d_gemm, h->cfact.gemm.size()));
+  CK(cudaMemcpy(h->cfact.d_gemm, h->cfact.gemm.data(), h->cfact.gemm.size() * sizeof(GemmTask), cudaMemcpyHostToDevice));
+  TRY(dalloc(h, &h->csolve.d_tasks, h->csolve.tasks.size()));
+  CK(cudaMemcpy(h->csolve.d_tasks, h->csolve.tasks.data(), h->csolve.tasks.size() * sizeof(SolveTask),
+                cudaMemcpyHostToDevice));
+  return MSGFEM_OK;
+}
+
 msgfem_status msgfem_coarse_assemble(msgfem_h h, int* coarse_dim_out) {
   return msgfem_coarse_assemble_threshold(h, 0.0, coarse_dim_out);
 }
@@ -1583,35 +1615,10 @@ msgfem_status msgfem_coarse_assemble_threshold(msgfem_h h, double t, int* coarse
       h->NcCap = NcPad;
     }
     h->NcPad = NcPad;
-    if (h->inv) {
-      TRY(coarse_inv_build(h));
-    } else {
-      {
-        // the coarse inverse's split rows: scratch tiles and the identity strip
-        size_t tiles = 0;
-        int maxc = 1;
-        coarse_inverse_split_sizes(NcPad / TILE, COARSE_INV_SPLIT, &tiles, &maxc);
-        dfree(h, h->d_cscr);
-        dfree(h, h->d_cid);
-        h->d_cscr = h->d_cid = nullptr;
-        TRY(dalloc(h, &h->d_cscr, std::max<size_t>(tiles, 1) * TILE * TILE));
-        std::vector<double> id((size_t)TILE * maxc * TILE, 0.0);
-        for (int r = 0; r < TILE; ++r)
-          for (int c = 0; c < maxc; ++c) id[(size_t)r * maxc * TILE + (size_t)c * TILE + r] = 1.0;
-        TRY(dalloc(h, &h->d_cid, id.size()));
-        CK(cudaMemcpy(h->d_cid, id.data(), id.size() * sizeof(double), cudaMemcpyHostToDevice));
-      }
-      build_coarse_schedules(h);
-      dfree(h, h->cfact.d_gemm);
-      dfree(h, h->csolve.d_tasks);
-      h->cfact.d_gemm = nullptr;
-      h->csolve.d_tasks = nullptr;
-      TRY(dalloc(h, &h->cfact.d_gemm, h->cfact.gemm.size()));
-      CK(cudaMemcpy(h->cfact.d_gemm, h->cfact.gemm.data(), h->cfact.gemm.size() * sizeof(GemmTask),
-                    cudaMemcpyHostToDevice));
-      TRY(dalloc(h, &h->csolve.d_tasks, h->csolve.tasks.size()));
-      CK(cudaMemcpy(h->csolve.d_tasks, h->csolve.tasks.data(), h->csolve.tasks.size() * sizeof(SolveTask),
-                    cudaMemcpyHostToDevice));
+    const msgfem_status bst = coarse_build(h);
+    if (bst != MSGFEM_OK) {
+      h->NcPad = 0;   // built again by the next call
+      return bst;
     }
   }
   h->Nc = Nc;

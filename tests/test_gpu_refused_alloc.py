@@ -1,0 +1,77 @@
+"""Device memory that the caller's allocator refuses in the middle of a call: the call
+returns ENOMEM, and once memory is there again the handle works as one that never met the
+refusal, bit for bit (the calls are deterministic).  Every allocation of the call is
+refused once, the first, the second and so on, each on a fresh handle."""
+from dataclasses import replace
+
+import numpy as np
+import pytest
+
+from workloads import element_angles, get_config
+
+pytestmark = pytest.mark.gpu
+
+
+class Refusing:
+    """PyTorch's caching allocator; the allocation number `at` after arm(at) is refused."""
+
+    def __init__(self):
+        import torch
+        self.torch, self.left, self.refused = torch, -1, False
+
+    def arm(self, at):
+        self.left, self.refused = at, False
+
+    def alloc(self, n):
+        if self.left == 0:
+            self.left, self.refused = -1, True
+            return None
+        self.left -= self.left > 0
+        return self.torch.cuda.caching_allocator_alloc(n, device=self.torch.cuda.current_device())
+
+    def free(self, p, n):
+        self.torch.cuda.caching_allocator_delete(p)
+
+    def refuse(self, at, call):
+        """call() with its allocation `at` refused (ENOMEM); False when it has no such allocation."""
+        from paper_2211_13893_gb300.msgfem import MsgfemError
+        self.arm(at)
+        try:
+            call()
+        except MsgfemError as err:
+            assert err.code == 2 and self.refused, err
+        met, self.left = self.refused, -1
+        return met
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(factor_schedule=1), dict(precision=1)])
+def test_coarse_assembly(kw):
+    from paper_2211_13893_gb300 import MSGFEM
+    cfg = replace(get_config("t3"), n_loc=24)
+    ang = element_angles(cfg)
+    ref = MSGFEM.from_config(cfg, ang, seed=5, **kw)
+    lam = ref.local_spaces(cfg.n_loc)
+    small = 1.0 / np.median(lam)                # a threshold that keeps a smaller coarse space
+    dims, sols = [], []
+    for t in (0.0, small):
+        dims.append(ref.coarse_assemble(threshold=t))
+        sols.append(ref.solve()[0])
+    ref.close()
+    assert -(-dims[1] // 64) < -(-dims[0] // 64)   # another number of tiles
+    mem = Refusing()
+    for first in (None, small):                 # the arrays grow from nothing, from the small coarse space
+        at = 0
+        while True:
+            m = MSGFEM.from_config(cfg, ang, seed=5, allocator=(mem.alloc, mem.free), **kw)
+            m.local_spaces(cfg.n_loc)
+            if first is not None:
+                m.coarse_assemble(threshold=first)
+            met = mem.refuse(at, m.coarse_assemble)
+            for t, dim, want in ((0.0, dims[0], sols[0]), (small, dims[1], sols[1])):
+                assert m.coarse_assemble(threshold=t) == dim
+                assert np.array_equal(m.solve()[0], want)
+            m.close()
+            if not met:
+                break
+            at += 1
+        assert at >= 4
