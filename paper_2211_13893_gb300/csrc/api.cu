@@ -1615,7 +1615,7 @@ msgfem_status msgfem_coarse_assemble_threshold(msgfem_h h, double t, int* coarse
       h->NcCap = NcPad;
     }
     h->NcPad = NcPad;
-    const msgfem_status bst = coarse_build(h);
+    const msgfem_status bst = NcPad > 0 ? coarse_build(h) : MSGFEM_OK;
     if (bst != MSGFEM_OK) {
       h->NcPad = 0;   // built again by the next call
       return bst;
@@ -1624,15 +1624,17 @@ msgfem_status msgfem_coarse_assemble_threshold(msgfem_h h, double t, int* coarse
   h->Nc = Nc;
   CK(cudaMemcpyAsync(h->d_coff, h->coff.data(), h->N * sizeof(int), cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(h->d_m, h->basis_m.data(), h->N * sizeof(int), cudaMemcpyHostToDevice, st));
-  CK(cudaMemsetAsync(h->d_AH, 0, (size_t)NcPad * NcPad * sizeof(double), st));
-  launch_coarse_blocks(h);
-  launch_coarse_rhs(h);
   CK(cudaMemsetAsync(h->d_notspd + h->N, 0, sizeof(int), st));
-  if (h->inv) {
-    CK(cudaMemcpyAsync(h->d_AHkeep, h->d_AH, (size_t)NcPad * NcPad * sizeof(double), cudaMemcpyDeviceToDevice, st));
-    coarse_inv_factor(h);
-  } else {
-    run_schedule(h->cfact, st);
+  if (Nc > 0) {   // (a threshold may leave no function at all: u^G = 0)
+    CK(cudaMemsetAsync(h->d_AH, 0, (size_t)NcPad * NcPad * sizeof(double), st));
+    launch_coarse_blocks(h);
+    launch_coarse_rhs(h);
+    if (h->inv) {
+      CK(cudaMemcpyAsync(h->d_AHkeep, h->d_AH, (size_t)NcPad * NcPad * sizeof(double), cudaMemcpyDeviceToDevice, st));
+      coarse_inv_factor(h);
+    } else {
+      run_schedule(h->cfact, st);
+    }
   }
   span_end(h, sp_c);
   CK_LAUNCH();

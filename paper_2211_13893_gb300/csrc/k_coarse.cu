@@ -262,11 +262,13 @@ void launch_coarse_restrict(msgfem* h, const double* r, cudaStream_t st) {
 }
 
 void launch_coarse_rhs(msgfem* h) {
+  if (h->Nc == 0) return;
   cudaMemsetAsync(h->d_bH, 0, sizeof(double) * (size_t)h->NcPad * PST, h->stream);
   launch_coarse_restrict(h, nullptr, h->stream);
 }
 
 void launch_coarse_solve(msgfem* h, cudaStream_t st, int refine) {
+  if (h->Nc == 0) return;
   if (h->inv == nullptr) {
     run_solve_mv(h->csolve, st, 0, 0, 0);
     return;

@@ -271,7 +271,11 @@ __global__ void k_chol_inv_small(const SubDev* __restrict__ subs, const int* __r
   if (active != nullptr && !active[sidx]) return;
   const SubDev& s = subs[sidx];
   const int n = ncol_sub ? ncol_sub[sidx] : nfixed;
-  if (n <= 0) return;
+  if (n <= 0) {   // no columns: nothing of an earlier factor stays
+    for (int e = threadIdx.x; e < PST * PST; e += blockDim.x) s.Y[e] = 0.0;
+    if (threadIdx.x == 0) s.status[2] = 0;
+    return;
+  }
   __shared__ double L[PST][PST + 1];
   __shared__ double U[PST][PST + 1];
   __shared__ double d[PST];
