@@ -403,6 +403,15 @@ void span_end(msgfem* h, int idx) {
   if (idx >= 0) cudaEventRecord(h->spans[idx].b, h->stream);
 }
 
+// spans that are not to be counted
+void drop_spans(msgfem* h) {
+  for (auto& sp : h->spans) {
+    h->ev_pool.push_back(sp.a);
+    h->ev_pool.push_back(sp.b);
+  }
+  h->spans.clear();
+}
+
 void spans_collect(msgfem* h) {
   if (h->spans.empty()) return;
   cudaStreamSynchronize(h->stream);
@@ -1285,6 +1294,7 @@ static msgfem_status local_spaces_run(msgfem_h h, const std::vector<int>& nl, do
   TRY(set_active(h, act));
   CK(cudaMemsetAsync(h->d_notspd, 0, (h->N + 1) * sizeof(int), st));
   for (auto& s : h->sub) CK(cudaMemsetAsync(s.status, 0, 4 * sizeof(int), st));
+  if (!h->inv_on) TRY(chol_lists(h));
   count_factor_flops(h);
   h->prof.solve_flops = 0.0;
   h->prof.solve_bytes = 0.0;
@@ -1823,14 +1833,38 @@ static msgfem_status autotune_run(msgfem_h h, int reps, msgfem_tuning* out);
 
 msgfem_status msgfem_autotune(msgfem_h h, int reps, msgfem_tuning* out) {
   if (!h) return MSGFEM_EINVAL;
+  if (h->stage < 2) return MSGFEM_ESTATE;
+  const bool use = h->inv_use;
+  const int left = h->factor_left, groups_f = h->ngroup_factor, tc = h->factor_tc, persistent = h->factor_persistent;
+  const int groups = h->ngroup, variant = h->solve_variant;
+  spans_collect(h);
+  const msgfem_profile prof = h->prof;
+  const long long launches = g_launch_count;
   const msgfem_status st = autotune_run(h, reps, out);
+  if (st != MSGFEM_OK) {
+    // the handle as before the call; the block Cholesky's task lists, half replaced, are
+    // built again when they are needed
+    cudaStreamSynchronize(h->stream);
+    drop_graphs(h);
+    h->inv_use = h->inv_on = use;
+    h->factor_left = left;
+    h->ngroup_factor = groups_f;
+    h->factor_tc = tc;
+    h->factor_persistent = persistent;
+    h->ngroup = groups;
+    h->solve_variant = variant;
+    drop_spans(h);
+    h->prof = prof;
+    g_launch_count = launches;
+    h->cur = 0;
+    h->base_act.assign(h->N, 1);
+    (void)set_active(h, h->base_act);
+  }
   const msgfem_status ke = check_stage_error(h);
   return ke != MSGFEM_OK ? ke : st;
 }
 
 static msgfem_status autotune_run(msgfem_h h, int reps, msgfem_tuning* out) {
-  if (!h) return MSGFEM_EINVAL;
-  if (h->stage < 2) return MSGFEM_ESTATE;
   if (reps <= 0) reps = 3;
   h->factored_wave = -1;   // the timed factorisations leave scratch in the pool
   h->inv_on = false;       // the block Cholesky's candidates first, then the inverse form against the best
@@ -1838,14 +1872,8 @@ static msgfem_status autotune_run(msgfem_h h, int reps, msgfem_tuning* out) {
   CK(cudaStreamSynchronize(st));
   // the task lists are re-uploaded below: drop every captured factorisation and
   // solve graph first, so that none can replay a freed task list
-  for (auto it = h->graphs.begin(); it != h->graphs.end();) {
-    if ((it->first >> 60) == 1 || (it->first >> 60) == 2) {
-      if (it->second.first) cudaGraphExecDestroy(it->second.first);
-      it = h->graphs.erase(it);
-    } else {
-      ++it;
-    }
-  }
+  drop_graphs(h);
+  h->chol_ready = false;
   // the last wave's factors are the ones resident in the pool
   const int last = (int)h->waves.size() - 1;
   WaveSched& wl = h->waves[last];
@@ -1996,16 +2024,6 @@ static msgfem_status autotune_run(msgfem_h h, int reps, msgfem_tuning* out) {
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
-  auto drop_graphs = [&]() {
-    for (auto it = h->graphs.begin(); it != h->graphs.end();) {
-      if ((it->first >> 60) == 1 || (it->first >> 60) == 2) {
-        if (it->second.first) cudaGraphExecDestroy(it->second.first);
-        it = h->graphs.erase(it);
-      } else {
-        ++it;
-      }
-    }
-  };
   // block-solve stream groups and kernel: each choice timed on applications
   // of the shift-invert operator as the eigensolver makes them (N-product
   // stencil, K solve, in mixed precision with its PCG refinement, and the
@@ -2019,14 +2037,14 @@ static msgfem_status autotune_run(msgfem_h h, int reps, msgfem_tuning* out) {
   for (int gi = 0; gi < 4; ++gi) {
     for (int vi = 0; vi < 4; ++vi) t.solve_ms[gi][vi] = -1.0;
     if (groups[gi] > h->ngroup_created) continue;
-    drop_graphs();
+    drop_graphs(h);
     h->ngroup = groups[gi];
     build_wave_solve_schedules(h, wl);
     TRY(upload_wave_solves(h, wl));
     for (int vi = 0; vi < 4; ++vi) {
       const int v = variants[vi];
       if ((v == SOLVE_ASYNC_RING || v == SOLVE_TMA_RING) && !h->mixed) continue;
-      drop_graphs();
+      drop_graphs(h);
       h->solve_variant = v;
       for (int r = 0; r <= reps; ++r) {
         if (r == 1) CK(cudaEventRecord(e0, st));
@@ -2046,7 +2064,7 @@ static msgfem_status autotune_run(msgfem_h h, int reps, msgfem_tuning* out) {
       }
     }
   }
-  drop_graphs();
+  drop_graphs(h);
   h->solve_variant = saved_variant;
   if (h->inv != nullptr) {
     // the inverse form: one factorisation and the same operator applications; kept
@@ -2075,11 +2093,7 @@ static msgfem_status autotune_run(msgfem_h h, int reps, msgfem_tuning* out) {
   CK(cudaEventDestroy(f0));
   CK(cudaEventDestroy(f1));
   CK(cudaStreamSynchronize(st));
-  for (auto& sp : h->spans) {   // the timing's phase spans are dropped
-    h->ev_pool.push_back(sp.a);
-    h->ev_pool.push_back(sp.b);
-  }
-  h->spans.clear();
+  drop_spans(h);   // the timing's phase spans
   h->prof = prof_kept;
   g_launch_count = launches_kept;
   CK(cudaEventDestroy(e0));

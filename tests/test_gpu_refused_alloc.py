@@ -75,3 +75,36 @@ def test_coarse_assembly(kw):
                 break
             at += 1
         assert at >= 4
+
+
+@pytest.mark.parametrize("waves", [1, 2])
+@pytest.mark.parametrize("kw", [dict(), dict(precision=1), dict(solve_kernel=2)])
+def test_autotuner(kw, waves):
+    """The local stage after a refused autotuner is the one before it, also of waves whose
+    task lists the autotuner had not reached."""
+    from paper_2211_13893_gb300 import MSGFEM, plan
+    cfg = get_config("t2")
+    ang = element_angles(cfg)
+    kw = dict(kw, wave_mb=0.0 if waves == 1 else 1.01 * plan(cfg, kw.get("precision", 0))["pool_mb"] / waves)
+    mem = Refusing()
+    at = 0
+    while True:
+        m = MSGFEM.from_config(cfg, ang, seed=5, allocator=(mem.alloc, mem.free), **kw)
+        lam = m.local_spaces(cfg.n_loc).copy()
+        before = m.profile()
+        assert before["waves"] >= waves
+        met = mem.refuse(at, lambda: m.autotune(reps=1))
+        if not met:
+            break
+        assert m.profile()["launches"] == before["launches"]
+        assert np.array_equal(m.local_spaces(cfg.n_loc), lam), at
+        after = m.profile()
+        assert after["factor_flops"] == before["factor_flops"]
+        assert after["factor_flops_executed"] == before["factor_flops_executed"]
+        m.coarse_assemble()
+        u, _ = m.solve()
+        assert np.all(np.isfinite(u))
+        m.close()
+        at = at + 1 if at < 6 else 2 * at
+    m.close()
+    assert at >= 6
