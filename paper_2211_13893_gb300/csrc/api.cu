@@ -145,22 +145,42 @@ msgfem_status set_angles(msgfem* h, const double* ang) {
   std::vector<int> etype, trep;
   element_types(h, layered, types, etype, trep);
   const bool geometric = !h->h_xyz.empty() || !h->h_frame.empty();
-  if ((int)types.size() > h->type_cap) {
-    h->type_cap = (int)types.size();
-    TRY(dalloc(h, &h->d_angles_type, types.size()));
-    TRY(dalloc(h, &h->d_Ke, types.size() * 576));
+  // arrays that grow: all of them are there before any of the handle's is replaced
+  const size_t nt = types.size();
+  const bool typed = geometric && !layered, grow = (int)nt > h->type_cap, grow_rep = typed && (int)nt > h->trep_cap;
+  double *ang_type = nullptr, *Ke = nullptr;
+  int *etype_dev = nullptr, *trep_dev = nullptr;
+  auto grow_all = [&]() -> msgfem_status {
+    if (grow) TRY(dalloc(h, &ang_type, nt));
+    if (grow) TRY(dalloc(h, &Ke, nt * 576));
+    if (typed && h->d_etype == nullptr) TRY(dalloc(h, &etype_dev, ntot));
+    if (grow_rep) TRY(dalloc(h, &trep_dev, nt));
+    return MSGFEM_OK;
+  };
+  const msgfem_status gst = grow_all();
+  if (gst != MSGFEM_OK) {
+    for (void* p : {(void*)ang_type, (void*)Ke, (void*)etype_dev, (void*)trep_dev}) dfree(h, p);
+    return gst;
   }
-  if (geometric && !layered) {
-    if (h->d_etype == nullptr) TRY(dalloc(h, &h->d_etype, ntot));
-    if ((int)types.size() > h->trep_cap) {
-      h->trep_cap = (int)types.size();
-      TRY(dalloc(h, &h->d_trep, types.size()));
-    }
+  if (grow) {
+    dfree(h, h->d_angles_type);
+    dfree(h, h->d_Ke);
+    h->d_angles_type = ang_type;
+    h->d_Ke = Ke;
+    h->type_cap = (int)nt;
+  }
+  if (etype_dev) h->d_etype = etype_dev;
+  if (grow_rep) {
+    dfree(h, h->d_trep);
+    h->d_trep = trep_dev;
+    h->trep_cap = (int)nt;
+  }
+  if (typed) {
     CK(cudaMemcpyAsync(h->d_etype, etype.data(), ntot * sizeof(int), cudaMemcpyHostToDevice, h->stream));
     CK(cudaMemcpyAsync(h->d_trep, trep.data(), trep.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream));
   }
   h->layered = layered ? 1 : 0;
-  h->typed = (geometric && !layered) ? 1 : 0;
+  h->typed = typed ? 1 : 0;
   h->ntypes = (int)types.size();
   CK(cudaMemcpyAsync(h->d_angles_type, types.data(), types.size() * sizeof(double), cudaMemcpyHostToDevice, h->stream));
   CK(cudaStreamSynchronize(h->stream));

@@ -108,3 +108,34 @@ def test_autotuner(kw, waves):
         at = at + 1 if at < 6 else 2 * at
     m.close()
     assert at >= 6
+
+
+def test_update_angles():
+    """Angles that need more element matrices than the earlier ones (per element instead of
+    per ply): refused, the earlier angles stay, also for the solution that is there."""
+    from paper_2211_13893_gb300 import MSGFEM
+    cfg = get_config("t2")
+    ang = element_angles(cfg)
+    other = ang + np.random.default_rng(2).standard_normal(ang.shape)
+    mem = Refusing()
+    ref = MSGFEM.from_config(cfg, other, seed=5)
+    want = ref.local_spaces(cfg.n_loc).copy()
+    ref.close()
+    u_ref = np.sin(np.arange(cfg.n_dof))
+    at = 0
+    while True:
+        m = MSGFEM.from_config(cfg, ang, seed=5, allocator=(mem.alloc, mem.free))
+        lam = m.local_spaces(cfg.n_loc).copy()
+        m.coarse_assemble()
+        _, err = m.solve(u_ref=u_ref)
+        met = mem.refuse(at, lambda: m.update_angles(other))
+        if met:
+            assert m.solve(u_ref=u_ref)[1] == err
+            assert np.array_equal(m.local_spaces(cfg.n_loc), lam)
+            m.update_angles(other)
+        assert np.array_equal(m.local_spaces(cfg.n_loc), want)
+        m.close()
+        if not met:
+            break
+        at += 1
+    assert at >= 2
