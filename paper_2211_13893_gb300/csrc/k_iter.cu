@@ -539,7 +539,7 @@ __global__ void k_colnorm_reduce(const SubDev* __restrict__ subs, const int* __r
     for (int w = 0; w < 3; ++w) t[w] += part[(((size_t)sidx * nchunk + c) * 3 + w) * 32 + lane];
   const double th = s.theta[lane];
   const double den = sqrt(t[1]) + fabs(th) * sqrt(t[2]);
-  s.resid[lane] = (lane < p && den > 0.0) ? sqrt(t[0]) / den : 0.0;
+  s.resid[lane] = (lane < p && den != 0.0) ? sqrt(t[0]) / den : 0.0;   // (a NaN stays one)
 }
 
 // D = diag(theta) X - Y on columns < p (zero elsewhere).

@@ -435,7 +435,7 @@ k_rr_jacobi(const SubDev* __restrict__ subs, const int* __restrict__ active, con
   __shared__ double d[MQ], id[MQ], al[MQ / 2], be[MQ / 2];
   __shared__ int pa[MQ / 2], pb[MQ / 2];
   __shared__ double red_off[16], red_tot[16];
-  __shared__ int again;
+  __shared__ int again, bad;
   const int tid = threadIdx.x, np = m / 2;      // m is a multiple of KB
   float* log = wk.log + (size_t)sidx * RR_ROUNDS * (MQ / 2);
   for (int e = tid; e < m * m; e += 512) {
@@ -468,6 +468,7 @@ k_rr_jacobi(const SubDev* __restrict__ subs, const int* __restrict__ active, con
       double so = 0.0, st = 0.0;
       for (int w = 0; w < 16; ++w) { so += red_off[w]; st += red_tot[w]; }
       again = so > 1e-30 * st;
+      bad = !(st <= 1.7e308);   // an operator with a NaN or an infinity has no Ritz pairs
     }
     __syncthreads();
     if (!again) break;
@@ -523,9 +524,10 @@ k_rr_jacobi(const SubDev* __restrict__ subs, const int* __restrict__ active, con
   if (tid < m) {
     int rank = 0;
     for (int j = 0; j < m; ++j) rank += (mu[j] > mu[tid] || (mu[j] == mu[tid] && j < tid)) ? 1 : 0;
+    if (bad) rank = tid;   // every rank is written: none keeps an earlier call's value
     if (rank < nw && rank < PST) {
       wk.perm[sidx * PST + rank] = tid;
-      wk.mu[sidx * PST + rank] = mu[tid];
+      wk.mu[sidx * PST + rank] = bad ? NAN : mu[tid];
     }
   }
   if (tid == 0) wk.rounds[sidx] = rounds;
