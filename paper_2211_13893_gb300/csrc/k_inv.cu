@@ -720,10 +720,10 @@ k_inv_condition(const InvMat* __restrict__ mats, const int* __restrict__ active,
 __host__ __device__ __forceinline__ int up4(int v) { return (v + 3) & ~3; }
 template <typename T>
 __global__ void k_inv_pack(const InvMat* __restrict__ mats, const int* __restrict__ active) {
-  const InvMat& m = mats[blockIdx.y];
+  const InvMat& m = mats[blockIdx.x];
   if (active != nullptr && !active[m.sub]) return;
   const int nn = m.n / 3, np = up4(nn);
-  for (int l = blockIdx.x; l < m.nL; l += gridDim.x) {
+  for (int l = blockIdx.y; l < m.nL; l += gridDim.y) {
     T* out = static_cast<T*>(m.L) + (size_t)l * m.b * m.b;
     for (int e = threadIdx.x; e < 2 * np * 81; e += blockDim.x) {
       const int dir = e / (np * 81), p = (e / 81) % np, s = e % 81, dk = dir ? 1 : -1;
@@ -1024,9 +1024,9 @@ __host__ __device__ __forceinline__ int f32_blocks(int n, int G) { return ((n + 
 // rows, then [column / 4][row of the strip][4]; zero outside the n x n matrix.
 __global__ void __launch_bounds__(256)
 k_inv_pack_f32(const InvMat* __restrict__ mats, const int* __restrict__ active, int last) {
-  const InvMat& m = mats[blockIdx.z];
+  const InvMat& m = mats[blockIdx.x];
   if (m.sg == 0 || (active != nullptr && !active[m.sub])) return;
-  const int l = last ? m.nL - 1 : blockIdx.y, rb = blockIdx.x, nb = (m.n + 31) / 32, kp = nb * 32;
+  const int l = last ? m.nL - 1 : blockIdx.y, rb = blockIdx.z, nb = (m.n + 31) / 32, kp = nb * 32;
   if (rb >= nb || (!last && l >= m.nL - 1)) return;
   __shared__ float4 tile[32][33];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
@@ -1338,9 +1338,9 @@ __device__ __forceinline__ int* row_exponents(const InvMat& m, int l) {
 // -S^{-1} of every layer to biased integers in fragment order, in place: one strip of 16 rows per CTA
 __global__ void __launch_bounds__(256)
 k_inv_digits(const InvMat* __restrict__ mats, const int* __restrict__ active) {
-  const InvMat& m = mats[blockIdx.z];
+  const InvMat& m = mats[blockIdx.x];
   if (active != nullptr && !active[m.sub]) return;
-  const int l = blockIdx.y, s = blockIdx.x, nkb = (m.n + 15) / 16;
+  const int l = blockIdx.y, s = blockIdx.z, nkb = (m.n + 15) / 16;
   if (l >= m.nL || s >= nkb) return;
   extern __shared__ __align__(16) unsigned char smem_dg[];
   double* v = reinterpret_cast<double*>(smem_dg);
@@ -2031,21 +2031,22 @@ static void inv_factor_t(msgfem* h, int w, cudaStream_t st) {
       cudaEventRecord(h->gs.join[g], h->gs.s[g]);
       cudaStreamWaitEvent(st, h->gs.join[g], 0);
     }
-  // inactive subdomains (other waves) are skipped by the kernels below
+  // inactive subdomains (other waves) are skipped by the kernels below (the matrices, two
+  // per subdomain, lie along x: the other grid dimensions end at 65,535)
   int maxl = 1;
   for (int i : wv.all) maxl = std::max(maxl, f.mats[i].nL);
   cudaMemsetAsync(f.d_cond, 0, 2 * (size_t)h->N * sizeof(int), st);
   k_inv_condition<T><<<dim3((int)f.mats.size(), maxl), 128, 0, st>>>(f.d_mats, h->d_flags, h->d_notspd, f.d_cond);
   ++g_launch_count;
   // packed couplings, over the sweep's scratch
-  k_inv_pack<T><<<dim3(maxl, (int)f.mats.size()), 256, 0, st>>>(f.d_mats, h->d_flags);
+  k_inv_pack<T><<<dim3((int)f.mats.size(), maxl), 256, 0, st>>>(f.d_mats, h->d_flags);
   ++g_launch_count;
   if (sizeof(T) == 4) {
     int kmax = 0;
     for (int i : wv.all)
       if (f.mats[i].sg > 0) kmax = std::max(kmax, (f.mats[i].n + 31) / 32);
     for (int last = 0; last < 2 && kmax > 0; ++last) {
-      k_inv_pack_f32<<<dim3(kmax, last ? 1 : maxl, (int)f.mats.size()), 256, 0, st>>>(f.d_mats, h->d_flags, last);
+      k_inv_pack_f32<<<dim3((int)f.mats.size(), last ? 1 : maxl, kmax), 256, 0, st>>>(f.d_mats, h->d_flags, last);
       ++g_launch_count;
     }
   }
@@ -2055,7 +2056,7 @@ static void inv_factor_t(msgfem* h, int w, cudaStream_t st) {
       bmax = std::max(bmax, f.mats[i].b);
       kmax = std::max(kmax, (f.mats[i].n + 15) / 16);
     }
-    k_inv_digits<<<dim3(kmax, maxl, (int)f.mats.size()), 256, 16 * (bmax + 2) * 8, st>>>(f.d_mats, h->d_flags);
+    k_inv_digits<<<dim3((int)f.mats.size(), maxl, kmax), 256, 16 * (bmax + 2) * 8, st>>>(f.d_mats, h->d_flags);
     ++g_launch_count;
   }
 }
