@@ -20,7 +20,7 @@ namespace {
 constexpr double KSIGMA = 1e-2;   // N = S + KSIGMA T
 
 // Rayleigh-Ritz work arrays: wanted mu (descending) and their indices [N][PST], the
-// rotations' tangents [N][rounds][MQ / 2], rounds run [N]
+// rotations' tangents [RR_BATCH or N][rounds][MQ / 2], rounds run [N]
 struct RrWork {
   double* mu;
   float* log;
@@ -407,6 +407,9 @@ __global__ void k_take_col_kb(const SubDev* __restrict__ subs, const int* __rest
 // rows, columns and vectors before).
 constexpr int RR_SWEEPS = 30;
 constexpr int RR_ROUNDS = RR_SWEEPS * (MQ - 1);
+// The log of a subdomain takes 547 KB (the most sweeps at the largest basis), so that of
+// the subdomains of one launch only is kept: two rounds of the two CTAs that an SM holds.
+constexpr int RR_BATCH = 608;
 
 // pair k of round r of the round-robin order of mm (even) indices
 __device__ __forceinline__ void rr_pair(int k, int r, int mm, int& a, int& b) {
@@ -424,8 +427,8 @@ __device__ __forceinline__ double rr_rsqrt(double w) {
 
 __global__ void __launch_bounds__(512)
 k_rr_jacobi(const SubDev* __restrict__ subs, const int* __restrict__ active, const int* __restrict__ mvec,
-            const int* __restrict__ nwvec, RrWork wk) {
-  const int sidx = blockIdx.x;
+            const int* __restrict__ nwvec, RrWork wk, int first) {
+  const int sidx = first + blockIdx.x;
   if (active != nullptr && !active[sidx]) return;
   const SubDev& s = subs[sidx];
   const int m = mvec[sidx], nw = nwvec[sidx];
@@ -437,7 +440,7 @@ k_rr_jacobi(const SubDev* __restrict__ subs, const int* __restrict__ active, con
   __shared__ double red_off[16], red_tot[16];
   __shared__ int again, bad;
   const int tid = threadIdx.x, np = m / 2;      // m is a multiple of KB
-  float* log = wk.log + (size_t)sidx * RR_ROUNDS * (MQ / 2);
+  float* log = wk.log + (size_t)blockIdx.x * RR_ROUNDS * (MQ / 2);
   for (int e = tid; e < m * m; e += 512) {
     const int r = e / m, c = e % m;
     if (c <= r) A[r][c] = 0.5 * (s.H[(size_t)r * MQ + c] + s.H[(size_t)c * MQ + r]);
@@ -537,8 +540,8 @@ constexpr int RR_CHUNK = 32;   // rounds whose rotations are staged at once
 
 __global__ void __launch_bounds__(4 * (MQ / 2))
 k_rr_vectors(const SubDev* __restrict__ subs, const int* __restrict__ active, const int* __restrict__ mvec,
-             const int* __restrict__ nwvec, RrWork wk) {
-  const int sidx = blockIdx.y;
+             const int* __restrict__ nwvec, RrWork wk, int first) {
+  const int sidx = first + blockIdx.y;
   if (active != nullptr && !active[sidx]) return;
   const SubDev& s = subs[sidx];
   const int m = mvec[sidx], nw = nwvec[sidx];
@@ -550,7 +553,7 @@ k_rr_vectors(const SubDev* __restrict__ subs, const int* __restrict__ active, co
   const int src = live ? wk.perm[sidx * PST + col] : -1;
   for (int a = k; a < MQ; a += MQ / 2) x[a][c] = (a == src) ? 1.0 : 0.0;
   if (blockIdx.x * 4 < nw) {
-    const float* log = wk.log + (size_t)sidx * RR_ROUNDS * (MQ / 2);
+    const float* log = wk.log + (size_t)blockIdx.y * RR_ROUNDS * (MQ / 2);
     // V e = J_1 (J_2 ( ... J_n e)), each round's disjoint rotations at once
     for (int r1 = wk.rounds[sidx]; r1 > 0; r1 -= RR_CHUNK) {
       const int r0 = max(0, r1 - RR_CHUNK);
@@ -758,7 +761,8 @@ void launch_zero_kb(msgfem* h, int which) {
 
 // bytes of the Rayleigh-Ritz work arrays of N subdomains
 size_t rr_bytes(int N) {
-  return (size_t)N * (PST * (sizeof(double) + sizeof(int)) + RR_ROUNDS * (MQ / 2) * sizeof(float) + 8);
+  return (size_t)N * (PST * (sizeof(double) + sizeof(int)) + 8) +
+         (size_t)std::min(N, RR_BATCH) * RR_ROUNDS * (MQ / 2) * sizeof(float);
 }
 
 void launch_rr_krylov(msgfem* h, const int* d_m, const int* d_nw) {
@@ -772,11 +776,14 @@ void launch_rr_krylov(msgfem* h, const int* d_m, const int* d_nw) {
   char* base = static_cast<char*>(h->d_rr);
   wk.mu = reinterpret_cast<double*>(base);
   wk.log = reinterpret_cast<float*>(wk.mu + (size_t)h->N * PST);
-  wk.perm = reinterpret_cast<int*>(wk.log + (size_t)h->N * RR_ROUNDS * (MQ / 2));
+  wk.perm = reinterpret_cast<int*>(wk.log + (size_t)std::min(h->N, RR_BATCH) * RR_ROUNDS * (MQ / 2));
   wk.rounds = wk.perm + (size_t)h->N * PST;
-  k_rr_jacobi<<<h->N, 512, smem, h->stream>>>(h->d_sub, h->d_flags, d_m, d_nw, wk);
-  k_rr_vectors<<<dim3(PST / 4, h->N), 4 * (MQ / 2), 0, h->stream>>>(h->d_sub, h->d_flags, d_m, d_nw, wk);
-  g_launch_count += 2;
+  for (int first = 0; first < h->N; first += RR_BATCH) {
+    const int n = std::min(RR_BATCH, h->N - first);
+    k_rr_jacobi<<<n, 512, smem, h->stream>>>(h->d_sub, h->d_flags, d_m, d_nw, wk, first);
+    k_rr_vectors<<<dim3(PST / 4, n), 4 * (MQ / 2), 0, h->stream>>>(h->d_sub, h->d_flags, d_m, d_nw, wk, first);
+    g_launch_count += 2;
+  }
 }
 
 void launch_ritz(msgfem* h, const int* d_m, const int* d_nw, int scale, bool masked, int src, int dst) {

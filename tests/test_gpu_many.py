@@ -1,6 +1,7 @@
 """More subdomains than half of a grid dimension: 33,000 in one handle, every instance of
 the same beam, so every instance has the first one's eigenvalues (1e-8, mixed 1e-5: the
-start blocks differ)."""
+start blocks differ).  And the storage per subdomain besides the pool: the working blocks
+of its 192 rows, 1.2 MB, with nothing of that order added per subdomain of a large batch."""
 from dataclasses import replace
 
 import numpy as np
@@ -49,3 +50,17 @@ def test_more_subdomains_than_half_a_grid(precision):
     one.close()
     scale = np.maximum(np.abs(ref).max(axis=1, keepdims=True), 1.0)
     assert (np.abs(lam - ref[None]) / scale[None]).max() <= (1e-8 if precision == 0 else 1e-5)
+
+
+def test_storage_per_subdomain():
+    from paper_2211_13893_gb300 import MSGFEM
+    cfg = replace(get_config("t3"), name="tiny", **TINY)
+    total = []
+    for inst in (700, 1400):
+        pool = _Bump(10 << 30)
+        ang = np.tile(element_angles(cfg).reshape(-1), inst)
+        m = MSGFEM.from_config(cfg, ang, seed=7, instances=inst, allocator=(pool.alloc, pool.free))
+        pool_mb = m.profile()["pool_mb"]
+        total.append(sum(pool.sizes) - pool_mb * 1048576)
+        m.close()
+    assert (total[1] - total[0]) / 1400 <= 1.4e6
