@@ -58,13 +58,14 @@ enum { EPI_PLAIN = 0, EPI_BIAS_TANH = 1, EPI_BIAS = 2, EPI_DTANH = 3, EPI_MSE = 
 // with the leading dimension of C.  EPI_PLAIN also writes the sums of A over k
 // (the bias gradient) to gb; EPI_MSE stores scale (C + bias - H) and adds one
 // partial sum of the squared differences per CTA to part.
-// A cluster of gridDim.z CTAs shares one output tile; rank z sums chunks
+// tn tiles along n; all output tiles lie along the grid's x (its other dimensions end at
+// 65,535).  A cluster of gridDim.z CTAs shares one output tile; rank z sums chunks
 // [z, z + 1) per of the inner dimension.
 template <bool AT, bool BT, int EPI>
 __global__ void __launch_bounds__(256)
 k_gemm(int M, int N, int K, const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
        float* __restrict__ C, int ldc, const float* __restrict__ bias, const float* __restrict__ H,
-       float* __restrict__ gb, float scale, double* __restrict__ part) {
+       float* __restrict__ gb, float scale, double* __restrict__ part, int tn) {
   namespace cg = cooperative_groups;
   __shared__ float As[GK][GT + 1];
   __shared__ float Bs[GK][GT + 1];
@@ -72,7 +73,7 @@ k_gemm(int M, int N, int K, const float* __restrict__ A, int lda, const float* _
   __shared__ float Ss[GT];           // sums of A over its chunks (EPI_PLAIN)
   __shared__ double red[8];
   const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-  const int m0 = blockIdx.y * GT, n0 = blockIdx.x * GT;
+  const int bx = blockIdx.x % tn, m0 = blockIdx.x / tn * GT, n0 = bx * GT;
   const int nch = (K + GK - 1) / GK, per = (nch + gridDim.z - 1) / gridDim.z;
   const int c0 = blockIdx.z * per, c1 = min(c0 + per, nch);
   float acc[2][2] = {};
@@ -142,7 +143,7 @@ k_gemm(int M, int N, int K, const float* __restrict__ A, int lda, const float* _
     }
     C[(size_t)gm * ldc + gn] = v;
   }
-  if (EPI == EPI_PLAIN && blockIdx.x == 0 && z == 0 && tid < GT && m0 + tid < M) {
+  if (EPI == EPI_PLAIN && bx == 0 && z == 0 && tid < GT && m0 + tid < M) {
     float v = 0.f;
     for (int q = 0; q < R; ++q) v += R > 1 ? *cl.map_shared_rank(&Ss[tid], q) : Ss[tid];
     gb[m0 + tid] = v;
@@ -154,7 +155,7 @@ k_gemm(int M, int N, int K, const float* __restrict__ A, int lda, const float* _
     if (tid == 0) {
       double t = 0.0;
       for (int w = 0; w < 8; ++w) t += red[w];
-      part[((size_t)blockIdx.y * gridDim.x + blockIdx.x) * R + z] = t;
+      part[(size_t)blockIdx.x * R + z] = t;
     }
   }
   if (R > 1) cl.sync();   // the partial tiles stay alive until every rank has read them
@@ -196,7 +197,8 @@ void gemm(cudaStream_t st, int M, int N, int K, const float* A, int lda, const f
           const float* bias = nullptr, const float* H = nullptr, float* gb = nullptr, float scale = 0.f,
           double* part = nullptr) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((N + GT - 1) / GT, (M + GT - 1) / GT, split_of(K));
+  const int tn = (N + GT - 1) / GT, tm = (M + GT - 1) / GT;
+  cfg.gridDim = dim3(tn * tm, 1, split_of(K));
   cfg.blockDim = dim3(256);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
@@ -206,7 +208,7 @@ void gemm(cudaStream_t st, int M, int N, int K, const float* A, int lda, const f
   at[0].val.clusterDim.z = cfg.gridDim.z;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_gemm<AT, BT, EPI>, M, N, K, A, lda, B, ldb, C, ldc, bias, H, gb, scale, part);
+  cudaLaunchKernelEx(&cfg, k_gemm<AT, BT, EPI>, M, N, K, A, lda, B, ldb, C, ldc, bias, H, gb, scale, part, tn);
   ++g_launch_count;
 }
 
