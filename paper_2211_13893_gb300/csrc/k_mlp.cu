@@ -2,13 +2,13 @@
 // mean-squared-error gradient and Adam, all in FP32 on the GPU.
 //
 // Every layer is one tiled GEMM (32 x 32 output tile per CTA, 2 x 2 outputs per
-// thread) with the bias, the tanh, the tanh derivative, the loss gradient and the
-// bias gradient fused into it:
+// thread; 64 x 64 and 4 x 4 where enough of them fill the chip) with the bias, the
+// tanh, the tanh derivative, the loss gradient and the bias gradient fused into it:
 //   forward      Z_l = H_{l-1} W_l^T + b_l, H_l = tanh(Z_l) (linear output layer)
 //   loss grad    G_L = 2 (Y - T) / (B d) in the output layer's epilogue
 //   weight grad  dW_l = G_l^T H_{l-1}, db_l = column sums of G_l
 //   data grad    G_{l-1} = (G_l W_l) * (1 - H_{l-1}^2)
-// The products are skinny: a hidden layer of 32 units is a handful of output tiles
+// The products are mostly skinny: a hidden layer of 32 units is a handful of output tiles
 // over an inner dimension of hundreds, so the time is latency, not arithmetic.
 // Long inner dimensions are split over the CTAs of a thread-block cluster (one
 // chunk of 64 each as far as 8 CTAs reach), whose partial tiles are summed in rank
@@ -47,10 +47,9 @@ struct msgfem_net {
 
 namespace {
 
-constexpr int GT = 32;    // output tile
-constexpr int GK = 64;    // K chunk
-
 enum { EPI_PLAIN = 0, EPI_BIAS_TANH = 1, EPI_BIAS = 2, EPI_DTANH = 3, EPI_MSE = 4 };
+
+constexpr int GK = 64;    // K chunk of a rank, and of a partial sum
 
 // C[m][n] = sum_k A(m, k) B(k, n) with A(m, k) = A[m lda + k] (or A[k lda + m]
 // when AT) and B(k, n) = B[k ldb + n] (or B[n ldb + k] when BT), followed by
@@ -58,17 +57,22 @@ enum { EPI_PLAIN = 0, EPI_BIAS_TANH = 1, EPI_BIAS = 2, EPI_DTANH = 3, EPI_MSE = 
 // with the leading dimension of C.  EPI_PLAIN also writes the sums of A over k
 // (the bias gradient) to gb; EPI_MSE stores scale (C + bias - H) and adds one
 // partial sum of the squared differences per CTA to part.
-// tn tiles along n; all output tiles lie along the grid's x (its other dimensions end at
-// 65,535).  A cluster of gridDim.z CTAs shares one output tile; rank z sums chunks
-// [z, z + 1) per of the inner dimension.
-template <bool AT, bool BT, int EPI>
+// GT x GT output tiles, GT / 16 squared outputs per thread; tn tiles along n, all tiles
+// along the grid's x (its other dimensions end at 65,535).
+// A cluster of gridDim.z CTAs shares one output tile; rank z sums chunks
+// [z, z + 1) per of the inner dimension.  Without a split a CTA of the larger tile adds
+// the same chunks, in the same order (the same bits up to 8 chunks).
+template <int GT, bool AT, bool BT, int EPI>
 __global__ void __launch_bounds__(256)
 k_gemm(int M, int N, int K, const float* __restrict__ A, int lda, const float* __restrict__ B, int ldb,
        float* __restrict__ C, int ldc, const float* __restrict__ bias, const float* __restrict__ H,
        float* __restrict__ gb, float scale, double* __restrict__ part, int tn) {
   namespace cg = cooperative_groups;
-  __shared__ float As[GK][GT + 1];
-  __shared__ float Bs[GK][GT + 1];
+  constexpr int R = GT / 16;             // outputs per thread and dimension
+  constexpr int KC = GT == 32 ? GK : 32;   // k staged at once
+  constexpr int LD = GT * KC / 256;      // loads per thread and operand
+  __shared__ float As[KC][GT + 1];
+  __shared__ float Bs[KC][GT + 1];
   __shared__ float Cs[GT][GT + 1];   // partial tile of this rank
   __shared__ float Ss[GT];           // sums of A over its chunks (EPI_PLAIN)
   __shared__ double red[8];
@@ -76,16 +80,15 @@ k_gemm(int M, int N, int K, const float* __restrict__ A, int lda, const float* _
   const int bx = blockIdx.x % tn, m0 = blockIdx.x / tn * GT, n0 = bx * GT;
   const int nch = (K + GK - 1) / GK, per = (nch + gridDim.z - 1) / gridDim.z;
   const int c0 = blockIdx.z * per, c1 = min(c0 + per, nch);
-  float acc[2][2] = {};
-  float asum = 0.f;
-  for (int c = c0; c < c1; ++c) {
-    const int k0 = c * GK;
-    float ra[8], rb[8];
+  float acc[R][R] = {}, sum[R][R] = {};
+  float asum = 0.f, atot = 0.f;
+  auto stage = [&](int k0) {   // KC of k
+    float ra[LD], rb[LD];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {   // every load of the chunk in flight at once
+    for (int i = 0; i < LD; ++i) {   // every load in flight at once
       const int e = tid + 256 * i;
-      const int am = AT ? e % GT : e / GK, ak = AT ? e / GT : e % GK;
-      const int bn = BT ? e / GK : e % GT, bk = BT ? e % GK : e / GT;
+      const int am = AT ? e % GT : e / KC, ak = AT ? e / GT : e % KC;
+      const int bn = BT ? e / KC : e % GT, bk = BT ? e % KC : e / GT;
       ra[i] = (m0 + am < M && k0 + ak < K)
                   ? (AT ? A[(size_t)(k0 + ak) * lda + m0 + am] : A[(size_t)(m0 + am) * lda + k0 + ak]) : 0.f;
       rb[i] = (n0 + bn < N && k0 + bk < K)
@@ -93,40 +96,61 @@ k_gemm(int M, int N, int K, const float* __restrict__ A, int lda, const float* _
     }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < LD; ++i) {
       const int e = tid + 256 * i;
-      if (AT) As[e / GT][e % GT] = ra[i]; else As[e % GK][e / GK] = ra[i];
-      if (BT) Bs[e % GK][e / GK] = rb[i]; else Bs[e / GT][e % GT] = rb[i];
+      if (AT) As[e / GT][e % GT] = ra[i]; else As[e % KC][e / KC] = ra[i];
+      if (BT) Bs[e % KC][e / KC] = rb[i]; else Bs[e / GT][e % GT] = rb[i];
     }
     __syncthreads();
 #pragma unroll 16
-    for (int kk = 0; kk < GK; ++kk) {
-      const float a0 = As[kk][ty], a1 = As[kk][ty + 16], b0 = Bs[kk][tx], b1 = Bs[kk][tx + 16];
-      acc[0][0] = fmaf(a0, b0, acc[0][0]);
-      acc[0][1] = fmaf(a0, b1, acc[0][1]);
-      acc[1][0] = fmaf(a1, b0, acc[1][0]);
-      acc[1][1] = fmaf(a1, b1, acc[1][1]);
+    for (int kk = 0; kk < KC; ++kk) {
+      float a[R], b[R];
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        a[i] = As[kk][ty + 16 * i];
+        b[i] = Bs[kk][tx + 16 * i];
+      }
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int j = 0; j < R; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
     }
     if (EPI == EPI_PLAIN && tid < GT)
-      for (int kk = 0; kk < GK; ++kk) asum += As[kk][tid];
+      for (int kk = 0; kk < KC; ++kk) asum += As[kk][tid];
+  };
+  for (int c = c0; c < c1; ++c) {
+    if constexpr (GT == 32) {
+      stage(c * GK);
+    } else {   // one CTA adds a long inner dimension: partial sums of GK terms
+      for (int k0 = c * GK; k0 < min(c * GK + GK, K); k0 += KC) stage(k0);
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+          sum[i][j] += acc[i][j];
+          acc[i][j] = 0.f;
+        }
+      atot += asum;
+      asum = 0.f;
+    }
   }
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+  for (int i = 0; i < R; ++i)
 #pragma unroll
-    for (int j = 0; j < 2; ++j) Cs[ty + 16 * i][tx + 16 * j] = acc[i][j];
-  if (EPI == EPI_PLAIN && tid < GT) Ss[tid] = asum;
-  // rank z finishes rows z, z + R, ... of the tile
+    for (int j = 0; j < R; ++j) Cs[ty + 16 * i][tx + 16 * j] = GT == 32 ? acc[i][j] : sum[i][j];
+  if (EPI == EPI_PLAIN && tid < GT) Ss[tid] = GT == 32 ? asum : atot;
+  // rank z finishes rows z, z + nr, ... of the tile
   cg::cluster_group cl = cg::this_cluster();
-  const int R = gridDim.z, z = blockIdx.z;
-  if (R > 1) cl.sync();
+  const int nr = gridDim.z, z = blockIdx.z;
+  if (nr > 1) cl.sync();
   else __syncthreads();
   double sq = 0.0;
   for (int e = tid; e < GT * GT; e += 256) {
     const int r = e / GT, cc = e % GT, gm = m0 + r, gn = n0 + cc;
-    if (r % R != z || gm >= M || gn >= N) continue;
+    if (r % nr != z || gm >= M || gn >= N) continue;
     float v = 0.f;
-    if (R > 1) {
-      for (int q = 0; q < R; ++q) v += *cl.map_shared_rank(&Cs[r][cc], q);
+    if (nr > 1) {
+      for (int q = 0; q < nr; ++q) v += *cl.map_shared_rank(&Cs[r][cc], q);
     } else {
       v = Cs[r][cc];
     }
@@ -145,7 +169,7 @@ k_gemm(int M, int N, int K, const float* __restrict__ A, int lda, const float* _
   }
   if (EPI == EPI_PLAIN && bx == 0 && z == 0 && tid < GT && m0 + tid < M) {
     float v = 0.f;
-    for (int q = 0; q < R; ++q) v += R > 1 ? *cl.map_shared_rank(&Ss[tid], q) : Ss[tid];
+    for (int q = 0; q < nr; ++q) v += nr > 1 ? *cl.map_shared_rank(&Ss[tid], q) : Ss[tid];
     gb[m0 + tid] = v;
   }
   if (EPI == EPI_MSE) {
@@ -155,10 +179,10 @@ k_gemm(int M, int N, int K, const float* __restrict__ A, int lda, const float* _
     if (tid == 0) {
       double t = 0.0;
       for (int w = 0; w < 8; ++w) t += red[w];
-      part[(size_t)blockIdx.x * R + z] = t;
+      part[(size_t)blockIdx.x * nr + z] = t;
     }
   }
-  if (R > 1) cl.sync();   // the partial tiles stay alive until every rank has read them
+  if (nr > 1) cl.sync();   // the partial tiles stay alive until every rank has read them
 }
 
 // loss = sum of the partials / n (fixed order: deterministic)
@@ -189,27 +213,49 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
   }
 }
 
-// CTAs that split the inner dimension: one chunk each, at most 8 (a portable cluster)
-int split_of(int K) { return std::min(8, (K + GK - 1) / GK); }
+// Output tile, and CTAs that split the inner dimension, of an M x N x K product
+struct GemmShape {
+  int tile, split;
+  long long tiles(int M, int N) const { return (long long)((M + tile - 1) / tile) * ((N + tile - 1) / tile); }
+};
 
-template <bool AT, bool BT, int EPI>
-void gemm(cudaStream_t st, int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C, int ldc,
-          const float* bias = nullptr, const float* H = nullptr, float* gb = nullptr, float scale = 0.f,
-          double* part = nullptr) {
-  cudaLaunchConfig_t cfg = {};
+// 32 x 32 tiles, one chunk of the inner dimension per CTA of a cluster as far as 8 reach;
+// from 128 tiles of 64 x 64 on those, without a split: four outputs per shared read instead
+// of one, and the chip is full without it.  One layer's forward pass, us, 32 / 64: 128
+// tiles with K = 512, 1,024, 4,096: 45 / 31, 78 / 56, 283 / 203; 256 with 64, 512, 1,024:
+// 14.6 / 12.6, 82 / 51, 148 / 95; 512 with 4,096: 1,091 / 731; but 64 with 512: 27 / 31, 16
+// with 1,024: 19 / 56.  Not where the larger tiles are half empty (65,536 x 32: 22.9 / 23.8).
+GemmShape gemm_shape(int M, int N, int K) {
+  const GemmShape small = {32, std::min(8, (K + GK - 1) / GK)}, large = {64, 1};
+  return large.tiles(M, N) >= 128 && small.tiles(M, N) >= 3 * large.tiles(M, N) ? large : small;
+}
+
+template <int GT, bool AT, bool BT, int EPI>
+void gemm_tile(cudaStream_t st, int split, int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C,
+               int ldc, const float* bias, const float* H, float* gb, float scale, double* part) {
   const int tn = (N + GT - 1) / GT, tm = (M + GT - 1) / GT;
-  cfg.gridDim = dim3(tn * tm, 1, split_of(K));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(tn * tm, 1, split);
   cfg.blockDim = dim3(256);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 1;
   at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = cfg.gridDim.z;
+  at[0].val.clusterDim.z = split;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_gemm<AT, BT, EPI>, M, N, K, A, lda, B, ldb, C, ldc, bias, H, gb, scale, part, tn);
+  cudaLaunchKernelEx(&cfg, k_gemm<GT, AT, BT, EPI>, M, N, K, A, lda, B, ldb, C, ldc, bias, H, gb, scale, part, tn);
   ++g_launch_count;
+}
+
+template <bool AT, bool BT, int EPI>
+void gemm(cudaStream_t st, int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C, int ldc,
+          const float* bias = nullptr, const float* H = nullptr, float* gb = nullptr, float scale = 0.f,
+          double* part = nullptr) {
+  const GemmShape g = gemm_shape(M, N, K);
+  auto run = g.tile == 32 ? gemm_tile<32, AT, BT, EPI> : gemm_tile<64, AT, BT, EPI>;
+  run(st, g.split, M, N, K, A, lda, B, ldb, C, ldc, bias, H, gb, scale, part);
 }
 
 // forward pass up to layer `layers`; the last layer's output goes to Y (or the
@@ -237,7 +283,8 @@ void gradient(msgfem_net* n, const float* X, const float* T, int B, bool want_lo
   gemm<false, true, EPI_MSE>(n->st, B, dout, din, hl, din, n->p + n->woff[n->L - 1], din, n->d1, dout,
                              n->p + n->boff[n->L - 1], T, nullptr, 2.f / (float)cnt, n->part);
   if (want_loss) {
-    const int np = ((dout + GT - 1) / GT) * ((B + GT - 1) / GT) * split_of(din);
+    const GemmShape g = gemm_shape(B, dout, din);
+    const int np = (int)(g.tiles(B, dout) * g.split);
     k_loss_final<<<1, 256, 0, n->st>>>(n->part, np, cnt, n->loss);
     ++g_launch_count;
   }
@@ -285,8 +332,10 @@ msgfem_status msgfem_net_create(int n_sizes, const int* sizes, int max_batch, co
   }
   for (int i = 0; i < n_sizes; ++i) wmax = sizes[i] > wmax ? sizes[i] : wmax;
   n->np = off;
-  // partial sums of the loss: one per output-layer CTA of the largest batch
-  const size_t loss_parts = (size_t)((sizes[n->L] + GT - 1) / GT) * ((max_batch + GT - 1) / GT) * split_of(sizes[n->L - 1]);
+  // partial sums of the loss: one per output-layer CTA, the most that a batch up to the
+  // largest has (the smaller tiles and their split)
+  const GemmShape small = {32, std::min(8, (sizes[n->L - 1] + GK - 1) / GK)};
+  const size_t loss_parts = (size_t)small.tiles(max_batch, sizes[n->L]) * small.split;
   n->act.assign(n->L + 1, nullptr);
   bool good = ok(cudaMalloc(&n->p, off * sizeof(float))) && ok(cudaMalloc(&n->g, off * sizeof(float))) &&
               ok(cudaMalloc(&n->m, off * sizeof(float))) && ok(cudaMalloc(&n->v, off * sizeof(float))) &&
