@@ -36,7 +36,7 @@ struct msgfem_net {
   float* g = nullptr;              // gradient
   float* m = nullptr;              // Adam moments
   float* v = nullptr;
-  std::vector<float*> act;         // act[l], l = 1..L-1: hidden outputs [bmax][sizes[l]]; act[L]: output
+  std::vector<float*> act;         // act[l], l = 1..L-1: hidden outputs [bmax][sizes[l]]
   float* d1 = nullptr;             // back-propagated gradients [bmax][max width] (ping-pong)
   float* d2 = nullptr;
   double* part = nullptr;          // loss partial sums
@@ -258,8 +258,7 @@ void gemm(cudaStream_t st, int M, int N, int K, const float* A, int lda, const f
   run(st, g.split, M, N, K, A, lda, B, ldb, C, ldc, bias, H, gb, scale, part);
 }
 
-// forward pass up to layer `layers`; the last layer's output goes to Y (or the
-// handle's output buffer when Y is null)
+// forward pass up to layer `layers`; the last layer's output goes to Y
 void forward(msgfem_net* n, const float* X, int B, float* Y, int layers) {
   const float* h = X;
   for (int l = 0; l < layers; ++l) {
@@ -267,7 +266,7 @@ void forward(msgfem_net* n, const float* X, int B, float* Y, int layers) {
     const float* W = n->p + n->woff[l];
     const float* b = n->p + n->boff[l];
     const bool last = l + 1 == n->L;
-    float* o = last ? (Y ? Y : n->act[n->L]) : n->act[l + 1];
+    float* o = last ? Y : n->act[l + 1];
     if (last) gemm<false, true, EPI_BIAS>(n->st, B, out, in, h, in, W, in, o, out, b);
     else gemm<false, true, EPI_BIAS_TANH>(n->st, B, out, in, h, in, W, in, o, out, b);
     h = o;
@@ -336,13 +335,13 @@ msgfem_status msgfem_net_create(int n_sizes, const int* sizes, int max_batch, co
   // largest has (the smaller tiles and their split)
   const GemmShape small = {32, std::min(8, (sizes[n->L - 1] + GK - 1) / GK)};
   const size_t loss_parts = (size_t)small.tiles(max_batch, sizes[n->L]) * small.split;
-  n->act.assign(n->L + 1, nullptr);
+  n->act.assign(n->L, nullptr);
   bool good = ok(cudaMalloc(&n->p, off * sizeof(float))) && ok(cudaMalloc(&n->g, off * sizeof(float))) &&
               ok(cudaMalloc(&n->m, off * sizeof(float))) && ok(cudaMalloc(&n->v, off * sizeof(float))) &&
               ok(cudaMalloc(&n->d1, (size_t)max_batch * wmax * sizeof(float))) &&
               ok(cudaMalloc(&n->d2, (size_t)max_batch * wmax * sizeof(float))) &&
               ok(cudaMalloc(&n->part, loss_parts * sizeof(double))) && ok(cudaMalloc(&n->loss, sizeof(double)));
-  for (int l = 1; good && l <= n->L; ++l) good = ok(cudaMalloc(&n->act[l], (size_t)max_batch * sizes[l] * sizeof(float)));
+  for (int l = 1; good && l < n->L; ++l) good = ok(cudaMalloc(&n->act[l], (size_t)max_batch * sizes[l] * sizeof(float)));
   if (!good) {
     msgfem_net_destroy(n);
     return MSGFEM_ENOMEM;
