@@ -1680,16 +1680,15 @@ constexpr int INV_SMEM = 225 * 1024;   // shared memory of one solve CTA
 // and from 65,000 on pivots turn non-positive where the block Cholesky's do not.
 constexpr float INV_COND_A11 = 1e3f, INV_COND_K = 1e5f, INV_COND_F32 = 5e4f;
 
-template <typename T>
-const void* solve_kernel_ptr(int rs, bool back) {
-  if (rs == 8) return back ? (const void*)k_inv_solve<T, 8, true> : (const void*)k_inv_solve<T, 8, false>;
-  return back ? (const void*)k_inv_solve<T, 4, true> : (const void*)k_inv_solve<T, 4, false>;
+template <typename T, int RS>
+const void* solve_kernel_ptr(bool back) {
+  return back ? (const void*)k_inv_solve<T, RS, true> : (const void*)k_inv_solve<T, RS, false>;
 }
 const void* solve_kernel(const msgfem* h, const InvForm& f, const InvForm::Solve& s, bool back) {
   if (s.rows32) return back ? (const void*)k_inv_solve_f32<true> : (const void*)k_inv_solve_f32<false>;
   if (f.digits) return back ? (const void*)k_inv_solve_fx<true> : (const void*)k_inv_solve_fx<false>;
-  const int rs = f.rs;
-  return h->mixed ? solve_kernel_ptr<float>(rs, back) : solve_kernel_ptr<double>(rs, back);
+  if (!h->mixed) return solve_kernel_ptr<double, 4>(back);
+  return f.rs == 8 ? solve_kernel_ptr<float, 8>(back) : solve_kernel_ptr<float, 4>(back);
 }
 
 int solve_threads(const InvForm& f) { return f.digits ? 32 * FX_WARPS : 256; }
@@ -1867,8 +1866,8 @@ bool inv_create(msgfem* h) {
       f->mats.push_back(m);
     }
   }
-  const int row = bmax * es;
-  f->rs = row <= 6144 ? 8 : 4;
+  // rows of at most 6 KiB: eight per stage (in FP64 those layers all take the digit products)
+  f->rs = h->mixed && bmax * es <= 6144 ? 8 : 4;
   // two stages of the widest layer and its vectors must fit with the widest cluster
   InvForm::Solve probe;
   for (int i = 0; i < (int)f->mats.size(); ++i)
@@ -1895,11 +1894,9 @@ void inv_destroy(msgfem* h) {
 msgfem_status inv_build(msgfem* h) {
   InvForm& f = *h->inv;
   // shared-memory limits (of the current device)
-  for (int rs : {4, 8})
-    for (bool back : {false, true}) {
-      CK(cudaFuncSetAttribute(solve_kernel_ptr<float>(rs, back), cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
-      CK(cudaFuncSetAttribute(solve_kernel_ptr<double>(rs, back), cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
-    }
+  for (bool back : {false, true})
+    for (const void* k : {solve_kernel_ptr<float, 8>(back), solve_kernel_ptr<float, 4>(back), solve_kernel_ptr<double, 4>(back)})
+      CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, INV_SMEM));
   CK(cudaFuncSetAttribute(k_inv_step<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, inv_step_smem<double>()));
   CK(cudaFuncSetAttribute(k_inv_step<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, inv_step_smem<float>()));
   for (const void* k : {(const void*)k_inv_solve_f32<false>, (const void*)k_inv_solve_f32<true>})
