@@ -294,7 +294,8 @@ typedef struct {
                                     (padding, whole diagonal tiles and inverses included) */
 } msgfem_profile;
 
-/* Launch shapes chosen by msgfem_autotune and what it measured. */
+/* Launch shapes of the block Cholesky chosen by msgfem_autotune, what it measured, and whether
+ * the handle keeps the inverse form instead. */
 typedef struct {
   int factor_schedule;  /* msgfem_options.factor_schedule chosen */
   int factor_streams;   /* stream groups of the factorisation schedules chosen (16 or 32) */
@@ -316,6 +317,13 @@ typedef struct {
   int factor_persistent;       /* msgfem_options.factor_persistent chosen (mixed precision) */
   double factor_ms_persistent[2];   /* the persistent FMA factorisation, [right-, left-looking];
                                        -1 = not run */
+  int inverse_form;            /* 1: the handle keeps inverses of the Schur complements (msgfem_profile).
+                                  The choices above, of the block Cholesky, then stand by for calls that
+                                  go over to it; they are not for the options of the next handle, where a
+                                  Cholesky schedule, tile kernel or solve kernel switches the inverse form
+                                  off: leave those at 0 there */
+  double inverse_ms[2];        /* the inverse form on the measured wave: its factorisation, one application
+                                  of the operator; -1 = not run */
 } msgfem_tuning;
 
 /* Per-subdomain diagnostics filled by msgfem_get_info. */

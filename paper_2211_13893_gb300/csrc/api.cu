@@ -1928,6 +1928,7 @@ static msgfem_status autotune_run(msgfem_h h, int reps, msgfem_tuning* out) {
   };
   t.tc_factor_diff = -1.0;
   t.fma_factor_diff = -1.0;
+  t.inverse_ms[0] = t.inverse_ms[1] = -1.0;
   for (int fv = 0; fv < 2; ++fv) {
     t.factor_ms_persistent[fv] = -1.0;
     for (int gi = 0; gi < 2; ++gi) t.factor_ms[fv][gi] = t.factor_ms_tc[fv][gi] = -1.0;
@@ -2107,6 +2108,8 @@ static msgfem_status autotune_run(msgfem_h h, int reps, msgfem_tuning* out) {
     CK_LAUNCH();
     CK(cudaEventElapsedTime(&fms, f0, f1));
     CK(cudaEventElapsedTime(&oms, e0, e1));
+    t.inverse_ms[0] = fms;
+    t.inverse_ms[1] = oms / reps;
     h->inv_use = fms + 10.0 * oms / reps <= best_fms + 10.0 * best;
   }
   h->inv_on = h->inv_use;
@@ -2138,6 +2141,7 @@ static msgfem_status autotune_run(msgfem_h h, int reps, msgfem_tuning* out) {
   t.streams = best_g;
   t.solve_kernel = best_v;
   t.best_ms = best;
+  t.inverse_form = h->inv_use ? 1 : 0;
   if (out) *out = t;
   return MSGFEM_OK;
 }

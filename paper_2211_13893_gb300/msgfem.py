@@ -74,7 +74,8 @@ class Tuning(C.Structure):
                 ("solve_ms", (C.c_double * 4) * 4), ("factor_kernel", C.c_int),
                 ("factor_ms_tc", (C.c_double * 2) * 2), ("tc_factor_diff", C.c_double),
                 ("fma_factor_diff", C.c_double), ("factor_persistent", C.c_int),
-                ("factor_ms_persistent", C.c_double * 2)]
+                ("factor_ms_persistent", C.c_double * 2), ("inverse_form", C.c_int),
+                ("inverse_ms", C.c_double * 2)]
 
 
 class Profile(C.Structure):
@@ -407,7 +408,8 @@ class MSGFEM:
                 "factor_ms_tc": [[t.factor_ms_tc[f][g] for g in range(2)] for f in range(2)],
                 "tc_factor_diff": t.tc_factor_diff, "fma_factor_diff": t.fma_factor_diff,
                 "factor_persistent": t.factor_persistent,
-                "factor_ms_persistent": [t.factor_ms_persistent[f] for f in range(2)]}
+                "factor_ms_persistent": [t.factor_ms_persistent[f] for f in range(2)],
+                "inverse_form": t.inverse_form, "inverse_ms": [t.inverse_ms[f] for f in range(2)]}
 
     def schwarz_solve(self, coarse=None, b=None, u0=None, rtol=0.0, max_iter=0, u_out=None, allow_noconv=False):
         """Two-level additive Schwarz PCG for the fine problem (include/msgfem.h

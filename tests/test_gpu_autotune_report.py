@@ -32,3 +32,22 @@ def test_executed_flops_after_autotune(precision, waves):
     assert np.isfinite(after["factor_flops_executed"])
     m.close()
     chol.close()
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(precision=1), dict(solve_kernel=2)])
+def test_tuning_names_the_form(kw):
+    """msgfem_tuning.inverse_form is the form of the next local stage, with both forms'
+    times; a handle set up by a Cholesky kernel measures the block Cholesky only."""
+    from paper_2211_13893_gb300 import MSGFEM
+    cfg = replace(get_config("t3"), NX=25, NY=7, NZ=8, sx=3, sy=2, overlap=2, oversampling=3, n_loc=9)
+    m = MSGFEM.from_config(cfg, element_angles(cfg), seed=7, **kw)
+    m.local_spaces(cfg.n_loc)
+    t = m.autotune(reps=1)
+    m.local_spaces(cfg.n_loc)
+    p = m.profile()
+    # (only the inverse form counts no separate inverses of diagonal factors)
+    assert t["inverse_form"] == (1 if p["factor_flops_inverse"] == p["factor_flops"] else 0)
+    assert all((v > 0.0) == ("solve_kernel" not in kw) for v in t["inverse_ms"])
+    if t["inverse_form"]:
+        assert t["inverse_ms"][1] > 0.0 and t["inverse_ms"][0] > 0.0
+    m.close()
