@@ -250,7 +250,7 @@ struct msgfem {
   int factor_tc = 0;                 // FP32 factorisation on the tensor cores (msgfem_options.factor_kernel)
   void* d_tc_maps = nullptr;         // device tensor maps of every subdomain's FP32 arrays (4 per subdomain)
   void* d_solve_maps = nullptr;      // the same arrays in 64 x 64 unswizzled boxes (TMA solve stages)
-  int* d_kerr = nullptr;             // set by a TMA solve stage that did not arrive in time
+  int* d_kerr = nullptr;             // KERR_* of a bounded wait that ran out
   int potrf_fp64 = 0;                // mixed: FP64 tile Cholesky after an FP32 one met a bad pivot
   InvForm* inv = nullptr;            // inverse form, when the handle is eligible
   bool inv_use = false;              // factorisations start in the inverse form (eligible, and kept by the autotuner)
@@ -362,6 +362,9 @@ enum { SOLVE_DEFAULT = 0, SOLVE_ASYNC_RING = 1, SOLVE_STREAM = 2, SOLVE_STREAM_C
 void set_solve_maps(const void* maps, int* err);
 msgfem_status solve_maps_build(msgfem* h);
 // MSGFEM_ECUDA (and the flag cleared) when a TMA solve stage reported a failure
+// what a bounded wait on the device waited for in vain (d_kerr), and its message (setup.cpp)
+enum { KERR_TMA_STAGE = 1, KERR_PERSISTENT = 2, KERR_SOLVE_COPY = 3 };
+const char* stage_error_text(int e);
 msgfem_status check_stage_error(msgfem* h);
 // allocate (once) and clear the device error flag of bounded waits (k_dense.cu)
 msgfem_status kerr_ensure(msgfem* h);

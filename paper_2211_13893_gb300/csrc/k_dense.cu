@@ -423,7 +423,7 @@ k_factor_persistent(const TileTaskT<float>* __restrict__ tasks, const int4* __re
     const int t = s_t;
     if (t >= ntask) return;
     if (!s_ok) {
-      if (threadIdx.x == 0) atomicExch(err, 2);
+      if (threadIdx.x == 0) atomicExch(err, KERR_PERSISTENT);
       return;
     }
     const int4 mt = meta[t];
@@ -1017,7 +1017,7 @@ k_solve_tma(const SolveTaskT<float>* __restrict__ tasks, const SubDev* __restric
     // a stage did not arrive: wait once more (bounded) for every copy issued, then report
     if (tid == 0) {
       for (int i = waited; i < issued; ++i) tc::mbar_wait(bar0 + 8 * (i % ASYNC_DEPTH), (i / ASYNC_DEPTH) & 1);
-      if (err != nullptr) atomicExch(err, 1);
+      if (err != nullptr) atomicExch(err, KERR_TMA_STAGE);
     }
     __syncthreads();
   }
@@ -1202,8 +1202,7 @@ msgfem_status check_stage_error(msgfem* h) {
   CK(cudaMemcpy(&e, h->d_kerr, sizeof(int), cudaMemcpyDeviceToHost));
   if (e == 0) return MSGFEM_OK;
   CK(cudaMemset(h->d_kerr, 0, sizeof(int)));
-  h->err = e == 2 ? "a task of the persistent factorisation waited more than two seconds for its predecessors"
-                  : "a tensor-memory-accelerator solve stage failed its slab check or did not arrive within a second";
+  h->err = stage_error_text(e);
   return MSGFEM_ECUDA;
 }
 

@@ -985,7 +985,7 @@ k_inv_solve(const InvSolveArgs a) {
     // a copy did not arrive within its limit: wait once more for those in flight, then report
     for (int i = waited; i < issued; ++i) tc::mbar_wait(bar0 + 8 * (i % a.ring), (i / a.ring) & 1);
     if (cphase > 0) tc::mbar_wait(bar0 + 64, (cphase - 1) & 1);
-    if (a.err != nullptr) atomicExch(a.err, 1);
+    if (a.err != nullptr) atomicExch(a.err, KERR_SOLVE_COPY);
   }
 }
 
@@ -1320,7 +1320,7 @@ k_inv_solve_f32(const InvSolveArgs a) {
       for (int i = max(0, issued - rg.depth); i < issued; ++i)
         tc::mbar_wait(rg.bar + 8 * (i % rg.depth), (i / rg.depth) & 1);
     if (tid == 0 && cphase > 0) tc::mbar_wait(cbar, (cphase - 1) & 1);
-    if (tid == 0 && a.err != nullptr) atomicExch(a.err, 1);
+    if (tid == 0 && a.err != nullptr) atomicExch(a.err, KERR_SOLVE_COPY);
   }
 }
 
@@ -1627,7 +1627,7 @@ k_inv_solve_fx(const InvSolveArgs a) {
     if (lane == 0)
       for (int i = max(0, issued - depth); i < issued; ++i) tc::mbar_wait(wbar + 8 * (i % depth), (i / depth) & 1);
     if (tid == 0 && cphase > 0) tc::mbar_wait(cbar, (cphase - 1) & 1);
-    if (tid == 0 && a.err != nullptr) atomicExch(a.err, 1);
+    if (tid == 0 && a.err != nullptr) atomicExch(a.err, KERR_SOLVE_COPY);
   }
 }
 

@@ -917,6 +917,14 @@ void build_coarse_schedules(msgfem* h) {
   flatten_solve(keys, h->csolve);
 }
 
+const char* stage_error_text(int e) {
+  switch (e) {
+    case KERR_PERSISTENT: return "a task of the persistent factorisation waited more than two seconds for its predecessors";
+    case KERR_SOLVE_COPY: return "a bulk copy of a block solve with inverse Schur complements did not arrive within a second";
+    default: return "a tensor-memory-accelerator solve stage failed its slab check or did not arrive within a second";
+  }
+}
+
 // Memory plan of a problem on the host (no handle, no CUDA call): the same
 // decomposition as msgfem_setup, the storage of every subdomain and the waves.
 extern "C" msgfem_status msgfem_plan(const msgfem_mesh* mesh, const msgfem_partition* part, int overlap,

@@ -765,4 +765,7 @@ int hc_merge_steps(void* p, int which, int g, int s) {
   return 0;
 }
 
+// message of a bounded wait that ran out
+const char* hc_stage_error_text(int e) { return stage_error_text(e); }
+
 }  // extern "C"
