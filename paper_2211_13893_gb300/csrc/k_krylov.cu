@@ -427,8 +427,8 @@ __device__ __forceinline__ double rr_rsqrt(double w) {
 
 __global__ void __launch_bounds__(512)
 k_rr_jacobi(const SubDev* __restrict__ subs, const int* __restrict__ active, const int* __restrict__ mvec,
-            const int* __restrict__ nwvec, RrWork wk, int first) {
-  const int sidx = first + blockIdx.x;
+            const int* __restrict__ nwvec, RrWork wk) {
+  const int sidx = blockIdx.x;
   if (active != nullptr && !active[sidx]) return;
   const SubDev& s = subs[sidx];
   const int m = mvec[sidx], nw = nwvec[sidx];
@@ -438,9 +438,9 @@ k_rr_jacobi(const SubDev* __restrict__ subs, const int* __restrict__ active, con
   __shared__ double d[MQ], id[MQ], al[MQ / 2], be[MQ / 2];
   __shared__ int pa[MQ / 2], pb[MQ / 2];
   __shared__ double red_off[16], red_tot[16];
-  __shared__ int again, bad;
+  __shared__ int again;
   const int tid = threadIdx.x, np = m / 2;      // m is a multiple of KB
-  float* log = wk.log + (size_t)blockIdx.x * RR_ROUNDS * (MQ / 2);
+  float* log = wk.log + (size_t)sidx * RR_ROUNDS * (MQ / 2);
   for (int e = tid; e < m * m; e += 512) {
     const int r = e / m, c = e % m;
     if (c <= r) A[r][c] = 0.5 * (s.H[(size_t)r * MQ + c] + s.H[(size_t)c * MQ + r]);
@@ -471,7 +471,6 @@ k_rr_jacobi(const SubDev* __restrict__ subs, const int* __restrict__ active, con
       double so = 0.0, st = 0.0;
       for (int w = 0; w < 16; ++w) { so += red_off[w]; st += red_tot[w]; }
       again = so > 1e-30 * st;
-      bad = !(st <= 1.7e308);   // an operator with a NaN or an infinity has no Ritz pairs
     }
     __syncthreads();
     if (!again) break;
@@ -527,7 +526,12 @@ k_rr_jacobi(const SubDev* __restrict__ subs, const int* __restrict__ active, con
   if (tid < m) {
     int rank = 0;
     for (int j = 0; j < m; ++j) rank += (mu[j] > mu[tid] || (mu[j] == mu[tid] && j < tid)) ? 1 : 0;
-    if (bad) rank = tid;   // every rank is written: none keeps an earlier call's value
+    // an operator with a NaN or an infinity has no Ritz pairs: every rank is written (none
+    // keeps an earlier call's value) as invalid
+    double mass = 0.0;
+    for (int w = 0; w < 16; ++w) mass += red_tot[w];
+    const bool bad = !(mass <= 1.7e308);
+    if (bad) rank = tid;
     if (rank < nw && rank < PST) {
       wk.perm[sidx * PST + rank] = tid;
       wk.mu[sidx * PST + rank] = bad ? NAN : mu[tid];
@@ -540,8 +544,8 @@ constexpr int RR_CHUNK = 32;   // rounds whose rotations are staged at once
 
 __global__ void __launch_bounds__(4 * (MQ / 2))
 k_rr_vectors(const SubDev* __restrict__ subs, const int* __restrict__ active, const int* __restrict__ mvec,
-             const int* __restrict__ nwvec, RrWork wk, int first) {
-  const int sidx = first + blockIdx.y;
+             const int* __restrict__ nwvec, RrWork wk) {
+  const int sidx = blockIdx.y;
   if (active != nullptr && !active[sidx]) return;
   const SubDev& s = subs[sidx];
   const int m = mvec[sidx], nw = nwvec[sidx];
@@ -553,7 +557,7 @@ k_rr_vectors(const SubDev* __restrict__ subs, const int* __restrict__ active, co
   const int src = live ? wk.perm[sidx * PST + col] : -1;
   for (int a = k; a < MQ; a += MQ / 2) x[a][c] = (a == src) ? 1.0 : 0.0;
   if (blockIdx.x * 4 < nw) {
-    const float* log = wk.log + (size_t)blockIdx.y * RR_ROUNDS * (MQ / 2);
+    const float* log = wk.log + (size_t)sidx * RR_ROUNDS * (MQ / 2);
     // V e = J_1 (J_2 ( ... J_n e)), each round's disjoint rotations at once
     for (int r1 = wk.rounds[sidx]; r1 > 0; r1 -= RR_CHUNK) {
       const int r0 = max(0, r1 - RR_CHUNK);
@@ -778,11 +782,15 @@ void launch_rr_krylov(msgfem* h, const int* d_m, const int* d_nw) {
   wk.log = reinterpret_cast<float*>(wk.mu + (size_t)h->N * PST);
   wk.perm = reinterpret_cast<int*>(wk.log + (size_t)std::min(h->N, RR_BATCH) * RR_ROUNDS * (MQ / 2));
   wk.rounds = wk.perm + (size_t)h->N * PST;
-  for (int first = 0; first < h->N; first += RR_BATCH) {
+  for (int first = 0; first < h->N; first += RR_BATCH) {   // the arrays from the batch's first subdomain on
     const int n = std::min(RR_BATCH, h->N - first);
-    k_rr_jacobi<<<n, 512, smem, h->stream>>>(h->d_sub, h->d_flags, d_m, d_nw, wk, first);
-    k_rr_vectors<<<dim3(PST / 4, n), 4 * (MQ / 2), 0, h->stream>>>(h->d_sub, h->d_flags, d_m, d_nw, wk, first);
+    k_rr_jacobi<<<n, 512, smem, h->stream>>>(h->d_sub + first, h->d_flags + first, d_m + first, d_nw + first, wk);
+    k_rr_vectors<<<dim3(PST / 4, n), 4 * (MQ / 2), 0, h->stream>>>(h->d_sub + first, h->d_flags + first, d_m + first,
+                                                                  d_nw + first, wk);
     g_launch_count += 2;
+    wk.mu += (size_t)RR_BATCH * PST;
+    wk.perm += (size_t)RR_BATCH * PST;
+    wk.rounds += RR_BATCH;
   }
 }
 
