@@ -355,7 +355,8 @@ def run_ours(args):
         dom, achieved, share = "k_tile_task<double> (layer-block Cholesky tile tasks)", fact_tf, prof["factor_ms"] / total_ms
     roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak, "traffic": None if inverse else NCU_TRAFFIC.get(args.config), "kernel": dom,
-            "traffic_note": "bytes per factorisation graph replay (one per step), from an ncu capture on p2 scaled "
+            "traffic_note": None if inverse else
+                            "bytes per factorisation graph replay (one per step), from an ncu capture on p2 scaled "
                             "to the workload's subdomains",
             "peak_note": "FP64 as 28 exact FP16 digit products: 152 SMs x 956 / 28 FMA/clk (measured mma.sync rate) x 2 "
                          "flop x 2070 MHz" if inverse else
