@@ -209,8 +209,9 @@ typedef struct {
      returns device memory of the current device, at least 256-byte aligned, or NULL
      (ENOMEM); dev_free(p, bytes, alloc_ctx) takes back a block (bytes as allocated).  Both
      are called on the thread of the API call, during msgfem_setup, msgfem_update_angles,
-     msgfem_local_spaces, msgfem_autotune, msgfem_get_basis and msgfem_destroy; the
-     library synchronises its stream before it frees a block.  Both NULL: cudaMalloc and
+     msgfem_local_spaces, msgfem_import_local, msgfem_coarse_assemble, msgfem_schwarz_solve,
+     msgfem_autotune, msgfem_get_basis, msgfem_export_local and msgfem_destroy; the library
+     synchronises its stream before it frees a block.  Both NULL: cudaMalloc and
      cudaFree.  One of them NULL: EINVAL.  (The network handles of msgfem_warm.h and the
      fixed scratch array of msgfem_energy_error_noalloc do not use them.) */
   void* (*dev_alloc)(size_t bytes, void* alloc_ctx);
