@@ -248,12 +248,14 @@ msgfem_status schwarz_run(msgfem_h hl, msgfem_h hc, const double* b_in, const do
   const int nclamp = 3 * (NY + 1) * (NZ + 1);
   if (hc) CK(cudaStreamSynchronize(hc->stream));   // the coarse handle's own work is complete
   TRY(schwarz_factors(h));
+  void* buf = nullptr;
   if (h->d_pcg_vec == nullptr) {
-    void* p = nullptr;
-    TRY(dev_alloc_bytes(h, &p, (size_t)6 * ndof * sizeof(double)));
-    h->d_pcg_vec = static_cast<double*>(p);
-    TRY(dev_alloc_bytes(h, &p, (size_t)2 * DOT_BLOCKS * sizeof(double)));
-    h->d_pcg_part = static_cast<double*>(p);
+    TRY(dev_alloc_bytes(h, &buf, (size_t)6 * ndof * sizeof(double)));
+    h->d_pcg_vec = static_cast<double*>(buf);
+  }
+  if (h->d_pcg_part == nullptr) {
+    TRY(dev_alloc_bytes(h, &buf, (size_t)2 * DOT_BLOCKS * sizeof(double)));
+    h->d_pcg_part = static_cast<double*>(buf);
   }
   double* x = h->d_pcg_vec;
   double* r = x + ndof;

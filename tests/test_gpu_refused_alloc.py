@@ -139,3 +139,25 @@ def test_update_angles():
             break
         at += 1
     assert at >= 2
+
+
+@pytest.mark.parametrize("kw", [dict(), dict(precision=1)])
+def test_schwarz_solve(kw):
+    from paper_2211_13893_gb300 import MSGFEM
+    cfg = get_config("t2")
+    cfg = replace(cfg, oversampling=cfg.overlap)
+    ang = element_angles(cfg)
+    ref = MSGFEM.from_config(cfg, ang, seed=5, **kw)
+    want, _ = ref.schwarz_solve()
+    ref.close()
+    mem = Refusing()
+    at = 0
+    while True:
+        m = MSGFEM.from_config(cfg, ang, seed=5, allocator=(mem.alloc, mem.free), **kw)
+        met = mem.refuse(at, m.schwarz_solve)
+        assert np.array_equal(m.schwarz_solve()[0], want)
+        m.close()
+        if not met:
+            break
+        at += 1
+    assert at >= 2
