@@ -1662,7 +1662,7 @@ struct InvForm {
   std::vector<SchedStep> csteps;
   int rs = 8;                      // rows per stage of the solves (by the widest layer and the type)
   bool digits = false;             // FP64: solves in digit products (k_inv_solve_fx)
-  int* d_cond = nullptr;           // [2 N + 2] conditioning of the matrices' Schur complements (float bits)
+  int* d_cond = nullptr;           // [2 N] conditioning of the matrices' Schur complements (float bits)
 };
 
 namespace {
@@ -1912,7 +1912,7 @@ msgfem_status inv_build(msgfem* h) {
   TRY(dev_alloc_bytes(h, &p, f.mats.size() * sizeof(InvMat)));
   f.d_mats = static_cast<InvMat*>(p);
   CK(cudaMemcpy(f.d_mats, f.mats.data(), f.mats.size() * sizeof(InvMat), cudaMemcpyHostToDevice));
-  TRY(dev_alloc_bytes(h, &p, (2 * (size_t)h->N + 2) * sizeof(int)));
+  TRY(dev_alloc_bytes(h, &p, 2 * (size_t)h->N * sizeof(int)));
   f.d_cond = static_cast<int*>(p);
   TRY(kerr_ensure(h));
   f.waves.resize(h->waves.size());
