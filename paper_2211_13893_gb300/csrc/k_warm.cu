@@ -173,8 +173,8 @@ msgfem_status warm_check(msgfem* h, std::vector<int>& bad) {
 // B2 row lists (ascending full-layout rows of the interface DoFs), built once
 msgfem_status warm_rows(msgfem* h) {
   if ((int)h->d_b2rows.size() == h->N) return MSGFEM_OK;
-  h->d_b2rows.assign(h->N, nullptr);
-  for (int j = 0; j < h->N; ++j) {
+  // (a call that ended early left the lists built so far: the next goes on from there)
+  for (int j = (int)h->d_b2rows.size(); j < h->N; ++j) {
     const SubDev& s = h->sub[j];
     std::vector<int> rows;
     for (int n = 0; n < s.nnode; ++n)
@@ -188,7 +188,7 @@ msgfem_status warm_rows(msgfem* h) {
     TRY(dev_alloc_bytes(h, &buf, std::max<size_t>(1, rows.size()) * sizeof(int)));
     int* d = static_cast<int*>(buf);
     if (!rows.empty()) CK(cudaMemcpy(d, rows.data(), rows.size() * sizeof(int), cudaMemcpyHostToDevice));
-    h->d_b2rows[j] = d;
+    h->d_b2rows.push_back(d);
   }
   return MSGFEM_OK;
 }

@@ -161,3 +161,53 @@ def test_schwarz_solve(kw):
             break
         at += 1
     assert at >= 2
+
+
+def test_start_block():
+    import torch
+    from paper_2211_13893_gb300 import MSGFEM
+    cfg = get_config("t2")
+    ang = element_angles(cfg)
+    mem = Refusing()
+    at, want = 0, None
+    while True:
+        m = MSGFEM.from_config(cfg, ang, seed=5, allocator=(mem.alloc, mem.free))
+        m.local_spaces(cfg.n_loc)
+        n2, _ = m.warm_sizes(m.N - 1, cfg.n_loc)
+        block = torch.zeros((n2, 8), dtype=torch.float32, device="cuda")
+        met = mem.refuse(at, lambda: m.warm_targets(m.N - 1, block, 8))
+        m.warm_targets(m.N - 1, block, 8)
+        m.set_start_block(m.N - 1, block, 8, 8)
+        got = (block.cpu().numpy(), m.local_spaces(cfg.n_loc).copy())
+        m.close()
+        want = got if want is None else want
+        assert np.any(got[0] != 0.0) and all(np.array_equal(a, b) for a, b in zip(got, want))
+        if not met:
+            break
+        at += 1
+    assert at >= 3
+
+
+def test_going_over_to_the_block_cholesky():
+    """The task lists that a local stage builds when its layers are too ill-conditioned for
+    the inverse form (fibres 25,000 times as stiff as the matrix, on cubes)."""
+    from paper_2211_13893_gb300 import MSGFEM
+    E = (1.62e5, 6.48, 6.48, 2.0, 2.0, 2.0, 0.3, 0.3, 0.3)
+    cfg = replace(get_config("t2"), hx=0.25, hy=0.25, material=E, n_loc=7)
+    ang = element_angles(cfg)
+    mem = Refusing()
+    ref = MSGFEM.from_config(cfg, ang, seed=5, precision=1)
+    want = ref.local_spaces(cfg.n_loc, allow_noconv=True).copy()
+    flops = ref.profile()
+    assert flops["factor_flops"] != flops["factor_flops_inverse"]     # it did go over
+    ref.close()
+    at = 0
+    while True:
+        m = MSGFEM.from_config(cfg, ang, seed=5, precision=1, allocator=(mem.alloc, mem.free))
+        met = mem.refuse(at, lambda: m.local_spaces(cfg.n_loc, allow_noconv=True))
+        assert np.array_equal(m.local_spaces(cfg.n_loc, allow_noconv=True), want)
+        m.close()
+        if not met:
+            break
+        at += 1
+    assert at >= 5
